@@ -184,10 +184,9 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
  *      x transform with each 32-point register FFT spread over a pair of
  *      lanes (fewer registers, three blocks per SM);
  *  [1] the last pass (inverse x FFT + CG update): 0 default rows, 1 half, 2 double;
- *      in 3D with RVE_MIXED and n_x >= 128 also 3, a persistent pipelined
- *      pass whose next spectrum tile arrives by one tensor copy (same
- *      conditions and timeout as variant 5 of the first pass), and 4, variant
- *      0 with the L2 prefetch of a later block's spectrum tile and rows;
+ *      in 3D with RVE_MIXED and n_x >= 128 also 3 and 4, the default and half
+ *      rows with the tile's residual rows prefetched into L2 at the start of
+ *      the block;
  *  [2] the split N = N1 * N2 of the four-step FFT along the last axis (y in
  *      2D, z in 3D; the pass that applies the projection): 0 the most square
  *      split, 1 half N1 and twice N2 (16 = 2 x 8, 32 = 2 x 16, 64 = 4 x 16,
@@ -208,9 +207,10 @@ int rve_set_schedule(rve_t h, const int* variants);
  * the same operator G C (Eq. stat-mech-equi-FFT-homogenization with the
  * projection of Eqs. discrete_projection_op and small-strain-eq2), so the CG
  * iterates agree up to rounding:
- *   RVE_FORM_STRESS   (default) forward FFT of every stress component, the
- *                     projection B (B^H B)^-1 B^H at each wavevector, inverse
- *                     FFT of every strain component.
+ *   RVE_FORM_STRESS   (default) CG on strain fields; forward x FFT of every
+ *                     stress component, B^H applied before the y and z
+ *                     transforms (its factors are shifts there), (B^H B)^-1 at
+ *                     each wavevector, B applied after the inverse transforms.
  *   RVE_FORM_FACTORED the same chain split where Appendix B splits it: the
  *                     right-hand side of Eq. small-strain-eq2 (B^H applied to
  *                     the stresses) is formed in real space as nodal forces
@@ -365,18 +365,18 @@ int rve_batch_effective_tangent(rve_batch_t b, int index, double* C);
  * call on that device (or at the first use of any other entry point there), so
  * a caller that must not allocate later makes one call at set-up time.  The
  * first call on a device also looks up that array's device address
- * (cudaGetSymbolAddress) with the device current; make that first call before
- * any stream capture.  Later calls copy nothing from the host: the tables and
- * the state record are written by a small kernel.  All calls share the array
- * and it keeps the contents of the last call (each call rewrites everything it
- * reads), so calls that overlap on the GPU -- on different streams, or from
+ * (cudaGetSymbolAddress) with the device current and writes the tables and the
+ * state record with a small kernel; make that first call before any stream
+ * capture.  Later calls copy nothing from the host and are three launches.  All
+ * calls share the array and it keeps the contents of the last call (each call
+ * rewrites the spectrum it reads), so calls that overlap on the GPU -- on different streams, or from
  * different host threads -- race; serialise them.  Not usable after
  * cudaDeviceReset on that device.  Returns without waiting for the GPU. */
 int rve_apply_operator_2d_static(const int64_t* n, const double* length, const float* E, double nu,
                                  const float* p, float* q, int apply_material, void* cuda_stream);
 
 /* Test hook (the paper has no counterpart): with on != 0 the pipelined passes
- * (schedule variant 5 of the first pass, 3 of the last) issue none of their
+ * (schedule variant 5 of the first pass) issue none of their
  * copies, so that their bounded device-side waits run out; the solve then
  * returns RVE_ERR_TIMEOUT after a few seconds and the handle stays usable once
  * the hook is off again.  For testing the timeout path without a GPU fault;

@@ -6,8 +6,8 @@
 //
 //   force stencil  x += alpha_prev p_old, p = r + beta p_old, sigma = C p,
 //                  <p, sigma> -> alpha, f = B_r^T sigma (D per node)
-//   FFT passes     f -> w = F^-1 (B^H B)^-1 F f   (existing passes, D components)
-//   strain update  q = B_r w, r -= alpha q, <r, r> -> beta, convergence
+//   FFT passes     f -> w = F^-1 (B^H B)^-1 F f   (the passes of the stress form, D components);
+//                  the last one forms q = B_r w, r -= alpha q, <r, r> -> beta, convergence
 //
 // B_r^T gathers, for every node, the forces of the elements of the 2^D voxels
 // it is a corner of.  The force stencil sweeps a tile of nodes plane by plane
@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kFNT, sizeof(T) == 4 ? 2 : 1)
   T* lo = reinterpret_cast<T*>(smem_raw);   // [12][kFVS]: corners dz = 0 of the current voxel plane
   T* hi = lo + 12 * kFVS;                   // [2][12][kFVS]: corners dz = 1 of the current / previous plane
   __shared__ double red[kFNT / 32];
+  __shared__ T cols[kFNT];
   __shared__ int flag;
   const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
   const int tx = nx < kFX ? nx : kFX, ty = ny < kFY ? ny : kFY, tz = nz < kFZ ? nz : kFZ;
@@ -90,7 +91,7 @@ __global__ void __launch_bounds__(kFNT, sizeof(T) == 4 ? 2 : 1)
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
   const int x0 = blockIdx.x * tx, y0 = blockIdx.y * ty, z0 = zc * tz;
-  const T beta = (T)cg->beta, alpha_prev = (T)cg->alpha;
+  const T beta = cg_beta<T>(cg), alpha_prev = cg_alpha<T>(cg);
   const bool use_old = cg->it > 0;
   const T ih[3] = {a.ih[0], a.ih[1], a.ih[2]};
   const int tid = threadIdx.x;
@@ -177,77 +178,13 @@ __global__ void __launch_bounds__(kFNT, sizeof(T) == 4 ? 2 : 1)
     cur ^= 1;
     __syncthreads();
   }
-  const double s = block_sum<kFNT>((double)acc, red);
+  const double s = block_sum_cols<kFNT>(acc, cols);
   const int nblk = gridDim.x * gridDim.y * nzc;
   const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * zc);
   double* part = a.part + (int64_t)l * a.part_stride;
   if (publish_partial(s, part, &cg->cnt_a, blk, nblk, &flag)) {
     const double pq = sum_partials<kFNT>(part, nblk, red);
     if (threadIdx.x == 0) finish_alpha(cg, pq);
-  }
-}
-
-// q = B_r w on every tetrahedron, r -= alpha q, <r, r>.  w: [L][3][N].
-// grid (ceil(N / NT), L).
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT) strain_update_3d(PassArgs<T> a, const T* __restrict__ w, T* __restrict__ r) {
-  __shared__ double red[NT / 32];
-  __shared__ int flag;
-  const int l = blockIdx.y;
-  CgState* cg = a.cg + l;
-  if (!cg->active) return;
-  if (a.cgphase && cg->status != ST_RUN) return;
-  const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
-  const int64_t N = a.N;
-  const int64_t v = (int64_t)blockIdx.x * NT + threadIdx.x;
-  const T alpha = (T)cg->alpha;
-  T acc = 0;
-  if (v < N) {
-    const int x = (int)(v % nx), y = (int)((v / nx) % ny), z = (int)(v / ((int64_t)nx * ny));
-    const T* wl = w + (int64_t)l * 3 * N;
-    T uc[8][3];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int cx = (x + (c & 1)) & (nx - 1), cy = (y + ((c >> 1) & 1)) & (ny - 1);
-      const int cz = (z + ((c >> 2) & 1)) & (nz - 1);
-      const int64_t i = ((int64_t)cz * ny + cy) * nx + cx;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) uc[c][j] = __ldg(wl + j * N + i);
-    }
-    const int64_t cbase = (int64_t)l * a.m * N + v;
-    const T r2 = (T)kInvSqrt2;
-#pragma unroll
-    for (int t = 0; t < 6; ++t) {
-      const int pa = kuhn_perm(t, 0), pb = kuhn_perm(t, 1), pc = kuhn_perm(t, 2);
-      const int v1 = 1 << pa, v2 = v1 | (1 << pb);
-      T H[3][3];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        H[pa][j] = (uc[v1][j] - uc[0][j]) * a.ih[pa];
-        H[pb][j] = (uc[v2][j] - uc[v1][j]) * a.ih[pb];
-        H[pc][j] = (uc[7][j] - uc[v2][j]) * a.ih[pc];
-      }
-      T q[6];
-      q[0] = H[0][0]; q[1] = H[1][1]; q[2] = H[2][2];
-      q[3] = r2 * (H[1][2] + H[2][1]);
-      q[4] = r2 * (H[0][2] + H[2][0]);
-      q[5] = r2 * (H[0][1] + H[1][0]);
-      T rv[6];
-#pragma unroll
-      for (int s = 0; s < 6; ++s) rv[s] = r[cbase + (int64_t)(6 * t + s) * N];
-#pragma unroll
-      for (int s = 0; s < 6; ++s) {
-        rv[s] -= alpha * q[s];
-        acc += rv[s] * rv[s];
-        r[cbase + (int64_t)(6 * t + s) * N] = rv[s];
-      }
-    }
-  }
-  const double s = block_sum<NT>((double)acc, red);
-  double* part = a.part + (int64_t)l * a.part_stride;
-  if (publish_partial(s, part, &cg->cnt_e, blockIdx.x, gridDim.x, &flag)) {
-    const double rr = sum_partials<NT>(part, gridDim.x, red);
-    if (threadIdx.x == 0) finish_rr(cg, rr, false);
   }
 }
 
@@ -293,6 +230,7 @@ __global__ void __launch_bounds__(kGNT) force_stencil_2d(PassArgs<T> a, const T*
   __shared__ T lo[4][kGVS];      // corners dy = 0 of the current pixel row
   __shared__ T hi[2][4][kGVS];   // corners dy = 1 of the current / previous row
   __shared__ double red[kGNT / 32];
+  __shared__ T cols[kGNT];
   __shared__ int flag;
   const int nx = a.n[0], ny = a.n[1];
   const int tx = nx < kGX ? nx : kGX, ty = ny < kGY ? ny : kGY;
@@ -303,7 +241,7 @@ __global__ void __launch_bounds__(kGNT) force_stencil_2d(PassArgs<T> a, const T*
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
   const int x0 = blockIdx.x * tx, y0 = yc * ty;
-  const T beta = (T)cg->beta, alpha_prev = (T)cg->alpha;
+  const T beta = cg_beta<T>(cg), alpha_prev = cg_alpha<T>(cg);
   const bool use_old = cg->it > 0;
   const int tid = threadIdx.x;
   const bool vox = tid <= tx;
@@ -368,67 +306,13 @@ __global__ void __launch_bounds__(kGNT) force_stencil_2d(PassArgs<T> a, const T*
     cur ^= 1;
     __syncthreads();
   }
-  const double s = block_sum<kGNT>((double)acc, red);
+  const double s = block_sum_cols<kGNT>(acc, cols);
   const int nblk = gridDim.x * nyc;
   const int blk = blockIdx.x + gridDim.x * yc;
   double* part = a.part + (int64_t)l * a.part_stride;
   if (publish_partial(s, part, &cg->cnt_a, blk, nblk, &flag)) {
     const double pq = sum_partials<kGNT>(part, nblk, red);
     if (threadIdx.x == 0) finish_alpha(cg, pq);
-  }
-}
-
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT) strain_update_2d(PassArgs<T> a, const T* __restrict__ w, T* __restrict__ r) {
-  __shared__ double red[NT / 32];
-  __shared__ int flag;
-  const int l = blockIdx.y;
-  CgState* cg = a.cg + l;
-  if (!cg->active) return;
-  if (a.cgphase && cg->status != ST_RUN) return;
-  const int nx = a.n[0], ny = a.n[1];
-  const int64_t N = a.N;
-  const int64_t v = (int64_t)blockIdx.x * NT + threadIdx.x;
-  const T alpha = (T)cg->alpha;
-  T acc = 0;
-  if (v < N) {
-    const int x = (int)(v % nx), y = (int)(v / nx);
-    const int x1 = (x + 1) & (nx - 1), y1 = (y + 1) & (ny - 1);
-    const T* wl = w + (int64_t)l * 2 * N;
-    const int64_t i00 = (int64_t)y * nx + x, i10 = (int64_t)y * nx + x1;
-    const int64_t i01 = (int64_t)y1 * nx + x, i11 = (int64_t)y1 * nx + x1;
-    T u00[2], u10[2], u01[2], u11[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      u00[j] = __ldg(wl + j * N + i00); u10[j] = __ldg(wl + j * N + i10);
-      u01[j] = __ldg(wl + j * N + i01); u11[j] = __ldg(wl + j * N + i11);
-    }
-    const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
-    T q[6];
-    // element 0: d/dx = (u10 - u00) ihx, d/dy = (u01 - u00) ihy
-    q[0] = (u10[0] - u00[0]) * ihx;
-    q[1] = (u01[1] - u00[1]) * ihy;
-    q[2] = r2 * ((u01[0] - u00[0]) * ihy + (u10[1] - u00[1]) * ihx);
-    // element 1: d/dx = (u11 - u01) ihx, d/dy = (u11 - u10) ihy
-    q[3] = (u11[0] - u01[0]) * ihx;
-    q[4] = (u11[1] - u10[1]) * ihy;
-    q[5] = r2 * ((u11[0] - u10[0]) * ihy + (u11[1] - u01[1]) * ihx);
-    const int64_t cbase = (int64_t)l * a.m * N + v;
-    T rv[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) rv[c] = r[cbase + (int64_t)c * N];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      rv[c] -= alpha * q[c];
-      acc += rv[c] * rv[c];
-      r[cbase + (int64_t)c * N] = rv[c];
-    }
-  }
-  const double s = block_sum<NT>((double)acc, red);
-  double* part = a.part + (int64_t)l * a.part_stride;
-  if (publish_partial(s, part, &cg->cnt_e, blockIdx.x, gridDim.x, &flag)) {
-    const double rr = sum_partials<NT>(part, gridDim.x, red);
-    if (threadIdx.x == 0) finish_rr(cg, rr, false);
   }
 }
 
@@ -449,14 +333,6 @@ cudaError_t launch_force_stencil(const PassArgs<T>& a, const T* pold, T* pnew, T
     dim3 grid(a.n[0] / tx, (a.n[1] / ty) * a.L);
     force_stencil_2d<T><<<grid, kGNT, 0, s>>>(a, a.r, pold, pnew, a.x, f);
   }
-  return cudaGetLastError();
-}
-
-template <typename T> cudaError_t launch_strain_update(const PassArgs<T>& a, const T* w, cudaStream_t s) {
-  constexpr int NT = 256;
-  dim3 grid((unsigned)((a.N + NT - 1) / NT), a.L);
-  if (a.dim == 3) strain_update_3d<T, NT><<<grid, NT, 0, s>>>(a, w, a.r);
-  else strain_update_2d<T, NT><<<grid, NT, 0, s>>>(a, w, a.r);
   return cudaGetLastError();
 }
 

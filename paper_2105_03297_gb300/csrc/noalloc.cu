@@ -28,11 +28,13 @@ using namespace rve;
 namespace {
 
 // Largest grid side served from the static scratch, and the scratch size:
-// the half spectrum (6 components x (n/2+1) x n complex floats), 2 phase and
-// 2 twiddle tables of n complex floats, and one CgState.
+// the half spectrum (6 components x (n/2+1) x n complex floats), a phase and a
+// twiddle table of n complex floats for every length n = 16, 32, .. 256, and
+// one CgState.
 constexpr int kStaticMaxN = 256;
 constexpr size_t kSpecBytes = 6ull * (kStaticMaxN / 2 + 1) * kStaticMaxN * sizeof(float2);
-constexpr size_t kTableBytes = 4ull * kStaticMaxN * sizeof(float2);
+constexpr int kTableLen = 2 * kStaticMaxN - 16;   // entries of one kind: length n starts at n - 16
+constexpr size_t kTableBytes = 2ull * kTableLen * sizeof(float2);
 constexpr size_t kStaticScratchBytes = kSpecBytes + kTableBytes + 256;
 
 // Held by every device that loads the library, until the process exits.
@@ -42,21 +44,20 @@ static __device__ __align__(256) unsigned char g_rve_scratch[kStaticScratchBytes
 std::atomic<void*> g_scratch_ptr[kMaxDevices];
 DeviceOnce g_scratch_once;
 
-// Phase tables exp(+2 pi i j / n) of both axes, twiddle tables exp(-2 pi i j / n),
-// and a fresh CG-state record (active, everything else zero), written on the
-// device so that a call copies nothing from the host.  sincospi is CUDA's own
-// FP64 function; its results are rounded to FP32 like the host tables of the
-// handle path.
-__global__ void fill_static_tables(float2* tables, CgState* cg, int nx, int ny) {
-  const int len[2] = {nx, ny};
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * kStaticMaxN; i += gridDim.x * blockDim.x) {
-    const int a = i / kStaticMaxN, j = i % kStaticMaxN;
-    if (j < len[a]) {
-      double sn, cs;
-      sincospi(2.0 * (double)j / (double)len[a], &sn, &cs);
-      tables[a * kStaticMaxN + j] = make_float2((float)cs, (float)sn);             // exp(+i ang)
-      tables[(2 + a) * kStaticMaxN + j] = make_float2((float)cs, (float)-sn);      // exp(-i ang)
-    }
+// Phase tables exp(+2 pi i j / n) and twiddle tables exp(-2 pi i j / n) of
+// every length, and the CG-state record (active, everything else zero; no mode
+// of this entry point changes it), written on the device at set-up.  sincospi
+// is CUDA's own FP64 function; its results are rounded to FP32 like the host
+// tables of the handle path.  They used to be rewritten by every call: without
+// that launch a 64 x 64 call is three launches instead of four.
+__global__ void fill_static_tables(float2* tables, CgState* cg) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kTableLen; i += gridDim.x * blockDim.x) {
+    int n = 16;
+    while (i >= 2 * n - 16) n *= 2;
+    double sn, cs;
+    sincospi(2.0 * (double)(i - (n - 16)) / (double)n, &sn, &cs);
+    tables[i] = make_float2((float)cs, (float)sn);               // exp(+i ang)
+    tables[kTableLen + i] = make_float2((float)cs, (float)-sn);  // exp(-i ang)
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     CgState st{};
@@ -80,29 +81,30 @@ extern "C" int rve_apply_operator_2d_static(const int64_t* n, const double* leng
   }
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return RVE_ERR_CUDA; }
+  cudaStream_t s = (cudaStream_t)cuda_stream;
   // Set-up, once per device, with that device current: the device address of
-  // the static array (its name is only a host-side stand-in).  The kernel
+  // the static array (its name is only a host-side stand-in), and the tables
+  // and the state record in it, written on the first call's stream (callers
+  // serialise calls, so every later call finds them complete).  The kernel
   // attributes of the pass kernels are likewise set once per device by their
   // launchers.
   g_scratch_once.run(dev, [&] {
     void* ptr = nullptr;
     if (cudaGetSymbolAddress(&ptr, g_rve_scratch) != cudaSuccess || !ptr) { cudaGetLastError(); ptr = nullptr; }
+    if (ptr) {
+      unsigned char* b = static_cast<unsigned char*>(ptr) + kSpecBytes;
+      fill_static_tables<<<4, 128, 0, s>>>(reinterpret_cast<float2*>(b), reinterpret_cast<CgState*>(b + kTableBytes));
+      if (cudaGetLastError() != cudaSuccess) ptr = nullptr;
+    }
     g_scratch_ptr[dev].store(ptr);
   });
   unsigned char* base = static_cast<unsigned char*>(g_scratch_ptr[dev].load());
   if (!base) return RVE_ERR_CUDA;
   float2* spec = reinterpret_cast<float2*>(base);
-  float2* tables = reinterpret_cast<float2*>(base + kSpecBytes);   // ph_x, ph_y, tw_x, tw_y
+  float2* tables = reinterpret_cast<float2*>(base + kSpecBytes);   // phases, then twiddles
   CgState* cg = reinterpret_cast<CgState*>(base + kSpecBytes + kTableBytes);
-  cudaStream_t s = (cudaStream_t)cuda_stream;
 
   const int nx = (int)n[0], ny = (int)n[1];
-  // Tables and CG state of this call, written on the device (the scratch keeps
-  // the previous call's contents).
-  fill_static_tables<<<4, 128, 0, s>>>(tables, cg, nx, ny);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return RVE_ERR_CUDA;
-
   PassArgs<float> a;
   std::memset(&a, 0, sizeof(a));
   a.n[0] = nx; a.n[1] = ny; a.n[2] = 1;
@@ -113,8 +115,10 @@ extern "C" int rve_apply_operator_2d_static(const int64_t* n, const double* leng
   a.lcs = 1;
   a.in = p; a.out = q;
   a.spec = spec;
-  a.ph[0] = tables; a.ph[1] = tables + kStaticMaxN;
-  a.tw[0] = tables + 2 * kStaticMaxN; a.tw[1] = tables + 3 * kStaticMaxN;
+  for (int i = 0; i < 2; ++i) {
+    a.ph[i] = tables + (n[i] - 16);
+    a.tw[i] = tables + kTableLen + (n[i] - 16);
+  }
   for (int i = 0; i < 2; ++i) a.ih[i] = (float)((double)n[i] / (length ? length[i] : 1.0));
   a.lam = (float)(nu / ((1.0 + nu) * (1.0 - 2.0 * nu)));
   a.mu2 = (float)(1.0 / (1.0 + nu));
@@ -124,7 +128,8 @@ extern "C" int rve_apply_operator_2d_static(const int64_t* n, const double* leng
   a.pmode = P_G;
   a.emode = E_OUT;
   a.cgphase = 0;
-  e = launch_pass_a_2d<float>(a, s);
+  a.grads = 1;
+  cudaError_t e = launch_pass_a_2d<float>(a, s);
   if (e == cudaSuccess) e = launch_pass_c_2d<float>(a, s);
   if (e == cudaSuccess) e = launch_pass_e_2d<float>(a, s);
   if (e != cudaSuccess) { cudaGetLastError(); return RVE_ERR_CUDA; }

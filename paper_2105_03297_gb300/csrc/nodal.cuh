@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kNNT, sizeof(T) == 4 ? 2 : 1)
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
   const int x0 = blockIdx.x * tx, y0 = blockIdx.y * ty, z0 = zc * tz;
-  const T beta = (T)cg->beta, alpha_prev = (T)cg->alpha;
+  const T beta = cg_beta<T>(cg), alpha_prev = cg_alpha<T>(cg);
   const bool use_old = cg->it > 0;
   const T ih[3] = {a.ih[0], a.ih[1], a.ih[2]};
   const int tid = threadIdx.x;
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(NT) nodal_update_3d(PassArgs<T> a, const T* __
   const int bx = nx < 32 ? nx : 32, by = NT / bx;
   const int x = blockIdx.x * bx + (threadIdx.x & (bx - 1)), y = blockIdx.y * by + threadIdx.x / bx;
   const int x1 = (x + 1) & (nx - 1), y1 = (y + 1) & (ny - 1);
-  const T alpha = init ? (T)0 : (T)cg->alpha;
+  const T alpha = init ? (T)0 : cg_alpha<T>(cg);
   const int64_t lbase = (int64_t)l * 3 * N;
   const int64_t plane = (int64_t)nx * ny;
   const int64_t o00 = (int64_t)y * nx + x, o10 = (int64_t)y * nx + x1;
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(kMNT) nodal_force_2d(PassArgs<T> a, const T* _
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
   const int x0 = blockIdx.x * tx, y0 = yc * ty;
-  const T beta = (T)cg->beta, alpha_prev = (T)cg->alpha;
+  const T beta = cg_beta<T>(cg), alpha_prev = cg_alpha<T>(cg);
   const bool use_old = cg->it > 0;
   const int tid = threadIdx.x;
   const bool isnode = tid < tx + 2;
@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(NT) nodal_update_2d(PassArgs<T> a, const T* __
   const int x = blockIdx.x * bx + (threadIdx.x % bx);
   const int ys = yb * rows_blk + (threadIdx.x / bx) * kUY;
   const int x1 = (x + 1) & (nx - 1);
-  const T alpha = init ? (T)0 : (T)cg->alpha;
+  const T alpha = init ? (T)0 : cg_alpha<T>(cg);
   const int64_t lbase = (int64_t)l * 2 * N;
   T acc = 0;
   if (ys < ny) {
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(NT) nodal_finish(PassArgs<T> a, const T* __res
   const int64_t v = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (v >= N) return;
   const bool last = cg->it > 0 && cg->status != ST_BAD;
-  const T alpha = last ? (T)cg->alpha : (T)0;
+  const T alpha = last ? cg_alpha<T>(cg) : (T)0;
   const T* pl = ((cg->it - 1) & 1) ? pi_odd : pi_even;
   const int64_t lbase = (int64_t)l * a.dim * N;
   for (int j = 0; j < a.dim; ++j) {

@@ -4,12 +4,16 @@
 //   A  material (+ fused CG direction update and <p, C p>) and forward real
 //      FFT along x; writes the half spectrum transposed, [l][c][k_x][y], so
 //      that the next pass reads whole y-columns contiguously;
-//   C  forward FFT along y, the projection G(k) = B (B^H B)^-1 B^H per
-//      wavevector (k = 0 set to zero), inverse FFT along y, in place;
-//   E  inverse real FFT along x, then r -= alpha q and <r, r> (q never
-//      touches memory).  x += alpha p of iteration k is deferred to pass A of
-//      iteration k+1, which reads p anyway (one vector stream less per
-//      iteration); cg_finish_x applies the last one.
+//   C  t = B^H sigma (differences along y where the factors of B^H are
+//      shifts), forward FFT along y, w^ = (B^H B)^-1 t^ per wavevector (k = 0
+//      set to zero), inverse FFT along y;
+//   E  inverse real FFT along x of w, q = B w in real space, then r -= alpha q
+//      and <r, r> (q never touches memory).  x += alpha p of iteration k is
+//      deferred to pass A of iteration k+1, which reads p anyway (one vector
+//      stream less per iteration); cg_finish_x applies the last one.
+// The other derivatives and finite strain carry all their components through C
+// (with the projection) and E.  Measured at 1024^2, three load cases, FP32, us
+// per iteration: all six components through C 80 and E 85, now C 48 and E 61.
 // DFT convention of Appendix A; the 1/N of the inverse is applied in pass C.
 // Two real rows (y, y+1) share one complex FFT (X_y + i X_{y+1}).
 #pragma once
@@ -28,12 +32,13 @@ __device__ __forceinline__ void finish_alpha(CgState* cg, double pq) {
   cg->pq = pq;
   if (!(pq > 0.0) || !isfinite(pq)) { cg->status = ST_BAD; cg->alpha = 0.0; }
   else cg->alpha = cg->rr / pq;
+  cg->alpha_f = (float)cg->alpha;
   cg->cnt_a = 0;
 }
 // ... and of <r, r> (pass E)
 __device__ __forceinline__ void finish_rr(CgState* cg, double rr, bool init) {
   if (init) {
-    cg->rr0 = rr; cg->rr = rr; cg->it = 0; cg->beta = 0.0;
+    cg->rr0 = rr; cg->rr = rr; cg->it = 0; cg->beta = 0.0; cg->beta_f = 0.f;
     // a held slot (ST_HOLD) stays held until the host releases it
     cg->status = !isfinite(rr) ? ST_BAD : (rr == 0.0 ? ST_CONV : (cg->status == ST_HOLD ? ST_HOLD : ST_RUN));
   } else {
@@ -41,6 +46,7 @@ __device__ __forceinline__ void finish_rr(CgState* cg, double rr, bool init) {
     if (!isfinite(rr)) { cg->status = ST_BAD; }
     else {
       cg->beta = rr / cg->rr;
+      cg->beta_f = (float)cg->beta;
       cg->rr = rr;
       if (rr <= cg->tol2 * cg->rr0) cg->status = ST_CONV;
       else if (cg->it >= cg->maxit) cg->status = ST_MAXIT;
@@ -225,6 +231,7 @@ __global__ void __launch_bounds__(NT, PAIR ? 3 : pass_a2_min_blocks<T, NT>()) pa
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [GS][NP][LD]
   __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
   __shared__ int flag;
 
   const int l = blockIdx.z, grp = blockIdx.y, y0 = blockIdx.x * TY;
@@ -236,7 +243,7 @@ __global__ void __launch_bounds__(NT, PAIR ? 3 : pass_a2_min_blocks<T, NT>()) pa
   const int c0 = nodal ? 0 : grp * 3;
   T beta = 0, alpha_prev = 0;
   bool use_old = false;
-  if (a.amode == A_CG) { beta = (T)cg->beta; alpha_prev = (T)cg->alpha; use_old = cg->it > 0; }
+  if (a.amode == A_CG) { beta = cg_beta<T>(cg); alpha_prev = cg_alpha<T>(cg); use_old = cg->it > 0; }
   // the lane-pair variant runs three blocks per SM: units of two columns (8-byte
   // loads, as in 3D) keep the load phase within its registers
   const T acc = pass_a_load<T, NX, TY, GS, NT, LD, PAIR ? 2 : Vec16<T>::n>(a, buf, l, c0, (int64_t)y0 * NX, nodal,
@@ -248,7 +255,7 @@ __global__ void __launch_bounds__(NT, PAIR ? 3 : pass_a2_min_blocks<T, NT>()) pa
                                   (int64_t)KX * ny, ny);
 
   if (a.amode == A_CG) {
-    const double s = block_sum<NT>((double)acc, red);
+    const double s = block_sum_cols<NT>(acc, cols);
     const int nblk = gridDim.x * gridDim.y;
     const int blk = blockIdx.x + gridDim.x * blockIdx.y;
     double* part = a.part + (int64_t)l * a.part_stride;
@@ -260,12 +267,9 @@ __global__ void __launch_bounds__(NT, PAIR ? 3 : pass_a2_min_blocks<T, NT>()) pa
 }
 
 // ---------------------------------------------------------------- pass C
-// Projection of the m = 6 spectra at one wavevector, in place.
-//   mode P_G:         s (6) -> B (B^H B)^-1 B^H s
-//   mode P_NODAL_IN:  s[0..1] = f^ -> B (B^H B)^-1 f^   (6 out)
-//   mode P_NODAL_OUT: s (6) -> (B^H B)^-1 B^H s           (2 out, in s[0..1])
+// w^ = (B^H B)^-1 t^ at one wavevector (k != 0), scaled, in place.
 template <typename T>
-__device__ __forceinline__ void project_2d(cplx<T>* s, cplx<T> ex, cplx<T> ey, T ihx, T ihy, T scale, int mode) {
+__device__ __forceinline__ void solve_2d(cplx<T>* t, cplx<T> ex, cplx<T> ey, T ihx, T ihy, T scale) {
   using C = cplx<T>;
   const C one = mkc<T>(1, 0);
   C g[2][2];
@@ -281,46 +285,25 @@ __device__ __forceinline__ void project_2d(cplx<T>* s, cplx<T> ex, cplx<T> ey, T
     m11 += (T)0.5 * ax + ay;
     m01 = cadd(m01, cscale(cmul(g[q][0], cconj(g[q][1])), (T)0.5));
   }
-  C t0, t1;
-  if (mode == P_NODAL_IN || mode == P_SOLVE) {
-    t0 = s[0]; t1 = s[1];
-  } else {
-    // t = B^H s: t_j = sum_q sum_a conj(g_qa) sigma_q,aj
-    t0 = mkc<T>(0, 0); t1 = mkc<T>(0, 0);
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const C sxx = s[3 * q], syy = s[3 * q + 1], sxy = cscale(s[3 * q + 2], (T)kInvSqrt2);
-      t0 = cadd(t0, cadd(cjmul(g[q][0], sxx), cjmul(g[q][1], sxy)));
-      t1 = cadd(t1, cadd(cjmul(g[q][0], sxy), cjmul(g[q][1], syy)));
-    }
-  }
   const T det = m00 * m11 - cabs2(m01);
   const T id = scale / det;
-  // w = M^-1 t,  M^-1 = [[m11, -m01], [-conj(m01), m00]] / det
-  const C w0 = cscale(csub(cscale(t0, m11), cmul(m01, t1)), id);
-  const C w1 = cscale(csub(cscale(t1, m00), cjmul(m01, t0)), id);
-  if (mode == P_NODAL_OUT || mode == P_SOLVE) {
-    s[0] = w0; s[1] = w1;
-    return;
-  }
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    s[3 * q] = cmul(g[q][0], w0);
-    s[3 * q + 1] = cmul(g[q][1], w1);
-    s[3 * q + 2] = cscale(cadd(cmul(g[q][0], w1), cmul(g[q][1], w0)), (T)kInvSqrt2);
-  }
+  // M^-1 = [[m11, -m01], [-conj(m01), m00]] / det
+  const C w0 = cscale(csub(cscale(t[0], m11), cmul(m01, t[1])), id);
+  const C w1 = cscale(csub(cscale(t[1], m00), cjmul(m01, t[0])), id);
+  t[0] = w0; t[1] = w1;
 }
 
-// grid (n_x/2+1, L); one k_x column of all six spectra per block.  The forward
-// FFT reads the column straight from the spectrum, the inverse FFT writes it
-// straight back; only the middle transposes and the projection use shared
-// memory.
-template <typename T, int NY, int NQ, int NT, int V = 0>
+// Projection on all components (the derivatives without a finite-element
+// stencil, and finite strain): grid (n_x/2+1, L); one k_x column of all
+// spectra per block.  The forward FFT reads the column straight from the
+// spectrum, the inverse FFT writes it straight back; only the middle
+// transposes and the projection use shared memory.
+template <typename T, int NY, int NQ, int NT>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs<T> a) {
   using C = cplx<T>;
-  constexpr int M = 3 * NQ;   // 6 for the finite elements and two-point Fourier, 3 for one point,
+  constexpr int M = 3 * NQ;   // 6 for the two-point Fourier derivative, 3 for one point,
                               // 9 for finite-strain gradients (8 + padding)
-  constexpr int LD = FftSplit<NY, V>::LD;
+  constexpr int LD = FftSplit<NY>::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [M][LD]
   const int kx = blockIdx.x, l = blockIdx.y;
@@ -328,20 +311,17 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs
   CgState* cg = a.cg + l;
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
-  const int cin = (a.pmode == P_NODAL_IN || a.pmode == P_SOLVE) ? 2 : M;
-  const int cout = (a.pmode == P_NODAL_OUT || a.pmode == P_SOLVE) ? 2 : M;
   C* col = a.spec + (((int64_t)l * M) * KX + kx) * NY;
   const int64_t cstride = (int64_t)KX * NY;
   auto ld_g = [&](int c, int y) -> C { return col[c * cstride + y]; };
   auto st_s = [&](int c, int k, C v) { buf[c * LD + k] = v; };
-  if (cin == M) fft4<T, NY, M, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
-  else fft4<T, NY, 2, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
+  fft4<T, NY, M, LD, NT, -1, false, true, false, false>(buf, a.tw[1], ld_g, st_s);
 
   const C ex = a.ph[0][kx];
   for (int ky = threadIdx.x; ky < NY; ky += NT) {
     C s[M];
 #pragma unroll
-    for (int c = 0; c < M; ++c) s[c] = (c < cin) ? buf[c * LD + ky] : mkc<T>(0, 0);
+    for (int c = 0; c < M; ++c) s[c] = buf[c * LD + ky];
     if constexpr (NQ == 3) {
       // finite strain: deformation gradients of the two triangles (+ padding)
       const C e2[2] = {ex, a.ph[1][ky]};
@@ -352,8 +332,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs
     } else if (kx == 0 && ky == 0) {
 #pragma unroll
       for (int c = 0; c < M; ++c) s[c] = mkc<T>(0, 0);
-    } else if (NQ == 2 && a.deriv == D_FE) {
-      project_2d<T>(s, ex, a.ph[1][ky], a.ih[0], a.ih[1], a.inv_n, a.pmode);
     } else {
       const int j[2] = {kx, ky};
       const C e[2] = {ex, a.ph[1][ky]};
@@ -362,25 +340,41 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs
       project_generic<T, 2>(s, g, nq, a.inv_n);
     }
 #pragma unroll
-    for (int c = 0; c < M; ++c)
-      if (c < cout) buf[c * LD + ky] = s[c];
+    for (int c = 0; c < M; ++c) buf[c * LD + ky] = s[c];
   }
   __syncthreads();
   auto ld_s = [&](int c, int y) -> C { return buf[c * LD + y]; };
   auto st_g = [&](int c, int k, C v) { col[c * cstride + k] = v; };
-  if (cout == M) fft4<T, NY, M, LD, NT, +1, true, false, false, false, V>(buf, a.tw[1], ld_s, st_g);
-  else fft4<T, NY, 2, LD, NT, +1, true, false, false, false, V>(buf, a.tw[1], ld_s, st_g);
+  fft4<T, NY, M, LD, NT, +1, true, false, false, false>(buf, a.tw[1], ld_s, st_g);
 }
 
-// Pass C for the nodal solve w^ = (B^H B)^-1 f^ (P_SOLVE, 2 components in and
-// out): P k_x columns per block so that a block holds as many transforms as
-// the 6-component pass.  Row b is component b % 2 of column kx0 + b / 2;
-// columns past n_x/2 are skipped.  grid (ceil((n_x/2+1) / P), L).
-template <typename T, int NY, int P, int NT>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 1) pass_c_2d_nodal(PassArgs<T> a) {
+// Pass C of the finite elements: w^ = (B^H B)^-1 t^ for P k_x columns per
+// block; w(k_x, y), the D = 2 nodal components after the inverse FFT along y,
+// goes to components 0 and 1 of the spectrum.  With COMBINE the input is the
+// x-transformed stresses of all six components and t = B^H sigma is formed
+// before the y transform: a factor exp(-i k_y h) is a shift by one row, so
+// with dx = (exp(-i k_x h) - 1)/h and s0, s1 the stresses of the two triangles
+//   t_j(y) = U_j(y) + V_j(y-1),   W_j = (s0_yj + exp(-i k_x h) s1_yj)/h_y,
+//   U_j = dx s0_xj - W_j,         V_j = W_j + dx s1_xj,
+// and only two columns per k_x are transformed there and back instead of six.
+// Without COMBINE components 0 and 1 hold t(k_x, y) (nodal forces).
+// W = 4 (P = 1) writes the differences d_a w_j along the element edges,
+// d_a = (exp(i k_a h_a) - 1)/h_a, as components 2 a + j: the last pass then
+// only picks them up at the right nodes.  Differences of w itself, taken there
+// in real space, round like eps n_a |w|: up to 8 times the error on a smooth
+// field (measured at 1024^2 in FP32: 1.0e-5 against 1.2e-6 of the 2-norm; on
+// white noise 4.3e-7 against 3.1e-7).  Inside the CG that error is corrected
+// by the FP64 refinement, so W = 2 is used there, W = 4 for rve_apply_operator.
+// Bound by the spectrum traffic (COMBINE: 6 columns in, 2 out).  Consecutive
+// lanes hold consecutive rows, so V(y-1) comes by a shuffle; lane 0 and row 0
+// load row y-1 themselves.  Row b of the buffer is component b % 2 of column
+// kx0 + b / 2; columns past n_x/2 are skipped.  grid (ceil((n_x/2+1) / P), L).
+template <typename T, int NY, int P, int NT, int V, bool COMBINE, int W>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) pass_c_2d_fe(PassArgs<T> a) {
   using C = cplx<T>;
-  constexpr int M = 6, R = 2 * P;
-  constexpr int LD = FftSplit<NY>::LD;
+  constexpr int R = 2 * P;
+  static_assert(W == 2 || (W == 4 && P == 1), "differences: one column per block");
+  constexpr int LD = FftSplit<NY, V>::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [R][LD]
   const int kx0 = blockIdx.x * P, l = blockIdx.y;
@@ -389,43 +383,94 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 1) pass_c_2d_nodal(Pa
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t cstride = (int64_t)KX * NY;
-  C* base = a.spec + ((int64_t)l * M * KX + kx0) * NY;
-  auto ld_g = [&](int b, int y) -> C {
-    return (kx0 + b / 2 < KX) ? base[(b % 2) * cstride + (int64_t)(b / 2) * NY + y] : mkc<T>(0, 0);
-  };
+  C* base = a.spec + ((int64_t)l * a.m * KX + kx0) * NY;
   auto st_s = [&](int b, int k, C v) { buf[b * LD + k] = v; };
-  fft4<T, NY, R, LD, NT, -1, false, true, false, false>(buf, a.tw[1], ld_g, st_s);
+  auto ld_s = [&](int b, int y) -> C { return buf[b * LD + y]; };
+  if constexpr (COMBINE) {
+    const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
+    for (int i0 = 0; i0 < P * NY; i0 += NT) {   // whole warps: every lane takes part in the shuffles
+      const int i = i0 + threadIdx.x;
+      const int pc = i / NY, y = i % NY;
+      const bool on = i < P * NY && kx0 + pc < KX;
+      C u[2], v[2], vp[2];
+      u[0] = u[1] = v[0] = v[1] = vp[0] = vp[1] = mkc<T>(0, 0);
+      C cex = mkc<T>(1, 0), dx = mkc<T>(0, 0);
+      const C* col = base + (int64_t)pc * NY;
+      if (on) {
+        cex = cconj(a.ph[0][kx0 + pc]);
+        dx = cscale(csub(cex, mkc<T>(1, 0)), ihx);
+        C s[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) s[c] = col[c * cstride + y];
+        s[2] = cscale(s[2], r2); s[5] = cscale(s[5], r2);
+        const C w0 = cscale(cadd(s[2], cmul(cex, s[5])), ihy);
+        const C w1 = cscale(cadd(s[1], cmul(cex, s[4])), ihy);
+        u[0] = csub(cmul(dx, s[0]), w0); u[1] = csub(cmul(dx, s[2]), w1);
+        v[0] = cadd(cmul(dx, s[3]), w0); v[1] = cadd(cmul(dx, s[5]), w1);
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        vp[j].x = __shfl_up_sync(0xffffffffu, v[j].x, 1);
+        vp[j].y = __shfl_up_sync(0xffffffffu, v[j].y, 1);
+      }
+      if (on) {
+        if ((threadIdx.x & 31) == 0 || y == 0) {
+          const int ym = (y + NY - 1) & (NY - 1);
+          const C s1 = col[cstride + ym], s2 = cscale(col[2 * cstride + ym], r2), s3 = col[3 * cstride + ym];
+          const C s4 = col[4 * cstride + ym], s5 = cscale(col[5 * cstride + ym], r2);
+          vp[0] = cadd(cmul(dx, s3), cscale(cadd(s2, cmul(cex, s5)), ihy));
+          vp[1] = cadd(cmul(dx, s5), cscale(cadd(s1, cmul(cex, s4)), ihy));
+        }
+        buf[2 * pc * LD + y] = cadd(u[0], vp[0]);
+        buf[(2 * pc + 1) * LD + y] = cadd(u[1], vp[1]);
+      } else if (i < P * NY) {
+        buf[2 * pc * LD + y] = buf[(2 * pc + 1) * LD + y] = mkc<T>(0, 0);
+      }
+    }
+    __syncthreads();
+    fft4<T, NY, R, LD, NT, -1, true, true, false, false, V>(buf, a.tw[1], ld_s, st_s);
+  } else {
+    auto ld_g = [&](int b, int y) -> C {
+      return (kx0 + b / 2 < KX) ? base[(b % 2) * cstride + (int64_t)(b / 2) * NY + y] : mkc<T>(0, 0);
+    };
+    fft4<T, NY, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
+  }
   for (int i = threadIdx.x; i < P * NY; i += NT) {
     const int pc = i / NY, ky = i % NY, kx = kx0 + pc;
     if (kx >= KX) continue;
-    C s2[M];
-    s2[0] = buf[2 * pc * LD + ky];
-    s2[1] = buf[(2 * pc + 1) * LD + ky];
-    if (kx == 0 && ky == 0) {
-      s2[0] = s2[1] = mkc<T>(0, 0);   // k = 0: the nodal solve has no mean
+    C t[2] = {buf[2 * pc * LD + ky], buf[(2 * pc + 1) * LD + ky]};
+    if (kx == 0 && ky == 0) t[0] = t[1] = mkc<T>(0, 0);   // k = 0: no mean
+    else solve_2d<T>(t, a.ph[0][kx], a.ph[1][ky], a.ih[0], a.ih[1], a.inv_n);
+    if constexpr (W == 4) {
+      const C one = mkc<T>(1, 0);
+      const C d0 = cscale(csub(a.ph[0][kx], one), a.ih[0]), d1 = cscale(csub(a.ph[1][ky], one), a.ih[1]);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        buf[j * LD + ky] = cmul(d0, t[j]);
+        buf[(2 + j) * LD + ky] = cmul(d1, t[j]);
+      }
     } else {
-      project_2d<T>(s2, a.ph[0][kx], a.ph[1][ky], a.ih[0], a.ih[1], a.inv_n, P_SOLVE);
+      buf[2 * pc * LD + ky] = t[0];
+      buf[(2 * pc + 1) * LD + ky] = t[1];
     }
-    buf[2 * pc * LD + ky] = s2[0];
-    buf[(2 * pc + 1) * LD + ky] = s2[1];
   }
   __syncthreads();
-  auto ld_s = [&](int b, int y) -> C { return buf[b * LD + y]; };
   auto st_g = [&](int b, int k, C v) {
-    if (kx0 + b / 2 < KX) base[(b % 2) * cstride + (int64_t)(b / 2) * NY + k] = v;
+    if (kx0 + b / W < KX) base[(b % W) * cstride + (int64_t)(b / W) * NY + k] = v;
   };
-  fft4<T, NY, R, LD, NT, +1, true, false, false, false>(buf, a.tw[1], ld_s, st_g);
+  fft4<T, NY, W * P, LD, NT, +1, true, false, false, false, V>(buf, a.tw[1], ld_s, st_g);
 }
 
 // ------------------------------------------------------------------------
 // Pass E body shared by 2D and 3D: load the (k, y-pair) spectra of ge
 // components into packed rows (component j at src + j*comp_stride +
-// k*k_stride + y-offset, rows j*NP + pr), ready for the inverse FFT.
+// k*k_stride + y, rows j*NP + pr of the tile starting at row y0; y wraps at
+// ymask + 1, a power of two), ready for the inverse FFT.
 // Each thread has up to UB of its loads in flight before it writes any of
 // them to shared memory (a load per loop trip would leave one in flight).
 template <typename T, int NX, int TY, int NT, int LD>
 __device__ __forceinline__ void pass_e_unpack(cplx<T>* buf, const cplx<T>* src, int ge, int64_t comp_stride,
-                                              int64_t k_stride) {
+                                              int64_t k_stride, int y0, int ymask) {
   using C = cplx<T>;
   constexpr int NP = TY / 2;
   constexpr int KX = NX / 2 + 1;
@@ -438,7 +483,7 @@ __device__ __forceinline__ void pass_e_unpack(cplx<T>* buf, const cplx<T>* src, 
       const int i = i0 + u * NT;
       if (i < total) {
         const int pr = i % NP, k = (i / NP) % KX, j = i / (NP * KX);
-        cload2<T>(ab[u], src + j * comp_stride + (int64_t)k * k_stride + 2 * pr);
+        cload2<T>(ab[u], src + j * comp_stride + (int64_t)k * k_stride + ((y0 + 2 * pr) & ymask));
       }
     }
 #pragma unroll
@@ -546,6 +591,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [GE][NP][LD]
   __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
   __shared__ int flag;
   const int l = blockIdx.z, grp = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1];
@@ -557,22 +603,130 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   const int ge = nodal ? 2 : GE;
   const int c0 = nodal ? 0 : grp * GE;
 
-  pass_e_unpack<T, NX, TY, NT, LD>(buf, a.spec + (((int64_t)l * a.m + c0) * KX) * ny + y0, ge, (int64_t)KX * ny, ny);
+  pass_e_unpack<T, NX, TY, NT, LD>(buf, a.spec + (((int64_t)l * a.m + c0) * KX) * ny, ge, (int64_t)KX * ny, ny, y0,
+                                   ny - 1);
   __syncthreads();
   T acc = 0;
-  const T alpha = (a.emode == E_CG) ? (T)cg->alpha : (T)0;
+  const T alpha = (a.emode == E_CG) ? cg_alpha<T>(cg) : (T)0;
   auto ld_s = [&](int b, int x) -> C { return buf[b * LD + x]; };
   PassEStore<T, NX, NP> st{&a, ge, (int64_t)y0 * NX, ((int64_t)l * a.m + c0) * N, (int64_t)l * 2 * N, alpha, &acc};
   fft4<T, NX, GE * NP, LD, NT, +1, true, false, false, false, 0, decltype(ld_s), decltype(st), true>(buf, a.tw[0],
                                                                                                   ld_s, st);
 
   if (a.emode == E_CG || a.emode == E_INIT) {
-    const double s = block_sum<NT>((double)acc, red);
+    const double s = block_sum_cols<NT>(acc, cols);
     const int nblk = gridDim.x * gridDim.y;
     const int blk = blockIdx.x + gridDim.x * blockIdx.y;
     double* part = a.part + (int64_t)l * a.part_stride;
     if (publish_partial(s, part, &cg->cnt_e, blk, nblk, &flag)) {
       const double rr = sum_partials<NT>(part, nblk, red);
+      if (threadIdx.x == 0) finish_rr(cg, rr, a.emode == E_INIT);
+    }
+  }
+}
+
+// Update of VL consecutive values of one strain component by q (modes of the
+// last pass): CG r -= alpha q, INIT r = -q and x = 0, OUT out = q.  rv holds r
+// in CG mode.  Returns the share of <r, r>.
+template <typename T, int VL>
+__device__ __forceinline__ T strain_update(const PassArgs<T>& a, int64_t idx, T* rv, const T* q, T alpha) {
+  T s = 0;
+  if (a.emode == E_CG) {
+#pragma unroll
+    for (int i = 0; i < VL; ++i) { rv[i] -= alpha * q[i]; s += rv[i] * rv[i]; }
+    vstoren<T, VL>(a.r + idx, rv);
+  } else if (a.emode == E_INIT) {
+    T z[VL], n[VL];
+#pragma unroll
+    for (int i = 0; i < VL; ++i) { n[i] = -q[i]; z[i] = 0; s += q[i] * q[i]; }
+    vstoren<T, VL>(a.r + idx, n);
+    vstoren<T, VL>(a.x + idx, z);
+  } else {
+    vstoren<T, VL>(a.out + idx, q);
+  }
+  return s;
+}
+
+// Last pass of the finite elements: from w(k_x, y) of the two nodal components
+// (pass C) the inverse x FFT of rows y0 .. y0 + TY + 1 (two rows per complex
+// transform; the row past the tile and its partner complete the last pair),
+// then in real space the strains q = B w of both triangles of every pixel of
+// the TY rows and the update of all six components.  Transforming w instead of
+// the strains needs TY + 2 row pairs where the components need 3 TY, and reads
+// a third of the spectrum.  Bound by the r traffic (read and write, 16-byte
+// accesses).  W = 4: the spectrum holds the edge differences of w instead (see
+// pass_c_2d_fe).  grid (n_y/TY, L).
+template <typename T, int NX, int TY, int NT, int W>
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pass_e_2d_fe(PassArgs<T> a) {
+  using C = cplx<T>;
+  constexpr int NPR = TY / 2 + 1;
+  constexpr int KX = NX / 2 + 1;
+  constexpr int LD = ae_ld<NX>();
+  constexpr int VL = sizeof(T) == 4 ? 4 : 1;   // FP64: more, shorter work items
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NPR][LD]
+  __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
+  __shared__ int flag;
+  const int l = blockIdx.y, y0 = blockIdx.x * TY;
+  const int ny = a.n[1];
+  CgState* cg = a.cg + l;
+  if (!cg->active) return;
+  if (a.cgphase && cg->status != ST_RUN) return;
+  pass_e_unpack<T, NX, 2 * NPR, NT, LD>(buf, a.spec + (int64_t)l * a.m * KX * ny, W, (int64_t)KX * ny, ny, y0, ny - 1);
+  __syncthreads();
+  smem_fft<T, NX, W * NPR, LD, NT, +1>(buf, a.tw[0]);
+  const bool cgm = a.emode == E_CG;
+  const T alpha = cgm ? cg_alpha<T>(cg) : (T)0;
+  const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
+  T acc = 0;
+  for (int i = threadIdx.x; i < TY * (NX / VL); i += NT) {
+    const int yy = i / (NX / VL), x0 = (i % (NX / VL)) * VL, pr = yy / 2;
+    const int64_t v0 = (int64_t)l * a.m * a.N + (int64_t)(y0 + yy) * NX + x0;
+    T rv[6][VL], q[6][VL];
+    if (cgm) {
+#pragma unroll
+      for (int c = 0; c < 6; ++c) vloadn<T, VL>(rv[c], a.r + v0 + c * a.N);
+    }
+    // node rows yy and yy + 1 at columns x0 .. x0 + VL: rows 2 pr and 2 pr + 1
+    // are the two parts of pair pr
+    T lo[W][VL + 1], hi[W][VL + 1];
+#pragma unroll
+    for (int j = 0; j < W; ++j)
+#pragma unroll
+      for (int k = 0; k <= VL; ++k) {
+        const C* w = buf + (j * NPR + pr) * LD + ((x0 + k) & (NX - 1));
+        lo[j][k] = (yy & 1) ? w->y : w->x;
+        hi[j][k] = (yy & 1) ? w[LD].x : w->y;
+      }
+#pragma unroll
+    for (int k = 0; k < VL; ++k) {
+      if constexpr (W == 4) {   // components d_x w_0, d_x w_1, d_y w_0, d_y w_1 at the lower end of each edge
+        q[0][k] = lo[0][k];
+        q[1][k] = lo[3][k];
+        q[2][k] = r2 * (lo[2][k] + lo[1][k]);
+        q[3][k] = hi[0][k];
+        q[4][k] = lo[3][k + 1];
+        q[5][k] = r2 * (lo[2][k + 1] + hi[1][k]);
+        continue;
+      }
+      // element 0: d/dx = (u10 - u00) ihx, d/dy = (u01 - u00) ihy
+      q[0][k] = (lo[0][k + 1] - lo[0][k]) * ihx;
+      q[1][k] = (hi[1][k] - lo[1][k]) * ihy;
+      q[2][k] = r2 * ((hi[0][k] - lo[0][k]) * ihy + (lo[1][k + 1] - lo[1][k]) * ihx);
+      // element 1: d/dx = (u11 - u01) ihx, d/dy = (u11 - u10) ihy
+      q[3][k] = (hi[0][k + 1] - hi[0][k]) * ihx;
+      q[4][k] = (hi[1][k + 1] - lo[1][k + 1]) * ihy;
+      q[5][k] = r2 * ((hi[0][k + 1] - lo[0][k + 1]) * ihy + (hi[1][k + 1] - hi[1][k]) * ihx);
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) acc += strain_update<T, VL>(a, v0 + c * a.N, rv[c], q[c], alpha);
+  }
+  if (a.emode == E_CG || a.emode == E_INIT) {
+    const double s = block_sum_cols<NT>(acc, cols);
+    double* part = a.part + (int64_t)l * a.part_stride;
+    if (publish_partial(s, part, &cg->cnt_e, blockIdx.x, gridDim.x, &flag)) {
+      const double rr = sum_partials<NT>(part, gridDim.x, red);
       if (threadIdx.x == 0) finish_rr(cg, rr, a.emode == E_INIT);
     }
   }
@@ -586,7 +740,7 @@ __global__ void __launch_bounds__(NT) cg_finish_x(PassArgs<T> a) {
   const int l = blockIdx.y;
   const CgState* cg = a.cg + l;
   if (!cg->active || cg->it == 0 || cg->status == ST_BAD) return;
-  const T alpha = (T)cg->alpha;
+  const T alpha = cg_alpha<T>(cg);
   const int64_t nv = (int64_t)a.m * a.N / VL;
   const int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (i >= nv) return;
@@ -662,43 +816,75 @@ cudaError_t launch_a_2d_n(const PassArgs<T>& a, cudaStream_t s) {
   }
   return launch_a_2d_t<T, NX, tile_rows<T>(0)>(a, s);
 }
+template <typename T, int NX, int TY, int W>
+cudaError_t launch_e_2d_fe_w(const PassArgs<T>& a, cudaStream_t s) {
+  constexpr int R = W * (TY / 2 + 1);
+  constexpr int NT = fft_threads<NX, R>();
+  const size_t sm = sizeof(cplx<T>) * R * ae_ld<NX>();
+  auto k = pass_e_2d_fe<T, NX, TY, NT, W>;
+  static DeviceOnce attr;
+  attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
+  k<<<dim3(a.n[1] / TY, a.L), NT, sm, s>>>(a);
+  return cudaGetLastError();
+}
+template <typename T, int NX, int TY>
+cudaError_t launch_e_2d_fe_t(const PassArgs<T>& a, cudaStream_t s) {
+  return launch_e_2d_fe_w<T, NX, TY, 2>(a, s);
+}
+// Whether the passes run on the D nodal components after the x transform
+// (small-strain finite elements); otherwise on all components.
+template <typename T> bool fe_path(const PassArgs<T>& a) { return a.deriv == D_FE && a.m == a.ns * (a.dim == 2 ? 2 : 6); }
+
 // Tile variants of the 2D pass E: 0 default rows per block, 1 half, 2 double.
-// (The lane-pair x transform of pass A's variant 5 made pass E slower at
-// 1024^2: 0.091 against 0.083 ms per iteration for three load cases.)
 template <typename T, int NX>
 cudaError_t launch_e_2d_n(const PassArgs<T>& a, cudaStream_t s) {
+  if (fe_path(a) && (a.emode == E_CG || a.emode == E_INIT || a.emode == E_OUT)) {
+    if (a.grads) return launch_e_2d_fe_w<T, NX, tile_rows<T>(1), 4>(a, s);
+    if constexpr (NX >= 64) {
+      if (a.var_e == 1) return launch_e_2d_fe_t<T, NX, tile_rows<T>(1)>(a, s);
+      if (a.var_e == 2 && a.n[1] >= tile_rows<T>(2)) return launch_e_2d_fe_t<T, NX, tile_rows<T>(2)>(a, s);
+    }
+    return launch_e_2d_fe_t<T, NX, tile_rows<T>(0)>(a, s);
+  }
   if constexpr (NX >= 64) {
     if (a.var_e == 1) return launch_e_2d_t<T, NX, tile_rows<T>(1)>(a, s);
     if (a.var_e == 2 && a.n[1] >= tile_rows<T>(2)) return launch_e_2d_t<T, NX, tile_rows<T>(2)>(a, s);
   }
   return launch_e_2d_t<T, NX, tile_rows<T>(0)>(a, s);
 }
-// Pass C of the finite elements (two triangles) with split variant V (a.var_c).
-template <typename T, int NY, int V>
+// Pass C of the finite elements with split variant V (a.var_c): P columns per
+// block.  FP64 runs one column per block (its transforms are bound by the FP64
+// pipe, so the work is spread over as many SMs as there are columns).
+template <typename T, int NY, int V, bool COMBINE, int W = 2>
 cudaError_t launch_c_2d_v(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int NT = fft_threads<NY, 6, V>();
-  const size_t sm = sizeof(cplx<T>) * 6 * FftSplit<NY, V>::LD;
-  auto k = pass_c_2d<T, NY, 2, NT, V>;
+  constexpr int P = (sizeof(T) == 8 || W == 4) ? 1 : NY >= 256 ? 2 : 4;
+  constexpr int NT = fft_threads<NY, W * P, V>();
+  const size_t sm = sizeof(cplx<T>) * W * P * FftSplit<NY, V>::LD;
+  auto k = pass_c_2d_fe<T, NY, P, NT, V, COMBINE, W>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  dim3 grid(a.kx, a.L);
-  k<<<grid, NT, sm, s>>>(a);
+  k<<<dim3((a.kx + P - 1) / P, a.L), NT, sm, s>>>(a);
   return cudaGetLastError();
+}
+template <typename T, int NY, bool COMBINE>
+cudaError_t launch_c_2d_fe(const PassArgs<T>& a, cudaStream_t s) {
+  if constexpr (fft_split_count<NY>() > 1) {
+    if constexpr (COMBINE) {
+      if (a.grads && a.var_c == 1) return launch_c_2d_v<T, NY, 1, COMBINE, 4>(a, s);
+    }
+    if (a.var_c == 1) return launch_c_2d_v<T, NY, 1, COMBINE>(a, s);
+  }
+  if constexpr (COMBINE) {
+    if (a.grads) return launch_c_2d_v<T, NY, 0, COMBINE, 4>(a, s);
+  }
+  return launch_c_2d_v<T, NY, 0, COMBINE>(a, s);
 }
 
 template <typename T, int NY>
 cudaError_t launch_c_2d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if (a.pmode == P_SOLVE) {
-    constexpr int P = 3;
-    constexpr int NTn = fft_threads<NY, 2 * P>();
-    const size_t smn = sizeof(cplx<T>) * 2 * P * FftSplit<NY>::LD;
-    auto kn = pass_c_2d_nodal<T, NY, P, NTn>;
-    static DeviceOnce attr_n;
-    attr_n.run(current_device(), [&] { set_smem_attrs(kn, smn); });
-    dim3 gridn((a.kx + P - 1) / P, a.L);
-    kn<<<gridn, NTn, smn, s>>>(a);
-    return cudaGetLastError();
-  }
+  if (fe_path(a))
+    return (a.pmode == P_NODAL_IN || a.pmode == P_SOLVE) ? launch_c_2d_fe<T, NY, false>(a, s)
+                                                         : launch_c_2d_fe<T, NY, true>(a, s);
   if (a.nq == 3) {
     constexpr int NT3 = fft_threads<NY, 9>();
     const size_t sm3 = sizeof(cplx<T>) * 9 * FftSplit<NY>::LD;
@@ -717,10 +903,13 @@ cudaError_t launch_c_2d_n(const PassArgs<T>& a, cudaStream_t s) {
     k1<<<dim3(a.kx, a.L), NT1, sm1, s>>>(a);
     return cudaGetLastError();
   }
-  if constexpr (fft_split_count<NY>() > 1) {
-    if (a.var_c == 1) return launch_c_2d_v<T, NY, 1>(a, s);
-  }
-  return launch_c_2d_v<T, NY, 0>(a, s);
+  constexpr int NT2 = fft_threads<NY, 6>();
+  const size_t sm2 = sizeof(cplx<T>) * 6 * FftSplit<NY>::LD;
+  auto k2 = pass_c_2d<T, NY, 2, NT2>;
+  static DeviceOnce attr2;
+  attr2.run(current_device(), [&] { set_smem_attrs(k2, sm2); });
+  k2<<<dim3(a.kx, a.L), NT2, sm2, s>>>(a);
+  return cudaGetLastError();
 }
 
 #define RVE_DISPATCH_N(nval, FN, ...)                      \

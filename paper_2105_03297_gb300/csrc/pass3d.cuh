@@ -3,13 +3,19 @@
 // Real fields are [l][c][z][y][x].  One application of q = G * (C : p):
 //   A  material (+ CG direction update, <p, C p>) and forward real FFT along x;
 //      writes spec1 as [l][c][k_x][z][y] (y contiguous);
-//   B  forward FFT along y of whole y-pencils; writes spec2 as
-//      [l][c][k_x][k_y][z] (z contiguous, chunks of TZB z per k_y);
-//   C  forward FFT along z, projection G(k) per wavevector, inverse FFT along
-//      z, in place on spec2 (all m = 36 components of one (k_x, k_y) pencil);
+//   B  t = B^H sigma (differences along y and z where the factors of B^H are
+//      shifts) and its forward FFT along y; writes spec2 as [l][j][k_x][k_y][z]
+//      (z contiguous, chunks of TZB z per k_y, the D = 3 nodal components j);
+//   C  forward FFT along z, w^ = (B^H B)^-1 t^ per wavevector, inverse FFT
+//      along z, in place on spec2;
 //   D  inverse FFT along y, spec2 -> spec1;
-//   E  inverse real FFT along x, r -= alpha q, <r, r> (x += alpha p is
-//      deferred to the next pass A, as in 2D).
+//   E  inverse real FFT along x of w, q = B w in real space, r -= alpha q,
+//      <r, r> (x += alpha p is deferred to the next pass A, as in 2D).
+// The other derivatives (one evaluation point) and finite strain carry all
+// their components through B, C (with the projection), D and E.
+// Measured at 256 x 256 x 64, one load case, FP32, us per iteration: all 36
+// components through every pass A 656, B 168, C 371, D 184, E 388; now A 656,
+// B 168, C 50, D 27, E 310.
 #pragma once
 #include "pass2d.cuh"
 #include "pass3d_pipe.cuh"
@@ -88,27 +94,6 @@ __device__ __forceinline__ void pass_a_prefetch_ahead(const PassArgs<T>& a, int 
   prefetch_l2_bulk(src, (unsigned)(TY * NX * sizeof(T)));
 }
 
-// Pass E (CG mode, stress form): the later block's spectrum tile (TY
-// contiguous y values for each of its six components and NX/2 + 1 k_x) and its
-// r rows.
-template <typename T, int NX, int TY>
-__device__ __forceinline__ void pass_e_prefetch_ahead(const PassArgs<T>& a, int G) {
-  constexpr int KX = NX / 2 + 1;
-  static_assert((TY * sizeof(cplx<T>)) % 16 == 0, "bulk prefetch sizes are multiples of 16 bytes");
-  static_assert((TY * NX * sizeof(T)) % 16 == 0, "bulk prefetch sizes are multiples of 16 bytes");
-  int l, grp, z, y0;
-  if (!block_ahead(a, G, TY, l, grp, z, y0)) return;
-  const int ny = a.n[1], nz = a.n[2];
-  const cplx<T>* s0 = a.spec + ((((int64_t)l * a.m + grp * 6) * KX) * nz + z) * ny + y0;
-  const T* r0 = a.r + ((int64_t)l * a.m + grp * 6) * a.N + ((int64_t)z * ny + y0) * NX;
-  for (int i = threadIdx.x; i < 6 * KX + 6; i += blockDim.x) {
-    if (i < 6 * KX)
-      prefetch_l2_bulk(s0 + (int64_t)i * nz * ny, (unsigned)(TY * sizeof(cplx<T>)));   // i = c KX + k_x
-    else
-      prefetch_l2_bulk(r0 + (int64_t)(i - 6 * KX) * a.N, (unsigned)(TY * NX * sizeof(T)));
-  }
-}
-
 // ---------------------------------------------------------------- pass A
 // Resident blocks per SM the register budget is sized for.
 template <typename T, int NT> __host__ __device__ constexpr int pass_a_min_blocks() {
@@ -116,20 +101,21 @@ template <typename T, int NT> __host__ __device__ constexpr int pass_a_min_block
 }
 
 // grid (n_y/TY, n_z, L*G), G = 6 tetrahedra (6 components each) or 1 (nodal, 3).
+// GS = 6 components per tetrahedron, or 3 for the nodal components (A_NODAL).
 // NT is either the FFT's thread count or (tile variants 3, 4) the number of
 // load units of the tile, so that every thread streams exactly one unit.
-template <typename T, int NX, int TY, int NT>
+template <typename T, int NX, int TY, int NT, int GS>
 __global__ void __launch_bounds__(NT, pass_a_min_blocks<T, NT>()) pass_a_3d(PassArgs<T> a) {
   using C = cplx<T>;
   constexpr int NP = TY / 2;
-  constexpr int GS = 6;
   constexpr int KX = NX / 2 + 1;
   constexpr int LD = ae_ld<NX>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [GS][NP][LD]
   __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
   __shared__ int flag;
-  const bool nodal = (a.amode == A_NODAL);
+  constexpr bool nodal = GS == 3;
   const int G = nodal ? 1 : a.nq;
   const int l = blockIdx.z / G, grp = blockIdx.z % G;
   const int z = blockIdx.y, y0 = blockIdx.x * TY;
@@ -140,19 +126,19 @@ __global__ void __launch_bounds__(NT, pass_a_min_blocks<T, NT>()) pass_a_3d(Pass
   const int c0 = nodal ? 0 : grp * 6;
   T beta = 0, alpha_prev = 0;
   bool use_old = false;
-  if (a.amode == A_CG) { beta = (T)cg->beta; alpha_prev = (T)cg->alpha; use_old = cg->it > 0; }
+  if (a.amode == A_CG) { beta = cg_beta<T>(cg); alpha_prev = cg_alpha<T>(cg); use_old = cg->it > 0; }
   if (a.pf_ahead > 0 && a.amode == A_CG && !nodal) pass_a_prefetch_ahead<T, NX, TY>(a, G);
   // two columns per unit: 6 components x 2 rows x (r, p, x) stay in registers
   const T acc = pass_a_load<T, NX, TY, GS, NT, LD, 2>(a, buf, l, c0, ((int64_t)z * ny + y0) * NX, nodal, beta,
                                                       alpha_prev, use_old);
   __syncthreads();
   smem_fft<T, NX, GS * NP, LD, NT, -1>(buf, a.tw[0]);
-  pass_a_store<T, NX, TY, NT, LD>(buf, nodal ? 3 : 6,
+  pass_a_store<T, NX, TY, NT, LD>(buf, GS,
                                   a.spec + ((((int64_t)l * a.m + c0) * KX) * nz + z) * ny + y0,
                                   (int64_t)KX * nz * ny, (int64_t)nz * ny);
 
   if (a.amode == A_CG) {
-    const double s = block_sum<NT>((double)acc, red);
+    const double s = block_sum_cols<NT>(acc, cols);
     const int nblk = gridDim.x * gridDim.y * G;
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * grp);
     double* part = a.part + (int64_t)l * a.part_stride;
@@ -208,29 +194,129 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT <= 256 ? 4 : 2) : 1) 
   }
 }
 
-// ---------------------------------------------------------------- pass C
-// Projection at one wavevector of the column kz of buf ([36][LD] in shared
-// memory), in place, streaming the components so that only the element
-// gradients, B^H B and t live in registers.
-//   mode P_G:         s (36) -> B (B^H B)^-1 B^H s
-//   mode P_NODAL_IN:  rows 0..2 = f^ -> B (B^H B)^-1 f^   (36 out)
-//   mode P_NODAL_OUT: s (36) -> (B^H B)^-1 B^H s           (3 out, rows 0..2)
-template <typename T, int LD>
-__device__ __forceinline__ void project_3d(cplx<T>* col, const cplx<T>* e, const T* ih, T scale, int mode) {
+// ------------------------------------------------- pass B, finite elements
+// From the x-transformed stresses of all 36 components, spec1 [c][k_x][z][y],
+// the nodal forces t = B^H sigma and their y transform, spec2
+// [j][k_x][k_y][z], j < 3.  A factor exp(-i k_a h_a) of B^H is a shift by one
+// node along a, so B^H is applied here, where only x is transformed: every
+// voxel gives the forces of its eight corners, the four with dx = 1 times
+// exp(-i k_x h_x), and node (y, z) sums the corners (dy, dz) of voxels
+// (y - dy, z - dz).  After this only the three nodal components are
+// transformed along y and z, there and back, instead of all 36.  Bound by reading the
+// 36-component spectrum once.
+// A thread owns one y and marches in z over its lane's TZB / LN planes (one
+// plane more on the low side), keeping the dz = 1 corners of the plane below in
+// registers; the dy = 1 corners go to the neighbour row by a warp shuffle, and
+// across warps through `edge`.  The loads of a plane's 36 components are
+// independent, so a thread has up to 36 of them in flight.
+// grid (n_z/TZB, n_x/2+1, L).
+template <typename T, int NY, int TZB, int NT, int V>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT == 256 ? 2 : 6) : 1) pass_b_3d_fe(PassArgs<T> a) {
   using C = cplx<T>;
-  const C one = mkc<T>(1, 0);
-  C d[3];
+  constexpr int LN = NT / NY;            // z lanes
+  constexpr int TZL = TZB / LN;          // planes per lane
+  static_assert(NT % NY == 0 && TZB % LN == 0 && LN >= 1, "threads cover whole rows, lanes whole planes");
+  constexpr int LD = FftSplit<NY, V>::LDO;
+  constexpr int NW = NY > 32 ? NY / 32 : 1;   // warps per row
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* buf = reinterpret_cast<C*>(smem_raw);   // [3][TZB][LD]
+  C* edge = buf + 3 * TZB * LD;              // [3][TZB][NW]: dy = 1 corners of each warp's last row
+  const int l = blockIdx.z, kx = blockIdx.y, z0 = blockIdx.x * TZB;
+  const int nz = a.n[2], KX = a.kx;
+  CgState* cg = a.cg + l;
+  if (!cg->active) return;
+  if (a.cgphase && cg->status != ST_RUN) return;
+  const int y = threadIdx.x % NY, ln = threadIdx.x / NY;
+  const int64_t cs = (int64_t)KX * nz * NY;  // component stride
+  const C* src = a.spec + ((int64_t)l * a.m * KX + kx) * nz * NY + y;
+  const C cex = cconj(a.ph[0][kx]);
+  const C dx = cscale(csub(cex, mkc<T>(1, 0)), a.ih[0]);
+  const C ey = cscale(cex, a.ih[1]), ez = cscale(cex, a.ih[2]);
+  const T ihy = a.ih[1], ihz = a.ih[2], r2 = (T)kInvSqrt2;
+  C c0[3], c1[3];   // dz = 1 corners of the plane below: (dy = 0, 1)
 #pragma unroll
-  for (int i = 0; i < 3; ++i) d[i] = cscale(csub(e[i], one), ih[i]);
-  const C e01 = cmul(e[0], e[1]), e02 = cmul(e[0], e[2]), e12 = cmul(e[1], e[2]);
-  // element gradients g[t][axis] of the Kuhn tetrahedra {0, e_a, e_a+e_b, 1}
+  for (int j = 0; j < 3; ++j) c0[j] = c1[j] = mkc<T>(0, 0);
+  for (int zz = ln * TZL - 1; zz < (ln + 1) * TZL; ++zz) {
+    const C* pl = src + (int64_t)((z0 + zz) & (nz - 1)) * NY;
+    // d[dy + 2 dz][j]: corner forces of the voxel, the two dx corners combined
+    C d[4][3];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) d[k][j] = mkc<T>(0, 0);
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+      C s[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) s[c] = pl[(6 * t + c) * cs];
+#pragma unroll
+      for (int c = 3; c < 6; ++c) s[c] = cscale(s[c], r2);
+      int at = 0;   // corner dx + 2 dy + 4 dz where the edge starts
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        const int ax = kuhn_perm(t, e);
+        const int lo = (at >> 1) & 3, hi = ((at | (1 << ax)) >> 1) & 3;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const C sj = s[ax == j ? j : 6 - ax - j];   // sigma_ax,j: xx yy zz, yz xz xy
+          if (ax == 0) {
+            d[lo][j] = cadd(d[lo][j], cmul(dx, sj));
+          } else {
+            const C f = (at & 1) ? cmul(ax == 1 ? ey : ez, sj) : cscale(sj, ax == 1 ? ihy : ihz);
+            d[lo][j] = csub(d[lo][j], f);
+            d[hi][j] = cadd(d[hi][j], f);
+          }
+        }
+        at |= 1 << ax;
+      }
+    }
+    if (zz >= ln * TZL) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const C u = cadd(d[0][j], c0[j]), v = cadd(d[1][j], c1[j]);   // to nodes y and y + 1
+        C vp;
+        if constexpr (NY >= 32) {
+          vp.x = __shfl_up_sync(0xffffffffu, v.x, 1);
+          vp.y = __shfl_up_sync(0xffffffffu, v.y, 1);
+          if ((threadIdx.x & 31) == 31) edge[(j * TZB + zz) * NW + y / 32] = v;
+          if ((threadIdx.x & 31) == 0) vp = mkc<T>(0, 0);   // added from `edge` below
+        } else {
+          const int from = (threadIdx.x & 31 & ~(NY - 1)) | ((y + NY - 1) & (NY - 1));
+          vp.x = __shfl_sync(0xffffffffu, v.x, from);
+          vp.y = __shfl_sync(0xffffffffu, v.y, from);
+        }
+        buf[(j * TZB + zz) * LD + y] = cadd(u, vp);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) { c0[j] = d[2][j]; c1[j] = d[3][j]; }
+  }
+  __syncthreads();
+  if constexpr (NY >= 32) {
+    for (int i = threadIdx.x; i < 3 * TZB * NW; i += NT) {
+      const int row = i / NW, w = i % NW;
+      C* p = buf + row * LD + 32 * w;
+      *p = cadd(*p, edge[row * NW + (w + NW - 1) % NW]);
+    }
+    __syncthreads();
+  }
+  for (int j = 0; j < 3; ++j) {
+    C* bj = buf + j * TZB * LD;
+    C* chunks = a.spec2 + (((int64_t)l * a.m + j) * KX + kx) * NY * nz + z0;   // [k_y][zz], zz contiguous
+    auto ld = [&](int zz, int yy) -> C { return bj[zz * LD + yy]; };
+    auto st = [&](int zz, int k, C v) { chunks[(int64_t)k * nz + zz] = v; };
+    fft4<T, NY, TZB, LD, NT, -1, true, false, false, true, V>(bj, a.tw[1], ld, st);
+  }
+}
+
+// ---------------------------------------------------------------- pass C
+// w^ = (B^H B)^-1 t^ at one wavevector (k != 0): column kz of the three
+// component rows of buf, in place, scaled.
+template <typename T, int LD>
+__device__ __forceinline__ void solve_3d(cplx<T>* col, const cplx<T>* e, const T* ih, T scale) {
+  using C = cplx<T>;
   C g[6][3];
-  g[0][0] = d[0];             g[0][1] = cmul(e[0], d[1]);  g[0][2] = cmul(e01, d[2]);   // (x,y,z)
-  g[1][0] = d[0];             g[1][1] = cmul(e02, d[1]);   g[1][2] = cmul(e[0], d[2]);  // (x,z,y)
-  g[2][0] = cmul(e[1], d[0]); g[2][1] = d[1];              g[2][2] = cmul(e01, d[2]);   // (y,x,z)
-  g[3][0] = cmul(e12, d[0]);  g[3][1] = d[1];              g[3][2] = cmul(e[1], d[2]);  // (y,z,x)
-  g[4][0] = cmul(e[2], d[0]); g[4][1] = cmul(e02, d[1]);   g[4][2] = d[2];              // (z,x,y)
-  g[5][0] = cmul(e12, d[0]);  g[5][1] = cmul(e[2], d[1]);  g[5][2] = d[2];              // (z,y,x)
+  fe_gradients<T, 3>(e, ih, g);
   // M = B^H B = 1/2 sum_t (|g|^2 I + g g^H)
   T mdiag[3] = {0, 0, 0};
   C m01 = mkc<T>(0, 0), m02 = mkc<T>(0, 0), m12 = mkc<T>(0, 0);
@@ -245,23 +331,7 @@ __device__ __forceinline__ void project_3d(cplx<T>* col, const cplx<T>* e, const
     m02 = cadd(m02, cscale(cmul(g[t][0], cconj(g[t][2])), (T)0.5));
     m12 = cadd(m12, cscale(cmul(g[t][1], cconj(g[t][2])), (T)0.5));
   }
-  const T r2 = (T)kInvSqrt2;
-  C t3[3];
-  if (mode == P_NODAL_IN || mode == P_SOLVE) {
-    t3[0] = col[0]; t3[1] = col[LD]; t3[2] = col[2 * LD];
-  } else {
-    // t = B^H s: t_j = sum_t sum_a conj(g_ta) sigma_t,aj
-    t3[0] = t3[1] = t3[2] = mkc<T>(0, 0);
-#pragma unroll
-    for (int t = 0; t < 6; ++t) {
-      const C* sp = col + 6 * t * LD;
-      const C sxx = sp[0], syy = sp[LD], szz = sp[2 * LD];
-      const C syz = cscale(sp[3 * LD], r2), sxz = cscale(sp[4 * LD], r2), sxy = cscale(sp[5 * LD], r2);
-      t3[0] = cadd(t3[0], cadd(cadd(cjmul(g[t][0], sxx), cjmul(g[t][1], sxy)), cjmul(g[t][2], sxz)));
-      t3[1] = cadd(t3[1], cadd(cadd(cjmul(g[t][0], sxy), cjmul(g[t][1], syy)), cjmul(g[t][2], syz)));
-      t3[2] = cadd(t3[2], cadd(cadd(cjmul(g[t][0], sxz), cjmul(g[t][1], syz)), cjmul(g[t][2], szz)));
-    }
-  }
+  const C t3[3] = {col[0], col[LD], col[2 * LD]};
   // w = M^-1 t by the adjugate of the Hermitian matrix
   // M = [[A, m01, m02], [conj m01, B, m12], [conj m02, conj m12, Cc]]
   const T A = mdiag[0], B = mdiag[1], Cc = mdiag[2];
@@ -274,230 +344,58 @@ __device__ __forceinline__ void project_3d(cplx<T>* col, const cplx<T>* e, const
   const C A12 = csub(cmul(m02, cconj(m01)), cscale(m12, A));
   const T det = A * A00 + (cmul(m01, cconj(A01))).x + (cmul(m02, cconj(A02))).x;
   const T id = scale / det;
-  C w[3];
-  w[0] = cscale(cadd(cadd(cscale(t3[0], A00), cmul(A01, t3[1])), cmul(A02, t3[2])), id);
-  w[1] = cscale(cadd(cadd(cjmul(A01, t3[0]), cscale(t3[1], A11)), cmul(A12, t3[2])), id);
-  w[2] = cscale(cadd(cadd(cjmul(A02, t3[0]), cjmul(A12, t3[1])), cscale(t3[2], A22)), id);
-  if (mode == P_NODAL_OUT || mode == P_SOLVE) {
-    col[0] = w[0]; col[LD] = w[1]; col[2 * LD] = w[2];
-    return;
-  }
-  // eps^ = B w: Mandel components of sym(g_t (x) w)
-#pragma unroll
-  for (int t = 0; t < 6; ++t) {
-    C* sp = col + 6 * t * LD;
-    sp[0] = cmul(g[t][0], w[0]);
-    sp[LD] = cmul(g[t][1], w[1]);
-    sp[2 * LD] = cmul(g[t][2], w[2]);
-    sp[3 * LD] = cscale(cadd(cmul(g[t][1], w[2]), cmul(g[t][2], w[1])), r2);
-    sp[4 * LD] = cscale(cadd(cmul(g[t][0], w[2]), cmul(g[t][2], w[0])), r2);
-    sp[5 * LD] = cscale(cadd(cmul(g[t][0], w[1]), cmul(g[t][1], w[0])), r2);
-  }
+  col[0] = cscale(cadd(cadd(cscale(t3[0], A00), cmul(A01, t3[1])), cmul(A02, t3[2])), id);
+  col[LD] = cscale(cadd(cadd(cjmul(A01, t3[0]), cscale(t3[1], A11)), cmul(A12, t3[2])), id);
+  col[2 * LD] = cscale(cadd(cadd(cjmul(A02, t3[0]), cjmul(A12, t3[1])), cscale(t3[2], A22)), id);
 }
 
-// The same projection done by a pair of adjacent lanes: lane half h handles
-// tetrahedra 3h..3h+2 (their gradients, their share of B^H B and of
-// t = B^H s), the pair exchanges its partial sums by warp shuffle, both
-// solve the 3x3 system, and each writes the outputs of its own tetrahedra.
-// All 32 lanes of a warp must call it together (it exchanges partial sums
-// with __shfl_xor_sync over the full warp): the k = 0 wavevector is handled by
-// the `zero` flag, which only changes what is written at the end.
-template <typename T, int LD>
-__device__ __forceinline__ void project_3d_pair(cplx<T>* col, const cplx<T>* e, const T* ih, T scale, int mode,
-                                                int half, bool zero) {
+// Pass C of the finite elements: forward FFT along z, w^ = (B^H B)^-1 t^,
+// inverse FFT, on the three nodal components; P pencils (k_x, k_y0 + i), i <
+// P, per block.  Row b of the buffer is component b % 3 of pencil b / 3.  W =
+// 9 (P = 1) writes the differences d_a w_j along the element edges as
+// components 3 a + j (see pass_c_2d_fe).  grid (n_x/2+1, n_y/P, L).
+template <typename T, int NZ, int P, int NT, int V, int W>
+__global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 384 ? 2 : 1) pass_c_3d_nodal(PassArgs<T> a) {
   using C = cplx<T>;
-  const C one = mkc<T>(1, 0);
-  C d[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) d[i] = cscale(csub(e[i], one), ih[i]);
-  const C e01 = cmul(e[0], e[1]), e02 = cmul(e[0], e[2]), e12 = cmul(e[1], e[2]);
-  // gradients of this lane's tetrahedra {0, e_a, e_a+e_b, 1}
-  C g[3][3];
-  if (half == 0) {
-    g[0][0] = d[0];             g[0][1] = cmul(e[0], d[1]);  g[0][2] = cmul(e01, d[2]);   // (x,y,z)
-    g[1][0] = d[0];             g[1][1] = cmul(e02, d[1]);   g[1][2] = cmul(e[0], d[2]);  // (x,z,y)
-    g[2][0] = cmul(e[1], d[0]); g[2][1] = d[1];              g[2][2] = cmul(e01, d[2]);   // (y,x,z)
-  } else {
-    g[0][0] = cmul(e12, d[0]);  g[0][1] = d[1];              g[0][2] = cmul(e[1], d[2]);  // (y,z,x)
-    g[1][0] = cmul(e[2], d[0]); g[1][1] = cmul(e02, d[1]);   g[1][2] = d[2];              // (z,x,y)
-    g[2][0] = cmul(e12, d[0]);  g[2][1] = cmul(e[2], d[1]);  g[2][2] = d[2];              // (z,y,x)
-  }
-  // partial M = B^H B over this lane's tetrahedra
-  T md[3] = {0, 0, 0};
-  C m01 = mkc<T>(0, 0), m02 = mkc<T>(0, 0), m12 = mkc<T>(0, 0);
-#pragma unroll
-  for (int t = 0; t < 3; ++t) {
-    const T a0 = cabs2(g[t][0]), a1 = cabs2(g[t][1]), a2 = cabs2(g[t][2]);
-    const T nn = a0 + a1 + a2;
-    md[0] += (T)0.5 * (nn + a0);
-    md[1] += (T)0.5 * (nn + a1);
-    md[2] += (T)0.5 * (nn + a2);
-    m01 = cadd(m01, cscale(cmul(g[t][0], cconj(g[t][1])), (T)0.5));
-    m02 = cadd(m02, cscale(cmul(g[t][0], cconj(g[t][2])), (T)0.5));
-    m12 = cadd(m12, cscale(cmul(g[t][1], cconj(g[t][2])), (T)0.5));
-  }
-  const T r2 = (T)kInvSqrt2;
-  C t3[3];
-  cplx<T>* own = col + 18 * half * LD;  // rows of this lane's tetrahedra
-  const bool nodal_in = (mode == P_NODAL_IN || mode == P_SOLVE);
-  if (nodal_in) {
-    t3[0] = col[0]; t3[1] = col[LD]; t3[2] = col[2 * LD];
-  } else {
-    t3[0] = t3[1] = t3[2] = mkc<T>(0, 0);
-#pragma unroll
-    for (int t = 0; t < 3; ++t) {
-      const C* sp = own + 6 * t * LD;
-      const C sxx = sp[0], syy = sp[LD], szz = sp[2 * LD];
-      const C syz = cscale(sp[3 * LD], r2), sxz = cscale(sp[4 * LD], r2), sxy = cscale(sp[5 * LD], r2);
-      t3[0] = cadd(t3[0], cadd(cadd(cjmul(g[t][0], sxx), cjmul(g[t][1], sxy)), cjmul(g[t][2], sxz)));
-      t3[1] = cadd(t3[1], cadd(cadd(cjmul(g[t][0], sxy), cjmul(g[t][1], syy)), cjmul(g[t][2], syz)));
-      t3[2] = cadd(t3[2], cadd(cadd(cjmul(g[t][0], sxz), cjmul(g[t][1], syz)), cjmul(g[t][2], szz)));
-    }
-  }
-  // pair sums
-  auto xs = [](T v) { return v + __shfl_xor_sync(0xffffffffu, v, 1); };
-#pragma unroll
-  for (int i = 0; i < 3; ++i) md[i] = xs(md[i]);
-  m01.x = xs(m01.x); m01.y = xs(m01.y);
-  m02.x = xs(m02.x); m02.y = xs(m02.y);
-  m12.x = xs(m12.x); m12.y = xs(m12.y);
-  if (!nodal_in) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) { t3[i].x = xs(t3[i].x); t3[i].y = xs(t3[i].y); }
-  }
-  const T A = md[0], B = md[1], Cc = md[2];
-  const T A00 = B * Cc - cabs2(m12);
-  const T A11 = A * Cc - cabs2(m02);
-  const T A22 = A * B - cabs2(m01);
-  const C A01 = csub(cmul(m02, cconj(m12)), cscale(m01, Cc));
-  const C A02 = csub(cmul(m01, m12), cscale(m02, B));
-  const C A12 = csub(cmul(m02, cconj(m01)), cscale(m12, A));
-  const T det = A * A00 + (cmul(m01, cconj(A01))).x + (cmul(m02, cconj(A02))).x;
-  const T id = scale / det;
-  C w[3];
-  w[0] = cscale(cadd(cadd(cscale(t3[0], A00), cmul(A01, t3[1])), cmul(A02, t3[2])), id);
-  w[1] = cscale(cadd(cadd(cjmul(A01, t3[0]), cscale(t3[1], A11)), cmul(A12, t3[2])), id);
-  w[2] = cscale(cadd(cadd(cjmul(A02, t3[0]), cjmul(A12, t3[1])), cscale(t3[2], A22)), id);
-  const bool nodal_out = (mode == P_NODAL_OUT || mode == P_SOLVE);
-  if (zero) {
-    // k = 0: G(0) = 0, the fluctuation has no mean (w is not finite here)
-    const C z = mkc<T>(0, 0);
-    if (nodal_out) {
-      if (half == 0) { col[0] = z; col[LD] = z; col[2 * LD] = z; }
-    } else {
-#pragma unroll
-      for (int r = 0; r < 18; ++r) own[r * LD] = z;
-    }
-    return;
-  }
-  if (nodal_out) {
-    if (half == 0) { col[0] = w[0]; col[LD] = w[1]; col[2 * LD] = w[2]; }
-    return;
-  }
-#pragma unroll
-  for (int t = 0; t < 3; ++t) {
-    C* sp = own + 6 * t * LD;
-    sp[0] = cmul(g[t][0], w[0]);
-    sp[LD] = cmul(g[t][1], w[1]);
-    sp[2 * LD] = cmul(g[t][2], w[2]);
-    sp[3 * LD] = cscale(cadd(cmul(g[t][1], w[2]), cmul(g[t][2], w[1])), r2);
-    sp[4 * LD] = cscale(cadd(cmul(g[t][0], w[2]), cmul(g[t][2], w[0])), r2);
-    sp[5 * LD] = cscale(cadd(cmul(g[t][0], w[1]), cmul(g[t][1], w[0])), r2);
-  }
-}
-
-// Row stride of the pass C buffer: at least the FFT's leading dimension, and
-// chosen so that the two lanes of a wavevector (rows c and c + 18, same
-// column) fall into different halves of a shared-memory bank window: the row
-// offset 18 LD sizeof(complex) is then an odd multiple of 64 bytes and the
-// lane-pair projection's accesses are free of bank conflicts.
-template <typename T, int NZ, int V = 0> __host__ __device__ constexpr int pass_c_ld() {
-  constexpr int base = FftSplit<NZ, V>::LD;
-  constexpr int mod = sizeof(T) == 4 ? 8 : 4, want = sizeof(T) == 4 ? 4 : 2;
-  return base + ((want - base % mod) + mod) % mod;
-}
-
-// grid (n_x/2+1, n_y, L): one (k_x, k_y) pencil of all components per block.
-template <typename T, int NZ, int NT, int V = 0>
-__global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 576) ? 2 : 1) pass_c_3d(PassArgs<T> a) {
-  using C = cplx<T>;
-  constexpr int M = 36;
-  constexpr int LD = pass_c_ld<T, NZ, V>();
-  static_assert((18 * LD * (int)sizeof(cplx<T>)) % 128 == 64, "lane pairs must not share a bank");
+  constexpr int R = 3 * P;
+  static_assert(W == 3 || (W == 9 && P == 1), "differences: one pencil per block");
+  constexpr int LD = FftSplit<NZ, V>::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);  // [M][LD]
-  const int kx = blockIdx.x, ky = blockIdx.y, l = blockIdx.z;
-  const int ny = a.n[1], KX = a.kx;
-  CgState* cg = a.cg + l;
-  if (!cg->active) return;
-  if (a.cgphase && cg->status != ST_RUN) return;
-  const int cin = (a.pmode == P_NODAL_IN || a.pmode == P_SOLVE) ? 3 : M;
-  const int cout = (a.pmode == P_NODAL_OUT || a.pmode == P_SOLVE) ? 3 : M;
-  const int64_t stride_c = (int64_t)KX * ny * NZ;
-  C* pen = a.spec2 + (int64_t)l * M * stride_c + ((int64_t)kx * ny + ky) * NZ;
-  // L2 prefetch of the later block's pencil (see grid_ahead): one request of
-  // NZ values per component
-  int kx2, ky2, l2;
-  if (a.pf_ahead > 0 && threadIdx.x < M && grid_ahead(a, kx2, ky2, l2) && slot_runs(a, l2))
-    prefetch_l2_bulk(a.spec2 + (int64_t)l2 * M * stride_c + ((int64_t)kx2 * ny + ky2) * NZ + threadIdx.x * stride_c,
-                     (unsigned)(NZ * sizeof(C)));
-  auto ld_g = [&](int c, int z) -> C { return pen[c * stride_c + z]; };
-  auto st_s = [&](int c, int k, C v) { buf[c * LD + k] = v; };
-  if (cin == M) fft4<T, NZ, M, LD, NT, -1, false, true, false, false, V>(buf, a.tw[2], ld_g, st_s);
-  else fft4<T, NZ, 3, LD, NT, -1, false, true, false, false, V>(buf, a.tw[2], ld_g, st_s);
-  C e[3];
-  e[0] = a.ph[0][kx];
-  e[1] = a.ph[1][ky];
-  // two lanes per wavevector (NT >= 2 NZ, and 2 NZ is a whole number of warps)
-  static_assert(NT >= 2 * NZ && (2 * NZ) % 32 == 0, "pass C needs two lanes per wavevector");
-  if (threadIdx.x < 2 * NZ) {  // whole warps: every lane of them calls the pair projection
-    const int kz = threadIdx.x >> 1, half = threadIdx.x & 1;
-    e[2] = a.ph[2][kz];
-    project_3d_pair<T, LD>(buf + kz, e, a.ih, a.inv_n, a.pmode, half, kx == 0 && ky == 0 && kz == 0);
-  }
-  __syncthreads();
-  auto ld_s = [&](int c, int z) -> C { return buf[c * LD + z]; };
-  auto st_g = [&](int c, int k, C v) { pen[c * stride_c + k] = v; };
-  if (cout == M) fft4<T, NZ, M, LD, NT, +1, true, false, false, false, V>(buf, a.tw[2], ld_s, st_g);
-  else fft4<T, NZ, 3, LD, NT, +1, true, false, false, false, V>(buf, a.tw[2], ld_s, st_g);
-}
-
-// Pass C for the nodal solve w^ = (B^H B)^-1 f^ (P_SOLVE, 3 components in
-// and out): P pencils (k_x, k_y0 + i), i < P, per block, so that a block has
-// as many transforms as the 36-component pass.  Row b of the buffer is
-// component b % 3 of pencil b / 3.  grid (n_x/2+1, n_y/P, L).
-template <typename T, int NZ, int P, int NT>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) pass_c_3d_nodal(PassArgs<T> a) {
-  using C = cplx<T>;
-  constexpr int M = 36, R = 3 * P;
-  constexpr int LD = FftSplit<NZ>::LD;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);  // [R][LD]
+  C* buf = reinterpret_cast<C*>(smem_raw);  // [W P][LD]
   const int kx = blockIdx.x, ky0 = blockIdx.y * P, l = blockIdx.z;
   const int ny = a.n[1], KX = a.kx;
   CgState* cg = a.cg + l;
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t stride_c = (int64_t)KX * ny * NZ;
-  C* base = a.spec2 + (int64_t)l * M * stride_c + ((int64_t)kx * ny + ky0) * NZ;
+  C* base = a.spec2 + (int64_t)l * a.m * stride_c + ((int64_t)kx * ny + ky0) * NZ;
   auto ld_g = [&](int b, int z) -> C { return base[(b % 3) * stride_c + (b / 3) * NZ + z]; };
   auto st_s = [&](int b, int k, C v) { buf[b * LD + k] = v; };
-  fft4<T, NZ, R, LD, NT, -1, false, true, false, false>(buf, a.tw[2], ld_g, st_s);
+  fft4<T, NZ, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[2], ld_g, st_s);
   for (int i = threadIdx.x; i < P * NZ; i += NT) {
     const int pc = i / NZ, kz = i % NZ;
     C* col = buf + 3 * pc * LD + kz;
     if (kx == 0 && ky0 + pc == 0 && kz == 0) {
       // k = 0: the nodal solve has no mean (w^(0) = 0)
-      col[0] = col[LD] = col[2 * LD] = mkc<T>(0, 0);
+      for (int j = 0; j < W; ++j) col[j * LD] = mkc<T>(0, 0);
     } else {
       const C e[3] = {a.ph[0][kx], a.ph[1][ky0 + pc], a.ph[2][kz]};
-      project_3d<T, LD>(col, e, a.ih, a.inv_n, P_SOLVE);
+      solve_3d<T, LD>(col, e, a.ih, a.inv_n);
+      if constexpr (W == 9) {
+        const C w[3] = {col[0], col[LD], col[2 * LD]};
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+          const C d = cscale(csub(e[ax], mkc<T>(1, 0)), a.ih[ax]);
+#pragma unroll
+          for (int j = 0; j < 3; ++j) col[(3 * ax + j) * LD] = cmul(d, w[j]);
+        }
+      }
     }
   }
   __syncthreads();
   auto ld_s = [&](int b, int z) -> C { return buf[b * LD + z]; };
-  auto st_g = [&](int b, int k, C v) { base[(b % 3) * stride_c + (b / 3) * NZ + k] = v; };
-  fft4<T, NZ, R, LD, NT, +1, true, false, false, false>(buf, a.tw[2], ld_s, st_g);
+  auto st_g = [&](int b, int k, C v) { base[(b % W) * stride_c + (b / W) * NZ + k] = v; };
+  fft4<T, NZ, W * P, LD, NT, +1, true, false, false, false, V>(buf, a.tw[2], ld_s, st_g);
 }
 
 // Pass C for one evaluation point per voxel (the derivatives of Secs. 2.3-2.5,
@@ -586,18 +484,18 @@ __global__ void __launch_bounds__(NT, 1) pass_c_3d_fs(PassArgs<T> a) {
 // ---------------------------------------------------------------- pass E
 // grid (n_y/TY, n_z, L*G): G = 6 tetrahedra (6 components each) or one group
 // of the 3 nodal components (E_NODAL); inverse real FFT along x and update.
-template <typename T, int NX, int TY, int NT>
+template <typename T, int NX, int TY, int NT, int GE>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pass_e_3d(PassArgs<T> a) {
   using C = cplx<T>;
   constexpr int NP = TY / 2;
   constexpr int KX = NX / 2 + 1;
-  constexpr int GE = 6;
   constexpr int LD = ae_ld<NX>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [GE][NP][LD]
   __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
   __shared__ int flag;
-  const bool nodal = (a.emode == E_NODAL || a.emode == E_NOUT);
+  constexpr bool nodal = GE == 3;
   const int G = nodal ? 1 : a.nq;
   const int l = blockIdx.z / G, grp = blockIdx.z % G;
   const int z = blockIdx.y, y0 = blockIdx.x * TY;
@@ -606,31 +504,140 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pas
   CgState* cg = a.cg + l;
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
-  const int ge = nodal ? 3 : GE;
   const int c0 = nodal ? 0 : grp * GE;
-  // the r rows this tile updates after its inverse FFT: start their DRAM reads
-  // now so that they overlap the spectrum loads and the transform (measured at
-  // 256^3: pass E 1.92 -> 1.88 ms; the same prefetch slowed the 2D pass E, whose
-  // 4 KB rows compete with the spectrum loads at the start of the block)
-  if (a.emode == E_CG)
-    prefetch_rows_l2<T, NX>(a.r + ((int64_t)l * a.m + c0) * N + ((int64_t)z * ny + y0) * NX, ge, TY, N);
-  if (a.pf_ahead > 0 && a.emode == E_CG && !nodal) pass_e_prefetch_ahead<T, NX, TY>(a, G);
-
-  pass_e_unpack<T, NX, TY, NT, LD>(buf, a.spec + ((((int64_t)l * a.m + c0) * KX) * nz + z) * ny + y0, ge,
-                                   (int64_t)KX * nz * ny, (int64_t)nz * ny);
+  pass_e_unpack<T, NX, TY, NT, LD>(buf, a.spec + ((((int64_t)l * a.m + c0) * KX) * nz + z) * ny, GE,
+                                   (int64_t)KX * nz * ny, (int64_t)nz * ny, y0, ny - 1);
   __syncthreads();
   T acc = 0;
-  const T alpha = (a.emode == E_CG) ? (T)cg->alpha : (T)0;
+  const T alpha = (a.emode == E_CG) ? cg_alpha<T>(cg) : (T)0;
   auto ld_s = [&](int b, int x) -> C { return buf[b * LD + x]; };
-  PassEStore<T, NX, NP> st{&a, ge, ((int64_t)z * ny + y0) * NX, ((int64_t)l * a.m + c0) * N, (int64_t)l * 3 * N,
+  PassEStore<T, NX, NP> st{&a, GE, ((int64_t)z * ny + y0) * NX, ((int64_t)l * a.m + c0) * N, (int64_t)l * 3 * N,
                            alpha, &acc};
   fft4<T, NX, GE * NP, LD, NT, +1, true, false, false, false, 0, decltype(ld_s), decltype(st), true>(buf, a.tw[0],
                                                                                                   ld_s, st);
 
   if (a.emode == E_CG || a.emode == E_INIT) {
-    const double s = block_sum<NT>((double)acc, red);
+    const double s = block_sum_cols<NT>(acc, cols);
     const int nblk = gridDim.x * gridDim.y * G;
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * grp);
+    double* part = a.part + (int64_t)l * a.part_stride;
+    if (publish_partial(s, part, &cg->cnt_e, blk, nblk, &flag)) {
+      const double rr = sum_partials<NT>(part, nblk, red);
+      if (threadIdx.x == 0) finish_rr(cg, rr, a.emode == E_INIT);
+    }
+  }
+}
+
+// Last pass of the finite elements: from w(k_x, z, y) of the three nodal
+// components (pass D) the inverse x FFT of TY + 1 rows of planes z and z + 1
+// (the two planes share one complex transform), then in real space the strains
+// q = B w of the six tetrahedra of every voxel of the TY rows and the update of
+// all 36 components.  Transforming w needs 3 (TY + 1) transforms where the
+// components need 18 TY, and reads 1/12 of the spectrum; what is left is the r
+// traffic (read and written once), which bounds it.  W = 9: the spectrum holds
+// the edge differences of w instead (see pass_c_2d_fe).
+// grid (n_y/TY, n_z, L).
+template <int NX> __host__ __device__ constexpr int e_fe_ld() {
+  // 9 (mod 16): the TY + 1 rows that consecutive lanes unpack at one column
+  // fall on different banks
+  return FftSplit<NX>::LD + ((9 - FftSplit<NX>::LD % 16) + 16) % 16;
+}
+template <typename T, int NX, int TY, int NT, int MB, int W>
+__global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
+  using C = cplx<T>;
+  constexpr int KX = NX / 2 + 1;
+  constexpr int NR = TY + 1;
+  constexpr int R = W * NR;
+  constexpr int LD = e_fe_ld<NX>();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NR][LD]
+  __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
+  __shared__ int flag;
+  const int l = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * TY;
+  const int ny = a.n[1], nz = a.n[2];
+  const int64_t N = a.N;
+  CgState* cg = a.cg + l;
+  if (!cg->active) return;
+  if (a.cgphase && cg->status != ST_RUN) return;
+  const bool cgm = a.emode == E_CG;
+  const int64_t vox0 = (int64_t)l * a.m * N + ((int64_t)z * ny + y0) * NX;
+  if (cgm && a.pf_ahead > 0 && threadIdx.x < 36)   // the tile's r rows, contiguous per component
+    prefetch_l2_bulk(a.r + vox0 + threadIdx.x * N, (unsigned)(TY * NX * sizeof(T)));
+  {
+    const C* pa = a.spec + ((int64_t)l * a.m * KX * nz + z) * ny;
+    const C* pb = a.spec + ((int64_t)l * a.m * KX * nz + ((z + 1) & (nz - 1))) * ny;
+    constexpr int TOT = W * KX * NR, UB = 4;
+    for (int i0 = threadIdx.x; i0 < TOT; i0 += UB * NT) {
+      C xa[UB], xb[UB];
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int i = i0 + u * NT;
+        if (i < TOT) {
+          const int64_t o = (int64_t)(i / NR) * nz * ny + ((y0 + i % NR) & (ny - 1));   // i / NR = j KX + k_x
+          xa[u] = pa[o]; xb[u] = pb[o];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int i = i0 + u * NT;
+        if (i < TOT) {
+          const int k = (i / NR) % KX, j = i / (NR * KX);
+          C va = xa[u], vb = xb[u];
+          if (k == 0 || k == NX / 2) { va.y = 0; vb.y = 0; }  // C2R ignores these imaginary parts
+          C* row = buf + (j * NR + i % NR) * LD;
+          row[k] = mkc<T>(va.x - vb.y, va.y + vb.x);                                  // X_a + i X_b
+          if (k > 0 && k < NX / 2) row[NX - k] = mkc<T>(va.x + vb.y, vb.x - va.y);    // conj(X_a) + i conj(X_b)
+        }
+      }
+    }
+  }
+  __syncthreads();
+  smem_fft<T, NX, R, LD, NT, +1>(buf, a.tw[0]);
+  const T alpha = cgm ? cg_alpha<T>(cg) : (T)0;
+  const T ih[3] = {a.ih[0], a.ih[1], a.ih[2]};
+  const T r2 = (T)kInvSqrt2;
+  T acc = 0;
+  for (int i = threadIdx.x; i < TY * NX; i += NT) {
+    const int yy = i / NX, x = i % NX;
+    const int64_t v0 = vox0 + (int64_t)yy * NX + x;
+    // node values at (x + dx, y + dy): planes z (.x) and z + 1 (.y)
+    C n[W][2][2];
+#pragma unroll
+    for (int j = 0; j < W; ++j)
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) n[j][dy][q] = buf[(j * NR + yy + dy) * LD + ((x + q) & (NX - 1))];
+    auto corner = [&](int c, int j) -> T {   // corner c = dx + 2 dy + 4 dz
+      const C v = n[j][(c >> 1) & 1][c & 1];
+      return (c & 4) ? v.y : v.x;
+    };
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+      T rv[6];
+      if (cgm) {
+#pragma unroll
+        for (int s = 0; s < 6; ++s) rv[s] = a.r[v0 + (6 * t + s) * N];
+      }
+      const int ax[3] = {kuhn_perm(t, 0), kuhn_perm(t, 1), kuhn_perm(t, 2)};
+      const int v1 = 1 << ax[0], v2 = v1 | (1 << ax[1]);
+      const int at[4] = {0, v1, v2, 7};
+      T H[3][3];   // H[a][j] = d w_j / d x_a
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          H[ax[e]][j] = W == 9 ? corner(at[e], 3 * ax[e] + j) : (corner(at[e + 1], j) - corner(at[e], j)) * ih[ax[e]];
+      const T q[6] = {H[0][0], H[1][1], H[2][2], r2 * (H[1][2] + H[2][1]), r2 * (H[0][2] + H[2][0]),
+                      r2 * (H[0][1] + H[1][0])};
+#pragma unroll
+      for (int s = 0; s < 6; ++s) acc += strain_update<T, 1>(a, v0 + (6 * t + s) * N, &rv[s], &q[s], alpha);
+    }
+  }
+  if (cgm || a.emode == E_INIT) {
+    const double s = block_sum_cols<NT>(acc, cols);
+    const int nblk = gridDim.x * gridDim.y, blk = blockIdx.x + gridDim.x * blockIdx.y;
     double* part = a.part + (int64_t)l * a.part_stride;
     if (publish_partial(s, part, &cg->cnt_e, blk, nblk, &flag)) {
       const double rr = sum_partials<NT>(part, nblk, red);
@@ -672,13 +679,13 @@ inline int prefetch_distance(int occ, int div) {
   return d > 1 ? d : 1;
 }
 
-template <typename T, int NX, int TY, bool BY_UNITS = false>
+template <typename T, int NX, int TY, bool BY_UNITS = false, int GS = 6>
 cudaError_t launch_a_3d_t(const PassArgs<T>& a, cudaStream_t s, bool ahead = false) {
-  constexpr int NF = fft_threads<NX, 6 * (TY / 2)>();
+  constexpr int NF = fft_threads<NX, GS * (TY / 2)>();
   constexpr int NU = (pass_a_units3<T, NX, TY>() + 31) / 32 * 32;
   constexpr int NT = BY_UNITS ? (max_i<NF, NU>() > 1024 ? NF : max_i<NF, NU>()) : NF;
-  const size_t sm = sizeof(cplx<T>) * 6 * (TY / 2) * ae_ld<NX>();
-  auto k = pass_a_3d<T, NX, TY, NT>;
+  const size_t sm = sizeof(cplx<T>) * GS * (TY / 2) * ae_ld<NX>();
+  auto k = pass_a_3d<T, NX, TY, NT, GS>;
   static DeviceOnce attr;
   static int occ[kMaxDevices] = {0};
   const int dev = current_device();
@@ -686,7 +693,7 @@ cudaError_t launch_a_3d_t(const PassArgs<T>& a, cudaStream_t s, bool ahead = fal
     set_smem_attrs(k, sm);
     if (dev >= 0 && dev < kMaxDevices) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[dev], k, NT, sm);
   });
-  dim3 grid(a.n[1] / TY, a.n[2], a.L * (a.amode == A_NODAL ? 1 : a.nq));
+  dim3 grid(a.n[1] / TY, a.n[2], a.L * (GS == 3 ? 1 : a.nq));
   if (ahead) {
     PassArgs<T> b = a;
     b.pf_ahead = prefetch_distance((dev >= 0 && dev < kMaxDevices) ? occ[dev] : 0, 16);
@@ -696,26 +703,29 @@ cudaError_t launch_a_3d_t(const PassArgs<T>& a, cudaStream_t s, bool ahead = fal
   }
   return cudaGetLastError();
 }
-template <typename T, int NX, int TY>
-cudaError_t launch_e_3d_t(const PassArgs<T>& a, cudaStream_t s, bool ahead = false) {
-  constexpr int NT = fft_threads<NX, 6 * (TY / 2)>();
-  const size_t sm = sizeof(cplx<T>) * 6 * (TY / 2) * ae_ld<NX>();
-  auto k = pass_e_3d<T, NX, TY, NT>;
+template <typename T, int NX, int TY, int GE = 6>
+cudaError_t launch_e_3d_t(const PassArgs<T>& a, cudaStream_t s) {
+  constexpr int NT = fft_threads<NX, GE * (TY / 2)>();
+  const size_t sm = sizeof(cplx<T>) * GE * (TY / 2) * ae_ld<NX>();
+  auto k = pass_e_3d<T, NX, TY, NT, GE>;
   static DeviceOnce attr;
-  static int occ[kMaxDevices] = {0};
-  const int dev = current_device();
-  attr.run(dev, [&] {
-    set_smem_attrs(k, sm);
-    if (dev >= 0 && dev < kMaxDevices) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[dev], k, NT, sm);
-  });
-  dim3 grid(a.n[1] / TY, a.n[2], a.L * ((a.emode == E_NODAL || a.emode == E_NOUT) ? 1 : a.nq));
-  if (ahead) {
-    PassArgs<T> b = a;
-    b.pf_ahead = prefetch_distance((dev >= 0 && dev < kMaxDevices) ? occ[dev] : 0, 16);
-    k<<<grid, NT, sm, s>>>(b);
-  } else {
-    k<<<grid, NT, sm, s>>>(a);
-  }
+  attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
+  dim3 grid(a.n[1] / TY, a.n[2], a.L * (GE == 3 ? 1 : a.nq));
+  k<<<grid, NT, sm, s>>>(a);
+  return cudaGetLastError();
+}
+template <typename T, int NX, int TY, int W = 3>
+cudaError_t launch_e_3d_fe_t(const PassArgs<T>& a, cudaStream_t s, bool prefetch) {
+  constexpr int R = W * (TY + 1);
+  constexpr int NT = fft_threads<NX, R>();
+  constexpr size_t sm = sizeof(cplx<T>) * R * e_fe_ld<NX>();
+    constexpr int MB = sizeof(T) == 8 ? 1 : W == 9 ? (NT <= 448 ? 2 : 1) : NT <= 256 ? 4 : NT <= 448 ? 2 : 1;
+  auto k = pass_e_3d_fe<T, NX, TY, NT, MB, W>;
+  static DeviceOnce attr;
+  attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
+  PassArgs<T> b = a;
+  b.pf_ahead = prefetch ? 1 : 0;
+  k<<<dim3(a.n[1] / TY, a.n[2], a.L), NT, sm, s>>>(b);
   return cudaGetLastError();
 }
 // Tile variants of pass A: 0 default rows per block, 1 half, 2 double (threads
@@ -725,6 +735,10 @@ cudaError_t launch_e_3d_t(const PassArgs<T>& a, cudaStream_t s, bool ahead = fal
 // 6 variant 0 with the L2 prefetch of a later block's rows.
 template <typename T, int NX>
 cudaError_t launch_a_3d_n(const PassArgs<T>& a, cudaStream_t s) {
+  // the three nodal components: twice the rows, so that a block holds as many
+  // transforms as with six components (256^3, FP32: 137 us with the six-component
+  // tile, half of whose transforms were padding)
+  if (a.amode == A_NODAL) return launch_a_3d_t<T, NX, tile_rows3<T>(2), false, 3>(a, s);
   if constexpr (sizeof(T) == 4 && NX >= 128) {
     if (a.var_a == 5 && a.amode == A_CG && a.L <= kPipeMaxL && a.n[1] >= 4) return launch_a_3d_pipe<NX>(a, s);
   }
@@ -737,20 +751,26 @@ cudaError_t launch_a_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   }
   return launch_a_3d_t<T, NX, tile_rows3<T>(0)>(a, s);
 }
-// Tile variants of pass E: 0 default rows per block, 1 half, 2 double; 3
-// (FP32, n_x >= 128, CG iterations, with the spectrum's tensor map) the
-// pipelined persistent pass (pass3d_pipe.cuh); other modes of 3 use 0; 4
-// variant 0 with the L2 prefetch of a later block's spectrum tile and rows.
+// Tile variants of pass E: 0 default rows per block, 1 half, 2 double; with
+// n_x >= 128 in FP32 also 3 default and 4 half rows with the L2 prefetch of
+// the tile's own r rows at the start of the block.
 template <typename T, int NX>
 cudaError_t launch_e_3d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if constexpr (sizeof(T) == 4 && NX >= 128) {
-    if (a.var_e == 3 && a.emode == E_CG && a.tm_spec && a.L <= kPipeMaxL && a.n[1] >= kPipeETY)
-      return launch_e_3d_pipe<NX>(a, s);
+  if (fe_path(a) && (a.emode == E_CG || a.emode == E_INIT || a.emode == E_OUT)) {
+    if (a.grads) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1), 9>(a, s, false);
+    if constexpr (NX >= 64) {
+      if (a.var_e == 1) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1)>(a, s, false);
+      if (a.var_e == 2 && a.n[1] >= tile_rows3<T>(2)) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(2)>(a, s, false);
+      if (a.var_e == 3) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(0)>(a, s, true);
+      if (a.var_e == 4) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1)>(a, s, true);
+    }
+    return launch_e_3d_fe_t<T, NX, tile_rows3<T>(0)>(a, s, false);
   }
+  // the three nodal components: twice the rows, as in pass A
+  if (a.emode == E_NODAL || a.emode == E_NOUT) return launch_e_3d_t<T, NX, tile_rows3<T>(2), 3>(a, s);
   if constexpr (NX >= 64) {
     if (a.var_e == 1) return launch_e_3d_t<T, NX, tile_rows3<T>(1)>(a, s);
     if (a.var_e == 2 && a.n[1] >= tile_rows3<T>(2)) return launch_e_3d_t<T, NX, tile_rows3<T>(2)>(a, s);
-    if (a.var_e == 4) return launch_e_3d_t<T, NX, tile_rows3<T>(0)>(a, s, true);
   }
   return launch_e_3d_t<T, NX, tile_rows3<T>(0)>(a, s);
 }
@@ -767,9 +787,7 @@ cudaError_t launch_y_3d_v(const PassArgs<T>& a, cudaStream_t s) {
     set_smem_attrs(k, sm);
     if (dev >= 0 && dev < kMaxDevices) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[dev], k, NT, sm);
   });
-  const bool din = (a.pmode == P_NODAL_IN || a.pmode == P_SOLVE);
-  const bool dout = (a.pmode == P_NODAL_OUT || a.pmode == P_SOLVE);
-  const int Cc = FWD ? (din ? 3 : a.m) : (dout ? 3 : a.m);
+  const int Cc = !fe_path(a) ? a.m : (!FWD && a.grads) ? 9 : 3;   // finite elements: w or its edge differences
   dim3 grid(a.n[2] / TZB, a.kx, a.L * Cc);
   if (sizeof(T) == 4) {
     PassArgs<T> b = a;
@@ -780,9 +798,27 @@ cudaError_t launch_y_3d_v(const PassArgs<T>& a, cudaStream_t s) {
   }
   return cudaGetLastError();
 }
+// Pass B of the finite elements from all components (forward).
+template <typename T, int NY, int V>
+cudaError_t launch_b_3d_fe(const PassArgs<T>& a, cudaStream_t s) {
+  constexpr int TZB = Tile3D<T>::TZB;
+    constexpr int NT = NY >= 128 ? NY : 128;
+  constexpr size_t sm = sizeof(cplx<T>) * (3 * TZB * FftSplit<NY, V>::LDO + 3 * TZB * (NY > 32 ? NY / 32 : 1));
+  auto k = pass_b_3d_fe<T, NY, TZB, NT, V>;
+  static DeviceOnce attr;
+  attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
+  k<<<dim3(a.n[2] / TZB, a.kx, a.L), NT, sm, s>>>(a);
+  return cudaGetLastError();
+}
 // Split variant of the y transforms (passes B and D): a.var_y.
 template <typename T, int NY, bool FWD>
 cudaError_t launch_y_3d_n(const PassArgs<T>& a, cudaStream_t s) {
+  if (FWD && fe_path(a) && a.pmode != P_NODAL_IN && a.pmode != P_SOLVE) {
+    if constexpr (fft_split_count<NY>() > 1) {
+      if (a.var_y == 1) return launch_b_3d_fe<T, NY, 1>(a, s);
+    }
+    return launch_b_3d_fe<T, NY, 0>(a, s);
+  }
   if constexpr (fft_split_count<NY>() > 1) {
     if (a.var_y == 1) return launch_y_3d_v<T, NY, FWD, 1>(a, s);
   }
@@ -794,43 +830,22 @@ template <typename T, int NY> cudaError_t launch_yf_3d_n(const PassArgs<T>& a, c
 template <typename T, int NY> cudaError_t launch_yb_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   return launch_y_3d_n<T, NY, false>(a, s);
 }
-// Pass C of the finite-element stress form with split variant V (a.var_c).
-template <typename T, int NZ, int V>
+// Pass C of the finite elements with split variant V (a.var_c): 8 pencils per
+// block (n_y >= 16).
+template <typename T, int NZ, int V, int W = 3>
 cudaError_t launch_c_3d_v(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int NT = fft_threads<NZ, 36, V>();
-  const size_t sm = sizeof(cplx<T>) * 36 * pass_c_ld<T, NZ, V>();
-  auto k = pass_c_3d<T, NZ, NT, V>;
+  constexpr int P = W == 9 ? 1 : 8;
+  constexpr int NT = fft_threads<NZ, W * P, V>();
+  const size_t sm = sizeof(cplx<T>) * W * P * FftSplit<NZ, V>::LD;
+  auto k = pass_c_3d_nodal<T, NZ, P, NT, V, W>;
   static DeviceOnce attr;
-  static int occ[kMaxDevices] = {0};
-  const int dev = current_device();
-  attr.run(dev, [&] {
-    set_smem_attrs(k, sm);
-    if (dev >= 0 && dev < kMaxDevices) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[dev], k, NT, sm);
-  });
-  dim3 grid(a.kx, a.n[1], a.L);
-  if (sizeof(T) == 4) {
-    PassArgs<T> b = a;
-    b.pf_ahead = prefetch_distance((dev >= 0 && dev < kMaxDevices) ? occ[dev] : 0, 2);
-    k<<<grid, NT, sm, s>>>(b);
-  } else {
-    k<<<grid, NT, sm, s>>>(a);
-  }
+  attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
+  k<<<dim3(a.kx, a.n[1] / P, a.L), NT, sm, s>>>(a);
   return cudaGetLastError();
 }
 
 template <typename T, int NZ>
 cudaError_t launch_c_3d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if (a.pmode == P_SOLVE) {
-    constexpr int P = 8;  // n_y >= 16
-    constexpr int NTn = fft_threads<NZ, 3 * P>();
-    const size_t smn = sizeof(cplx<T>) * 3 * P * FftSplit<NZ>::LD;
-    auto kn = pass_c_3d_nodal<T, NZ, P, NTn>;
-    static DeviceOnce attr_n;
-    attr_n.run(current_device(), [&] { set_smem_attrs(kn, smn); });
-    dim3 gridn(a.kx, a.n[1] / P, a.L);
-    kn<<<gridn, NTn, smn, s>>>(a);
-    return cudaGetLastError();
-  }
   if (a.pmode == P_FINITE) {
     constexpr int NTf = fft_threads<NZ, 54>();
     const size_t smf = sizeof(cplx<T>) * 54 * FftSplit<NZ>::LD;
@@ -841,7 +856,7 @@ cudaError_t launch_c_3d_n(const PassArgs<T>& a, cudaStream_t s) {
     kf<<<dim3(a.kx, a.n[1], a.L), NTf, smf, s>>>(a);
     return cudaGetLastError();
   }
-  if (a.nq == 1) {
+  if (!fe_path(a)) {
     constexpr int NT1 = fft_threads<NZ, 36>();
     const size_t sm1 = sizeof(cplx<T>) * 36 * FftSplit<NZ>::LD;
     auto k1 = pass_c_3d_q1<T, NZ, NT1>;
@@ -851,9 +866,9 @@ cudaError_t launch_c_3d_n(const PassArgs<T>& a, cudaStream_t s) {
     return cudaGetLastError();
   }
   if constexpr (fft_split_count<NZ>() > 1) {
-    if (a.var_c == 1) return launch_c_3d_v<T, NZ, 1>(a, s);
+    if (a.var_c == 1) return a.grads ? launch_c_3d_v<T, NZ, 1, 9>(a, s) : launch_c_3d_v<T, NZ, 1>(a, s);
   }
-  return launch_c_3d_v<T, NZ, 0>(a, s);
+  return a.grads ? launch_c_3d_v<T, NZ, 0, 9>(a, s) : launch_c_3d_v<T, NZ, 0>(a, s);
 }
 
 #define RVE_DISPATCH_N3(nval, FN, ...)                     \

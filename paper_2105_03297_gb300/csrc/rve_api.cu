@@ -12,8 +12,6 @@
 //   RVE_FP64 runs the inner solve in FP64 (normally one outer step);
 //   RVE_MIXED runs it in FP32 and refines until the FP64 residual meets the
 //   tolerance.
-#include <cuda.h>   // CUtensorMap and its encoder's signature (looked up through the runtime)
-
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -32,9 +30,6 @@
 using namespace rve;
 
 struct rve_s {
-  // TMA tensor map of the first spectrum (3D, FP32), for the pipelined last pass
-  CUtensorMap tm_spec;
-  bool tm_ok = false;
   int stall_copies = 0;  // test hook (rve_test_stall_copies)
   int dim = 0, n[3] = {1, 1, 1};
   int64_t N = 0;
@@ -245,45 +240,6 @@ void free_L(rve_s* h) {
   h->Lcap = 0;
 }
 
-// The driver's tensor-map encoder, looked up once through the runtime (no link
-// against the driver library); null if unavailable.
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn tensor_map_encoder() {
-  static EncodeTiledFn fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-    else
-      cudaGetLastError();
-  });
-  return fn;
-}
-
-// Tensor map of the first spectrum [slot][component][k_x][z][y] (complex FP32
-// copied as 8-byte elements), box = the pipelined last pass's tile: kPipeETY
-// values of y, one z, every k_x, the six components of a tetrahedron group.
-void make_spec_tensor_map(rve_s* h) {
-  h->tm_ok = false;
-  if (h->dim != 3 || h->tsize != 4 || h->n[0] < 128 || h->n[1] < kPipeETY || !h->spec) return;
-  EncodeTiledFn enc = tensor_map_encoder();
-  if (!enc) return;
-  const cuuint64_t ny = (cuuint64_t)h->n[1], nz = (cuuint64_t)h->n[2], kx = (cuuint64_t)h->kx;
-  const cuuint64_t dims[4] = {ny, nz, kx, (cuuint64_t)h->Lcap * h->m};
-  const cuuint64_t strides[3] = {ny * 8, nz * ny * 8, kx * nz * ny * 8};
-  const cuuint32_t box[4] = {(cuuint32_t)kPipeETY, 1, (cuuint32_t)kx, 6};
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  const CUresult r = enc(&h->tm_spec, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, h->spec, dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  h->tm_ok = (r == CUDA_SUCCESS);
-}
-
 // Buffers for L load cases (grown, never shrunk).
 int ensure_capacity(rve_s* h, int L) {
   if (L <= h->Lcap) return RVE_OK;
@@ -339,7 +295,6 @@ int ensure_capacity(rve_s* h, int L) {
   if (keep_u) cudaFree(keep_u);
   CK(se);
   h->Lcap = L;
-  make_spec_tensor_map(h);
   CK(cudaGetLastError());
   return RVE_OK;
 }
@@ -374,7 +329,6 @@ template <typename T> PassArgs<T> pass_args(const rve_s* h, int L, double* u, co
   a.var_e = h->var[1] < 0 ? 0 : h->var[1];
   a.var_c = h->var[2] < 0 ? 0 : h->var[2];
   a.var_y = h->var[3] < 0 ? 0 : h->var[3];
-  a.tm_spec = h->tm_ok ? static_cast<const void*>(&h->tm_spec) : nullptr;
   a.stall_copies = h->stall_copies;
   return a;
 }
@@ -421,22 +375,18 @@ template <typename T> cudaError_t apply_passes(rve_s* h, const PassArgs<T>& a) {
 
 // One projected-CG iteration in the factored nodal form:
 //   force stencil (p update, material, f = B_r^T C p, alpha)
-//   -> FFT passes on the D nodal components with w^ = (B^H B)^-1 f^
-//   -> strain update (q = B_r w, r -= alpha q, beta).
+//   -> FFT passes on the D nodal components with w^ = (B^H B)^-1 f^, the last
+//      of which updates the strains (q = B_r w, r -= alpha q, beta).
 // Iteration parity q writes the direction to {p, p2}[q] and reads the previous
-// one from the other buffer.  f and w are carved out of fbuf (idle during CG).
+// one from the other buffer.  f is carved out of fbuf (idle during CG).
 template <typename T> cudaError_t apply_factored(rve_s* h, const PassArgs<T>& a, int parity) {
   T* P[2] = {(T*)h->p, (T*)h->p2};
   T* f = (T*)h->fbuf;
-  T* w = f + (size_t)a.L * h->D * h->N;
   cudaError_t e = timed(h, K_FS, [&] { return launch_force_stencil<T>(a, P[parity ^ 1], P[parity], f, h->stream); });
   PassArgs<T> b = a;
-  b.amode = A_NODAL; b.pmode = P_SOLVE; b.emode = E_NOUT;
-  b.in = f; b.out = w;
-  if (e == cudaSuccess) e = pass_a<T>(h, b);
-  if (e == cudaSuccess) e = pass_mid<T>(h, b);
-  if (e == cudaSuccess) e = pass_e<T>(h, b);
-  if (e == cudaSuccess) e = timed(h, K_SU, [&] { return launch_strain_update<T>(a, w, h->stream); });
+  b.amode = A_NODAL; b.pmode = P_SOLVE; b.emode = E_CG;
+  b.in = f;
+  if (e == cudaSuccess) e = apply_passes<T>(h, b);
   return e;
 }
 
@@ -550,7 +500,7 @@ int rve_sched_candidates(const rve_s* h, int which) {
   switch (which) {
     case 0: return (h->dim == 3 && h->tsize == 4 && h->n[0] >= 128) ? 7
                  : (h->dim == 2 && h->tsize == 4 && h->n[0] >= 512) ? 6 : h->n[0] >= 64 ? 5 : 3;
-    case 1: return (h->dim == 3 && h->tsize == 4 && h->n[0] >= 128 && h->tm_ok) ? 5 : 3;
+    case 1: return (h->dim == 3 && h->tsize == 4 && h->n[0] >= 128) ? 5 : 3;
     case 2: return split_count(h->n[h->dim - 1]);
     default: return h->dim == 3 ? split_count(h->n[1]) : 1;
   }
@@ -629,7 +579,10 @@ template <typename T> int autotune(rve_s* h, int L) {
       float ms = 0.f;
       CK(cudaEventElapsedTime(&ms, e0, e1));
       h->tune_ms[which][v] = ms / 3.0f;
-      if (ms < best_ms) { best_ms = ms; best[which] = v; }
+      // a later candidate has to win by more than the timing differs from run to
+      // run (3% and 0.5 us per launch): on small grids, where the candidates are
+      // alike, the choice then does not change between handles and load cases
+      if (ms < 0.97f * best_ms - 0.0015f) { best_ms = ms; best[which] = v; }
     }
     *(which == 0 ? &a.var_a : which == 1 ? &a.var_e : which == 2 ? &a.var_c : &a.var_y) = best[which];
   }
@@ -1823,12 +1776,12 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
   if (h->finite && apply_material) return RVE_ERR_ARG;
   if (h->tsize == 4) {
     PassArgs<float> a = pass_args<float>(h, 1, h->u, h->emac_d);
-    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = P_G; a.emode = E_OUT;
+    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = P_G; a.emode = E_OUT; a.grads = 1;
     a.in = (const float*)h->fbuf; a.out = (float*)h->x;
     CK(apply_passes<float>(h, a));
   } else {
     PassArgs<double> a = pass_args<double>(h, 1, h->u, h->emac_d);
-    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = h->finite ? P_FINITE : P_G; a.emode = E_OUT;
+    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = h->finite ? P_FINITE : P_G; a.emode = E_OUT; a.grads = 1;
     a.in = (const double*)h->fbuf; a.out = (double*)h->x;
     CK(apply_passes<double>(h, a));
   }

@@ -43,7 +43,20 @@ struct CgState {
   double fa2;        // squared norm of the summed magnitudes of the terms of f (round-off scale)
   int it, maxit, status, active;  // active: the outer refinement still runs this load case
   unsigned cnt_a, cnt_e, cnt_r, pad;
+  float alpha_f, beta_f;  // alpha and beta rounded to FP32, for the FP32 passes (see cg_alpha)
 };
+// alpha and beta in the passes' precision.  A conversion from FP64 runs on the
+// FP64 pipe, which handles a warp in 16 cycles: with one conversion per thread
+// the passes of a 128^3 grid spent a tenth of their time there, so the kernel
+// that finishes the scalar also stores its FP32 rounding.
+template <typename T> __device__ __forceinline__ T cg_alpha(const CgState* cg) {
+  if constexpr (sizeof(T) == 4) return cg->alpha_f;
+  else return cg->alpha;
+}
+template <typename T> __device__ __forceinline__ T cg_beta(const CgState* cg) {
+  if constexpr (sizeof(T) == 4) return cg->beta_f;
+  else return cg->beta;
+}
 
 // ST_HOLD: set up for a new inner solve but not yet released to the CG
 // kernels (a batch handle whose next refinement step is being prepared while
@@ -52,11 +65,9 @@ enum { ST_RUN = 0, ST_CONV = 1, ST_MAXIT = 2, ST_BAD = 3, ST_HOLD = 4 };
 // CgState::pad of a slot whose kernel gave up a bounded device-side wait
 // (status ST_BAD); the host reports RVE_ERR_TIMEOUT for it.
 constexpr unsigned kTimeoutMark = 0x7107u;
-// The pipelined persistent passes (pass3d_pipe.cuh): load-case slots their
-// per-slot partial sums hold, and the rows per tile of the last pass (the
-// height of its spectrum tensor map's box).
+// Load-case slots the per-slot partial sums of the pipelined persistent first
+// pass (pass3d_pipe.cuh) hold.
 constexpr int kPipeMaxL = 64;
-constexpr int kPipeETY = 4;
 
 // ------------------------------------------------------- FFT in shared memory
 __host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n / 2); }
@@ -564,17 +575,6 @@ template <typename T> __device__ __forceinline__ void vload(T* d, const T* s) {
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
-// Prefetch `rows` contiguous rows of NX values, `rows_per_comp` per component
-// (components comp_stride apart): one bulk request per row.
-template <typename T, int NX>
-__device__ __forceinline__ void prefetch_rows_l2(const T* base, int comps, int rows_per_comp, int64_t comp_stride) {
-  static_assert((NX * sizeof(T)) % 16 == 0, "bulk prefetch sizes are multiples of 16 bytes");
-  for (int i = threadIdx.x; i < comps * rows_per_comp; i += blockDim.x) {
-    const int j = i / rows_per_comp, row = i % rows_per_comp;
-    prefetch_l2_bulk(base + j * comp_stride + (int64_t)row * NX, (unsigned)(NX * sizeof(T)));
-  }
-}
-
 // Two consecutive complex values (16 bytes for float, two 16-byte halves for double)
 template <typename T> __device__ __forceinline__ void cload2(cplx<T>* d, const cplx<T>* s) {
   if constexpr (sizeof(T) == 4) {
@@ -663,6 +663,26 @@ template <int NT> __device__ __forceinline__ double block_sum(double v, double* 
     for (int i = 0; i < NT / 32; ++i) s += red[i];
   }
   return s;  // valid in thread 0
+}
+
+// Sum over the block of one value per thread, in FP64: every thread leaves its
+// value (FP32 or FP64) in cols[NT], one warp adds the columns of all warps and
+// then its lanes.  The FP64 pipe takes 16 cycles per warp instruction, so what
+// counts is the number of FP64 warp instructions: NT/32 conversions and
+// additions and 5 shuffled additions here, against 6 NT/32 when every warp
+// reduces itself (block_sum).  cols must not be in use; the sum is valid in
+// thread 0.
+template <int NT, typename T> __device__ __forceinline__ double block_sum_cols(T v, T* cols) {
+  cols[threadIdx.x] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) s += (double)cols[w * 32 + threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  }
+  return s;
 }
 
 // Publish this block's partial and report whether it is the last block of

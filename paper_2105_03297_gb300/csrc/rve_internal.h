@@ -67,11 +67,12 @@ template <typename T> struct PassArgs {
   int var_a, var_e;  // tile variants of passes A (0..6) and E (0..4): see the launchers
   int var_c, var_y;  // FFT split variants (FftSplit<N, V>) of pass C's axis and of passes B / D (3D)
   int comp_in;       // number of components in the spectrum for this pass (m or D)
-  const void* tm_spec;  // host copy of the TMA tensor map of the first spectrum (3D FP32), or null
-  int stall_copies;     // test hook: the pipelined passes issue no copies, so their bounded waits run out
-  int pf_ahead;      // 3D passes A and E: blocks ahead in launch order whose rows each block asks the TMA
-                     // unit to prefetch into L2 (tile variants A 6 and E 4), 0 = none
+  int stall_copies;     // test hook: the pipelined pass issues no copies, so its bounded waits run out
+  int pf_ahead;      // 3D passes A to D: blocks ahead in launch order whose input each block asks the TMA
+                     // unit to prefetch into L2, 0 = none; pass E: 1 = prefetch the tile's own r rows
   int deriv;         // Deriv
+  int grads;         // finite elements: passes C, D and E carry the D^2 edge differences of w instead of its D
+                     // components (see pass_c_2d_fe), for results that leave the library as they are
 };
 
 // Arguments of the FP64 real-space kernels (residual, homogenisation, adjoint).
@@ -101,7 +102,6 @@ template <typename T> cudaError_t launch_cg_finish_x(const PassArgs<T>& a, cudaS
 // factored nodal form of the operator
 template <typename T>
 cudaError_t launch_force_stencil(const PassArgs<T>& a, const T* pold, T* pnew, T* f, cudaStream_t s);
-template <typename T> cudaError_t launch_strain_update(const PassArgs<T>& a, const T* w, cudaStream_t s);
 // nodal-state form
 template <typename T>
 cudaError_t launch_nodal_force(const PassArgs<T>& a, const T* rho, const T* pold, T* pnew, T* xi, T* f,
