@@ -349,15 +349,11 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs
 }
 
 // Pass C of the finite elements: w^ = (B^H B)^-1 t^ for P k_x columns per
-// block; w(k_x, y), the D = 2 nodal components after the inverse FFT along y,
-// goes to components 0 and 1 of the spectrum.  With COMBINE the input is the
-// x-transformed stresses of all six components and t = B^H sigma is formed
-// before the y transform: a factor exp(-i k_y h) is a shift by one row, so
-// with dx = (exp(-i k_x h) - 1)/h and s0, s1 the stresses of the two triangles
-//   t_j(y) = U_j(y) + V_j(y-1),   W_j = (s0_yj + exp(-i k_x h) s1_yj)/h_y,
-//   U_j = dx s0_xj - W_j,         V_j = W_j + dx s1_xj,
-// and only two columns per k_x are transformed there and back instead of six.
-// Without COMBINE components 0 and 1 hold t(k_x, y) (nodal forces).
+// block, from t(k_x, y) in components 0 and 1 of the spectrum (pass A or the
+// force pass) to w(k_x, y) in place.  Bound by the FFT arithmetic (80
+// registers at 512 and 1024 points: six blocks of four warps per SM; at 150
+// registers and three blocks the 1024^2 pass took 65 us, now 48 with the
+// combination of all six components it then still did).
 // W = 4 (P = 1) writes the differences d_a w_j along the element edges,
 // d_a = (exp(i k_a h_a) - 1)/h_a, as components 2 a + j: the last pass then
 // only picks them up at the right nodes.  Differences of w itself, taken there
@@ -365,11 +361,9 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs
 // field (measured at 1024^2 in FP32: 1.0e-5 against 1.2e-6 of the 2-norm; on
 // white noise 4.3e-7 against 3.1e-7).  Inside the CG that error is corrected
 // by the FP64 refinement, so W = 2 is used there, W = 4 for rve_apply_operator.
-// Bound by the spectrum traffic (COMBINE: 6 columns in, 2 out).  Consecutive
-// lanes hold consecutive rows, so V(y-1) comes by a shuffle; lane 0 and row 0
-// load row y-1 themselves.  Row b of the buffer is component b % 2 of column
-// kx0 + b / 2; columns past n_x/2 are skipped.  grid (ceil((n_x/2+1) / P), L).
-template <typename T, int NY, int P, int NT, int V, bool COMBINE, int W>
+// Row b of the buffer is component b % 2 of column kx0 + b / 2; columns past
+// n_x/2 are skipped.  grid (ceil((n_x/2+1) / P), L).
+template <typename T, int NY, int P, int NT, int V, int W>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) pass_c_2d_fe(PassArgs<T> a) {
   using C = cplx<T>;
   constexpr int R = 2 * P;
@@ -386,55 +380,10 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
   C* base = a.spec + ((int64_t)l * a.m * KX + kx0) * NY;
   auto st_s = [&](int b, int k, C v) { buf[b * LD + k] = v; };
   auto ld_s = [&](int b, int y) -> C { return buf[b * LD + y]; };
-  if constexpr (COMBINE) {
-    const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
-    for (int i0 = 0; i0 < P * NY; i0 += NT) {   // whole warps: every lane takes part in the shuffles
-      const int i = i0 + threadIdx.x;
-      const int pc = i / NY, y = i % NY;
-      const bool on = i < P * NY && kx0 + pc < KX;
-      C u[2], v[2], vp[2];
-      u[0] = u[1] = v[0] = v[1] = vp[0] = vp[1] = mkc<T>(0, 0);
-      C cex = mkc<T>(1, 0), dx = mkc<T>(0, 0);
-      const C* col = base + (int64_t)pc * NY;
-      if (on) {
-        cex = cconj(a.ph[0][kx0 + pc]);
-        dx = cscale(csub(cex, mkc<T>(1, 0)), ihx);
-        C s[6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) s[c] = col[c * cstride + y];
-        s[2] = cscale(s[2], r2); s[5] = cscale(s[5], r2);
-        const C w0 = cscale(cadd(s[2], cmul(cex, s[5])), ihy);
-        const C w1 = cscale(cadd(s[1], cmul(cex, s[4])), ihy);
-        u[0] = csub(cmul(dx, s[0]), w0); u[1] = csub(cmul(dx, s[2]), w1);
-        v[0] = cadd(cmul(dx, s[3]), w0); v[1] = cadd(cmul(dx, s[5]), w1);
-      }
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        vp[j].x = __shfl_up_sync(0xffffffffu, v[j].x, 1);
-        vp[j].y = __shfl_up_sync(0xffffffffu, v[j].y, 1);
-      }
-      if (on) {
-        if ((threadIdx.x & 31) == 0 || y == 0) {
-          const int ym = (y + NY - 1) & (NY - 1);
-          const C s1 = col[cstride + ym], s2 = cscale(col[2 * cstride + ym], r2), s3 = col[3 * cstride + ym];
-          const C s4 = col[4 * cstride + ym], s5 = cscale(col[5 * cstride + ym], r2);
-          vp[0] = cadd(cmul(dx, s3), cscale(cadd(s2, cmul(cex, s5)), ihy));
-          vp[1] = cadd(cmul(dx, s5), cscale(cadd(s1, cmul(cex, s4)), ihy));
-        }
-        buf[2 * pc * LD + y] = cadd(u[0], vp[0]);
-        buf[(2 * pc + 1) * LD + y] = cadd(u[1], vp[1]);
-      } else if (i < P * NY) {
-        buf[2 * pc * LD + y] = buf[(2 * pc + 1) * LD + y] = mkc<T>(0, 0);
-      }
-    }
-    __syncthreads();
-    fft4<T, NY, R, LD, NT, -1, true, true, false, false, V>(buf, a.tw[1], ld_s, st_s);
-  } else {
-    auto ld_g = [&](int b, int y) -> C {
-      return (kx0 + b / 2 < KX) ? base[(b % 2) * cstride + (int64_t)(b / 2) * NY + y] : mkc<T>(0, 0);
-    };
-    fft4<T, NY, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
-  }
+  auto ld_g = [&](int b, int y) -> C {
+    return (kx0 + b / 2 < KX) ? base[(b % 2) * cstride + (int64_t)(b / 2) * NY + y] : mkc<T>(0, 0);
+  };
+  fft4<T, NY, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
   for (int i = threadIdx.x; i < P * NY; i += NT) {
     const int pc = i / NY, ky = i % NY, kx = kx0 + pc;
     if (kx >= KX) continue;
@@ -666,7 +615,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NPR][LD]
   __shared__ double red[NT / 32];
-  __shared__ T cols[NT];
+  __shared__ T cols[2 * NT];
   __shared__ int flag;
   const int l = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1];
@@ -679,7 +628,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   const bool cgm = a.emode == E_CG;
   const T alpha = cgm ? cg_alpha<T>(cg) : (T)0;
   const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
-  T acc = 0;
+  Acc<T> acc;
   for (int i = threadIdx.x; i < TY * (NX / VL); i += NT) {
     const int yy = i / (NX / VL), x0 = (i % (NX / VL)) * VL, pr = yy / 2;
     const int64_t v0 = (int64_t)l * a.m * a.N + (int64_t)(y0 + yy) * NX + x0;
@@ -719,11 +668,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
       q[4][k] = (hi[1][k + 1] - lo[1][k + 1]) * ihy;
       q[5][k] = r2 * ((hi[0][k + 1] - lo[0][k + 1]) * ihy + (hi[1][k + 1] - hi[1][k]) * ihx);
     }
+    T s = 0;
 #pragma unroll
-    for (int c = 0; c < 6; ++c) acc += strain_update<T, VL>(a, v0 + c * a.N, rv[c], q[c], alpha);
+    for (int c = 0; c < 6; ++c) s += strain_update<T, VL>(a, v0 + c * a.N, rv[c], q[c], alpha);
+    acc.add(s);
   }
   if (a.emode == E_CG || a.emode == E_INIT) {
-    const double s = block_sum_cols<NT>(acc, cols);
+    const double s = block_sum_acc<NT>(acc, cols);
     double* part = a.part + (int64_t)l * a.part_stride;
     if (publish_partial(s, part, &cg->cnt_e, blockIdx.x, gridDim.x, &flag)) {
       const double rr = sum_partials<NT>(part, gridDim.x, red);
@@ -844,6 +795,8 @@ cudaError_t launch_e_2d_n(const PassArgs<T>& a, cudaStream_t s) {
       if (a.var_e == 1) return launch_e_2d_fe_t<T, NX, tile_rows<T>(1)>(a, s);
       if (a.var_e == 2 && a.n[1] >= tile_rows<T>(2)) return launch_e_2d_fe_t<T, NX, tile_rows<T>(2)>(a, s);
     }
+    // variant 0: half the rows where the default ones leave SMs without a block
+    if ((int64_t)a.n[1] * a.L / tile_rows<T>(0) < device_sm_count()) return launch_e_2d_fe_t<T, NX, tile_rows<T>(1)>(a, s);
     return launch_e_2d_fe_t<T, NX, tile_rows<T>(0)>(a, s);
   }
   if constexpr (NX >= 64) {
@@ -855,36 +808,26 @@ cudaError_t launch_e_2d_n(const PassArgs<T>& a, cudaStream_t s) {
 // Pass C of the finite elements with split variant V (a.var_c): P columns per
 // block.  FP64 runs one column per block (its transforms are bound by the FP64
 // pipe, so the work is spread over as many SMs as there are columns).
-template <typename T, int NY, int V, bool COMBINE, int W = 2>
+template <typename T, int NY, int V, int W>
 cudaError_t launch_c_2d_v(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int P = (sizeof(T) == 8 || W == 4) ? 1 : NY >= 256 ? 2 : 4;
   constexpr int NT = fft_threads<NY, W * P, V>();
   const size_t sm = sizeof(cplx<T>) * W * P * FftSplit<NY, V>::LD;
-  auto k = pass_c_2d_fe<T, NY, P, NT, V, COMBINE, W>;
+  auto k = pass_c_2d_fe<T, NY, P, NT, V, W>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   k<<<dim3((a.kx + P - 1) / P, a.L), NT, sm, s>>>(a);
   return cudaGetLastError();
 }
-template <typename T, int NY, bool COMBINE>
-cudaError_t launch_c_2d_fe(const PassArgs<T>& a, cudaStream_t s) {
-  if constexpr (fft_split_count<NY>() > 1) {
-    if constexpr (COMBINE) {
-      if (a.grads && a.var_c == 1) return launch_c_2d_v<T, NY, 1, COMBINE, 4>(a, s);
-    }
-    if (a.var_c == 1) return launch_c_2d_v<T, NY, 1, COMBINE>(a, s);
-  }
-  if constexpr (COMBINE) {
-    if (a.grads) return launch_c_2d_v<T, NY, 0, COMBINE, 4>(a, s);
-  }
-  return launch_c_2d_v<T, NY, 0, COMBINE>(a, s);
-}
 
 template <typename T, int NY>
 cudaError_t launch_c_2d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if (fe_path(a))
-    return (a.pmode == P_NODAL_IN || a.pmode == P_SOLVE) ? launch_c_2d_fe<T, NY, false>(a, s)
-                                                         : launch_c_2d_fe<T, NY, true>(a, s);
+  if (fe_path(a)) {
+    if constexpr (fft_split_count<NY>() > 1) {
+      if (a.var_c == 1) return a.grads ? launch_c_2d_v<T, NY, 1, 4>(a, s) : launch_c_2d_v<T, NY, 1, 2>(a, s);
+    }
+    return a.grads ? launch_c_2d_v<T, NY, 0, 4>(a, s) : launch_c_2d_v<T, NY, 0, 2>(a, s);
+  }
   if (a.nq == 3) {
     constexpr int NT3 = fft_threads<NY, 9>();
     const size_t sm3 = sizeof(cplx<T>) * 9 * FftSplit<NY>::LD;

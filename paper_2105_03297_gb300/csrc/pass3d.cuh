@@ -176,7 +176,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT <= 256 ? 4 : 2) : 1) 
     const int64_t cb2 = (((int64_t)(lc2 / Cc) * a.m + lc2 % Cc) * KX + kx2);
     const int z2 = zb2 * TZB;
     if (FWD) {
-      if (threadIdx.x == 0) prefetch_l2_bulk(a.spec + (cb2 * nz + z2) * NY, (unsigned)(TZB * NY * sizeof(C)));
+      if (threadIdx.x < (a.pair ? 2 : 1))
+        prefetch_l2_bulk(a.spec + ((cb2 + 3 * (int64_t)threadIdx.x * KX) * nz + z2) * NY, (unsigned)(TZB * NY * sizeof(C)));
     } else {
       for (int k = threadIdx.x; k < NY; k += blockDim.x)
         prefetch_l2_bulk(a.spec2 + cb2 * NY * nz + z2 + (int64_t)k * nz, (unsigned)(TZB * sizeof(C)));
@@ -184,9 +185,17 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT <= 256 ? 4 : 2) : 1) 
   }
   if (FWD) {
     // step 1 reads whole y-pencils, step 2 writes z-chunks (zz fastest)
-    auto ld = [&](int zz, int y) -> C { return pencils[(int64_t)zz * NY + y]; };
     auto st = [&](int zz, int k, C v) { chunks[(int64_t)k * nz + zz] = v; };
-    fft4<T, NY, TZB, LD, NT, -1, false, false, false, true, V>(buf, a.tw[1], ld, st);
+    if (a.pair) {   // the two parts of the nodal forces (force_3d)
+      const C* other = pencils + 3 * (int64_t)KX * nz * NY;
+      auto ld = [&](int zz, int y) -> C {
+        return cadd(pencils[(int64_t)zz * NY + y], other[(int64_t)zz * NY + y]);
+      };
+      fft4<T, NY, TZB, LD, NT, -1, false, false, false, true, V>(buf, a.tw[1], ld, st);
+    } else {
+      auto ld = [&](int zz, int y) -> C { return pencils[(int64_t)zz * NY + y]; };
+      fft4<T, NY, TZB, LD, NT, -1, false, false, false, true, V>(buf, a.tw[1], ld, st);
+    }
   } else {
     auto ld = [&](int zz, int k) -> C { return chunks[(int64_t)k * nz + zz]; };
     auto st = [&](int zz, int y, C v) { pencils[(int64_t)zz * NY + y] = v; };
@@ -552,7 +561,7 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NR][LD]
   __shared__ double red[NT / 32];
-  __shared__ T cols[NT];
+  __shared__ T cols[2 * NT];
   __shared__ int flag;
   const int l = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1], nz = a.n[2];
@@ -597,7 +606,7 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   const T alpha = cgm ? cg_alpha<T>(cg) : (T)0;
   const T ih[3] = {a.ih[0], a.ih[1], a.ih[2]};
   const T r2 = (T)kInvSqrt2;
-  T acc = 0;
+  Acc<T> acc;
   for (int i = threadIdx.x; i < TY * NX; i += NT) {
     const int yy = i / NX, x = i % NX;
     const int64_t v0 = vox0 + (int64_t)yy * NX + x;
@@ -613,6 +622,7 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
       const C v = n[j][(c >> 1) & 1][c & 1];
       return (c & 4) ? v.y : v.x;
     };
+    T vs = 0;
 #pragma unroll
     for (int t = 0; t < 6; ++t) {
       T rv[6];
@@ -632,11 +642,12 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
       const T q[6] = {H[0][0], H[1][1], H[2][2], r2 * (H[1][2] + H[2][1]), r2 * (H[0][2] + H[2][0]),
                       r2 * (H[0][1] + H[1][0])};
 #pragma unroll
-      for (int s = 0; s < 6; ++s) acc += strain_update<T, 1>(a, v0 + (6 * t + s) * N, &rv[s], &q[s], alpha);
+      for (int s = 0; s < 6; ++s) vs += strain_update<T, 1>(a, v0 + (6 * t + s) * N, &rv[s], &q[s], alpha);
     }
+    acc.add(vs);
   }
   if (cgm || a.emode == E_INIT) {
-    const double s = block_sum_cols<NT>(acc, cols);
+    const double s = block_sum_acc<NT>(acc, cols);
     const int nblk = gridDim.x * gridDim.y, blk = blockIdx.x + gridDim.x * blockIdx.y;
     double* part = a.part + (int64_t)l * a.part_stride;
     if (publish_partial(s, part, &cg->cnt_e, blk, nblk, &flag)) {
@@ -813,7 +824,7 @@ cudaError_t launch_b_3d_fe(const PassArgs<T>& a, cudaStream_t s) {
 // Split variant of the y transforms (passes B and D): a.var_y.
 template <typename T, int NY, bool FWD>
 cudaError_t launch_y_3d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if (FWD && fe_path(a) && a.pmode != P_NODAL_IN && a.pmode != P_SOLVE) {
+  if (FWD && fe_path(a) && !a.pair && a.pmode != P_NODAL_IN && a.pmode != P_SOLVE) {
     if constexpr (fft_split_count<NY>() > 1) {
       if (a.var_y == 1) return launch_b_3d_fe<T, NY, 1>(a, s);
     }

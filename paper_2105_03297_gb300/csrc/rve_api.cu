@@ -49,7 +49,6 @@ struct rve_s {
   double* E64 = nullptr;
   void* Ein = nullptr;  // E in the inner precision (aliases E64 for FP64)
   void* x = nullptr; void* r = nullptr; void* p = nullptr;
-  void* p2 = nullptr;   // second direction buffer (factored operator form only)
   void* fbuf = nullptr;
   void* spec = nullptr; void* spec2 = nullptr;
   double* u = nullptr;
@@ -230,7 +229,7 @@ int64_t spec_elems(const rve_s* h) {
 }
 
 void free_L(rve_s* h) {
-  free_dev(h->x); free_dev(h->r); free_dev(h->p); free_dev(h->p2); free_dev(h->fbuf);
+  free_dev(h->x); free_dev(h->r); free_dev(h->p); free_dev(h->fbuf);
   free_devp(h->Fs); free_devp(h->fmac_d);
   free_dev(h->spec); free_dev(h->spec2);
   free_devp(h->u); free_devp(h->uadj); free_devp(h->part); free_devp(h->cg);
@@ -269,8 +268,6 @@ int ensure_capacity(rve_s* h, int L) {
       (rc = dev_alloc(&h->fbuf, fld)) || (rc = dev_alloc(&h->spec, sp)))
     { free_L(h); if (keep_u) cudaFree(keep_u); return rc; }
   if (h->dim == 3 && (rc = dev_alloc(&h->spec2, sp))) { free_L(h); if (keep_u) cudaFree(keep_u); return rc; }
-  if (h->op_form == RVE_FORM_FACTORED && (rc = dev_alloc(&h->p2, fld)))
-    { free_L(h); if (keep_u) cudaFree(keep_u); return rc; }
   if ((rc = dev_alloc((void**)&h->u, (size_t)L * h->D * h->N * sizeof(double))) ||
       (rc = dev_alloc((void**)&h->uadj, (size_t)h->ns * h->D * h->N * sizeof(double))))
     { free_L(h); if (keep_u) cudaFree(keep_u); return rc; }
@@ -286,7 +283,6 @@ int ensure_capacity(rve_s* h, int L) {
     cudaGetLastError(); free_L(h); if (keep_u) cudaFree(keep_u); return RVE_ERR_OOM;
   }
   cudaMemsetAsync(h->p, 0, fld, h->stream);
-  if (h->p2) cudaMemsetAsync(h->p2, 0, fld, h->stream);
   cudaMemsetAsync(h->x, 0, fld, h->stream);
   cudaMemsetAsync(h->part, 0, (size_t)Lp * h->part_stride * sizeof(double), h->stream);
   if (keep_u)
@@ -297,6 +293,24 @@ int ensure_capacity(rve_s* h, int L) {
   h->Lcap = L;
   CK(cudaGetLastError());
   return RVE_OK;
+}
+
+// Whether the first pass of an iteration is the force pass (small-strain finite
+// elements); the pipelined first pass (stress form, tile variant 5) transforms
+// the stresses instead.
+bool force_pass(const rve_s* h, int var_a) {
+  if (h->deriv != D_FE || h->finite) return false;
+  return !(h->op_form == RVE_FORM_STRESS && var_a == 5 && h->dim == 3 && h->tsize == 4 && h->n[0] >= 128);
+}
+// The force pass on strain fields with iteration parity q: the direction
+// alternates between p and fbuf (idle during CG), because the row below a tile
+// is read by two blocks.
+template <typename T> void set_force(const rve_s* h, PassArgs<T>& a, int q) {
+  T* P[2] = {(T*)h->p, (T*)h->fbuf};
+  a.force = 1;
+  a.pair = h->dim == 3;
+  a.pold = P[q ^ 1];
+  a.pnew = P[q];
 }
 
 template <typename T> PassArgs<T> pass_args(const rve_s* h, int L, double* u, const double* emac) {
@@ -311,7 +325,7 @@ template <typename T> PassArgs<T> pass_args(const rve_s* h, int L, double* u, co
   a.E = (const T*)h->Ein;
   a.lcs = h->lcs > 0 ? h->lcs : L;
   a.x = (T*)h->x; a.r = (T*)h->r; a.p = (T*)h->p;
-  a.p2 = h->op_form == RVE_FORM_FACTORED ? (T*)h->p2 : nullptr;
+  a.p2 = force_pass(h, h->var[0]) ? (T*)h->fbuf : nullptr;
   a.in = (const T*)h->fbuf; a.out = (T*)h->fbuf;
   a.u64 = u;
   a.spec = (cplx<T>*)h->spec; a.spec2 = (cplx<T>*)h->spec2;
@@ -347,7 +361,9 @@ Fp64Args fp64_args(const rve_s* h, int L, const double* u, const double* emac, C
 }
 
 template <typename T> cudaError_t pass_a(rve_s* h, const PassArgs<T>& a) {
-  return timed(h, a.cgphase ? K_A : K_OTHER, [&] {
+  const int kind = !a.cgphase ? K_OTHER : a.force && h->op_form != RVE_FORM_STRESS ? K_FS : K_A;
+  return timed(h, kind, [&] {
+    if (a.force) return h->dim == 2 ? launch_force_2d<T>(a, h->stream) : launch_force_3d<T>(a, h->stream);
     return h->dim == 2 ? launch_pass_a_2d<T>(a, h->stream) : launch_pass_a_3d<T>(a, h->stream);
   });
 }
@@ -373,23 +389,6 @@ template <typename T> cudaError_t apply_passes(rve_s* h, const PassArgs<T>& a) {
   return e;
 }
 
-// One projected-CG iteration in the factored nodal form:
-//   force stencil (p update, material, f = B_r^T C p, alpha)
-//   -> FFT passes on the D nodal components with w^ = (B^H B)^-1 f^, the last
-//      of which updates the strains (q = B_r w, r -= alpha q, beta).
-// Iteration parity q writes the direction to {p, p2}[q] and reads the previous
-// one from the other buffer.  f is carved out of fbuf (idle during CG).
-template <typename T> cudaError_t apply_factored(rve_s* h, const PassArgs<T>& a, int parity) {
-  T* P[2] = {(T*)h->p, (T*)h->p2};
-  T* f = (T*)h->fbuf;
-  cudaError_t e = timed(h, K_FS, [&] { return launch_force_stencil<T>(a, P[parity ^ 1], P[parity], f, h->stream); });
-  PassArgs<T> b = a;
-  b.amode = A_NODAL; b.pmode = P_SOLVE; b.emode = E_CG;
-  b.in = f;
-  if (e == cudaSuccess) e = apply_passes<T>(h, b);
-  return e;
-}
-
 // Nodal-state buffers: xi, rho[2], pi[2], f, w, each [L][D][N] of the inner
 // precision, carved out of the strain-form fields (m >= 2 D components).
 template <typename T> struct NodalBufs {
@@ -404,19 +403,16 @@ template <typename T> struct NodalBufs {
 };
 
 // One projected-CG iteration on the nodal state (parity q of the iteration):
-// force kernel (pi, xi, f = B^T C B pi, alpha) -> FFT passes with
-// w^ = (B^H B)^-1 f^ -> update kernel (rho -= alpha w, <B rho, B rho>, beta).
+// force pass (pi, xi, f = B^T C B pi, alpha), the other FFT passes with
+// w^ = (B^H B)^-1 f^, update kernel (rho -= alpha w, <B rho, B rho>, beta).
 template <typename T> cudaError_t apply_nodal(rve_s* h, const PassArgs<T>& a, int q) {
   NodalBufs<T> nb(h, a.L);
-  cudaError_t e = timed(h, K_FS, [&] {
-    return launch_nodal_force<T>(a, nb.rho[q], nb.pi[q ^ 1], nb.pi[q], nb.xi, nb.f, h->stream);
-  });
   PassArgs<T> b = a;
-  b.amode = A_NODAL; b.pmode = P_SOLVE; b.emode = E_NOUT;
-  b.in = nb.f; b.out = nb.w;
-  if (e == cudaSuccess) e = pass_a<T>(h, b);
-  if (e == cudaSuccess) e = pass_mid<T>(h, b);
-  if (e == cudaSuccess) e = pass_e<T>(h, b);
+  b.amode = A_CG; b.pmode = P_G; b.emode = E_NOUT;
+  b.force = 2; b.pair = h->dim == 3;
+  b.rho = nb.rho[q]; b.pold = nb.pi[q ^ 1]; b.pnew = nb.pi[q]; b.xi = nb.xi;
+  b.out = nb.w;
+  cudaError_t e = apply_passes<T>(h, b);
   if (e == cudaSuccess)
     e = timed(h, K_SU, [&] { return launch_nodal_update<T>(a, nb.rho[q], nb.w, nb.rho[q ^ 1], nb.xi, 0, h->stream); });
   return e;
@@ -443,9 +439,11 @@ template <typename T> cudaError_t cg_iteration(rve_s* h, const PassArgs<T>& a, i
   if constexpr (std::is_same<T, double>::value) {
     if (h->finite) return apply_finite(h, a);
   }
-  if (h->op_form == RVE_FORM_FACTORED) return apply_factored<T>(h, a, k & 1);
   if (h->op_form == RVE_FORM_NODAL) return apply_nodal<T>(h, a, k & 1);
-  return apply_passes<T>(h, a);
+  if (!force_pass(h, a.var_a)) return apply_passes<T>(h, a);
+  PassArgs<T> b = a;
+  set_force(h, b, k & 1);
+  return apply_passes<T>(h, b);
 }
 
 int read_state(rve_s* h, int L) {
@@ -543,11 +541,19 @@ template <typename T> int autotune(rve_s* h, int L) {
   a.cgphase = 0; a.amode = A_CG; a.pmode = P_G; a.emode = E_CG;
   a.in = (const T*)h->fbuf; a.out = (T*)h->x;
   a.var_a = a.var_e = a.var_c = a.var_y = 0;
+  auto first_pass = [&] {   // the kind of first pass a.var_a stands for
+    a.force = a.pair = 0;
+    if (force_pass(h, a.var_a)) set_force(h, a, 1);
+  };
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   const bool d3 = (h->dim == 3);
-  auto pass_a_l = [&]() { return d3 ? launch_pass_a_3d<T>(a, h->stream) : launch_pass_a_2d<T>(a, h->stream); };
+  auto pass_a_l = [&]() {
+    first_pass();
+    if (a.force) return d3 ? launch_force_3d<T>(a, h->stream) : launch_force_2d<T>(a, h->stream);
+    return d3 ? launch_pass_a_3d<T>(a, h->stream) : launch_pass_a_2d<T>(a, h->stream);
+  };
   auto pass_b_l = [&]() { return d3 ? launch_pass_b_3d<T>(a, h->stream) : cudaSuccess; };
   auto pass_c_l = [&]() { return d3 ? launch_pass_c_3d<T>(a, h->stream) : launch_pass_c_2d<T>(a, h->stream); };
   auto pass_d_l = [&]() { return d3 ? launch_pass_d_3d<T>(a, h->stream) : cudaSuccess; };
@@ -559,6 +565,7 @@ template <typename T> int autotune(rve_s* h, int L) {
     const int nc = rve_sched_candidates(h, which);
     float best_ms = 1e30f;
     for (int v = 0; v < nc; ++v) {
+      if (which == 0 && v == 6 && force_pass(h, v)) continue;   // the force pass has no prefetching tile: 6 is 0
       int* slot = which == 0 ? &a.var_a : which == 1 ? &a.var_e : which == 2 ? &a.var_c : &a.var_y;
       *slot = v;
       auto one = [&]() -> cudaError_t {
@@ -832,9 +839,12 @@ template <typename T> struct FeSolve {
     }
     // u += (B^H B)^-1 B^H delta  (delta = CG iterate x; the nodal state added xi above)
     if (h->op_form != RVE_FORM_NODAL) {
-      a.cgphase = 0; a.amode = A_BARE; a.pmode = P_NODAL_OUT; a.emode = E_NODAL;
-      a.in = (const T*)h->x;
-      CK(apply_passes<T>(h, a));
+      a.cgphase = 0;
+      PassArgs<T> b = a;
+      set_force(h, b, 0);
+      b.amode = A_BARE; b.pmode = P_NODAL_OUT; b.emode = E_NODAL;
+      b.in = (const T*)h->x;
+      CK(apply_passes<T>(h, b));
     }
     for (int l = 0; l < L; ++l)
       if (bad[l]) { active[l] = 0; h->cg_h[l].active = 0; }
@@ -1777,11 +1787,13 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
   if (h->tsize == 4) {
     PassArgs<float> a = pass_args<float>(h, 1, h->u, h->emac_d);
     a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = P_G; a.emode = E_OUT; a.grads = 1;
+    set_force(h, a, 0);
     a.in = (const float*)h->fbuf; a.out = (float*)h->x;
     CK(apply_passes<float>(h, a));
   } else {
     PassArgs<double> a = pass_args<double>(h, 1, h->u, h->emac_d);
     a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = h->finite ? P_FINITE : P_G; a.emode = E_OUT; a.grads = 1;
+    if (force_pass(h, 0)) set_force(h, a, 0);
     a.in = (const double*)h->fbuf; a.out = (double*)h->x;
     CK(apply_passes<double>(h, a));
   }
@@ -1815,12 +1827,6 @@ int rve_set_operator_form(rve_t h, int form) {
   if (form != RVE_FORM_STRESS && (h->deriv != D_FE || h->finite)) return RVE_ERR_ARG;
   if (int jr = join_user(h)) return jr;
   CK(cudaStreamSynchronize(h->stream));
-  if (form == RVE_FORM_FACTORED && h->Lcap > 0 && !h->p2) {
-    const size_t fld = (size_t)h->Lcap * h->m * h->N * h->tsize;
-    if (int rc = dev_alloc(&h->p2, fld)) return rc;
-    CK(cudaMemsetAsync(h->p2, 0, fld, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-  }
   h->op_form = form;
   return RVE_OK;
 }

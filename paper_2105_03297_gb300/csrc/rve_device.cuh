@@ -685,6 +685,39 @@ template <int NT, typename T> __device__ __forceinline__ double block_sum_cols(T
   return s;
 }
 
+// Sum of many FP32 values with the rounding errors of the additions carried
+// along (two-sum), so that a thread's share of an inner product over a whole
+// column is no less exact than short FP32 sums added in FP64, without the FP64
+// pipe.  In FP64 a plain sum.
+template <typename T> struct Acc {
+  T hi = 0, lo = 0;
+  __device__ __forceinline__ void add(T v) {
+    if constexpr (sizeof(T) == 4) {
+      const T s = hi + v, b = s - hi;
+      lo += (hi - (s - b)) + (v - b);
+      hi = s;
+    } else {
+      hi += v;
+    }
+  }
+};
+template <int NT, typename T> __device__ __forceinline__ double block_sum_acc(const Acc<T>& v, T* cols /*[2 NT]*/) {
+  cols[threadIdx.x] = v.hi;
+  if constexpr (sizeof(T) == 4) cols[NT + threadIdx.x] = v.lo;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) {
+      s += (double)cols[w * 32 + threadIdx.x];
+      if constexpr (sizeof(T) == 4) s += (double)cols[NT + w * 32 + threadIdx.x];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  }
+  return s;
+}
+
 // Publish this block's partial and report whether it is the last block of
 // the load case to do so.  The last block then sums all partials in block
 // order, so the result does not depend on scheduling.

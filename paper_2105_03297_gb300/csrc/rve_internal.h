@@ -46,7 +46,7 @@ template <typename T> struct PassArgs {
   const T* E;        // [L / lcs][N] Young's modulus (one field per material)
   int lcs;           // load-case slots per material: slot l uses field l / lcs
   T* x; T* r; T* p;  // [L][m][N] CG vectors
-  T* p2;             // second direction buffer of the factored form (p alternates p, p2), else null
+  T* p2;             // second direction buffer (the direction alternates p, p2), or null
   const T* in;       // [L][m or D][N] input field (A_FIELD / A_BARE / A_NODAL)
   T* out;            // [L][m][N] output field (E_OUT)
   double* u64;       // [L][D][N] FP64 nodal displacement (E_NODAL)
@@ -71,6 +71,12 @@ template <typename T> struct PassArgs {
   int pf_ahead;      // 3D passes A to D: blocks ahead in launch order whose input each block asks the TMA
                      // unit to prefetch into L2, 0 = none; pass E: 1 = prefetch the tile's own r rows
   int deriv;         // Deriv
+  int force;         // first pass of the finite elements: 1 strain fields, 2 nodal fields (pass_force.cuh)
+  const T* pold;     // previous and new search direction of the force pass (different arrays)
+  T* pnew;
+  const T* rho;      // nodal state: residual and iterate of the force pass
+  T* xi;
+  int pair;          // 3D: the spectrum holds F0 and F1 (components j and 3 + j), pass B adds them
   int grads;         // finite elements: passes C, D and E carry the D^2 edge differences of w instead of its D
                      // components (see pass_c_2d_fe), for results that leave the library as they are
 };
@@ -99,13 +105,10 @@ template <typename T> cudaError_t launch_pass_c_2d(const PassArgs<T>& a, cudaStr
 template <typename T> cudaError_t launch_pass_e_2d(const PassArgs<T>& a, cudaStream_t s);
 
 template <typename T> cudaError_t launch_cg_finish_x(const PassArgs<T>& a, cudaStream_t s);
-// factored nodal form of the operator
-template <typename T>
-cudaError_t launch_force_stencil(const PassArgs<T>& a, const T* pold, T* pnew, T* f, cudaStream_t s);
+// material, nodal forces and x transform of the finite elements
+template <typename T> cudaError_t launch_force_2d(const PassArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t launch_force_3d(const PassArgs<T>& a, cudaStream_t s);
 // nodal-state form
-template <typename T>
-cudaError_t launch_nodal_force(const PassArgs<T>& a, const T* rho, const T* pold, T* pnew, T* xi, T* f,
-                               cudaStream_t s);
 template <typename T>
 cudaError_t launch_nodal_update(const PassArgs<T>& a, const T* rho_old, const T* w, T* rho_new, T* xi, int init,
                                 cudaStream_t s);
