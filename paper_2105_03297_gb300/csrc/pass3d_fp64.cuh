@@ -48,6 +48,76 @@ __device__ __forceinline__ void stress_3d(const double* eps, double e, double la
   for (int j = 3; j < 6; ++j) sig[j] = e * mu2 * eps[j];
 }
 
+// Corner forces f = B_e^T sigma_e of the six tetrahedra of a voxel and their
+// summed term magnitudes fa, for the strain E + B u of the corner displacements
+// uc; ec[a][j] are the parts of E added to the difference d u_j / d x_a (the
+// whole shear 2 E_aj to the one with a < j).  The FP64 pipe is the bound, so
+// the tetrahedra are taken round the diagonal: each shares one edge with the
+// next (the first edges of tetrahedra 0 and 1, the last ones of 1 and 4, ..),
+// whose difference is taken once and whose stresses are summed before they go
+// to the corners.  About 370 FP64 operations per voxel with the node sums,
+// against 560 with every tetrahedron on its own.
+__device__ __forceinline__ void voxel_residual_3d(const double uc[8][3], double e, double lam, double mu2,
+                                                  const double* ih, const double ec[3][3], double f[8][3],
+                                                  double fa[8][3]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) f[c][0] = f[c][1] = f[c][2] = fa[c][0] = fa[c][1] = fa[c][2] = 0.0;
+  const double le = e * lam, me = e * mu2, mh = 0.5 * me;
+  auto diff = [&](int a, int c0, double* d) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) d[j] = (uc[c0 | (1 << a)][j] - uc[c0][j]) * ih[a] + ec[a][j];
+  };
+  auto give = [&](int a, int c0, const double* s, const double* m) {   // edge force to its corners
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      f[c0][j] -= ih[a] * s[j];
+      f[c0 | (1 << a)][j] += ih[a] * s[j];
+      fa[c0][j] += ih[a] * m[j];
+      fa[c0 | (1 << a)][j] += ih[a] * m[j];
+    }
+  };
+  double d[3][3];          // by axis
+  double hs[3], hm[3];     // stresses and magnitudes of the edge shared with the previous tetrahedron
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int t = i == 0 ? 0 : i == 1 ? 1 : i == 2 ? 4 : i == 3 ? 5 : i == 4 ? 3 : 2;
+    const int pa = kuhn_perm(t, 0), pb = kuhn_perm(t, 1), pc = kuhn_perm(t, 2);
+    const int v1 = 1 << pa, v2 = v1 | (1 << pb);
+    if (!(i & 1)) diff(pa, 0, d[pa]);            // odd i: the previous one's first edge
+    diff(pb, v1, d[pb]);
+    if ((i & 1) || i == 0) diff(pc, v2, d[pc]);  // even i > 0: the previous one's last edge
+    const double tr = le * (d[0][0] + d[1][1] + d[2][2]);
+    double S[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) S[a][a] = me * d[a][a] + tr;
+    S[1][2] = S[2][1] = mh * (d[1][2] + d[2][1]);
+    S[0][2] = S[2][0] = mh * (d[0][2] + d[2][0]);
+    S[0][1] = S[1][0] = mh * (d[0][1] + d[1][0]);
+    double M[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) M[a][j] = fabs(S[a][j]);
+    give(pb, v1, S[pb], M[pb]);
+    const int sh = (i & 1) ? pa : pc, c0 = (i & 1) ? 0 : v2;   // the edge shared with the previous tetrahedron
+    if (i == 0) {
+      give(pc, v2, S[pc], M[pc]);
+    } else {
+      double s[3], m[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) { s[j] = hs[j] + S[sh][j]; m[j] = hm[j] + M[sh][j]; }
+      give(sh, c0, s, m);
+    }
+    const int nx = (i & 1) ? pc : pa;                          // the edge shared with the next one
+    if (i == 5) {
+      give(pc, v2, S[pc], M[pc]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) { hs[j] = S[nx][j]; hm[j] = M[nx][j]; }
+    }
+  }
+}
+
 // f = B^T C (E + B u) per node, its squared norm, the squared norm of the
 // summed term magnitudes (round-off scale) and the copy of f in the inner
 // precision.  A block sweeps a node tile of (at most) 32 x 8 nodes through a
@@ -101,6 +171,11 @@ __global__ void __launch_bounds__(kR3NT, 1) residual_3d(Fp64Args a) {
     }
   };
   load_plane(-1, un);
+  double ec[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ec[i][j] = i == j ? em[i] : i < j ? 1.41421356237309504880 * em[6 - i - j] : 0.0;
   double acc = 0.0, acca = 0.0;
   int cur = 0;
   for (int zz = -1; zz < tz; ++zz) {
@@ -119,45 +194,7 @@ __global__ void __launch_bounds__(kR3NT, 1) residual_3d(Fp64Args a) {
       }
       const double e = Eb[(int64_t)((z0 + zz) & (nz - 1)) * plane + vox_xy];
       double f[8][3], fa[8][3];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) f[c][0] = f[c][1] = f[c][2] = fa[c][0] = fa[c][1] = fa[c][2] = 0.0;
-#pragma unroll
-      for (int t = 0; t < 6; ++t) {
-        const int pa = kuhn_perm(t, 0), pb = kuhn_perm(t, 1), pc = kuhn_perm(t, 2);
-        const int v1 = 1 << pa, v2 = v1 | (1 << pb);
-        double H[3][3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          H[pa][j] = (uc[v1][j] - uc[0][j]) * a.ih[pa];
-          H[pb][j] = (uc[v2][j] - uc[v1][j]) * a.ih[pb];
-          H[pc][j] = (uc[7][j] - uc[v2][j]) * a.ih[pc];
-        }
-        double eps[6], sg[6];
-        eps[0] = em[0] + H[0][0];
-        eps[1] = em[1] + H[1][1];
-        eps[2] = em[2] + H[2][2];
-        eps[3] = em[3] + kInvSqrt2 * (H[1][2] + H[2][1]);
-        eps[4] = em[4] + kInvSqrt2 * (H[0][2] + H[2][0]);
-        eps[5] = em[5] + kInvSqrt2 * (H[0][1] + H[1][0]);
-        stress_3d(eps, e, a.lam, a.mu2, sg);
-        double S[3][3];
-        S[0][0] = sg[0]; S[1][1] = sg[1]; S[2][2] = sg[2];
-        S[1][2] = S[2][1] = kInvSqrt2 * sg[3];
-        S[0][2] = S[2][0] = kInvSqrt2 * sg[4];
-        S[0][1] = S[1][0] = kInvSqrt2 * sg[5];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const double Pa = a.ih[pa] * S[pa][j], Pb = a.ih[pb] * S[pb][j], Pc = a.ih[pc] * S[pc][j];
-          f[0][j] -= Pa;
-          f[v1][j] += Pa - Pb;
-          f[v2][j] += Pb - Pc;
-          f[7][j] += Pc;
-          fa[0][j] += fabs(Pa);
-          fa[v1][j] += fabs(Pa) + fabs(Pb);
-          fa[v2][j] += fabs(Pb) + fabs(Pc);
-          fa[7][j] += fabs(Pc);
-        }
-      }
+      voxel_residual_3d(uc, e, a.lam, a.mu2, a.ih, ec, f, fa);
       double* hc = hi + cur * 12 * kR3VS;
       double* hca = hia + cur * 12 * kR3VS;
 #pragma unroll
