@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(kFT) fs_dir_tangent(PassArgs<double> a, const 
   __shared__ int flag;
   const int l = blockIdx.y;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t v = (int64_t)blockIdx.x * kFT + threadIdx.x;
@@ -241,9 +242,8 @@ cudaError_t launch_fs_stress(const PassArgs<double>& a, const double* F, double*
 
 cudaError_t launch_fs_dir_tangent(const PassArgs<double>& a, const double* F, double* t, cudaStream_t s) {
   dim3 grid((unsigned)((a.N + kFT - 1) / kFT), a.L);
-  if (a.dim == 2) fs_dir_tangent<2><<<grid, kFT, 0, s>>>(a, F, t);
-  else fs_dir_tangent<3><<<grid, kFT, 0, s>>>(a, F, t);
-  return cudaGetLastError();
+  return a.dim == 2 ? launch_pass(a.pdl, fs_dir_tangent<2>, grid, kFT, 0, s, a, F, t)
+                    : launch_pass(a.pdl, fs_dir_tangent<3>, grid, kFT, 0, s, a, F, t);
 }
 
 cudaError_t launch_fs_add(const PassArgs<double>& a, double* F, cudaStream_t s) {

@@ -7,7 +7,5 @@ template cudaError_t launch_pass_c_2d<float>(const PassArgs<float>&, cudaStream_
 template cudaError_t launch_pass_e_2d<float>(const PassArgs<float>&, cudaStream_t);
 template cudaError_t launch_cg_finish_x<float>(const PassArgs<float>&, cudaStream_t);
 template cudaError_t launch_force_2d<float>(const PassArgs<float>&, cudaStream_t);
-template cudaError_t launch_nodal_update<float>(const PassArgs<float>&, const float*, const float*, float*, float*, int,
-                                              cudaStream_t);
 template cudaError_t launch_nodal_finish<float>(const PassArgs<float>&, const float*, const float*, const float*, cudaStream_t);
 }  // namespace rve

@@ -129,6 +129,7 @@ extern "C" int rve_apply_operator_2d_static(const int64_t* n, const double* leng
   a.emode = E_OUT;
   a.cgphase = 0;
   a.grads = 1;
+  a.pdl = 1;
   a.force = 1;
   cudaError_t e = launch_force_2d<float>(a, s);
   if (e == cudaSuccess) e = launch_pass_c_2d<float>(a, s);

@@ -237,6 +237,7 @@ __global__ void __launch_bounds__(NT, PAIR ? 3 : pass_a2_min_blocks<T, NT>()) pa
   const int l = blockIdx.z, grp = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1];
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const bool nodal = (a.amode == A_NODAL);
@@ -309,6 +310,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs
   const int kx = blockIdx.x, l = blockIdx.y;
   const int KX = a.kx;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   C* col = a.spec + (((int64_t)l * M) * KX + kx) * NY;
@@ -348,6 +350,21 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) pass_c_2d(PassArgs
   fft4<T, NY, M, LD, NT, +1, true, false, false, false>(buf, a.tw[1], ld_s, st_g);
 }
 
+// Nodal state: the block's share of <rho, R> in wavevector space (Parseval: the
+// half spectrum counts twice except k_x = 0 and n_x/2; w^ carries the 1/N), all
+// of it the square |B rho|^2 >= 0 of one wavevector each, so nothing cancels;
+// the last block finishes the CG step.
+template <int NT, typename T>
+__device__ __forceinline__ void publish_rr(const PassArgs<T>& a, CgState* cg, const Acc<T>& acc, T* cols, double* red,
+                                           int* flag, double weight, int blk, int nblk, int l) {
+  const double s = weight * block_sum_acc<NT>(acc, cols);
+  double* part = a.part + (int64_t)l * a.part_stride;
+  if (publish_partial(s, part, &cg->cnt_e, blk, nblk, flag)) {
+    const double rr = sum_partials<NT>(part, nblk, red);
+    if (threadIdx.x == 0) finish_rr(cg, rr, a.dot == 2);
+  }
+}
+
 // Pass C of the finite elements: w^ = (B^H B)^-1 t^ for P k_x columns per
 // block, from t(k_x, y) in components 0 and 1 of the spectrum (pass A or the
 // force pass) to w(k_x, y) in place.  Bound by the FFT arithmetic (80
@@ -371,25 +388,64 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
   constexpr int LD = FftSplit<NY, V>::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [R][LD]
+  __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
+  __shared__ int flag;
   const int kx0 = blockIdx.x * P, l = blockIdx.y;
   const int KX = a.kx;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t cstride = (int64_t)KX * NY;
   C* base = a.spec + ((int64_t)l * a.m * KX + kx0) * NY;
   auto st_s = [&](int b, int k, C v) { buf[b * LD + k] = v; };
   auto ld_s = [&](int b, int y) -> C { return buf[b * LD + y]; };
-  auto ld_g = [&](int b, int y) -> C {
-    return (kx0 + b / 2 < KX) ? base[(b % 2) * cstride + (int64_t)(b / 2) * NY + y] : mkc<T>(0, 0);
-  };
-  fft4<T, NY, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
+  if (a.resid) {   // nodal state: keep the residual force R and transform it (as pass_y_3d)
+    const bool upd = a.resid == 2;
+    const T alpha = upd ? cg_alpha<T>(cg) : (T)1;
+    constexpr int TOT = R * NY, U = 4;
+    for (int i0 = threadIdx.x; i0 < TOT; i0 += U * NT) {
+      C v[U], r[U];
+      int64_t o[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * NT, b = i / NY;
+        o[u] = (i < TOT && kx0 + b / 2 < KX) ? (b % 2) * cstride + (int64_t)(b / 2) * NY + i % NY : -1;
+        v[u] = r[u] = mkc<T>(0, 0);
+        if (o[u] >= 0) {
+          v[u] = base[o[u]];
+          if (upd) r[u] = base[o[u] + 2 * cstride];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * NT;
+        v[u] = csub(r[u], cscale(v[u], alpha));
+        if (o[u] >= 0) base[o[u] + 2 * cstride] = v[u];
+        if (i < TOT) buf[(i / NY) * LD + i % NY] = v[u];
+      }
+    }
+    __syncthreads();
+    fft4<T, NY, R, LD, NT, -1, true, true, false, false, V>(buf, a.tw[1], ld_s, st_s);
+  } else {
+    auto ld_g = [&](int b, int y) -> C {
+      return (kx0 + b / 2 < KX) ? base[(b % 2) * cstride + (int64_t)(b / 2) * NY + y] : mkc<T>(0, 0);
+    };
+    fft4<T, NY, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
+  }
+  Acc<T> acc;
   for (int i = threadIdx.x; i < P * NY; i += NT) {
     const int pc = i / NY, ky = i % NY, kx = kx0 + pc;
     if (kx >= KX) continue;
     C t[2] = {buf[2 * pc * LD + ky], buf[(2 * pc + 1) * LD + ky]};
+    const C r0 = t[0], r1 = t[1];
     if (kx == 0 && ky == 0) t[0] = t[1] = mkc<T>(0, 0);   // k = 0: no mean
     else solve_2d<T>(t, a.ph[0][kx], a.ph[1][ky], a.ih[0], a.ih[1], a.inv_n);
+    if (a.dot) {
+      const T d = r0.x * t[0].x + r0.y * t[0].y + r1.x * t[1].x + r1.y * t[1].y;
+      acc.add(kx == 0 || kx == KX - 1 ? d : (T)2 * d);
+    }
     if constexpr (W == 4) {
       const C one = mkc<T>(1, 0);
       const C d0 = cscale(csub(a.ph[0][kx], one), a.ih[0]), d1 = cscale(csub(a.ph[1][ky], one), a.ih[1]);
@@ -404,6 +460,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
     }
   }
   __syncthreads();
+  if (a.dot) publish_rr<NT>(a, cg, acc, cols, red, &flag, 1.0, blockIdx.x, gridDim.x, l);
   auto st_g = [&](int b, int k, C v) {
     if (kx0 + b / W < KX) base[(b % W) * cstride + (int64_t)(b / W) * NY + k] = v;
   };
@@ -546,6 +603,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   const int ny = a.n[1];
   const int64_t N = a.N;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const bool nodal = (a.emode == E_NODAL || a.emode == E_NOUT);
@@ -615,11 +673,12 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NPR][LD]
   __shared__ double red[NT / 32];
-  __shared__ T cols[2 * NT];
+  __shared__ T cols[NT];
   __shared__ int flag;
   const int l = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1];
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   pass_e_unpack<T, NX, 2 * NPR, NT, LD>(buf, a.spec + (int64_t)l * a.m * KX * ny, W, (int64_t)KX * ny, ny, y0, ny - 1);
@@ -736,8 +795,7 @@ cudaError_t launch_a_2d_t(const PassArgs<T>& a, cudaStream_t s) {
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   dim3 grid(a.n[1] / TY, a.amode == A_NODAL ? 1 : a.nq, a.L);
-  k<<<grid, NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, grid, NT, sm, s, a);
 }
 template <typename T, int NX, int TY>
 cudaError_t launch_e_2d_t(const PassArgs<T>& a, cudaStream_t s) {
@@ -747,8 +805,7 @@ cudaError_t launch_e_2d_t(const PassArgs<T>& a, cudaStream_t s) {
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   dim3 grid(a.n[1] / TY, (a.emode == E_NODAL || a.emode == E_NOUT) ? 1 : a.nq, a.L);
-  k<<<grid, NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, grid, NT, sm, s, a);
 }
 // Tile variants of the 2D pass A: 0 default rows per block, 1 half, 2 double
 // (threads = the FFT's); 3 default rows and 4 half rows with one thread per
@@ -775,8 +832,7 @@ cudaError_t launch_e_2d_fe_w(const PassArgs<T>& a, cudaStream_t s) {
   auto k = pass_e_2d_fe<T, NX, TY, NT, W>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  k<<<dim3(a.n[1] / TY, a.L), NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.L), NT, sm, s, a);
 }
 template <typename T, int NX, int TY>
 cudaError_t launch_e_2d_fe_t(const PassArgs<T>& a, cudaStream_t s) {
@@ -816,8 +872,7 @@ cudaError_t launch_c_2d_v(const PassArgs<T>& a, cudaStream_t s) {
   auto k = pass_c_2d_fe<T, NY, P, NT, V, W>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  k<<<dim3((a.kx + P - 1) / P, a.L), NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, dim3((a.kx + P - 1) / P, a.L), NT, sm, s, a);
 }
 
 template <typename T, int NY>
@@ -834,8 +889,7 @@ cudaError_t launch_c_2d_n(const PassArgs<T>& a, cudaStream_t s) {
     auto k3 = pass_c_2d<T, NY, 3, NT3>;
     static DeviceOnce attr3;
     attr3.run(current_device(), [&] { set_smem_attrs(k3, sm3); });
-    k3<<<dim3(a.kx, a.L), NT3, sm3, s>>>(a);
-    return cudaGetLastError();
+    return launch_pass(a.pdl, k3, dim3(a.kx, a.L), NT3, sm3, s, a);
   }
   if (a.nq == 1) {
     constexpr int NT1 = fft_threads<NY, 3>();
@@ -843,16 +897,14 @@ cudaError_t launch_c_2d_n(const PassArgs<T>& a, cudaStream_t s) {
     auto k1 = pass_c_2d<T, NY, 1, NT1>;
     static DeviceOnce attr1;
     attr1.run(current_device(), [&] { set_smem_attrs(k1, sm1); });
-    k1<<<dim3(a.kx, a.L), NT1, sm1, s>>>(a);
-    return cudaGetLastError();
+    return launch_pass(a.pdl, k1, dim3(a.kx, a.L), NT1, sm1, s, a);
   }
   constexpr int NT2 = fft_threads<NY, 6>();
   const size_t sm2 = sizeof(cplx<T>) * 6 * FftSplit<NY>::LD;
   auto k2 = pass_c_2d<T, NY, 2, NT2>;
   static DeviceOnce attr2;
   attr2.run(current_device(), [&] { set_smem_attrs(k2, sm2); });
-  k2<<<dim3(a.kx, a.L), NT2, sm2, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k2, dim3(a.kx, a.L), NT2, sm2, s, a);
 }
 
 #define RVE_DISPATCH_N(nval, FN, ...)                      \

@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(NT, pass_a_min_blocks<T, NT>()) pass_a_3d(Pass
   const int z = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1], nz = a.n[2];
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int c0 = nodal ? 0 : grp * 6;
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT <= 256 ? 4 : 2) : 1) 
   const int kx = blockIdx.y, z0 = blockIdx.x * TZB;
   const int nz = a.n[2], KX = a.kx;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t cbase = (((int64_t)l * a.m + c) * KX + kx);
@@ -186,7 +188,41 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT <= 256 ? 4 : 2) : 1) 
   if (FWD) {
     // step 1 reads whole y-pencils, step 2 writes z-chunks (zz fastest)
     auto st = [&](int zz, int k, C v) { chunks[(int64_t)k * nz + zz] = v; };
-    if (a.pair) {   // the two parts of the nodal forces (force_3d)
+    if (a.resid) {
+      // nodal state: this pass keeps the residual force R and transforms it (the
+      // loads of several values come before their stores, which the compiler
+      // could not reorder)
+      const C* f1 = pencils + 3 * (int64_t)KX * nz * NY;
+      C* res = pencils + 6 * (int64_t)KX * nz * NY;
+      const bool upd = a.resid == 2;
+      const T alpha = upd ? cg_alpha<T>(cg) : (T)1;
+      constexpr int TOT = TZB * NY, U = 4;
+      static_assert(TOT % NT == 0, "whole rounds");
+      for (int i0 = threadIdx.x; i0 < TOT; i0 += U * NT) {
+        C v[U], w[U], r[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u * NT;
+          if (i < TOT) {
+            v[u] = pencils[i];
+            if (upd) { w[u] = f1[i]; r[u] = res[i]; }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u * NT;
+          if (i < TOT) {
+            if (upd) v[u] = csub(r[u], cscale(cadd(v[u], w[u]), alpha));
+            else v[u] = cscale(v[u], (T)-1);
+            res[i] = v[u];
+            buf[(i / NY) * LD + i % NY] = v[u];
+          }
+        }
+      }
+      __syncthreads();
+      auto ld = [&](int zz, int y) -> C { return buf[zz * LD + y]; };
+      fft4<T, NY, TZB, LD, NT, -1, true, false, false, true, V>(buf, a.tw[1], ld, st);
+    } else if (a.pair) {   // the two parts of the nodal forces (force_3d)
       const C* other = pencils + 3 * (int64_t)KX * nz * NY;
       auto ld = [&](int zz, int y) -> C {
         return cadd(pencils[(int64_t)zz * NY + y], other[(int64_t)zz * NY + y]);
@@ -233,6 +269,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT == 256 ? 2 : 6) : 1) 
   const int l = blockIdx.z, kx = blockIdx.y, z0 = blockIdx.x * TZB;
   const int nz = a.n[2], KX = a.kx;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int y = threadIdx.x % NY, ln = threadIdx.x / NY;
@@ -371,9 +408,13 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 38
   constexpr int LD = FftSplit<NZ, V>::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [W P][LD]
+  __shared__ double red[NT / 32];
+  __shared__ T cols[NT];
+  __shared__ int flag;
   const int kx = blockIdx.x, ky0 = blockIdx.y * P, l = blockIdx.z;
   const int ny = a.n[1], KX = a.kx;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t stride_c = (int64_t)KX * ny * NZ;
@@ -381,6 +422,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 38
   auto ld_g = [&](int b, int z) -> C { return base[(b % 3) * stride_c + (b / 3) * NZ + z]; };
   auto st_s = [&](int b, int k, C v) { buf[b * LD + k] = v; };
   fft4<T, NZ, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[2], ld_g, st_s);
+  Acc<T> acc;
   for (int i = threadIdx.x; i < P * NZ; i += NT) {
     const int pc = i / NZ, kz = i % NZ;
     C* col = buf + 3 * pc * LD + kz;
@@ -389,7 +431,14 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 38
       for (int j = 0; j < W; ++j) col[j * LD] = mkc<T>(0, 0);
     } else {
       const C e[3] = {a.ph[0][kx], a.ph[1][ky0 + pc], a.ph[2][kz]};
+      const C t[3] = {col[0], col[LD], col[2 * LD]};
       solve_3d<T, LD>(col, e, a.ih, a.inv_n);
+      if (a.dot) {
+        T d = 0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) d += t[j].x * col[j * LD].x + t[j].y * col[j * LD].y;
+        acc.add(d);
+      }
       if constexpr (W == 9) {
         const C w[3] = {col[0], col[LD], col[2 * LD]};
 #pragma unroll
@@ -405,6 +454,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 38
   auto ld_s = [&](int b, int z) -> C { return buf[b * LD + z]; };
   auto st_g = [&](int b, int k, C v) { base[(b % W) * stride_c + (b / W) * NZ + k] = v; };
   fft4<T, NZ, W * P, LD, NT, +1, true, false, false, false, V>(buf, a.tw[2], ld_s, st_g);
+  if (a.dot) publish_rr<NT>(a, cg, acc, cols, red, &flag, kx == 0 || kx == KX - 1 ? 1.0 : 2.0, blockIdx.x + gridDim.x * blockIdx.y,
+                            gridDim.x * gridDim.y, l);
 }
 
 // Pass C for one evaluation point per voxel (the derivatives of Secs. 2.3-2.5,
@@ -421,6 +472,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) pass_c_3d_q1(PassA
   const int kx = blockIdx.x, ky0 = blockIdx.y * P, l = blockIdx.z;
   const int ny = a.n[1], KX = a.kx;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t stride_c = (int64_t)KX * ny * NZ;
@@ -470,6 +522,7 @@ __global__ void __launch_bounds__(NT, 1) pass_c_3d_fs(PassArgs<T> a) {
   const int kx = blockIdx.x, ky = blockIdx.y, l = blockIdx.z;
   const int ny = a.n[1], KX = a.kx;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t stride_c = (int64_t)KX * ny * NZ;
@@ -511,6 +564,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pas
   const int ny = a.n[1], nz = a.n[2];
   const int64_t N = a.N;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int c0 = nodal ? 0 : grp * GE;
@@ -546,6 +600,15 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pas
 // traffic (read and written once), which bounds it.  W = 9: the spectrum holds
 // the edge differences of w instead (see pass_c_2d_fe).
 // grid (n_y/TY, n_z, L).
+// In FP32 the r loads of the update go through a ring of the thread's own
+// shared-memory slots (cp.async, six tetrahedra deep): issued before the
+// spectrum is unpacked, they keep DRAM busy during the transforms, and in the
+// update every store no longer waits for the loads behind it (us per iteration,
+// without and with: 256 x 256 x 64 309, 289; 128^3 156, 149; 64^3, six load
+// cases 147, 114).
+template <typename T, int NT, int W> __host__ __device__ constexpr bool e_fe_ring() {
+  return sizeof(T) == 4 && W == 3 && NT <= 256;   // else it does not fit beside the rows
+}
 template <int NX> __host__ __device__ constexpr int e_fe_ld() {
   // 9 (mod 16): the TY + 1 rows that consecutive lanes unpack at one column
   // fall on different banks
@@ -561,18 +624,36 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NR][LD]
   __shared__ double red[NT / 32];
-  __shared__ T cols[2 * NT];
+  __shared__ T cols[NT];
   __shared__ int flag;
   const int l = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1], nz = a.n[2];
   const int64_t N = a.N;
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const bool cgm = a.emode == E_CG;
   const int64_t vox0 = (int64_t)l * a.m * N + ((int64_t)z * ny + y0) * NX;
-  if (cgm && a.pf_ahead > 0 && threadIdx.x < 36)   // the tile's r rows, contiguous per component
-    prefetch_l2_bulk(a.r + vox0 + threadIdx.x * N, (unsigned)(TY * NX * sizeof(T)));
+  // the r values of this thread's next six tetrahedra, copied into its own
+  // slots while the spectrum is unpacked and transformed (see e_fe_ring)
+  constexpr bool RING = e_fe_ring<T, NT, W>();
+  constexpr int VL = (RING && NX >= 256) ? 2 : 1; // voxels of a thread's unit (256: 298 -> 289 us; 64^3: 114, 130 with 2)
+  constexpr int UNITS = TY * (NX / VL);
+  T* ring = reinterpret_cast<T*>(buf + R * LD);   // [6][6][NT] units
+  auto issue = [&](int i, int t) {
+    if (cgm && i < UNITS) {
+      const T* src = a.r + vox0 + VL * i;
+#pragma unroll
+      for (int s = 0; s < 6; ++s)
+        copy_async<VL * (int)sizeof(T)>(ring + ((6 * t + s) * NT + threadIdx.x) * VL, src + (6 * t + s) * N);
+    }
+    copy_async_commit();
+  };
+  if constexpr (RING) {
+#pragma unroll
+    for (int t = 0; t < 6; ++t) issue(threadIdx.x, t);
+  }
   {
     const C* pa = a.spec + ((int64_t)l * a.m * KX * nz + z) * ny;
     const C* pb = a.spec + ((int64_t)l * a.m * KX * nz + ((z + 1) & (nz - 1))) * ny;
@@ -607,42 +688,52 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   const T ih[3] = {a.ih[0], a.ih[1], a.ih[2]};
   const T r2 = (T)kInvSqrt2;
   Acc<T> acc;
-  for (int i = threadIdx.x; i < TY * NX; i += NT) {
-    const int yy = i / NX, x = i % NX;
+  for (int i = threadIdx.x; i < UNITS; i += NT) {
+    const int yy = i / (NX / VL), x = (i % (NX / VL)) * VL;
     const int64_t v0 = vox0 + (int64_t)yy * NX + x;
-    // node values at (x + dx, y + dy): planes z (.x) and z + 1 (.y)
-    C n[W][2][2];
+    // node values at (x + q, y + dy): planes z (.x) and z + 1 (.y)
+    C n[W][2][VL + 1];
 #pragma unroll
     for (int j = 0; j < W; ++j)
 #pragma unroll
       for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
-        for (int q = 0; q < 2; ++q) n[j][dy][q] = buf[(j * NR + yy + dy) * LD + ((x + q) & (NX - 1))];
-    auto corner = [&](int c, int j) -> T {   // corner c = dx + 2 dy + 4 dz
-      const C v = n[j][(c >> 1) & 1][c & 1];
+        for (int q = 0; q <= VL; ++q) n[j][dy][q] = buf[(j * NR + yy + dy) * LD + ((x + q) & (NX - 1))];
+    auto corner = [&](int c, int j, int q) -> T {   // corner c = dx + 2 dy + 4 dz of voxel x + q
+      const C v = n[j][(c >> 1) & 1][q + (c & 1)];
       return (c & 4) ? v.y : v.x;
     };
     T vs = 0;
 #pragma unroll
     for (int t = 0; t < 6; ++t) {
-      T rv[6];
+      T rv[6][VL];
       if (cgm) {
+        if constexpr (RING) copy_async_wait<5>();
 #pragma unroll
-        for (int s = 0; s < 6; ++s) rv[s] = a.r[v0 + (6 * t + s) * N];
+        for (int s = 0; s < 6; ++s)
+          vloadn<T, VL>(rv[s], RING ? ring + ((6 * t + s) * NT + threadIdx.x) * VL : a.r + v0 + (6 * t + s) * N);
       }
+      if constexpr (RING) issue(i + NT, t);
       const int ax[3] = {kuhn_perm(t, 0), kuhn_perm(t, 1), kuhn_perm(t, 2)};
       const int v1 = 1 << ax[0], v2 = v1 | (1 << ax[1]);
       const int at[4] = {0, v1, v2, 7};
-      T H[3][3];   // H[a][j] = d w_j / d x_a
+      T q[6][VL];
 #pragma unroll
-      for (int e = 0; e < 3; ++e)
+      for (int k = 0; k < VL; ++k) {
+        T H[3][3];   // H[a][j] = d w_j / d x_a
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-          H[ax[e]][j] = W == 9 ? corner(at[e], 3 * ax[e] + j) : (corner(at[e + 1], j) - corner(at[e], j)) * ih[ax[e]];
-      const T q[6] = {H[0][0], H[1][1], H[2][2], r2 * (H[1][2] + H[2][1]), r2 * (H[0][2] + H[2][0]),
-                      r2 * (H[0][1] + H[1][0])};
+        for (int e = 0; e < 3; ++e)
 #pragma unroll
-      for (int s = 0; s < 6; ++s) vs += strain_update<T, 1>(a, v0 + (6 * t + s) * N, &rv[s], &q[s], alpha);
+          for (int j = 0; j < 3; ++j)
+            H[ax[e]][j] = W == 9 ? corner(at[e], 3 * ax[e] + j, k)
+                                 : (corner(at[e + 1], j, k) - corner(at[e], j, k)) * ih[ax[e]];
+        q[0][k] = H[0][0]; q[1][k] = H[1][1]; q[2][k] = H[2][2];
+        q[3][k] = r2 * (H[1][2] + H[2][1]);
+        q[4][k] = r2 * (H[0][2] + H[2][0]);
+        q[5][k] = r2 * (H[0][1] + H[1][0]);
+      }
+#pragma unroll
+      for (int s = 0; s < 6; ++s) vs += strain_update<T, VL>(a, v0 + (6 * t + s) * N, rv[s], q[s], alpha);
     }
     acc.add(vs);
   }
@@ -708,9 +799,9 @@ cudaError_t launch_a_3d_t(const PassArgs<T>& a, cudaStream_t s, bool ahead = fal
   if (ahead) {
     PassArgs<T> b = a;
     b.pf_ahead = prefetch_distance((dev >= 0 && dev < kMaxDevices) ? occ[dev] : 0, 16);
-    k<<<grid, NT, sm, s>>>(b);
+    return launch_pass(b.pdl, k, grid, NT, sm, s, b);
   } else {
-    k<<<grid, NT, sm, s>>>(a);
+    return launch_pass(a.pdl, k, grid, NT, sm, s, a);
   }
   return cudaGetLastError();
 }
@@ -722,22 +813,18 @@ cudaError_t launch_e_3d_t(const PassArgs<T>& a, cudaStream_t s) {
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   dim3 grid(a.n[1] / TY, a.n[2], a.L * (GE == 3 ? 1 : a.nq));
-  k<<<grid, NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, grid, NT, sm, s, a);
 }
 template <typename T, int NX, int TY, int W = 3>
-cudaError_t launch_e_3d_fe_t(const PassArgs<T>& a, cudaStream_t s, bool prefetch) {
+cudaError_t launch_e_3d_fe_t(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int R = W * (TY + 1);
   constexpr int NT = fft_threads<NX, R>();
-  constexpr size_t sm = sizeof(cplx<T>) * R * e_fe_ld<NX>();
-    constexpr int MB = sizeof(T) == 8 ? 1 : W == 9 ? (NT <= 448 ? 2 : 1) : NT <= 256 ? 4 : NT <= 448 ? 2 : 1;
+  constexpr size_t sm = sizeof(cplx<T>) * R * e_fe_ld<NX>() + (e_fe_ring<T, NT, W>() ? sizeof(T) * 36 * (NX >= 256 ? 2 : 1) * NT : 0);
+    constexpr int MB = sizeof(T) == 8 ? 1 : W == 9 ? (NT <= 448 ? 2 : 1) : NT <= 256 ? (NX >= 256 ? 2 : 4) : NT <= 448 ? 2 : 1;
   auto k = pass_e_3d_fe<T, NX, TY, NT, MB, W>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  PassArgs<T> b = a;
-  b.pf_ahead = prefetch ? 1 : 0;
-  k<<<dim3(a.n[1] / TY, a.n[2], a.L), NT, sm, s>>>(b);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.n[2], a.L), NT, sm, s, a);
 }
 // Tile variants of pass A: 0 default rows per block, 1 half, 2 double (threads
 // = the FFT's); 3 default rows and 4 half rows with one thread per load unit;
@@ -763,19 +850,16 @@ cudaError_t launch_a_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   return launch_a_3d_t<T, NX, tile_rows3<T>(0)>(a, s);
 }
 // Tile variants of pass E: 0 default rows per block, 1 half, 2 double; with
-// n_x >= 128 in FP32 also 3 default and 4 half rows with the L2 prefetch of
-// the tile's own r rows at the start of the block.
+// n_x >= 128 in FP32 also 3 and 4, the same tiles as 0 and 1.
 template <typename T, int NX>
 cudaError_t launch_e_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   if (fe_path(a) && (a.emode == E_CG || a.emode == E_INIT || a.emode == E_OUT)) {
-    if (a.grads) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1), 9>(a, s, false);
+    if (a.grads) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1), 9>(a, s);
     if constexpr (NX >= 64) {
-      if (a.var_e == 1) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1)>(a, s, false);
-      if (a.var_e == 2 && a.n[1] >= tile_rows3<T>(2)) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(2)>(a, s, false);
-      if (a.var_e == 3) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(0)>(a, s, true);
-      if (a.var_e == 4) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1)>(a, s, true);
+      if (a.var_e == 1 || a.var_e == 4) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(1)>(a, s);
+      if (a.var_e == 2 && a.n[1] >= tile_rows3<T>(2)) return launch_e_3d_fe_t<T, NX, tile_rows3<T>(2)>(a, s);
     }
-    return launch_e_3d_fe_t<T, NX, tile_rows3<T>(0)>(a, s, false);
+    return launch_e_3d_fe_t<T, NX, tile_rows3<T>(0)>(a, s);
   }
   // the three nodal components: twice the rows, as in pass A
   if (a.emode == E_NODAL || a.emode == E_NOUT) return launch_e_3d_t<T, NX, tile_rows3<T>(2), 3>(a, s);
@@ -803,9 +887,9 @@ cudaError_t launch_y_3d_v(const PassArgs<T>& a, cudaStream_t s) {
   if (sizeof(T) == 4) {
     PassArgs<T> b = a;
     b.pf_ahead = prefetch_distance((dev >= 0 && dev < kMaxDevices) ? occ[dev] : 0, 2);
-    k<<<grid, NT, sm, s>>>(b, Cc);
+    return launch_pass(b.pdl, k, grid, NT, sm, s, b, Cc);
   } else {
-    k<<<grid, NT, sm, s>>>(a, Cc);
+    return launch_pass(a.pdl, k, grid, NT, sm, s, a, Cc);
   }
   return cudaGetLastError();
 }
@@ -818,8 +902,7 @@ cudaError_t launch_b_3d_fe(const PassArgs<T>& a, cudaStream_t s) {
   auto k = pass_b_3d_fe<T, NY, TZB, NT, V>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  k<<<dim3(a.n[2] / TZB, a.kx, a.L), NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, dim3(a.n[2] / TZB, a.kx, a.L), NT, sm, s, a);
 }
 // Split variant of the y transforms (passes B and D): a.var_y.
 template <typename T, int NY, bool FWD>
@@ -851,8 +934,7 @@ cudaError_t launch_c_3d_v(const PassArgs<T>& a, cudaStream_t s) {
   auto k = pass_c_3d_nodal<T, NZ, P, NT, V, W>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  k<<<dim3(a.kx, a.n[1] / P, a.L), NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, dim3(a.kx, a.n[1] / P, a.L), NT, sm, s, a);
 }
 
 template <typename T, int NZ>
@@ -864,8 +946,7 @@ cudaError_t launch_c_3d_n(const PassArgs<T>& a, cudaStream_t s) {
     auto kf = pass_c_3d_fs<T, NZ, NTf>;
     static DeviceOnce attrf;
     attrf.run(current_device(), [&] { set_smem_attrs(kf, smf); });
-    kf<<<dim3(a.kx, a.n[1], a.L), NTf, smf, s>>>(a);
-    return cudaGetLastError();
+    return launch_pass(a.pdl, kf, dim3(a.kx, a.n[1], a.L), NTf, smf, s, a);
   }
   if (!fe_path(a)) {
     constexpr int NT1 = fft_threads<NZ, 36>();
@@ -873,8 +954,7 @@ cudaError_t launch_c_3d_n(const PassArgs<T>& a, cudaStream_t s) {
     auto k1 = pass_c_3d_q1<T, NZ, NT1>;
     static DeviceOnce attr1;
     attr1.run(current_device(), [&] { set_smem_attrs(k1, sm1); });
-    k1<<<dim3(a.kx, (a.n[1] + 5) / 6, a.L), NT1, sm1, s>>>(a);
-    return cudaGetLastError();
+    return launch_pass(a.pdl, k1, dim3(a.kx, (a.n[1] + 5) / 6, a.L), NT1, sm1, s, a);
   }
   if constexpr (fft_split_count<NZ>() > 1) {
     if (a.var_c == 1) return a.grads ? launch_c_3d_v<T, NZ, 1, 9>(a, s) : launch_c_3d_v<T, NZ, 1>(a, s);

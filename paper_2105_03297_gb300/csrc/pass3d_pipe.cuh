@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(NT, 2) pass_a_3d_pipe(PassArgs<float> a) {
     bulk_copy_g2s(stage + 3 * GS * ROW, a.E + (int64_t)(l / a.lcs) * N + v0, bytes, &bar);
   };
 
+  pdl_begin();
   if (tid == 0) {
     mbar_init(&bar, 1);
     mbar_init_fence();
@@ -275,8 +276,7 @@ cudaError_t launch_a_3d_pipe(const PassArgs<float>& a, cudaStream_t s) {
   const int nsm = (dev >= 0 && dev < kMaxDevices && sms[dev] > 0) ? sms[dev] : 152;
   const int64_t tiles = (int64_t)(a.n[1] / TY) * a.n[2] * a.nq * a.L;
   const int blocks = (int)std::min<int64_t>(tiles, 2 * (int64_t)nsm);
-  k<<<blocks, NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, blocks, NT, sm, s, a);
 }
 
 }  // namespace rve

@@ -46,17 +46,6 @@ template <int NX, typename T> __device__ __forceinline__ T from_next(T v) {
   else return __shfl_sync(0xffffffffu, v, (threadIdx.x & 31 & ~(NX - 1)) | ((threadIdx.x + 1) & (NX - 1)));
 }
 
-// Asynchronous copy of one value from global to this thread's shared memory.
-template <typename T> __device__ __forceinline__ void copy_async(T* dst, const T* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
-               "n"((int)sizeof(T))
-               : "memory");
-}
-__device__ __forceinline__ void copy_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void copy_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // ---------------------------------------------------------------- 3D
 // Corner forces of tetrahedron t (added to f) from its scaled stress rows.
 template <typename T>
@@ -160,11 +149,12 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
   T* edge = reinterpret_cast<T*>(buf + 3 * TY * LD);              // [LN][TYL + 1][NW][12], NX > 32
   T* ring = edge + (NX > 32 ? 12 * (TY + LN) * NW : 0);           // strain source: [stages][18][NT]
   __shared__ double red[NT / 32];
-  __shared__ T cols[2 * NT];
+  __shared__ T cols[NT];
   __shared__ int flag;
   const int l = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1], nz = a.n[2];
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
@@ -230,13 +220,13 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
         const unsigned o = off(yy);
         T* slot = ring + (t % ST) * 18 * NT + threadIdx.x;
 #pragma unroll
-        for (int s = 0; s < 6; ++s) copy_async(slot + s * NT, rp + (6 * t + s) * N + o);
+        for (int s = 0; s < 6; ++s) copy_async<(int)sizeof(T)>(slot + s * NT, rp + (6 * t + s) * N + o);
         if (use_old) {
 #pragma unroll
-          for (int s = 0; s < 6; ++s) copy_async(slot + (6 + s) * NT, po + (6 * t + s) * N + o);
+          for (int s = 0; s < 6; ++s) copy_async<(int)sizeof(T)>(slot + (6 + s) * NT, po + (6 * t + s) * N + o);
           if (yy >= ln * TYL) {
 #pragma unroll
-            for (int s = 0; s < 6; ++s) copy_async(slot + (12 + s) * NT, xp + (6 * t + s) * N + o);
+            for (int s = 0; s < 6; ++s) copy_async<(int)sizeof(T)>(slot + (12 + s) * NT, xp + (6 * t + s) * N + o);
           }
         }
       }
@@ -464,11 +454,12 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
   C* buf = reinterpret_cast<C*>(smem_raw);             // [TY][LD]: f_0 + i f_1
   T* edge = reinterpret_cast<T*>(buf + TY * LD);       // [LN][TYL + 1][NW][4], NX > 32
   __shared__ double red[NT / 32];
-  __shared__ T cols[2 * NT];
+  __shared__ T cols[NT];
   __shared__ int flag;
   const int l = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1];
   CgState* cg = a.cg + l;
+  pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
@@ -697,15 +688,16 @@ cudaError_t launch_force_3d_t(const PassArgs<T>& a, cudaStream_t s) {
   auto k = force_3d<T, NX, TY, NT, MB, SRC>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  k<<<dim3(a.n[1] / TY, a.n[2], a.L), NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.n[2], a.L), NT, sm, s, a);
 }
 // Rows per block and threads.  Long rows need the shared memory for fewer of
 // them; short ones are marched side by side, with few rows per lane.
 template <typename T, int NX> constexpr int force_rows3() { return NX >= 128 ? 8 : 16; }
 template <int NX> constexpr int force_threads3() { return NX >= 256 ? 256 : NX >= 64 ? 128 : 64; }
 // Tile variants: 0 default rows, 1 half, 2 double (n_x >= 128: 16 rows, FP32),
-// 3 and 4 the rows of 0 and 1 with twice the threads; 6 as 0.
+// 3 and 4 the rows of 0 and 1 with twice the threads; 6 as 0 (an L2 prefetch of
+// the rows two steps ahead, 2 KB of each of the 108 fields, made the pass
+// slower: 256 x 256 x 64 657 -> 770 us).
 template <typename T, int NX>
 cudaError_t launch_force_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int TY = force_rows3<T, NX>(), NT = force_threads3<NX>();
@@ -733,8 +725,7 @@ cudaError_t launch_force_2d_t(const PassArgs<T>& a, cudaStream_t s) {
   auto k = force_2d<T, NX, TY, NT, MB, SRC>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
-  k<<<dim3(a.n[1] / TY, a.L), NT, sm, s>>>(a);
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.L), NT, sm, s, a);
 }
 // Threads: at most two rows in a row of steps (TY = 2: one lane per row).
 template <int NX, int TY> constexpr int force_threads2() {

@@ -284,7 +284,8 @@ int ensure_capacity(rve_s* h, int L) {
   if ((rc = dev_alloc((void**)&h->u, (size_t)L * h->D * h->N * sizeof(double))) ||
       (rc = dev_alloc((void**)&h->uadj, (size_t)h->ns * h->D * h->N * sizeof(double))))
     { free_L(h); if (keep_u) cudaFree(keep_u); return rc; }
-  h->part_stride = (int)(h->N / 128 + (int64_t)h->n[1] * h->n[2] * h->m / 2 + 64);
+  // one partial per block of any reducing pass (the 2D pass C: one per k_x)
+  h->part_stride = (int)(h->N / 128 + (int64_t)h->n[1] * h->n[2] * h->m / 2 + h->kx + 64);
   const int Lp = L > h->ns ? L : h->ns;
   if ((rc = dev_alloc((void**)&h->part, (size_t)Lp * h->part_stride * sizeof(double))) ||
       (rc = dev_alloc((void**)&h->cg, (size_t)Lp * sizeof(CgState))) ||
@@ -402,33 +403,30 @@ template <typename T> cudaError_t apply_passes(rve_s* h, const PassArgs<T>& a) {
   return e;
 }
 
-// Nodal-state buffers: xi, rho[2], pi[2], f, w, each [L][D][N] of the inner
-// precision, carved out of the strain-form fields (m >= 2 D components).
+// Nodal-state buffers: xi, rho, pi[2], f (the FP64 residual), each [L][D][N] of
+// the inner precision, carved out of the strain-form fields (m >= 2 D components).
 template <typename T> struct NodalBufs {
-  T* xi; T* rho[2]; T* pi[2]; T* f; T* w;
+  T* xi; T* rho; T* pi[2]; T* f;
   NodalBufs(const rve_s* h, int L) {
     const size_t nd = (size_t)L * h->D * h->N;
     xi = (T*)h->x;
-    rho[0] = (T*)h->r; rho[1] = rho[0] + nd;
+    rho = (T*)h->r;
     pi[0] = (T*)h->p; pi[1] = pi[0] + nd;
-    f = (T*)h->fbuf; w = f + nd;
+    f = (T*)h->fbuf;
   }
 };
 
 // One projected-CG iteration on the nodal state (parity q of the iteration):
-// force pass (pi, xi, f = B^T C B pi, alpha), the other FFT passes with
-// w^ = (B^H B)^-1 f^, update kernel (rho -= alpha w, <B rho, B rho>, beta).
+// force pass (pi, xi, f = B^T C B pi, alpha), then R -= alpha f,
+// rho = (B^T B)^-1 R and <rho, R> -> beta in the other passes.
 template <typename T> cudaError_t apply_nodal(rve_s* h, const PassArgs<T>& a, int q) {
   NodalBufs<T> nb(h, a.L);
   PassArgs<T> b = a;
   b.amode = A_CG; b.pmode = P_G; b.emode = E_NOUT;
-  b.force = 2; b.pair = h->dim == 3;
-  b.rho = nb.rho[q]; b.pold = nb.pi[q ^ 1]; b.pnew = nb.pi[q]; b.xi = nb.xi;
-  b.out = nb.w;
-  cudaError_t e = apply_passes<T>(h, b);
-  if (e == cudaSuccess)
-    e = timed(h, K_SU, [&] { return launch_nodal_update<T>(a, nb.rho[q], nb.w, nb.rho[q ^ 1], nb.xi, 0, h->stream); });
-  return e;
+  b.force = 2; b.pair = h->dim == 3; b.resid = 2; b.dot = 1;
+  b.rho = nb.rho; b.pold = nb.pi[q ^ 1]; b.pnew = nb.pi[q]; b.xi = nb.xi;
+  b.out = nb.rho;
+  return apply_passes<T>(h, b);
 }
 
 // The k-th CG iteration of a batch (k counts from 0 at the start of an inner
@@ -578,7 +576,7 @@ template <typename T> int autotune(rve_s* h, int L) {
     const int nc = rve_sched_candidates(h, which);
     float best_ms = 1e30f;
     for (int v = 0; v < nc; ++v) {
-      if (which == 0 && v == 6 && force_pass(h, v)) continue;   // the force pass has no prefetching tile: 6 is 0
+      if (force_pass(h, 0) && ((which == 0 && v == 6) || (which == 1 && v >= 3))) continue;   // same kernel as 0 or 1
       int* slot = which == 0 ? &a.var_a : which == 1 ? &a.var_e : which == 2 ? &a.var_c : &a.var_y;
       *slot = v;
       auto one = [&]() -> cudaError_t {
@@ -817,9 +815,10 @@ template <typename T> struct FeSolve {
       NodalBufs<T> nb(h, L);
       PassArgs<T> b = a;
       b.amode = A_NODAL; b.pmode = P_SOLVE; b.emode = E_NOUT;
-      b.in = nb.f; b.out = nb.w;
+      b.resid = 1; b.dot = 2;
+      b.in = nb.f; b.out = nb.rho;
+      CK(cudaMemsetAsync(nb.xi, 0, (size_t)L * h->D * h->N * sizeof(T), h->stream));
       CK(apply_passes<T>(h, b));
-      CK(timed(h, K_OTHER, [&] { return launch_nodal_update<T>(a, nullptr, nb.w, nb.rho[0], nb.xi, 1, h->stream); }));
     } else {
       a.amode = A_NODAL; a.pmode = P_NODAL_IN; a.emode = E_INIT;
       a.in = (const T*)h->fbuf;
@@ -1844,6 +1843,7 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
     a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = P_G; a.emode = E_OUT; a.grads = 1;
     set_force(h, a, 0);
     a.cg = h->cg_op;
+    a.pdl = !h->timing;
     a.in = (const float*)in; a.out = (float*)out;
     CK(apply_passes<float>(h, a));
   } else {

@@ -77,6 +77,10 @@ template <typename T> struct PassArgs {
   const T* rho;      // nodal state: residual and iterate of the force pass
   T* xi;
   int pair;          // 3D: the spectrum holds F0 and F1 (components j and 3 + j), pass B adds them
+  int pdl;           // launch with the programmatic-serialization attribute (see pdl_begin)
+  int resid;         // nodal state: the pass that loads the x spectra keeps the residual force R(k_x, ..) there
+                     // (components 2 D .. 3 D - 1 in 3D, D .. 2 D - 1 in 2D): 1 R = -f, 2 R -= alpha f
+  int dot;           // nodal state: pass C sums <rho, R> = |B rho|^2 -> beta (2: start of an inner solve)
   int grads;         // finite elements: passes C, D and E carry the D^2 edge differences of w instead of its D
                      // components (see pass_c_2d_fe), for results that leave the library as they are
 };
@@ -109,9 +113,6 @@ template <typename T> cudaError_t launch_cg_finish_x(const PassArgs<T>& a, cudaS
 template <typename T> cudaError_t launch_force_2d(const PassArgs<T>& a, cudaStream_t s);
 template <typename T> cudaError_t launch_force_3d(const PassArgs<T>& a, cudaStream_t s);
 // nodal-state form
-template <typename T>
-cudaError_t launch_nodal_update(const PassArgs<T>& a, const T* rho_old, const T* w, T* rho_new, T* xi, int init,
-                                cudaStream_t s);
 template <typename T>
 cudaError_t launch_nodal_finish(const PassArgs<T>& a, const T* pi_even, const T* pi_odd, const T* xi,
                                 cudaStream_t s);
