@@ -22,11 +22,12 @@
 
 namespace rve {
 
-// wrapped angle of index j on an axis of n points (exactly 0 at j = 0 and j = n/2)
-template <typename T> __device__ __forceinline__ T wrapped_theta(int j, int n) {
+// wrapped angle of index j on an axis of n points (inv_n = 1/n) (exactly 0 at j = 0 and j = n/2)
+template <typename T> __device__ __forceinline__ T wrapped_theta(int j, int n, double inv_n) {
   int w = (2 * j < n) ? j : j - n;
   if (2 * j == n) w = 0;
-  return (T)(6.283185307179586477 * (double)w / (double)n);
+  // n is a power of two: 1/n is exact, and the product rounds like the quotient
+  return (T)(6.283185307179586477 * (double)w * inv_n);
 }
 
 template <typename T> __device__ __forceinline__ void sincos_t(T x, T* s, T* c);
@@ -69,7 +70,7 @@ __device__ __forceinline__ int deriv_symbols(int deriv, const int* j, const int*
   }
   T th[3];
 #pragma unroll
-  for (int a = 0; a < D; ++a) th[a] = wrapped_theta<T>(j[a], n[a]);
+  for (int a = 0; a < D; ++a) th[a] = wrapped_theta<T>(j[a], n[a], __hiloint2double((1023 - (31 - __clz(n[a]))) << 20, 0));
   if (deriv == D_FOURIER) {
 #pragma unroll
     for (int a = 0; a < D; ++a) g[0][a] = mkc<T>((T)0, th[a] * ih[a]);

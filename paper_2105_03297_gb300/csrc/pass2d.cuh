@@ -440,8 +440,16 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
     if (kx >= KX) continue;
     C t[2] = {buf[2 * pc * LD + ky], buf[(2 * pc + 1) * LD + ky]};
     const C r0 = t[0], r1 = t[1];
-    if (kx == 0 && ky == 0) t[0] = t[1] = mkc<T>(0, 0);   // k = 0: no mean
-    else solve_2d<T>(t, a.ph[0][kx], a.ph[1][ky], a.ih[0], a.ih[1], a.inv_n);
+    if (kx == 0 && ky == 0) {
+      t[0] = t[1] = mkc<T>(0, 0);   // k = 0: no mean
+    } else if (a.pmode == P_FINITE) {   // B^H B = sum |g|^2 I; both triangles have |g_a| = |e_a - 1| / h_a
+      const C ex = a.ph[0][kx], ey = a.ph[1][ky];
+      const T dx = a.ih[0] * a.ih[0] * (((ex.x - (T)1) * (ex.x - (T)1)) + ex.y * ex.y);
+      const T dy = a.ih[1] * a.ih[1] * (((ey.x - (T)1) * (ey.x - (T)1)) + ey.y * ey.y);
+      const T id = a.inv_n / ((T)2 * (dx + dy));
+      t[0] = cscale(t[0], id);
+      t[1] = cscale(t[1], id);
+    } else solve_2d<T>(t, a.ph[0][kx], a.ph[1][ky], a.ih[0], a.ih[1], a.inv_n);
     if (a.dot) {
       const T d = r0.x * t[0].x + r0.y * t[0].y + r1.x * t[1].x + r1.y * t[1].y;
       acc.add(kx == 0 || kx == KX - 1 ? d : (T)2 * d);
@@ -663,7 +671,7 @@ __device__ __forceinline__ T strain_update(const PassArgs<T>& a, int64_t idx, T*
 // a third of the spectrum.  Bound by the r traffic (read and write, 16-byte
 // accesses).  W = 4: the spectrum holds the edge differences of w instead (see
 // pass_c_2d_fe).  grid (n_y/TY, L).
-template <typename T, int NX, int TY, int NT, int W>
+template <typename T, int NX, int TY, int NT, int W, bool GRAD = false>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pass_e_2d_fe(PassArgs<T> a) {
   using C = cplx<T>;
   constexpr int NPR = TY / 2 + 1;
@@ -691,10 +699,11 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   for (int i = threadIdx.x; i < TY * (NX / VL); i += NT) {
     const int yy = i / (NX / VL), x0 = (i % (NX / VL)) * VL, pr = yy / 2;
     const int64_t v0 = (int64_t)l * a.m * a.N + (int64_t)(y0 + yy) * NX + x0;
-    T rv[6][VL], q[6][VL];
+    constexpr int NC = GRAD ? 8 : 6;   // GRAD: finite strain, q = grad w, component 4 q + 2 i + a
+    T rv[NC][VL], q[NC][VL];
     if (cgm) {
 #pragma unroll
-      for (int c = 0; c < 6; ++c) vloadn<T, VL>(rv[c], a.r + v0 + c * a.N);
+      for (int c = 0; c < NC; ++c) vloadn<T, VL>(rv[c], a.r + v0 + c * a.N);
     }
     // node rows yy and yy + 1 at columns x0 .. x0 + VL: rows 2 pr and 2 pr + 1
     // are the two parts of pair pr
@@ -709,6 +718,16 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
       }
 #pragma unroll
     for (int k = 0; k < VL; ++k) {
+      if constexpr (GRAD) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          q[2 * j][k] = (lo[j][k + 1] - lo[j][k]) * ihx;
+          q[2 * j + 1][k] = (hi[j][k] - lo[j][k]) * ihy;
+          q[4 + 2 * j][k] = (hi[j][k + 1] - hi[j][k]) * ihx;
+          q[5 + 2 * j][k] = (hi[j][k + 1] - lo[j][k + 1]) * ihy;
+        }
+        continue;
+      }
       if constexpr (W == 4) {   // components d_x w_0, d_x w_1, d_y w_0, d_y w_1 at the lower end of each edge
         q[0][k] = lo[0][k];
         q[1][k] = lo[3][k];
@@ -729,7 +748,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
     }
     T s = 0;
 #pragma unroll
-    for (int c = 0; c < 6; ++c) s += strain_update<T, VL>(a, v0 + c * a.N, rv[c], q[c], alpha);
+    for (int c = 0; c < NC; ++c) s += strain_update<T, VL>(a, v0 + c * a.N, rv[c], q[c], alpha);
+    if (GRAD && a.emode == E_INIT) {   // the padding component
+      T z[VL];
+#pragma unroll
+      for (int k = 0; k < VL; ++k) z[k] = 0;
+      strain_update<T, VL>(a, v0 + 8 * a.N, z, z, alpha);
+    }
     acc.add(s);
   }
   if (a.emode == E_CG || a.emode == E_INIT) {
@@ -824,12 +849,12 @@ cudaError_t launch_a_2d_n(const PassArgs<T>& a, cudaStream_t s) {
   }
   return launch_a_2d_t<T, NX, tile_rows<T>(0)>(a, s);
 }
-template <typename T, int NX, int TY, int W>
+template <typename T, int NX, int TY, int W, bool GRAD = false>
 cudaError_t launch_e_2d_fe_w(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int R = W * (TY / 2 + 1);
   constexpr int NT = fft_threads<NX, R>();
   const size_t sm = sizeof(cplx<T>) * R * ae_ld<NX>();
-  auto k = pass_e_2d_fe<T, NX, TY, NT, W>;
+  auto k = pass_e_2d_fe<T, NX, TY, NT, W, GRAD>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.L), NT, sm, s, a);
@@ -845,6 +870,9 @@ template <typename T> bool fe_path(const PassArgs<T>& a) { return a.deriv == D_F
 // Tile variants of the 2D pass E: 0 default rows per block, 1 half, 2 double.
 template <typename T, int NX>
 cudaError_t launch_e_2d_n(const PassArgs<T>& a, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {   // finite strain after the force pass
+    if (a.force == 3) return launch_e_2d_fe_w<T, NX, tile_rows<T>(1), 2, true>(a, s);
+  }
   if (fe_path(a) && (a.emode == E_CG || a.emode == E_INIT || a.emode == E_OUT)) {
     if (a.grads) return launch_e_2d_fe_w<T, NX, tile_rows<T>(1), 4>(a, s);
     if constexpr (NX >= 64) {
@@ -877,7 +905,7 @@ cudaError_t launch_c_2d_v(const PassArgs<T>& a, cudaStream_t s) {
 
 template <typename T, int NY>
 cudaError_t launch_c_2d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if (fe_path(a)) {
+  if (fe_path(a) || a.force == 3) {
     if constexpr (fft_split_count<NY>() > 1) {
       if (a.var_c == 1) return a.grads ? launch_c_2d_v<T, NY, 1, 4>(a, s) : launch_c_2d_v<T, NY, 1, 2>(a, s);
     }

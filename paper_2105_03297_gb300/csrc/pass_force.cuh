@@ -27,12 +27,14 @@
 //   S_NODAL   CG on nodal fields: pi = rho + beta pi_old, xi += alpha_prev
 //             pi_old, sigma = C B pi, <B pi, sigma> -> alpha.  Bound by issue:
 //             about 300 arithmetic instructions per voxel.
+//   S_GRAD    finite strain (2D): the divergence of the stress field in, 4
+//             components P_ia per triangle.
 #pragma once
 #include "pass3d.cuh"
 
 namespace rve {
 
-enum { S_STRAIN = 0, S_NODAL = 1 };
+enum { S_STRAIN = 0, S_NODAL = 1, S_GRAD = 2 };
 
 // Value of the previous (next) column of the same row; at the row's start (end)
 // inside a warp the row wraps, at a warp's first (last) lane of a longer row
@@ -439,6 +441,20 @@ template <typename T, int NX, int TY, int LN> constexpr size_t force_2d_smem() {
   return sizeof(cplx<T>) * TY * force_ld<T, NX, TY>() + sizeof(T) * 4 * (NX > 32 ? (TY + LN) * (NX / 32) : 0);
 }
 
+// The same for a field of first Piola-Kirchhoff stresses P[q][i][a] (finite
+// strain; not symmetric).
+template <typename T>
+__device__ __forceinline__ void pixel_divergence(const T P[8], T ihx, T ihy, T f[4][2]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const T x0 = ihx * P[2 * i], y0 = ihy * P[2 * i + 1], x1 = ihx * P[4 + 2 * i], y1 = ihy * P[5 + 2 * i];
+    f[0][i] = -x0 - y0;
+    f[1][i] = x0 - y1;
+    f[2][i] = y0 - x1;
+    f[3][i] = x1 + y1;
+  }
+}
+
 // grid (n_y/TY, L).  NT < NX: a thread marches NX / NT columns one after the
 // other; NT > NX: NT / NX rows side by side.
 template <typename T, int NX, int TY, int NT, int MB, int SRC>
@@ -496,7 +512,17 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
       carry[0] = s[1][0];
       carry[1] = s[1][1];
     };
-    if constexpr (SRC == S_STRAIN) {
+    if constexpr (SRC == S_GRAD) {
+      const T* __restrict__ in = a.in + (int64_t)l * a.m * N + x;
+      for (int yy = first; yy < end; ++yy) {
+        const int64_t o = (int64_t)((y0 + yy) & (ny - 1)) * NX;
+        T P[8], f[4][2];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) P[s] = in[o + s * N];
+        pixel_divergence<T>(P, ihx, ihy, f);
+        node_row(yy, f, yy >= ln * TYL);
+      }
+    } else if constexpr (SRC == S_STRAIN) {
       const int64_t base = (int64_t)l * a.m * N + x;
       const T* __restrict__ rp = (cgm ? a.r : a.in) + base;
       const T* __restrict__ po = a.pold + base;
@@ -753,6 +779,9 @@ template <typename T, int NX>
 cudaError_t launch_force_2d_n(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int TY = sizeof(T) == 4 ? 8 : 4;
   if (a.force == 2) return launch_force_2d_auto<T, NX, S_NODAL>(a, s);
+  if constexpr (sizeof(T) == 8) {
+    if (a.force == 3) return launch_force_2d_auto<T, NX, S_GRAD>(a, s);
+  }
   if constexpr (NX >= 64) {
     constexpr int NT = force_threads2<NX, TY>();
     if (a.var_a == 1) return launch_force_2d_r<T, NX, TY / 2, S_STRAIN>(a, s);

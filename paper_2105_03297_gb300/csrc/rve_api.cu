@@ -440,6 +440,7 @@ inline cudaError_t apply_finite(rve_s* h, const PassArgs<double>& a) {
   PassArgs<double> b = a;
   b.amode = A_BARE; b.pmode = P_FINITE; b.emode = E_CG;
   b.in = (const double*)h->fbuf;
+  b.force = h->dim == 2 ? 3 : 0;   // 2D: the transforms carry the divergence, two components instead of nine
   if (e == cudaSuccess) e = pass_a<double>(h, b);
   if (e == cudaSuccess) e = pass_mid<double>(h, b);
   if (e == cudaSuccess) e = pass_e<double>(h, b);
@@ -1242,6 +1243,7 @@ int solve_finite(rve_s* h, const double* Fmac_host, int L, double rel_tol, int m
     PassArgs<double> b = a;
     b.amode = A_BARE; b.pmode = P_FINITE; b.emode = E_INIT;
     b.in = (const double*)h->fbuf;
+    b.force = h->dim == 2 ? 3 : 0;
     CK(apply_passes<double>(h, b));
     if ((rc = read_state(h, L))) return rc;
     bool any = false;

@@ -71,7 +71,8 @@ template <typename T> struct PassArgs {
   int pf_ahead;      // 3D passes A to D: blocks ahead in launch order whose input each block asks the TMA
                      // unit to prefetch into L2, 0 = none; pass E: 1 = prefetch the tile's own r rows
   int deriv;         // Deriv
-  int force;         // first pass of the finite elements: 1 strain fields, 2 nodal fields (pass_force.cuh)
+  int force;         // first pass of the finite elements: 1 strain fields, 2 nodal fields, 3 stress
+                     // field of finite strain (2D) (pass_force.cuh)
   const T* pold;     // previous and new search direction of the force pass (different arrays)
   T* pnew;
   const T* rho;      // nodal state: residual and iterate of the force pass
