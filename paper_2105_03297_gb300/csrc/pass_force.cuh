@@ -2,7 +2,7 @@
 // real space, and the forward x FFT of the D nodal components.
 //
 // A block owns TY voxel rows of one z plane over the whole of x and marches
-// along y.  A thread owns one column x: per voxel it forms the element
+// along y.  A thread owns one column x (3D, FP32: two): per voxel it forms the element
 // stresses and the forces of the voxel's 2^D corners (the row below the tile,
 // which also acts on the tile's first node row, is computed again: one row in
 // TY more).  The corners with dx = 1 go to the next column by a warp shuffle,
@@ -23,7 +23,10 @@
 //             sigma = C p, <p, sigma> -> alpha (A_CG); or sigma = C in
 //             (A_FIELD), sigma = in (A_BARE).  p_old and p_new are different
 //             arrays: the row below the tile is read by two blocks.
-//             Bound by the 5 m N values per iteration.
+//             Bound by the 5 m N values per iteration (256 x 256 x 64 in FP32:
+//             622 us, 4.9 TB/s of r, p_old, x in and p, x out; a probe that
+//             marches the same rows without the arithmetic reaches 5.6: each
+//             1 KB row of 36 components opens DRAM pages of its own).
 //   S_NODAL   CG on nodal fields: pi = rho + beta pi_old, xi += alpha_prev
 //             pi_old, sigma = C B pi, <B pi, sigma> -> alpha.  Bound by issue:
 //             about 300 arithmetic instructions per voxel.
@@ -132,24 +135,27 @@ template <typename T, int NX, int TY> __host__ __device__ constexpr int force_ld
 }
 // Stages of the strain source's ring (18 values a thread each).
 template <typename T> __host__ __device__ constexpr int force_stages() { return sizeof(T) == 4 ? 3 : 2; }
-template <typename T, int NX, int TY, int NT, int SRC> constexpr size_t force_3d_smem() {
-  return (SRC == S_STRAIN ? sizeof(T) * force_stages<T>() * 18 * NT : 0) + sizeof(cplx<T>) * 3 * TY * force_ld<T, NX, TY>() +
-         sizeof(T) * 12 * (NX > 32 ? (TY + NT / NX) * (NX / 32) : 0);
+template <typename T, int NX, int TY, int NT, int VL, int SRC> constexpr size_t force_3d_smem() {
+  return (SRC == S_STRAIN ? sizeof(T) * force_stages<T>() * 18 * NT * VL : 0) +
+         sizeof(cplx<T>) * 3 * TY * force_ld<T, NX, TY>() +
+         sizeof(T) * 12 * (NX / VL > 32 ? (TY + NT * VL / NX) * (NX / VL / 32) : 0);
 }
 
-// grid (n_y/TY, n_z, L); NT / NX rows are marched side by side.
-template <typename T, int NX, int TY, int NT, int MB, int SRC>
+// grid (n_y/TY, n_z, L).  A thread owns VL neighbouring columns, TPR threads a
+// row; NT / TPR rows are marched side by side.
+template <typename T, int NX, int TY, int NT, int MB, int VL, int SRC>
 __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
   using C = cplx<T>;
   constexpr int KX = NX / 2 + 1;
   constexpr int LD = force_ld<T, NX, TY>();
-  constexpr int LN = NT / NX, TYL = TY / LN;     // row lanes, rows per lane
-  constexpr int NW = NX > 32 ? NX / 32 : 1;      // warps per row
-  static_assert(NT % NX == 0 && TY % LN == 0, "threads cover whole rows");
+  constexpr int TPR = NX / VL;                   // threads per row
+  constexpr int LN = NT / TPR, TYL = TY / LN;    // row lanes, rows per lane
+  constexpr int NW = TPR > 32 ? TPR / 32 : 1;    // warps per row
+  static_assert(NT % TPR == 0 && TY % LN == 0, "threads cover whole rows");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);                        // [3][TY][LD]
-  T* edge = reinterpret_cast<T*>(buf + 3 * TY * LD);              // [LN][TYL + 1][NW][12], NX > 32
-  T* ring = edge + (NX > 32 ? 12 * (TY + LN) * NW : 0);           // strain source: [stages][18][NT]
+  T* edge = reinterpret_cast<T*>(buf + 3 * TY * LD);              // [LN][TYL + 1][NW][12], TPR > 32
+  T* ring = edge + (TPR > 32 ? 12 * (TY + LN) * NW : 0);          // strain source: [stages][18][NT] x VL
   __shared__ double red[NT / 32];
   __shared__ T cols[NT];
   __shared__ int flag;
@@ -160,21 +166,24 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
-  const int x = threadIdx.x % NX, ln = threadIdx.x / NX;
+  const int tx = threadIdx.x % TPR, ln = threadIdx.x / TPR, x = tx * VL;
   const int lane = threadIdx.x & 31;
   const bool cgm = a.amode == A_CG;
   const bool use_old = cgm && cg->it > 0;
   const T beta = use_old ? cg_beta<T>(cg) : (T)0, alpha_prev = use_old ? cg_alpha<T>(cg) : (T)0;
   const T ih[3] = {a.ih[0], a.ih[1], a.ih[2]};
   const T* Ep = a.E + (int64_t)(l / a.lcs) * N + (int64_t)z * ny * NX + x;
+  const int first = ln * TYL - 1, end = (ln + 1) * TYL;
   Acc<T> acc;
-  T carry[2][3];   // [dz][j]: dy = 1 corners of the row below
+  T carry[VL][2][3];   // [column][dz][j]: dy = 1 corners of the row below
 #pragma unroll
-  for (int j = 0; j < 3; ++j) carry[0][j] = carry[1][j] = 0;
+  for (int k = 0; k < VL; ++k)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) carry[k][0][j] = carry[k][1][j] = 0;
+  auto load_e = [&](int yy, T* e) { vloadn<T, VL>(e, Ep + (int64_t)((y0 + yy) & (ny - 1)) * NX); };
 
-  // corner forces of row yy -> node row yy
-  auto node_row = [&](int yy, const T f[8][3], bool own) {
-    T s[2][2][3];   // [dy][dz][j]
+  // corners with dx = 1 of the last column (f) -> first column of the next thread
+  auto pass_on = [&](int yy, const T f[8][3], T pv[2][2][3]) {
 #pragma unroll
     for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
@@ -182,25 +191,40 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
           const T u = f[1 + 2 * dy + 4 * dz][j];
-          T p = from_prev<NX>(u);
-          if constexpr (NX > 32) {
-            if (lane == 31) edge[((ln * (TYL + 1) + yy + 1 - ln * TYL) * NW + x / 32) * 12 + dy * 6 + dz * 3 + j] = u;
-            if (lane == 0) p = 0;
-          } else if constexpr (NX == 32) {
+          T q = from_prev<TPR>(u);
+          if constexpr (TPR > 32) {
+            if (lane == 31) edge[((ln * (TYL + 1) + yy - first) * NW + tx / 32) * 12 + dy * 6 + dz * 3 + j] = u;
+            if (lane == 0) q = 0;
+          } else if constexpr (TPR == 32) {
             const T w = __shfl_sync(0xffffffffu, u, 31);
-            if (lane == 0) p = w;
+            if (lane == 0) q = w;
           }
-          s[dy][dz][j] = f[2 * dy + 4 * dz][j] + p;
+          pv[dy][dz][j] = q;
         }
-    if (own) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        buf[(j * TY + yy) * LD + x] = mkc<T>(s[0][0][j] + carry[0][j], s[0][1][j] + carry[1][j]);
-    }
+  };
+  // column k of row yy: corners dx = 0 of its voxel (f) and dx = 1 of the voxel before (pv)
+  auto put_column = [&](int yy, int k, const T f[8][3], const T pv[2][2][3]) {
+    const bool own = yy > first;
+    T v[2][3];
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) carry[dz][j] = s[1][dz][j];
+      for (int j = 0; j < 3; ++j) {
+        v[dz][j] = f[4 * dz][j] + pv[0][dz][j] + carry[k][dz][j];
+        carry[k][dz][j] = f[2 + 4 * dz][j] + pv[1][dz][j];
+      }
+    if (own) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) buf[(j * TY + yy) * LD + x + k] = mkc<T>(v[0][j], v[1][j]);
+    }
+  };
+  auto right = [&](const T f[8][3], T pv[2][2][3]) {   // within the thread
+#pragma unroll
+    for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+      for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) pv[dy][dz][j] = f[1 + 2 * dy + 4 * dz][j];
   };
 
   if constexpr (SRC == S_STRAIN) {
@@ -215,20 +239,20 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
     T* pn = a.pnew + base;
     T* xp = a.x + base;
     const bool mat = a.amode != A_BARE;
-    const int first = ln * TYL - 1, end = (ln + 1) * TYL;
     auto off = [&](int yy) -> unsigned { return (unsigned)(((y0 + yy) & (ny - 1)) * NX + x); };
+    auto slot = [&](int t, int s) -> T* { return ring + (((t % ST) * 18 + s) * NT + threadIdx.x) * VL; };
     auto issue = [&](int yy, int t) {   // step (yy, t) into slot t % ST
       if (yy < end) {
         const unsigned o = off(yy);
-        T* slot = ring + (t % ST) * 18 * NT + threadIdx.x;
+        constexpr int B = VL * (int)sizeof(T);
 #pragma unroll
-        for (int s = 0; s < 6; ++s) copy_async<(int)sizeof(T)>(slot + s * NT, rp + (6 * t + s) * N + o);
+        for (int s = 0; s < 6; ++s) copy_async<B>(slot(t, s), rp + (6 * t + s) * N + o);
         if (use_old) {
 #pragma unroll
-          for (int s = 0; s < 6; ++s) copy_async<(int)sizeof(T)>(slot + (6 + s) * NT, po + (6 * t + s) * N + o);
-          if (yy >= ln * TYL) {
+          for (int s = 0; s < 6; ++s) copy_async<B>(slot(t, 6 + s), po + (6 * t + s) * N + o);
+          if (yy > first) {
 #pragma unroll
-            for (int s = 0; s < 6; ++s) copy_async<(int)sizeof(T)>(slot + (12 + s) * NT, xp + (6 * t + s) * N + o);
+            for (int s = 0; s < 6; ++s) copy_async<B>(slot(t, 12 + s), xp + (6 * t + s) * N + o);
           }
         }
       }
@@ -237,55 +261,76 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
     const T r2 = (T)kInvSqrt2;
 #pragma unroll
     for (int t = 0; t < ST - 1; ++t) issue(first, t);
-    T e = mat ? Ep[(int64_t)((y0 + first) & (ny - 1)) * NX] : (T)1;
-    for (int yy = first; yy < end; ++yy) {
-      const bool own = yy >= ln * TYL;
-      const unsigned o = off(yy);
-      const T en = (mat && yy + 1 < end) ? Ep[(int64_t)((y0 + yy + 1) & (ny - 1)) * NX] : (T)1;
-      T f[8][3];
+    T e[VL], en[VL];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) f[c][0] = f[c][1] = f[c][2] = 0;
+    for (int k = 0; k < VL; ++k) e[k] = en[k] = 1;
+    if (mat) load_e(first, e);
+    for (int yy = first; yy < end; ++yy) {
+      const bool own = yy > first;
+      const unsigned o = off(yy);
+      if (mat && yy + 1 < end) load_e(yy + 1, en);
+      T f[VL][8][3];
+#pragma unroll
+      for (int k = 0; k < VL; ++k)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) f[k][c][0] = f[k][c][1] = f[k][c][2] = 0;
       T pq = 0;
 #pragma unroll
       for (int t = 0; t < 6; ++t) {
         issue(t + ST - 1 < 6 ? yy : yy + 1, (t + ST - 1) % 6);
         copy_async_wait<ST - 1>();
-        const T* slot = ring + (t % ST) * 18 * NT + threadIdx.x;
-        T p[6];
+        T p[6][VL];
 #pragma unroll
-        for (int s = 0; s < 6; ++s) p[s] = slot[s * NT];
+        for (int s = 0; s < 6; ++s) vloadn<T, VL>(p[s], slot(t, s));
         if (use_old) {
-          T v[6];
 #pragma unroll
-          for (int s = 0; s < 6; ++s) { v[s] = slot[(6 + s) * NT]; p[s] += beta * v[s]; }
-          if (own) {
+          for (int s = 0; s < 6; ++s) {
+            T v[VL];
+            vloadn<T, VL>(v, slot(t, 6 + s));
 #pragma unroll
-            for (int s = 0; s < 6; ++s) xp[(6 * t + s) * N + o] = slot[(12 + s) * NT] + alpha_prev * v[s];
+            for (int k = 0; k < VL; ++k) p[s][k] += beta * v[k];
+            if (own) {
+              T xv[VL];
+              vloadn<T, VL>(xv, slot(t, 12 + s));
+#pragma unroll
+              for (int k = 0; k < VL; ++k) xv[k] += alpha_prev * v[k];
+              vstoren<T, VL>(xp + (6 * t + s) * N + o, xv);
+            }
           }
         }
         if (cgm && own) {
 #pragma unroll
-          for (int s = 0; s < 6; ++s) pn[(6 * t + s) * N + o] = p[s];
+          for (int s = 0; s < 6; ++s) vstoren<T, VL>(pn + (6 * t + s) * N + o, p[s]);
         }
-        T S[3][3];
-        if (mat) {
-          const T tr = e * (a.lam * (p[0] + p[1] + p[2])), me = e * a.mu2;
+#pragma unroll
+        for (int k = 0; k < VL; ++k) {
           T sg[6];
+          if (mat) {
+            const T tr = e[k] * (a.lam * (p[0][k] + p[1][k] + p[2][k])), me = e[k] * a.mu2;
 #pragma unroll
-          for (int s = 0; s < 6; ++s) sg[s] = s < 3 ? tr + me * p[s] : me * p[s];
+            for (int s = 0; s < 6; ++s) sg[s] = s < 3 ? tr + me * p[s][k] : me * p[s][k];
 #pragma unroll
-          for (int s = 0; s < 6; ++s) pq += p[s] * sg[s];
+            for (int s = 0; s < 6; ++s) pq += p[s][k] * sg[s];
+          } else {
+#pragma unroll
+            for (int s = 0; s < 6; ++s) sg[s] = p[s][k];
+          }
+          T S[3][3];
           S[0][0] = sg[0]; S[1][1] = sg[1]; S[2][2] = sg[2];
           S[1][2] = S[2][1] = r2 * sg[3]; S[0][2] = S[2][0] = r2 * sg[4]; S[0][1] = S[1][0] = r2 * sg[5];
-        } else {
-          S[0][0] = p[0]; S[1][1] = p[1]; S[2][2] = p[2];
-          S[1][2] = S[2][1] = r2 * p[3]; S[0][2] = S[2][0] = r2 * p[4]; S[0][1] = S[1][0] = r2 * p[5];
+          tet_forces<T>(t, S, ih, f[k]);
         }
-        tet_forces<T>(t, S, ih, f);
       }
       if (own) acc.add(pq);
-      node_row(yy, f, own);
-      e = en;
+      T pv[2][2][3];
+      pass_on(yy, f[VL - 1], pv);
+#pragma unroll
+      for (int k = 0; k < VL; ++k) {
+        put_column(yy, k, f[k], pv);
+        right(f[k], pv);
+      }
+#pragma unroll
+      for (int k = 0; k < VL; ++k) e[k] = en[k];
     }
     copy_async_wait<0>();
   } else {
@@ -296,23 +341,27 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
     const T* __restrict__ po = a.pold;
     T* __restrict__ pn = a.pnew;
     T* __restrict__ xi = a.xi;
-    const bool last = NX > 32 && lane == 31;   // the next column belongs to another warp
-    // values of node row yy in flight: planes z and z + 1, own column and (last
+    const bool last = TPR > 32 && lane == 31;   // the next column belongs to another warp
+    // values of node row yy in flight: planes z and z + 1, own columns and (last
     // lane) the next one; p_old counts as 0 in the first iteration
-    T rv[2][3], pv[2][3], xv[3], re[2][3], pe[2][3];
+    T rv[2][3][VL], pv[2][3][VL], xv[3][VL], re[2][3], pe[2][3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) pv[0][j] = pv[1][j] = re[0][j] = re[1][j] = pe[0][j] = pe[1][j] = xv[j] = 0;
+    for (int j = 0; j < 3; ++j) {
+      re[0][j] = re[1][j] = pe[0][j] = pe[1][j] = 0;
+#pragma unroll
+      for (int k = 0; k < VL; ++k) pv[0][j][k] = pv[1][j][k] = xv[j][k] = 0;
+    }
     auto fetch = [&](int yy) {
       const unsigned row = (unsigned)(((y0 + yy) & (ny - 1)) * NX), o = row + x;
 #pragma unroll
       for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          rv[dz][j] = (rho + zo[dz] + j * N)[o];
-          if (use_old) pv[dz][j] = (po + zo[dz] + j * N)[o];
+          vloadn<T, VL>(rv[dz][j], rho + zo[dz] + j * N + o);
+          if (use_old) vloadn<T, VL>(pv[dz][j], po + zo[dz] + j * N + o);
         }
       if (last) {
-        const unsigned on = row + ((x + 1) & (NX - 1));
+        const unsigned on = row + ((x + VL) & (NX - 1));
 #pragma unroll
         for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
@@ -321,76 +370,111 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
             if (use_old) pe[dz][j] = (po + zo[dz] + j * N)[on];
           }
       }
-      if (use_old && yy >= ln * TYL && yy < (ln + 1) * TYL) {
+      if (use_old && yy > first && yy < end) {
 #pragma unroll
-        for (int j = 0; j < 3; ++j) xv[j] = (xi + zo[0] + j * N)[o];
+        for (int j = 0; j < 3; ++j) vloadn<T, VL>(xv[j], xi + zo[0] + j * N + o);
       }
     };
-    // pi of node row yy at columns x and x + 1: u[dx + 2 dz][j]
-    auto commit = [&](int yy, T u[4][3]) {
+    // pi of node row yy at columns x .. x + VL: u[dz][column][j]
+    auto commit = [&](int yy, T u[2][VL + 1][3]) {
 #pragma unroll
       for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          const T p = rv[dz][j] + beta * pv[dz][j];
-          u[2 * dz][j] = p;
-          T q = from_next<NX>(p);
-          if constexpr (NX > 32) {
+#pragma unroll
+          for (int k = 0; k < VL; ++k) u[dz][k][j] = rv[dz][j][k] + beta * pv[dz][j][k];
+          T q = from_next<TPR>(u[dz][0][j]);
+          if constexpr (TPR > 32) {
             if (last) q = re[dz][j] + beta * pe[dz][j];
-          } else if constexpr (NX == 32) {
-            const T w = __shfl_sync(0xffffffffu, p, 0);
+          } else if constexpr (TPR == 32) {
+            const T w = __shfl_sync(0xffffffffu, u[dz][0][j], 0);
             if (lane == 31) q = w;
           }
-          u[2 * dz + 1][j] = q;
+          u[dz][VL][j] = q;
         }
-      if (yy >= ln * TYL && yy < (ln + 1) * TYL) {
+      if (yy > first && yy < end) {
         const unsigned o = (unsigned)(((y0 + yy) & (ny - 1)) * NX + x);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          (pn + zo[0] + j * N)[o] = u[0][j];
-          if (use_old) (xi + zo[0] + j * N)[o] = xv[j] + alpha_prev * pv[0][j];
+          T s[VL];
+#pragma unroll
+          for (int k = 0; k < VL; ++k) s[k] = u[0][k][j];
+          vstoren<T, VL>(pn + zo[0] + j * N + o, s);
+          if (use_old) {
+#pragma unroll
+            for (int k = 0; k < VL; ++k) s[k] = xv[j][k] + alpha_prev * pv[0][j][k];
+            vstoren<T, VL>(xi + zo[0] + j * N + o, s);
+          }
         }
       }
     };
-    T lo[4][3], hi[4][3];
-    const int first = ln * TYL - 1, end = (ln + 1) * TYL;
+    T lo[2][VL + 1][3], hi[2][VL + 1][3];
     fetch(first);
     commit(first, lo);
     fetch(first + 1);
-    T e = Ep[(int64_t)((y0 + first) & (ny - 1)) * NX];
+    T e[VL], en[VL];
+    load_e(first, e);
+#pragma unroll
+    for (int k = 0; k < VL; ++k) en[k] = 0;
     for (int yy = first; yy < end; ++yy) {
       commit(yy + 1, hi);
-      T en = 0;
       if (yy + 1 < end) {
         fetch(yy + 2);
-        en = Ep[(int64_t)((y0 + yy + 1) & (ny - 1)) * NX];
+        load_e(yy + 1, en);
       }
-      T uc[8][3], f[8][3];
+      const bool own = yy > first;
+      T pq = 0, keep[2][2][3], f[8][3], pv1[2][2][3];
+      // from the last column back, so that one column's forces are live at a time:
+      // its dx = 0 corners wait in keep for the dx = 1 corners of the column before
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
+      for (int k = VL - 1; k >= 0; --k) {
+        T uc[8][3];
 #pragma unroll
-        for (int j = 0; j < 3; ++j) uc[c][j] = ((c >> 1) & 1 ? hi : lo)[(c & 1) + 2 * (c >> 2)][j];
-      const T pq = voxel_forces_3d<T>(uc, e, a.lam, a.mu2, ih, f);
-      const bool own = yy >= ln * TYL;
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) uc[c][j] = ((c >> 1) & 1 ? hi : lo)[c >> 2][k + (c & 1)][j];
+        pq += voxel_forces_3d<T>(uc, e[k], a.lam, a.mu2, ih, f);
+        if (k == VL - 1) pass_on(yy, f, pv1);
+        if (k < VL - 1) {   // finish column k + 1
+          T g[8][3], pr[2][2][3];
+          right(f, pr);
+#pragma unroll
+          for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+            for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+              for (int j = 0; j < 3; ++j) g[2 * dy + 4 * dz][j] = keep[dy][dz][j];
+          put_column(yy, k + 1, g, pr);
+        }
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+          for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) keep[dy][dz][j] = f[2 * dy + 4 * dz][j];
+      }
+      put_column(yy, 0, f, pv1);
       if (own) acc.add(pq);
-      node_row(yy, f, own);
-      e = en;
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+      for (int k = 0; k < VL; ++k) e[k] = en[k];
 #pragma unroll
-        for (int j = 0; j < 3; ++j) lo[c][j] = hi[c][j];
+      for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+        for (int c = 0; c <= VL; ++c)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) lo[dz][c][j] = hi[dz][c][j];
     }
   }
 
   __syncthreads();
-  if constexpr (NX > 32) {
+  if constexpr (TPR > 32) {
     for (int i = threadIdx.x; i < 3 * TY * NW; i += NT) {
       const int w = i % NW, yy = (i / NW) % TY, j = i / (NW * TY);
       const int q = yy / TYL, lr = yy % TYL + 1;   // the lane's rows: 0 is the row below its first
       const int wp = (w + NW - 1) % NW;
       const T* r0 = edge + ((q * (TYL + 1) + lr) * NW + wp) * 12 + j;        // dy = 0 of row yy
       const T* r1 = edge + ((q * (TYL + 1) + lr - 1) * NW + wp) * 12 + 6 + j;   // dy = 1 of row yy - 1
-      C* p = buf + (j * TY + yy) * LD + 32 * w;
+      C* p = buf + (j * TY + yy) * LD + 32 * VL * w;
       *p = mkc<T>(p->x + r0[0] + r1[0], p->y + r0[3] + r1[3]);
     }
     __syncthreads();
@@ -706,39 +790,50 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
 }
 
 // ------------------------------------------------------------ launchers
-template <typename T, int NX, int TY, int NT, int SRC>
+template <typename T, int NX, int TY, int NT, int VL, int SRC>
 cudaError_t launch_force_3d_t(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int MB = sizeof(T) == 8 ? 1 : NT <= 64 ? 8 : NT <= 128 ? 4 : NT <= 256 ? 2 : 1;
-  constexpr size_t sm = force_3d_smem<T, NX, TY, NT, SRC>();
+  // resident blocks the registers are sized for (shared memory holds two of the
+  // strain source's 128-thread blocks)
+  constexpr int MB = sizeof(T) == 8 ? 1 : VL == 2 ? (NT <= 64 ? 2 : 1) * (SRC == S_NODAL ? 3 : 2) / (NT <= 128 ? 1 : 2)
+                                         : NT <= 64 ? 8 : NT <= 128 ? 4 : NT <= 256 ? 2 : 1;
+  constexpr size_t sm = force_3d_smem<T, NX, TY, NT, VL, SRC>();
   static_assert(sm <= 222 * 1024, "shared memory of the tile");
-  auto k = force_3d<T, NX, TY, NT, MB, SRC>;
+  auto k = force_3d<T, NX, TY, NT, MB, VL, SRC>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.n[2], a.L), NT, sm, s, a);
 }
+// Columns per thread: two in FP32 where a row still fills a warp (8-byte
+// accesses: half the load and store instructions, which throttled the pass, and
+// half the shuffles).  us per iteration, one and two columns: strain source 256 x
+// 256 x 64 657, 622, 64^3 (six load cases) 265, 253, 128^3 342, 341; nodal source
+// 256 x 256 x 128 319, 248, 64^3 71, 58, 128^3 (two) 187, 164.
+template <typename T, int NX> constexpr int force_cols3() { return sizeof(T) == 4 && NX >= 64 ? 2 : 1; }
 // Rows per block and threads.  Long rows need the shared memory for fewer of
 // them; short ones are marched side by side, with few rows per lane.
 template <typename T, int NX> constexpr int force_rows3() { return NX >= 128 ? 8 : 16; }
-template <int NX> constexpr int force_threads3() { return NX >= 256 ? 256 : NX >= 64 ? 128 : 64; }
+template <int NX, int VL> constexpr int force_threads3() { return (NX >= 256 ? 256 : NX >= 64 ? 128 : 64) / (NX >= 64 ? VL : 1); }
 // Tile variants: 0 default rows, 1 half, 2 double (n_x >= 128: 16 rows, FP32),
 // 3 and 4 the rows of 0 and 1 with twice the threads; 6 as 0 (an L2 prefetch of
 // the rows two steps ahead, 2 KB of each of the 108 fields, made the pass
 // slower: 256 x 256 x 64 657 -> 770 us).
 template <typename T, int NX>
 cudaError_t launch_force_3d_n(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int TY = force_rows3<T, NX>(), NT = force_threads3<NX>();
-  if (a.force == 2) return launch_force_3d_t<T, NX, TY, NT, S_NODAL>(a, s);
+  constexpr int TY = force_rows3<T, NX>();
+  constexpr int VS = force_cols3<T, NX>();
+  constexpr int NT = force_threads3<NX, VS>();
+  if (a.force == 2) return launch_force_3d_t<T, NX, TY, NT, VS, S_NODAL>(a, s);
   if constexpr (NX >= 64) {
-    if (a.var_a == 1) return launch_force_3d_t<T, NX, TY / 2, NT, S_STRAIN>(a, s);
+    if (a.var_a == 1) return launch_force_3d_t<T, NX, TY / 2, NT, VS, S_STRAIN>(a, s);
     if constexpr (NX >= 128 && sizeof(T) == 4) {
-      if (a.var_a == 2) return launch_force_3d_t<T, NX, 2 * TY, NT, S_STRAIN>(a, s);
+      if (a.var_a == 2) return launch_force_3d_t<T, NX, 2 * TY, NT, VS, S_STRAIN>(a, s);
     }
     if constexpr (NX < 256 || sizeof(T) == 4) {   // else the shared memory does not hold the ring
-      if (a.var_a == 3) return launch_force_3d_t<T, NX, TY, 2 * NT, S_STRAIN>(a, s);
-      if (a.var_a == 4) return launch_force_3d_t<T, NX, TY / 2, 2 * NT, S_STRAIN>(a, s);
+      if (a.var_a == 3) return launch_force_3d_t<T, NX, TY, 2 * NT, VS, S_STRAIN>(a, s);
+      if (a.var_a == 4) return launch_force_3d_t<T, NX, TY / 2, 2 * NT, VS, S_STRAIN>(a, s);
     }
   }
-  return launch_force_3d_t<T, NX, TY, NT, S_STRAIN>(a, s);
+  return launch_force_3d_t<T, NX, TY, NT, VS, S_STRAIN>(a, s);
 }
 template <typename T> cudaError_t launch_force_3d(const PassArgs<T>& a, cudaStream_t s) {
   RVE_DISPATCH_N3(a.n[0], launch_force_3d_n, a, s)
