@@ -228,6 +228,31 @@ def model_bytes(dim, n, s, L_iters, form="stress"):
     return out
 
 
+def pass_bytes(dim, n, s, form="stress"):
+    """Bytes the passes of one CG iteration cannot do without, per load case
+    (model_bytes counts all m components through every transform; the passes
+    transform the D nodal ones).  s: bytes per real scalar of the inner
+    precision.  The first pass (kind force_stencil in the factored and nodal
+    forms) reads r, p_old, x, E and writes p, x (nodal: rho, pi_old, xi, E; pi, xi)
+    and the force spectra, two partial sums per component in 3D; pass B adds
+    them; pass C reads and writes D components; pass E reads D components and
+    reads and writes r (nodal: writes rho).  The nodal form also reads and writes
+    the spectra of the residual force in pass B (2D: C)."""
+    D, m, N = dim, (6 if dim == 2 else 36), int(np.prod(n))
+    spec = (n[0] // 2 + 1) * (N // n[0]) * 2 * s      # one component
+    parts = D if dim == 2 else 2 * D
+    nodal = form == "nodal"
+    first = "pass_a" if form == "stress" else "force_stencil"
+    res = 2 * D * spec if nodal else 0
+    out = {first: ((6 * D if nodal else 5 * m) + 1) * N * s + parts * spec,
+           "pass_c": 2 * D * spec + (res if dim == 2 else 0),
+           "pass_e": D * spec + (D if nodal else 2 * m) * N * s}
+    if dim == 3:
+        out["pass_b"] = (parts + D) * spec + res
+        out["pass_d"] = 2 * D * spec
+    return out
+
+
 def iteration_bytes(dim, n, s, form, mb):
     """Bytes of one CG iteration of one load case and the model's description: the
     scope table's model for the stress form, the sum of the form's per-kernel model
@@ -512,10 +537,10 @@ def run_batch(args, world, rank, local, dist):
         torch.cuda.synchronize()
         dt = (time.perf_counter() - t0) / args.steps
     dt = max_over_ranks(dt, dist if world > 1 else None, "cuda")
-    # model bytes of every slot's CG iterations in this step (7 vector + 4 spectrum streams, FP32)
+    # bytes of every slot's CG iterations in this step (FP32)
     total_bytes = 0.0
     for (n, _), rv in zip(rves, info):
-        mb = model_bytes(2, n, 4, None)
+        mb = pass_bytes(2, n, 4)
         total_bytes += sum(v["iterations"] for v in rv) * (mb["pass_a"] + mb["pass_c"] + mb["pass_e"])
     peak, peak_kind = peaks()
     achieved = total_bytes / dt / 1e9
@@ -610,7 +635,7 @@ def run_extension(args):
     }
     if "Fm" not in x and "W" not in x and "derivative" not in x and args.form == "stress":
         # small-strain FE stress form: the byte model of the headline workloads applies
-        mb = model_bytes(dim, n, s, 1)
+        mb = pass_bytes(dim, n, s)
         fr = hbm_fractions(mb, kt, lc_iters, 1, peak)
         out["kernels_hbm_frac"] = fr
         if fr:
@@ -623,7 +648,7 @@ def run_extension(args):
 def other_workload(name, form, stream, reps=3):
     """Timed solves of another headline workload (same form, precision and
     tolerance as its WORKLOADS entry), with its error against the stored oracle
-    result and its per-iteration HBM fraction on the scope table's model."""
+    result and its per-iteration HBM fraction (pass_bytes)."""
     import torch
     import microstructures as ms
     from paper_2105_03297_gb300 import RVE
@@ -655,9 +680,9 @@ def other_workload(name, form, stream, reps=3):
     cg_iters = float(np.mean([max(v) for v in its]))
     lc_iters = float(np.sum(its)) / reps
     s = 4 if prec == "mixed" else 8
-    mb = model_bytes(dim, n, s, lc_iters, form)
+    mb = pass_bytes(dim, n, s, form)
     cg_ms = sum(v[0] for k, v in kt.items() if k in mb) / (cg_iters * reps)
-    it_bytes = iteration_bytes(dim, n, s, form, mb)[0] * lc_iters / cg_iters
+    it_bytes = sum(mb.values()) * lc_iters / cg_iters
     peak, _ = peaks()
     err = oracle_error(cfg_name, C=C if L == ns else None, S=C if L != ns else None)
     return {"grid": list(n), "load_cases": L, "precision": prec, "rel_tol": tol, "status": code,
@@ -736,7 +761,7 @@ def run_gpu(args):
     lc_iters = float(np.sum(iters)) / args.steps          # load-case iterations per solve
     cg_iters = float(np.mean([max(v) for v in iters]))   # batched iterations per solve
     s = 4 if prec == "mixed" else 8
-    mb = model_bytes(dim, n, s, lc_iters, args.form)
+    mb = pass_bytes(dim, n, s, args.form)
     # dominant kernel: the CG-iteration pass with the most device time
     cand = {k: v for k, v in kt.items() if k in mb and v[1] > 0}
     dom = max(cand, key=lambda k: cand[k][0])
@@ -745,10 +770,9 @@ def run_gpu(args):
     achieved = bytes_total / (dom_ms * 1e-3) / 1e9
     peak, peak_kind = peaks()
     cg_ms = sum(v[0] for k, v in kt.items() if k in mb) / (cg_iters * args.steps)
-    # whole CG iteration: the scope table's model for the stress form (V = 8 vector,
-    # S spectrum streams), the form's own per-kernel model for the others
-    it_bytes, it_model = iteration_bytes(dim, n, s, args.form, mb)
-    it_bytes *= lc_iters / cg_iters
+    # whole CG iteration: what its passes cannot do without
+    it_bytes = sum(mb.values()) * lc_iters / cg_iters
+    it_model = "sum of pass_bytes over the passes of one CG iteration, all load cases; CUDA-event times"
     it_achieved = it_bytes / (cg_ms * 1e-3) / 1e9
 
     # end to end through the C ABI with host buffers: E host->device, C_eff device->host
