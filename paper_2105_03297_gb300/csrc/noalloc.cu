@@ -43,6 +43,7 @@ static __device__ __align__(256) unsigned char g_rve_scratch[kStaticScratchBytes
 // Device address of g_rve_scratch, per device (nullptr = not set up yet).
 std::atomic<void*> g_scratch_ptr[kMaxDevices];
 DeviceOnce g_scratch_once;
+std::atomic<bool> g_tables_written[kMaxDevices];
 
 // Phase tables exp(+2 pi i j / n) and twiddle tables exp(-2 pi i j / n) of
 // every length, and the CG-state record (active, everything else zero; no mode
@@ -83,19 +84,12 @@ extern "C" int rve_apply_operator_2d_static(const int64_t* n, const double* leng
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return RVE_ERR_CUDA; }
   cudaStream_t s = (cudaStream_t)cuda_stream;
   // Set-up, once per device, with that device current: the device address of
-  // the static array (its name is only a host-side stand-in), and the tables
-  // and the state record in it, written on the first call's stream (callers
-  // serialise calls, so every later call finds them complete).  The kernel
+  // the static array (its name is only a host-side stand-in).  The kernel
   // attributes of the pass kernels are likewise set once per device by their
   // launchers.
   g_scratch_once.run(dev, [&] {
     void* ptr = nullptr;
     if (cudaGetSymbolAddress(&ptr, g_rve_scratch) != cudaSuccess || !ptr) { cudaGetLastError(); ptr = nullptr; }
-    if (ptr) {
-      unsigned char* b = static_cast<unsigned char*>(ptr) + kSpecBytes;
-      fill_static_tables<<<4, 128, 0, s>>>(reinterpret_cast<float2*>(b), reinterpret_cast<CgState*>(b + kTableBytes));
-      if (cudaGetLastError() != cudaSuccess) ptr = nullptr;
-    }
     g_scratch_ptr[dev].store(ptr);
   });
   unsigned char* base = static_cast<unsigned char*>(g_scratch_ptr[dev].load());
@@ -103,6 +97,17 @@ extern "C" int rve_apply_operator_2d_static(const int64_t* n, const double* leng
   float2* spec = reinterpret_cast<float2*>(base);
   float2* tables = reinterpret_cast<float2*>(base + kSpecBytes);   // phases, then twiddles
   CgState* cg = reinterpret_cast<CgState*>(base + kSpecBytes + kTableBytes);
+  // The tables and the state record, on the first call's stream (callers
+  // serialise calls, so every later call finds them complete).  A call that is
+  // being captured runs later, if at all: it carries the kernel in its own graph
+  // and leaves it to the next call too.
+  if (!g_tables_written[dev].load()) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool known = cudaStreamIsCapturing(s, &cap) == cudaSuccess;
+    fill_static_tables<<<4, 128, 0, s>>>(tables, cg);
+    if (cudaGetLastError() != cudaSuccess) return RVE_ERR_CUDA;
+    if (known && cap == cudaStreamCaptureStatusNone) g_tables_written[dev].store(true);
+  }
 
   const int nx = (int)n[0], ny = (int)n[1];
   PassArgs<float> a;
