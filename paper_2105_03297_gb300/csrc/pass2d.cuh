@@ -1,11 +1,11 @@
 // 2D projected-operator passes (two linear triangles per pixel, Sec. 2.6).
 //
 // One application of q = G * (C : p) is three launches:
-//   A  material (+ fused CG direction update and <p, C p>) and forward real
-//      FFT along x; writes the half spectrum transposed, [l][c][k_x][y], so
-//      that the next pass reads whole y-columns contiguously;
-//   C  t = B^H sigma (differences along y where the factors of B^H are
-//      shifts), forward FFT along y, w^ = (B^H B)^-1 t^ per wavevector (k = 0
+//   A  force pass (pass_force.cuh): material, CG direction update, <p, C p>,
+//      nodal forces t = B^H sigma in real space, forward real FFT along x;
+//      writes the half spectrum transposed, [l][j][k_x][y], so that the next
+//      pass reads whole y-columns contiguously;
+//   C  forward FFT along y, w^ = (B^H B)^-1 t^ per wavevector (k = 0
 //      set to zero), inverse FFT along y;
 //   E  inverse real FFT along x of w, q = B w in real space, then r -= alpha q
 //      and <r, r> (q never touches memory).  x += alpha p of iteration k is
@@ -13,7 +13,7 @@
 //      stream less per iteration); cg_finish_x applies the last one.
 // The other derivatives and finite strain carry all their components through C
 // (with the projection) and E.  Measured at 1024^2, three load cases, FP32, us
-// per iteration: all six components through C 80 and E 85, now C 48 and E 61.
+// per iteration: all six components through A 113, C 80 and E 85, now A 108, C 35 and E 61.
 // DFT convention of Appendix A; the 1/N of the inverse is applied in pass C.
 // Two real rows (y, y+1) share one complex FFT (X_y + i X_{y+1}).
 #pragma once
@@ -218,11 +218,8 @@ template <typename T, int NT> __host__ __device__ constexpr int pass_a2_min_bloc
 
 // NT is either the FFT's thread count or (tile variants 3, 4) the number of
 // load units of the tile, so that every thread streams exactly one unit.
-// PAIR (n_x = 512 or 1024, tile variant 5): the x transform spreads each
-// 32-point register FFT of its first step over a lane pair (smem_fft_pair),
-// NT = 2 N1 per transform, three blocks per SM.
-template <typename T, int NX, int TY, int NT, bool PAIR = false>
-__global__ void __launch_bounds__(NT, PAIR ? 3 : pass_a2_min_blocks<T, NT>()) pass_a_2d(PassArgs<T> a) {
+template <typename T, int NX, int TY, int NT>
+__global__ void __launch_bounds__(NT, pass_a2_min_blocks<T, NT>()) pass_a_2d(PassArgs<T> a) {
   using C = cplx<T>;
   constexpr int NP = TY / 2;
   constexpr int GS = 3;
@@ -245,13 +242,10 @@ __global__ void __launch_bounds__(NT, PAIR ? 3 : pass_a2_min_blocks<T, NT>()) pa
   T beta = 0, alpha_prev = 0;
   bool use_old = false;
   if (a.amode == A_CG) { beta = cg_beta<T>(cg); alpha_prev = cg_alpha<T>(cg); use_old = cg->it > 0; }
-  // the lane-pair variant runs three blocks per SM: units of two columns (8-byte
-  // loads, as in 3D) keep the load phase within its registers
-  const T acc = pass_a_load<T, NX, TY, GS, NT, LD, PAIR ? 2 : Vec16<T>::n>(a, buf, l, c0, (int64_t)y0 * NX, nodal,
-                                                                          beta, alpha_prev, use_old);
+  const T acc = pass_a_load<T, NX, TY, GS, NT, LD, Vec16<T>::n>(a, buf, l, c0, (int64_t)y0 * NX, nodal, beta,
+                                                                alpha_prev, use_old);
   __syncthreads();
-  if constexpr (PAIR) smem_fft_pair<T, NX, GS * NP, LD, NT, -1>(buf, a.tw[0]);
-  else smem_fft<T, NX, GS * NP, LD, NT, -1>(buf, a.tw[0]);
+  smem_fft<T, NX, GS * NP, LD, NT, -1>(buf, a.tw[0]);
   pass_a_store<T, NX, TY, NT, LD>(buf, nodal ? 2 : 3, a.spec + (((int64_t)l * a.m + c0) * KX) * ny + y0,
                                   (int64_t)KX * ny, ny);
 
@@ -782,7 +776,7 @@ __global__ void __launch_bounds__(NT) cg_finish_x(PassArgs<T> a) {
   const int64_t idx = (int64_t)l * a.m * a.N + i * VL;
   T xv[VL], pv[VL];
   vload(xv, a.x + idx);
-  // the factored form alternates the direction between p (even iterations) and p2 (odd)
+  // the force pass alternates the direction between p (even iterations) and p2 (odd)
   const T* pl = (a.p2 != nullptr && ((cg->it - 1) & 1)) ? a.p2 : a.p;
   vload(pv, pl + idx);
 #pragma unroll
@@ -809,14 +803,14 @@ template <typename T> constexpr int tile_rows(int v) {
   return v == 1 ? Tile2D<T>::TY / 2 : v == 2 ? Tile2D<T>::TY * 2 : Tile2D<T>::TY;
 }
 
-template <typename T, int NX, int TY, bool BY_UNITS = false, bool PAIR = false>
+template <typename T, int NX, int TY, bool BY_UNITS = false>
 cudaError_t launch_a_2d_t(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int NF = PAIR ? 2 * FftSplit<NX>::N1 * 3 * (TY / 2) : fft_threads<NX, 3 * (TY / 2)>();
+  constexpr int NF = fft_threads<NX, 3 * (TY / 2)>();
   constexpr int NU = ((TY / 2) * (NX / Vec16<T>::n) + 31) / 32 * 32;   // load units of a tile
   constexpr int NT = (BY_UNITS && NU > NF && NU <= 1024) ? NU : NF;
   static_assert(NT <= 1024, "threads per block");
   const size_t sm = sizeof(cplx<T>) * 3 * (TY / 2) * ae_ld<NX>();
-  auto k = pass_a_2d<T, NX, TY, NT, PAIR>;
+  auto k = pass_a_2d<T, NX, TY, NT>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   dim3 grid(a.n[1] / TY, a.amode == A_NODAL ? 1 : a.nq, a.L);
@@ -832,16 +826,14 @@ cudaError_t launch_e_2d_t(const PassArgs<T>& a, cudaStream_t s) {
   dim3 grid(a.n[1] / TY, (a.emode == E_NODAL || a.emode == E_NOUT) ? 1 : a.nq, a.L);
   return launch_pass(a.pdl, k, grid, NT, sm, s, a);
 }
-// Tile variants of the 2D pass A: 0 default rows per block, 1 half, 2 double
-// (threads = the FFT's); 3 default rows and 4 half rows with one thread per
-// load unit; 5 (FP32, n_x = 512 or 1024) the lane-pair x transform with 384
-// threads (default rows at 512, half rows at 1024).
+// Tile variants of the 2D pass A on all components (FP64: the derivatives
+// without a finite-element stencil, and finite strain): 0 default rows per
+// block, 1 half, 2 double (threads = the FFT's); 3 default rows and 4 half rows
+// with one thread per load unit.  FP32 transforms only nodal residuals here,
+// once per refinement step.
 template <typename T, int NX>
 cudaError_t launch_a_2d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if constexpr ((NX == 512 || NX == 1024) && sizeof(T) == 4) {
-    if (a.var_a == 5) return launch_a_2d_t<T, NX, NX == 1024 ? tile_rows<T>(1) : tile_rows<T>(0), false, true>(a, s);
-  }
-  if constexpr (NX >= 64) {
+  if constexpr (NX >= 64 && sizeof(T) == 8) {
     if (a.var_a == 1) return launch_a_2d_t<T, NX, tile_rows<T>(1)>(a, s);
     if (a.var_a == 2 && a.n[1] >= tile_rows<T>(2)) return launch_a_2d_t<T, NX, tile_rows<T>(2)>(a, s);
     if (a.var_a == 3) return launch_a_2d_t<T, NX, tile_rows<T>(0), true>(a, s);
@@ -911,28 +903,31 @@ cudaError_t launch_c_2d_n(const PassArgs<T>& a, cudaStream_t s) {
     }
     return a.grads ? launch_c_2d_v<T, NY, 0, 4>(a, s) : launch_c_2d_v<T, NY, 0, 2>(a, s);
   }
-  if (a.nq == 3) {
-    constexpr int NT3 = fft_threads<NY, 9>();
-    const size_t sm3 = sizeof(cplx<T>) * 9 * FftSplit<NY>::LD;
-    auto k3 = pass_c_2d<T, NY, 3, NT3>;
-    static DeviceOnce attr3;
-    attr3.run(current_device(), [&] { set_smem_attrs(k3, sm3); });
-    return launch_pass(a.pdl, k3, dim3(a.kx, a.L), NT3, sm3, s, a);
+  if constexpr (sizeof(T) == 4) return cudaErrorInvalidValue;   // all components: FP64 only
+  else {
+    if (a.nq == 3) {
+      constexpr int NT3 = fft_threads<NY, 9>();
+      const size_t sm3 = sizeof(cplx<T>) * 9 * FftSplit<NY>::LD;
+      auto k3 = pass_c_2d<T, NY, 3, NT3>;
+      static DeviceOnce attr3;
+      attr3.run(current_device(), [&] { set_smem_attrs(k3, sm3); });
+      return launch_pass(a.pdl, k3, dim3(a.kx, a.L), NT3, sm3, s, a);
+    }
+    if (a.nq == 1) {
+      constexpr int NT1 = fft_threads<NY, 3>();
+      const size_t sm1 = sizeof(cplx<T>) * 3 * FftSplit<NY>::LD;
+      auto k1 = pass_c_2d<T, NY, 1, NT1>;
+      static DeviceOnce attr1;
+      attr1.run(current_device(), [&] { set_smem_attrs(k1, sm1); });
+      return launch_pass(a.pdl, k1, dim3(a.kx, a.L), NT1, sm1, s, a);
+    }
+    constexpr int NT2 = fft_threads<NY, 6>();
+    const size_t sm2 = sizeof(cplx<T>) * 6 * FftSplit<NY>::LD;
+    auto k2 = pass_c_2d<T, NY, 2, NT2>;
+    static DeviceOnce attr2;
+    attr2.run(current_device(), [&] { set_smem_attrs(k2, sm2); });
+    return launch_pass(a.pdl, k2, dim3(a.kx, a.L), NT2, sm2, s, a);
   }
-  if (a.nq == 1) {
-    constexpr int NT1 = fft_threads<NY, 3>();
-    const size_t sm1 = sizeof(cplx<T>) * 3 * FftSplit<NY>::LD;
-    auto k1 = pass_c_2d<T, NY, 1, NT1>;
-    static DeviceOnce attr1;
-    attr1.run(current_device(), [&] { set_smem_attrs(k1, sm1); });
-    return launch_pass(a.pdl, k1, dim3(a.kx, a.L), NT1, sm1, s, a);
-  }
-  constexpr int NT2 = fft_threads<NY, 6>();
-  const size_t sm2 = sizeof(cplx<T>) * 6 * FftSplit<NY>::LD;
-  auto k2 = pass_c_2d<T, NY, 2, NT2>;
-  static DeviceOnce attr2;
-  attr2.run(current_device(), [&] { set_smem_attrs(k2, sm2); });
-  return launch_pass(a.pdl, k2, dim3(a.kx, a.L), NT2, sm2, s, a);
 }
 
 #define RVE_DISPATCH_N(nval, FN, ...)                      \

@@ -1,21 +1,24 @@
 // 3D projected-operator passes (six Kuhn tetrahedra per voxel).
 //
 // Real fields are [l][c][z][y][x].  One application of q = G * (C : p):
-//   A  material (+ CG direction update, <p, C p>) and forward real FFT along x;
-//      writes spec1 as [l][c][k_x][z][y] (y contiguous);
-//   B  t = B^H sigma (differences along y and z where the factors of B^H are
-//      shifts) and its forward FFT along y; writes spec2 as [l][j][k_x][k_y][z]
-//      (z contiguous, chunks of TZB z per k_y, the D = 3 nodal components j);
+//   A  force pass (pass_force.cuh): material, CG direction update, <p, C p>,
+//      nodal forces t = B^H sigma in real space, forward real FFT along x;
+//      writes spec1 as [l][j][k_x][z][y] (y contiguous), two partial sums of
+//      t (planes z and z + 1) for each of the D = 3 nodal components j;
+//   B  their sum and its forward FFT along y; writes spec2 as [l][j][k_x][k_y][z]
+//      (z contiguous, chunks of TZB z per k_y);
 //   C  forward FFT along z, w^ = (B^H B)^-1 t^ per wavevector, inverse FFT
 //      along z, in place on spec2;
 //   D  inverse FFT along y, spec2 -> spec1;
 //   E  inverse real FFT along x of w, q = B w in real space, r -= alpha q,
 //      <r, r> (x += alpha p is deferred to the next pass A, as in 2D).
+// Tile variant 5 (pass3d_pipe.cuh) transforms all 36 stress components along x
+// instead, and B forms t from them (differences along y and z).
 // The other derivatives (one evaluation point) and finite strain carry all
 // their components through B, C (with the projection), D and E.
 // Measured at 256 x 256 x 64, one load case, FP32, us per iteration: all 36
-// components through every pass A 656, B 168, C 371, D 184, E 388; now A 656,
-// B 168, C 50, D 27, E 310.
+// components through every pass A 656, B 168, C 371, D 184, E 388; now A 622,
+// B 38, C 50, D 28, E 289.
 #pragma once
 #include "pass2d.cuh"
 #include "pass3d_pipe.cuh"
@@ -39,9 +42,8 @@ __host__ __device__ constexpr int kuhn_perm(int t, int i) {
 // a.pf_ahead = D > 0 every block asks the TMA unit to bring the input of
 // block b + D (b its own linear index) into L2 (bulk prefetches: no data
 // reaches the SM and nothing waits on them), so that DRAM keeps streaming a
-// later tile while this block transforms its own (passes A and E: tile
-// variants 6 and 4; passes B, C and D: always in FP32; the distances are in
-// prefetch_distance).
+// later tile while this block transforms its own (passes B and D, always in
+// FP32; the distance is in prefetch_distance).
 //
 // Block coordinates (x, y, z) of the block a.pf_ahead places after this one in
 // launch order; false past the end of the grid.
@@ -61,39 +63,6 @@ template <typename T> __device__ __forceinline__ bool slot_runs(const PassArgs<T
   const CgState* cg = a.cg + l;
   return cg->active && !(a.cgphase && cg->status != ST_RUN);
 }
-// Passes A and E (grid (n_y/TY, n_z, L*G)): tile (l, grp, z, y0) of the later
-// block; false past the end of the grid or for a load case whose CG has stopped.
-template <typename T>
-__device__ __forceinline__ bool block_ahead(const PassArgs<T>& a, int G, int TY, int& l, int& grp, int& z, int& y0) {
-  int bx, bz;
-  if (!grid_ahead(a, bx, z, bz)) return false;
-  y0 = bx * TY;
-  l = bz / G;
-  grp = bz % G;
-  return slot_runs(a, l);
-}
-
-// Pass A (CG mode, stress form): the r, E and (after the first iteration)
-// p_old and x rows of the later block: TY contiguous rows of NX values per
-// component, 19 requests of TY * NX * sizeof(T) bytes, one per thread.
-template <typename T, int NX, int TY>
-__device__ __forceinline__ void pass_a_prefetch_ahead(const PassArgs<T>& a, int G) {
-  static_assert((TY * NX * sizeof(T)) % 16 == 0, "bulk prefetch sizes are multiples of 16 bytes");
-  const int t = threadIdx.x;
-  if (t >= 19) return;
-  int l, grp, z, y0;
-  if (!block_ahead(a, G, TY, l, grp, z, y0)) return;
-  if (t >= 7 && a.cg[l].it == 0) return;   // no p_old or x reads in the first iteration
-  const int64_t N = a.N;
-  const int64_t row0 = ((int64_t)z * a.n[1] + y0) * NX;
-  const int64_t comp = ((int64_t)l * a.m + grp * 6) * N + row0;
-  const T* src = t < 6 ? a.r + comp + t * N
-               : t == 6 ? a.E + (int64_t)(l / a.lcs) * N + row0
-               : t < 13 ? a.p + comp + (t - 7) * N
-                        : a.x + comp + (t - 13) * N;
-  prefetch_l2_bulk(src, (unsigned)(TY * NX * sizeof(T)));
-}
-
 // ---------------------------------------------------------------- pass A
 // Resident blocks per SM the register budget is sized for.
 template <typename T, int NT> __host__ __device__ constexpr int pass_a_min_blocks() {
@@ -128,7 +97,6 @@ __global__ void __launch_bounds__(NT, pass_a_min_blocks<T, NT>()) pass_a_3d(Pass
   T beta = 0, alpha_prev = 0;
   bool use_old = false;
   if (a.amode == A_CG) { beta = cg_beta<T>(cg); alpha_prev = cg_alpha<T>(cg); use_old = cg->it > 0; }
-  if (a.pf_ahead > 0 && a.amode == A_CG && !nodal) pass_a_prefetch_ahead<T, NX, TY>(a, G);
   // two columns per unit: 6 components x 2 rows x (r, p, x) stay in registers
   const T acc = pass_a_load<T, NX, TY, GS, NT, LD, 2>(a, buf, l, c0, ((int64_t)z * ny + y0) * NX, nodal, beta,
                                                       alpha_prev, use_old);
@@ -764,46 +732,28 @@ template <int A, int B> constexpr int max_i() { return A > B ? A : B; }
 
 // Prefetch distance (blocks ahead, see grid_ahead): the blocks resident at once
 // (occ per SM x SMs) divided by div.  What pays is about 4 to 10 MB of
-// prefetched rows in flight, so the divisor depends on a block's input.
-// Measured at 256^3 (FP32, ms per CG iteration):
-//   pass A (152 KB per block, three blocks per SM), div 16 (28 blocks): 2.88
-//     without, 2.53 at div 16, 2.56 at div 32 to 152, 2.62 at div 8 and 3.26
-//     at div 2 (35 MB in flight crowd L2);
+// prefetched rows in flight.  Measured at 256^3 with all 36 components (FP32,
+// ms per CG iteration):
 //   pass B (32 KB per block): 0.86 without, 0.81 / 0.77 / 0.72 / 0.69 / 0.72
 //     at div 16 / 8 / 4 / 2 / 1;
-//   pass C (72 KB per block): 1.52 without, 1.55 / 1.53 / 1.47 / 1.41 / 1.43;
 //   pass D (32 KB per block, scattered z-chunks): 0.85 without, 0.83 / 0.82 /
-//     0.82 / 0.82 / 0.84;
-//   pass E (tile variant 4, 97 KB per block): 1.82 without, 1.80 at div 16, 8
-//     and 4, 1.87 at div 2 (the pipelined variant 3, 1.74, stays faster).
+//     0.82 / 0.82 / 0.84.
 inline int prefetch_distance(int occ, int div) {
   const int d = occ * device_sm_count() / div;
   return d > 1 ? d : 1;
 }
 
 template <typename T, int NX, int TY, bool BY_UNITS = false, int GS = 6>
-cudaError_t launch_a_3d_t(const PassArgs<T>& a, cudaStream_t s, bool ahead = false) {
+cudaError_t launch_a_3d_t(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int NF = fft_threads<NX, GS * (TY / 2)>();
   constexpr int NU = (pass_a_units3<T, NX, TY>() + 31) / 32 * 32;
   constexpr int NT = BY_UNITS ? (max_i<NF, NU>() > 1024 ? NF : max_i<NF, NU>()) : NF;
   const size_t sm = sizeof(cplx<T>) * GS * (TY / 2) * ae_ld<NX>();
   auto k = pass_a_3d<T, NX, TY, NT, GS>;
   static DeviceOnce attr;
-  static int occ[kMaxDevices] = {0};
-  const int dev = current_device();
-  attr.run(dev, [&] {
-    set_smem_attrs(k, sm);
-    if (dev >= 0 && dev < kMaxDevices) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[dev], k, NT, sm);
-  });
+  attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   dim3 grid(a.n[1] / TY, a.n[2], a.L * (GS == 3 ? 1 : a.nq));
-  if (ahead) {
-    PassArgs<T> b = a;
-    b.pf_ahead = prefetch_distance((dev >= 0 && dev < kMaxDevices) ? occ[dev] : 0, 16);
-    return launch_pass(b.pdl, k, grid, NT, sm, s, b);
-  } else {
-    return launch_pass(a.pdl, k, grid, NT, sm, s, a);
-  }
-  return cudaGetLastError();
+  return launch_pass(a.pdl, k, grid, NT, sm, s, a);
 }
 template <typename T, int NX, int TY, int GE = 6>
 cudaError_t launch_e_3d_t(const PassArgs<T>& a, cudaStream_t s) {
@@ -826,11 +776,12 @@ cudaError_t launch_e_3d_fe_t(const PassArgs<T>& a, cudaStream_t s) {
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.n[2], a.L), NT, sm, s, a);
 }
-// Tile variants of pass A: 0 default rows per block, 1 half, 2 double (threads
-// = the FFT's); 3 default rows and 4 half rows with one thread per load unit;
-// 5 (FP32, n_x >= 128, CG iterations) the pipelined persistent pass with
-// bulk-copied rows (pass3d_pipe.cuh); other modes of variant 5 use variant 0;
-// 6 variant 0 with the L2 prefetch of a later block's rows.
+// Tile variants of pass A on all components: 0 default rows per block, 1 half,
+// 2 double (threads = the FFT's); 3 default rows and 4 half rows with one
+// thread per load unit (FP64: the derivatives without a finite-element stencil,
+// and finite strain); 5 (FP32, n_x >= 128, CG iterations) the pipelined
+// persistent pass with bulk-copied rows (pass3d_pipe.cuh), which uses variant 0
+// for more load cases than it keeps sums for.
 template <typename T, int NX>
 cudaError_t launch_a_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   // the three nodal components: twice the rows, so that a block holds as many
@@ -840,12 +791,11 @@ cudaError_t launch_a_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   if constexpr (sizeof(T) == 4 && NX >= 128) {
     if (a.var_a == 5 && a.amode == A_CG && a.L <= kPipeMaxL && a.n[1] >= 4) return launch_a_3d_pipe<NX>(a, s);
   }
-  if constexpr (NX >= 64) {
+  if constexpr (NX >= 64 && sizeof(T) == 8) {
     if (a.var_a == 1) return launch_a_3d_t<T, NX, tile_rows3<T>(1)>(a, s);
     if (a.var_a == 2 && a.n[1] >= tile_rows3<T>(2)) return launch_a_3d_t<T, NX, tile_rows3<T>(2)>(a, s);
     if (a.var_a == 3) return launch_a_3d_t<T, NX, tile_rows3<T>(0), true>(a, s);
     if (a.var_a == 4) return launch_a_3d_t<T, NX, tile_rows3<T>(1), true>(a, s);
-    if (a.var_a == 6) return launch_a_3d_t<T, NX, tile_rows3<T>(0)>(a, s, true);
   }
   return launch_a_3d_t<T, NX, tile_rows3<T>(0)>(a, s);
 }
@@ -863,11 +813,14 @@ cudaError_t launch_e_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   }
   // the three nodal components: twice the rows, as in pass A
   if (a.emode == E_NODAL || a.emode == E_NOUT) return launch_e_3d_t<T, NX, tile_rows3<T>(2), 3>(a, s);
-  if constexpr (NX >= 64) {
-    if (a.var_e == 1) return launch_e_3d_t<T, NX, tile_rows3<T>(1)>(a, s);
-    if (a.var_e == 2 && a.n[1] >= tile_rows3<T>(2)) return launch_e_3d_t<T, NX, tile_rows3<T>(2)>(a, s);
+  if constexpr (sizeof(T) == 4) return cudaErrorInvalidValue;   // all components: FP64 only
+  else {
+    if constexpr (NX >= 64) {
+      if (a.var_e == 1) return launch_e_3d_t<T, NX, tile_rows3<T>(1)>(a, s);
+      if (a.var_e == 2 && a.n[1] >= tile_rows3<T>(2)) return launch_e_3d_t<T, NX, tile_rows3<T>(2)>(a, s);
+    }
+    return launch_e_3d_t<T, NX, tile_rows3<T>(0)>(a, s);
   }
-  return launch_e_3d_t<T, NX, tile_rows3<T>(0)>(a, s);
 }
 template <typename T, int NY, bool FWD, int V>
 cudaError_t launch_y_3d_v(const PassArgs<T>& a, cudaStream_t s) {
@@ -907,11 +860,13 @@ cudaError_t launch_b_3d_fe(const PassArgs<T>& a, cudaStream_t s) {
 // Split variant of the y transforms (passes B and D): a.var_y.
 template <typename T, int NY, bool FWD>
 cudaError_t launch_y_3d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if (FWD && fe_path(a) && !a.pair && a.pmode != P_NODAL_IN && a.pmode != P_SOLVE) {
-    if constexpr (fft_split_count<NY>() > 1) {
-      if (a.var_y == 1) return launch_b_3d_fe<T, NY, 1>(a, s);
+  if constexpr (FWD && sizeof(T) == 4) {   // after the pipelined first pass (tile variant 5, FP32)
+    if (fe_path(a) && !a.pair && a.pmode != P_NODAL_IN && a.pmode != P_SOLVE) {
+      if constexpr (fft_split_count<NY>() > 1) {
+        if (a.var_y == 1) return launch_b_3d_fe<T, NY, 1>(a, s);
+      }
+      return launch_b_3d_fe<T, NY, 0>(a, s);
     }
-    return launch_b_3d_fe<T, NY, 0>(a, s);
   }
   if constexpr (fft_split_count<NY>() > 1) {
     if (a.var_y == 1) return launch_y_3d_v<T, NY, FWD, 1>(a, s);
@@ -939,22 +894,24 @@ cudaError_t launch_c_3d_v(const PassArgs<T>& a, cudaStream_t s) {
 
 template <typename T, int NZ>
 cudaError_t launch_c_3d_n(const PassArgs<T>& a, cudaStream_t s) {
-  if (a.pmode == P_FINITE) {
-    constexpr int NTf = fft_threads<NZ, 54>();
-    const size_t smf = sizeof(cplx<T>) * 54 * FftSplit<NZ>::LD;
-    if (smf > 227 * 1024) return cudaErrorInvalidConfiguration;   // FP64 at n_z = 256
-    auto kf = pass_c_3d_fs<T, NZ, NTf>;
-    static DeviceOnce attrf;
-    attrf.run(current_device(), [&] { set_smem_attrs(kf, smf); });
-    return launch_pass(a.pdl, kf, dim3(a.kx, a.n[1], a.L), NTf, smf, s, a);
-  }
-  if (!fe_path(a)) {
-    constexpr int NT1 = fft_threads<NZ, 36>();
-    const size_t sm1 = sizeof(cplx<T>) * 36 * FftSplit<NZ>::LD;
-    auto k1 = pass_c_3d_q1<T, NZ, NT1>;
-    static DeviceOnce attr1;
-    attr1.run(current_device(), [&] { set_smem_attrs(k1, sm1); });
-    return launch_pass(a.pdl, k1, dim3(a.kx, (a.n[1] + 5) / 6, a.L), NT1, sm1, s, a);
+  if constexpr (sizeof(T) == 8) {   // all components: FP64 only
+    if (a.pmode == P_FINITE) {
+      constexpr int NTf = fft_threads<NZ, 54>();
+      const size_t smf = sizeof(cplx<T>) * 54 * FftSplit<NZ>::LD;
+      if (smf > 227 * 1024) return cudaErrorInvalidConfiguration;   // FP64 at n_z = 256
+      auto kf = pass_c_3d_fs<T, NZ, NTf>;
+      static DeviceOnce attrf;
+      attrf.run(current_device(), [&] { set_smem_attrs(kf, smf); });
+      return launch_pass(a.pdl, kf, dim3(a.kx, a.n[1], a.L), NTf, smf, s, a);
+    }
+    if (!fe_path(a)) {
+      constexpr int NT1 = fft_threads<NZ, 36>();
+      const size_t sm1 = sizeof(cplx<T>) * 36 * FftSplit<NZ>::LD;
+      auto k1 = pass_c_3d_q1<T, NZ, NT1>;
+      static DeviceOnce attr1;
+      attr1.run(current_device(), [&] { set_smem_attrs(k1, sm1); });
+      return launch_pass(a.pdl, k1, dim3(a.kx, (a.n[1] + 5) / 6, a.L), NT1, sm1, s, a);
+    }
   }
   if constexpr (fft_split_count<NZ>() > 1) {
     if (a.var_c == 1) return a.grads ? launch_c_3d_v<T, NZ, 1, 9>(a, s) : launch_c_3d_v<T, NZ, 1>(a, s);

@@ -68,8 +68,8 @@ template <typename T> struct PassArgs {
   int var_c, var_y;  // FFT split variants (FftSplit<N, V>) of pass C's axis and of passes B / D (3D)
   int comp_in;       // number of components in the spectrum for this pass (m or D)
   int stall_copies;     // test hook: the pipelined pass issues no copies, so its bounded waits run out
-  int pf_ahead;      // 3D passes A to D: blocks ahead in launch order whose input each block asks the TMA
-                     // unit to prefetch into L2, 0 = none; pass E: 1 = prefetch the tile's own r rows
+  int pf_ahead;      // 3D passes B and D: blocks ahead in launch order whose input each block asks the
+                     // TMA unit to prefetch into L2, 0 = none
   int deriv;         // Deriv
   int force;         // first pass of the finite elements: 1 strain fields, 2 nodal fields, 3 stress
                      // field of finite strain (2D) (pass_force.cuh)
