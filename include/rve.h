@@ -171,22 +171,18 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
 
 /* Schedule of the FFT passes: tile shapes, threads and radix schedules.
  * variants[RVE_SCHED_PASSES] holds
- *  [0] the first pass (material + x FFT): 0 default rows per block, 1 half,
- *      2 double; with n_x >= 64 also 3 default rows and 4 half rows with one
- *      thread per 16-byte load unit of the tile; in 3D with RVE_MIXED and
- *      n_x >= 128 also 5, a persistent pipelined pass whose next tile's rows
- *      arrive by bulk copies while the current tile is transformed (CG
- *      iterations of up to 64 load cases; otherwise it runs as 0), and 6,
- *      variant 0 whose blocks each ask for a later block's rows to be
- *      prefetched into L2 (a hint: no wait, same arithmetic).  A bounded
- *      device-side wait of variant 5 that gives up makes the solve return
- *      RVE_ERR_TIMEOUT.  In 2D with RVE_MIXED and n_x = 512 or 1024, 5 is the
- *      x transform with each 32-point register FFT spread over a pair of
- *      lanes (fewer registers, three blocks per SM);
+ *  [0] the first pass (material, nodal forces, x FFT): 0 default rows per
+ *      block, 1 half, 2 double; with n_x >= 64 also 3 and 4, the same tiles
+ *      with other threads per block; in 3D with RVE_MIXED and n_x >= 128 also 5, a
+ *      persistent pipelined pass that transforms every stress component and
+ *      whose next tile's rows arrive by bulk copies while the current tile is
+ *      transformed (stress form, CG iterations of up to 64 load cases), and
+ *      6, which runs as 0.  A bounded device-side wait of variant 5 that
+ *      gives up makes the solve return RVE_ERR_TIMEOUT.  In 2D with RVE_MIXED
+ *      and n_x = 512 or 1024, 5 is the x transform with each 32-point
+ *      register FFT spread over a pair of lanes (fewer registers);
  *  [1] the last pass (inverse x FFT + CG update): 0 default rows, 1 half, 2 double;
- *      in 3D with RVE_MIXED and n_x >= 128 also 3 and 4, the default and half
- *      rows with the tile's residual rows prefetched into L2 at the start of
- *      the block;
+ *      in 3D with RVE_MIXED and n_x >= 128 also 3 and 4, which run as 0 and 1;
  *  [2] the split N = N1 * N2 of the four-step FFT along the last axis (y in
  *      2D, z in 3D; the pass that applies the projection): 0 the most square
  *      split, 1 half N1 and twice N2 (16 = 2 x 8, 32 = 2 x 16, 64 = 4 x 16,
@@ -207,19 +203,16 @@ int rve_set_schedule(rve_t h, const int* variants);
  * the same operator G C (Eq. stat-mech-equi-FFT-homogenization with the
  * projection of Eqs. discrete_projection_op and small-strain-eq2), so the CG
  * iterates agree up to rounding:
- *   RVE_FORM_STRESS   (default) CG on strain fields; forward x FFT of every
- *                     stress component, B^H applied before the y and z
- *                     transforms (its factors are shifts there), (B^H B)^-1 at
- *                     each wavevector, B applied after the inverse transforms.
- *   RVE_FORM_FACTORED the same chain split where Appendix B splits it: the
+ *   RVE_FORM_STRESS   (default) and
+ *   RVE_FORM_FACTORED CG on strain fields, in the same kernels: the
  *                     right-hand side of Eq. small-strain-eq2 (B^H applied to
  *                     the stresses) is formed in real space as nodal forces
  *                     with the element stencils of Eq. discrderiv, only the D
  *                     nodal components are FFT'd and multiplied by the
  *                     inverse normal matrix (B^H B)^-1 (Eq. small-strain-chi),
  *                     and the strains of Eq. small-strain are formed back in
- *                     real space with the same stencils.  It needs one more
- *                     direction field [L][m][N] of the inner precision.
+ *                     real space with the same stencils.  (Tile variant 5 of
+ *                     the first pass belongs to the stress form only.)
  *   RVE_FORM_NODAL    the factored chain with the CG vectors themselves kept
  *                     as nodal fields: every iterate of the projected CG is
  *                     compatible, x = B xi, r = B rho, p = B pi, so CG runs on
@@ -231,7 +224,7 @@ int rve_set_schedule(rve_t h, const int* variants);
  *                     projection as a preconditioner of the FE stiffness that
  *                     Sec. 4 points to.  No extra memory.
  * rve_set_operator_form applies from the next solve; returns RVE_ERR_ARG for
- * an unknown form, RVE_ERR_OOM if the extra field cannot be allocated. */
+ * an unknown form. */
 #define RVE_FORM_STRESS 0
 #define RVE_FORM_FACTORED 1
 #define RVE_FORM_NODAL 2

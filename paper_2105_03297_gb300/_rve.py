@@ -259,15 +259,15 @@ class RVE:
         _check(load().rve_set_schedule(self.h, v), "rve_set_schedule")
 
     def test_stall_copies(self, on):
-        """Test hook: make the pipelined passes' bounded waits run out (see include/rve.h)."""
+        """Test hook: make the pipelined pass's bounded waits run out (see include/rve.h)."""
         _check(load().rve_test_stall_copies(self.h, 1 if on else 0), "rve_test_stall_copies")
 
     FORMS = {"stress": 0, "factored": 1, "nodal": 2}
 
     def set_operator_form(self, form):
-        """'stress' (default: FFT of every stress component), 'factored'
-        (real-space nodal forces, FFT of the D nodal components only) or
-        'nodal' (the factored chain with the CG vectors kept as nodal fields)."""
+        """'stress' (default) or 'factored' (CG on strains: real-space nodal
+        forces, FFT of the D nodal components, strains back in real space) or
+        'nodal' (the same chain with the CG vectors kept as nodal fields)."""
         _check(load().rve_set_operator_form(self.h, self.FORMS[form]), "rve_set_operator_form")
 
     def operator_form(self):
@@ -325,8 +325,8 @@ class RVE:
         _check(load().rve_get_deformation(self.h, int(load_case), p, flag), "rve_get_deformation")
         return out
 
-    # kind 7: real-space material kernel of the factored / nodal forms and of
-    # finite strain; kind 8: real-space update kernel of the factored / nodal forms
+    # kind 7: the first pass (with its x transform) of the factored and nodal forms,
+    # and the material kernel of finite strain; kind 8 is not used any more
     KINDS = ("pass_a", "pass_b", "pass_c", "pass_d", "pass_e", "residual", "other", "force_stencil",
              "strain_update")
 

@@ -472,11 +472,11 @@ int write_state(rve_s* h, int L) {
 
 // ---- autotuner: the schedule of the FFT passes --------------------------
 // Candidates per pass (rve_sched_candidates): pass A rows per block (default,
-// half, double) and one thread per load unit at the default and half rows;
-// pass E rows per block (default, half, double); in 3D FP32 with n_x >= 128
-// also the pipelined persistent passes and the default tiles with the L2
-// prefetch of a later block's rows (A 5 and 6, E 3 and 4); in 2D FP32 with
-// n_x = 512 or 1024 also pass A with the lane-pair x transform (A 5); the FFT split (radix
+// half, double) and other threads per block (A 3 and 4); pass E rows per block
+// (default, half, double); in 3D FP32 with n_x >= 128 also the pipelined
+// persistent first pass (A 5; A 6 and E 3, E 4 are accepted and run the tiles
+// of 0 and 1, so they are not timed on the force path); in 2D FP32 with n_x =
+// 512 or 1024 also pass A with the lane-pair x transform (A 5); the FFT split (radix
 // schedule) of pass C's axis; in 3D the split of the y axis (passes B and D,
 // timed together).  Each candidate is timed on the handle's own buffers
 // (CG-iteration modes on zeroed fields of the solve's load cases, at most
@@ -896,7 +896,7 @@ template <typename T> struct FeSolve {
   }
 };
 
-constexpr int kCheckEvery = 8;  // CG iterations per graph; even: the factored form alternates its buffers
+constexpr int kCheckEvery = 8;  // CG iterations per graph; even: the direction alternates its buffers
 
 template <typename T>
 int solve_impl(rve_s* h, const double* emac_host, int L, double rel_tol, int max_iter, rve_info* info,
