@@ -349,7 +349,8 @@ int rve_batch_effective_tangent(rve_batch_t b, int index, double* C);
  *             return RVE_ERR_SCRATCH_LIMIT;
  *  length[2]  cell lengths (NULL = unit cell);
  *  E[N]       device pointer, FP32 Young's moduli (may be NULL if apply_material = 0);
- *  p, q       device pointers, [6][N] FP32 fields (layout as rve_get_strain);
+ *  p, q       device pointers, [6][N] FP32 fields (layout as rve_get_strain); E, p
+ *             and q need the alignment of a float only, and q may be p;
  *  cuda_stream  stream to run on (NULL = default stream).
  * Scratch: one static device array of about 1.6 MB (spectrum, tables and a
  * state record), which every GPU that loads the library holds until the process

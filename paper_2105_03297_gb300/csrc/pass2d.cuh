@@ -650,6 +650,11 @@ __device__ __forceinline__ T strain_update(const PassArgs<T>& a, int64_t idx, T*
     for (int i = 0; i < VL; ++i) { n[i] = -q[i]; z[i] = 0; s += q[i] * q[i]; }
     vstoren<T, VL>(a.r + idx, n);
     vstoren<T, VL>(a.x + idx, z);
+  } else if (VL > 1 && (reinterpret_cast<uintptr_t>(a.out) & 15)) {
+    // a caller's own field (the entry point without a handle) of any element
+    // alignment; the handle's and the other fields are 16-byte aligned
+#pragma unroll
+    for (int i = 0; i < VL; ++i) a.out[idx + i] = q[i];
   } else {
     vstoren<T, VL>(a.out + idx, q);
   }

@@ -94,3 +94,38 @@ def test_static_operator_under_capture(n):
         call(ref, torch.cuda.current_stream())   # same stream: after the replay
         torch.cuda.synchronize()
         assert torch.equal(q, ref) and bool((q != 0).any())
+
+
+@pytest.mark.parametrize("n", [(16, 16), (256, 64)])
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_static_operator_on_any_element_alignment(n, shift):
+    """E, p and q of the entry point without a handle may start at any float,
+    and q may be p: the same bits as on aligned fields, and nothing outside."""
+    import ctypes as C
+    import torch
+    from paper_2105_03297_gb300 import _rve
+    lib = _rve.load()
+    N = n[0] * n[1]
+    E = torch.tensor(lognormal(n, 148).astype(np.float32), device="cuda").view(-1)
+    p = torch.tensor(np.random.default_rng(149).standard_normal(6 * N).astype(np.float32), device="cuda")
+    q = torch.empty_like(p)
+
+    def call(E, p, q):
+        assert 0 == lib.rve_apply_operator_2d_static(
+            (C.c_int64 * 2)(*n), None, C.c_void_p(E.data_ptr()), 0.3, C.c_void_p(p.data_ptr()),
+            C.c_void_p(q.data_ptr()), 1, C.c_void_p(torch.cuda.current_stream().cuda_stream))
+
+    def shifted(t):
+        w = torch.full((t.numel() + 8,), 7.0, device="cuda")
+        v = w[shift:shift + t.numel()]
+        v.copy_(t)
+        return w, v
+
+    call(E, p, q)
+    (_, Es), (pw, ps), (qw, qs) = shifted(E), shifted(p), shifted(torch.zeros_like(p))
+    call(Es, ps, qs)
+    assert torch.equal(qs, q) and torch.equal(ps, p)
+    call(Es, ps, ps)
+    assert torch.equal(ps, q)
+    for w in (pw, qw):
+        assert bool((w[:shift] == 7).all()) and bool((w[shift + 6 * N:] == 7).all())
