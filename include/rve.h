@@ -119,7 +119,10 @@ int rve_destroy(rve_t h);
  * C_eff and the strains of every element with E > 0 are unique (the energy is
  * strictly convex in them); strains of zero-stiffness elements, and the
  * adjoint gradient at zero-stiffness voxels, can carry any null-space
- * component and are not. */
+ * component and are not.
+ * A device field (RVE_PTR_DEVICE) is read after the work queued before the call
+ * on the handle's cuda_stream, on the legacy default stream and on every stream
+ * that synchronises with it; other streams are the caller's to order. */
 int rve_set_material(rve_t h, const void* E, int E_dtype, double nu, int ptr_flags);
 
 /* Solve L load cases together.  E_macro[L][n_s] (host, Mandel) are the

@@ -1473,16 +1473,21 @@ __global__ void __launch_bounds__(256) copy_moduli_k(const S* __restrict__ E, do
 }
 // Material of a handle from a field on its device: checked there, then copied
 // and rounded, so that the field does not cross to the host and back (256^3:
-// 24.1 ms of host loops and copies before, 0.1 ms now; 32^2: 0.18 ms, 0.03).
-// Invalid moduli leave the handle's material as it was.
+// 24.1 ms of host loops and copies, 0.3 ms this way; 32^2: 0.18 ms, 0.03).
+// Invalid moduli leave the handle's material as it was.  The check runs on the
+// legacy default stream, which waits for the work queued there and on every
+// blocking stream (the handle's own stream is waited for on the host): a field
+// written on the default stream is complete when it is read, whichever stream
+// the handle was created with.
 template <typename S> int device_material_t(rve_s* h, const S* E) {
   const int64_t want = (h->N + 255) / 256, most = 8 * (int64_t)device_sm_count();
   const unsigned blocks = (unsigned)(want < most ? want : most);
-  CK(cudaMemsetAsync(h->flag_d, 0, sizeof(unsigned), h->stream));
-  check_moduli_k<S><<<blocks, 256, 0, h->stream>>>(E, h->N, h->flag_d);
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(h->flag_h, h->flag_d, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  CK(cudaMemsetAsync(h->flag_d, 0, sizeof(unsigned), cudaStreamLegacy));
+  check_moduli_k<S><<<blocks, 256, 0, cudaStreamLegacy>>>(E, h->N, h->flag_d);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(h->flag_h, h->flag_d, sizeof(unsigned), cudaMemcpyDeviceToHost, cudaStreamLegacy));
+  CK(cudaStreamSynchronize(cudaStreamLegacy));
   if (*h->flag_h != 2u) return RVE_ERR_ARG;
   copy_moduli_k<S><<<blocks, 256, 0, h->stream>>>(E, h->E64, h->precision == RVE_MIXED ? (float*)h->Ein : nullptr, h->N);
   CK(cudaGetLastError());

@@ -42,6 +42,32 @@ def test_device_moduli(n, dtype, prec):
         assert np.array_equal(r.apply_operator(p), ref)
 
 
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_device_moduli_written_on_the_default_stream(own_stream):
+    """Moduli that are still being computed on the default stream when
+    set_material is called, on a handle of the default stream and on one of a
+    stream that does not wait for it."""
+    import torch
+    from paper_2105_03297_gb300 import RVE
+    n = (64, 64)
+    E = lognormal(n, 150)
+    p = np.random.default_rng(151).standard_normal((6, E.size))
+    a = torch.full((4096, 4096), 1.0 / 4096, device="cuda")
+    b, Ed = torch.empty_like(a), torch.ones(E.shape, dtype=torch.float64, device="cuda")
+    Eh = torch.tensor(E, device="cuda")
+    side = torch.cuda.Stream()   # non-blocking
+    with RVE(n, stream=side.cuda_stream if own_stream else None) as r:
+        r.set_material(E, 0.3)
+        ref = r.apply_operator(p)
+        torch.mm(a, a, out=b)
+        torch.cuda.synchronize()
+        for _ in range(60):   # some milliseconds of queued work
+            torch.mm(a, a, out=b)
+        Ed.copy_(Eh)
+        r.set_material(Ed, 0.3)
+        assert np.array_equal(r.apply_operator(p), ref)
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 @pytest.mark.parametrize("n", [(32, 16), (16, 16, 16)])
 def test_operator_on_device_tensors(n, prec):
