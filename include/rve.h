@@ -193,11 +193,13 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
  *  [3] in 3D the same choice for the y transforms (0 or 1); 0 in 2D.
  * -1 = choose by timing the candidates on the handle's buffers at the next
  * solve, with that solve's load cases (at most 8) (the default; the choice is
- * cached per grid, precision and number of load cases timed for the
- * process).  rve_set_schedule rejects a variant the grid does not have.
+ * cached per grid, precision, number of load cases timed, operator form and
+ * derivative for the process, and made again after a change of form or
+ * derivative).  rve_set_schedule rejects a variant the grid does not have.
  * rve_schedule also returns the measured candidate times
  * candidate_ms[RVE_SCHED_PASSES][RVE_SCHED_VARIANTS] (0 where a candidate does
- * not exist or was not timed; may be NULL). */
+ * not exist, runs as another one or was not timed; where variant 5 of the first
+ * pass is timed in 3D, [0] includes the first y transform; may be NULL). */
 enum { RVE_SCHED_PASSES = 4, RVE_SCHED_VARIANTS = 7 };
 int rve_schedule(rve_t h, int* variants, float* candidate_ms);
 int rve_set_schedule(rve_t h, const int* variants);

@@ -85,6 +85,7 @@ struct rve_s {
   // FFT split of pass C's axis and of passes B / D (3D); -1 = autotune at the
   // first solve
   int var[RVE_SCHED_PASSES] = {-1, -1, -1, -1};
+  unsigned tuned = 0;   // entries of var that the autotuner chose (bit w)
   float tune_ms[RVE_SCHED_PASSES][RVE_SCHED_VARIANTS] = {{0}};  // candidate times of the last tuning
   int op_form = RVE_FORM_STRESS;          // order of the operator inside projected CG
   int deriv = D_FE;                       // discrete derivative of the projection (RVE_DERIV_*)
@@ -419,14 +420,17 @@ template <typename T> struct NodalBufs {
 // One projected-CG iteration on the nodal state (parity q of the iteration):
 // force pass (pi, xi, f = B^T C B pi, alpha), then R -= alpha f,
 // rho = (B^T B)^-1 R and <rho, R> -> beta in the other passes.
-template <typename T> cudaError_t apply_nodal(rve_s* h, const PassArgs<T>& a, int q) {
+template <typename T> PassArgs<T> nodal_args(const rve_s* h, const PassArgs<T>& a, int q) {
   NodalBufs<T> nb(h, a.L);
   PassArgs<T> b = a;
   b.amode = A_CG; b.pmode = P_G; b.emode = E_NOUT;
   b.force = 2; b.pair = h->dim == 3; b.resid = 2; b.dot = 1;
   b.rho = nb.rho; b.pold = nb.pi[q ^ 1]; b.pnew = nb.pi[q]; b.xi = nb.xi;
   b.out = nb.rho;
-  return apply_passes<T>(h, b);
+  return b;
+}
+template <typename T> cudaError_t apply_nodal(rve_s* h, const PassArgs<T>& a, int q) {
+  return apply_passes<T>(h, nodal_args<T>(h, a, q));
 }
 
 // The k-th CG iteration of a batch (k counts from 0 at the start of an inner
@@ -482,12 +486,17 @@ int write_state(rve_s* h, int L) {
 // (CG-iteration modes on zeroed fields of the solve's load cases, at most
 // kTuneMaxL; 2 warm-up and 3 timed launches, CUDA events on the handle's
 // stream), passes in the order A, E, C, B/D with the winners of the earlier
-// ones, and the fastest is kept; choices are cached per (dimension, grid,
-// precision, load cases timed) for the process.
+// ones, and the fastest is kept.  Where A 5 is a candidate of the 3D force path
+// the first pass is timed together with pass B, which then has 36 components to
+// read instead of two force spectra (256 x 256 x 64: 168 against 38 us).
+// Choices are cached for the process per grid, precision, load cases timed,
+// operator form and derivative: the variants of the form's or derivative's own
+// kernels are not those of another.
 struct TuneKey {
-  int dim, n0, n1, n2, tsize, nl;
+  int dim, n0, n1, n2, tsize, nl, form, deriv;
   bool operator<(const TuneKey& o) const {
-    return std::tie(dim, n0, n1, n2, tsize, nl) < std::tie(o.dim, o.n0, o.n1, o.n2, o.tsize, o.nl);
+    return std::tie(dim, n0, n1, n2, tsize, nl, form, deriv) <
+           std::tie(o.dim, o.n0, o.n1, o.n2, o.tsize, o.nl, o.form, o.deriv);
   }
 };
 std::map<TuneKey, std::array<int, RVE_SCHED_PASSES>> g_tuned;
@@ -516,6 +525,14 @@ int rve_sched_candidates(const rve_s* h, int which) {
   }
 }
 
+// The tuner's choices hold for the operator form and derivative they were timed
+// in; entries the caller set stay.
+void retune(rve_s* h) {
+  for (int w = 0; w < RVE_SCHED_PASSES; ++w)
+    if (h->tuned & (1u << w)) h->var[w] = -1;
+  h->tuned = 0;
+}
+
 // Load cases the candidates are timed with: those of the solve that asks for
 // the tuning (the grids of the passes scale with them, and with them how full
 // the last wave of blocks is), at most kTuneMaxL.
@@ -523,13 +540,16 @@ constexpr int kTuneMaxL = 8;
 
 template <typename T> int autotune(rve_s* h, int L) {
   const int Lt = L < 1 ? 1 : (L > kTuneMaxL ? kTuneMaxL : L);
-  const TuneKey key{h->dim, h->n[0], h->n[1], h->n[2], (int)h->tsize, Lt};
+  const TuneKey key{h->dim, h->n[0], h->n[1], h->n[2], (int)h->tsize, Lt, h->op_form, h->deriv};
+  auto choose = [&](const std::array<int, RVE_SCHED_PASSES>& c) {
+    for (int w = 0; w < RVE_SCHED_PASSES; ++w)
+      if (h->var[w] < 0) { h->var[w] = c[w]; h->tuned |= 1u << w; }
+  };
   {
     std::lock_guard<std::mutex> lk(g_tune_mutex);
     auto it = g_tuned.find(key);
     if (it != g_tuned.end()) {
-      for (int w = 0; w < RVE_SCHED_PASSES; ++w)
-        if (h->var[w] < 0) h->var[w] = it->second[w];
+      choose(it->second);
       return RVE_OK;
     }
   }
@@ -553,7 +573,10 @@ template <typename T> int autotune(rve_s* h, int L) {
   a.cgphase = 0; a.amode = A_CG; a.pmode = P_G; a.emode = E_CG;
   a.in = (const T*)h->fbuf; a.out = (T*)h->x;
   a.var_a = a.var_e = a.var_c = a.var_y = 0;
+  const bool nodal = h->op_form == RVE_FORM_NODAL;
+  if (nodal) a = nodal_args(h, a, 1);
   auto first_pass = [&] {   // the kind of first pass a.var_a stands for
+    if (nodal) return;
     a.force = a.pair = 0;
     if (force_pass(h, a.var_a)) set_force(h, a, 1);
   };
@@ -570,20 +593,35 @@ template <typename T> int autotune(rve_s* h, int L) {
   auto pass_c_l = [&]() { return d3 ? launch_pass_c_3d<T>(a, h->stream) : launch_pass_c_2d<T>(a, h->stream); };
   auto pass_d_l = [&]() { return d3 ? launch_pass_d_3d<T>(a, h->stream) : cudaSuccess; };
   auto pass_e_l = [&]() { return d3 ? launch_pass_e_3d<T>(a, h->stream) : launch_pass_e_2d<T>(a, h->stream); };
-  int best[RVE_SCHED_PASSES] = {0, 0, 0, 0};
+  std::array<int, RVE_SCHED_PASSES> best{};
   for (int w = 0; w < RVE_SCHED_PASSES; ++w)
     for (int v = 0; v < RVE_SCHED_VARIANTS; ++v) h->tune_ms[w][v] = 0.f;
+  // candidates that run the kernel of an earlier one on this handle's path
+  auto same = [&](int which, int v) {
+    if (!force_pass(h, 0) || v == 0) return false;
+    if (which == 0) return nodal || v == 6 || (d3 && v == 5 && force_pass(h, 5));
+    return which == 1 && (v >= 3 || (nodal && d3));
+  };
+  const bool with_b = d3 && force_pass(h, 0) && !force_pass(h, 5);
+  if (nodal) {   // start the residual force from the zeroed fields
+    a.resid = 1;
+    CK(pass_a_l()); CK(pass_b_l()); CK(pass_c_l());
+    a.resid = 2;
+  }
   for (int which = 0; which < RVE_SCHED_PASSES; ++which) {
     const int nc = rve_sched_candidates(h, which);
     float best_ms = 1e30f;
     for (int v = 0; v < nc; ++v) {
-      if (force_pass(h, 0) && ((which == 0 && v == 6) || (which == 1 && v >= 3))) continue;   // same kernel as 0 or 1
+      if (same(which, v)) continue;
       int* slot = which == 0 ? &a.var_a : which == 1 ? &a.var_e : which == 2 ? &a.var_c : &a.var_y;
       *slot = v;
       auto one = [&]() -> cudaError_t {
-        if (which == 0) return pass_a_l();
         if (which == 1) return pass_e_l();
         if (which == 2) return pass_c_l();
+        if (which == 0) {
+          cudaError_t e = pass_a_l();
+          return e == cudaSuccess && with_b ? pass_b_l() : e;
+        }
         cudaError_t e = pass_b_l();
         return e == cudaSuccess ? pass_d_l() : e;
       };
@@ -607,13 +645,9 @@ template <typename T> int autotune(rve_s* h, int L) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  std::array<int, RVE_SCHED_PASSES> chosen;
-  for (int w = 0; w < RVE_SCHED_PASSES; ++w) {
-    if (h->var[w] < 0) h->var[w] = best[w];
-    chosen[w] = best[w];
-  }
+  choose(best);
   std::lock_guard<std::mutex> lk(g_tune_mutex);
-  g_tuned[key] = chosen;
+  g_tuned[key] = best;
   return RVE_OK;
 }
 
@@ -1882,6 +1916,7 @@ int rve_set_schedule(rve_t h, const int* variants) {
   for (int w = 0; w < RVE_SCHED_PASSES; ++w)
     if (variants[w] < -1 || variants[w] >= rve_sched_candidates(h, w)) return RVE_ERR_ARG;
   for (int w = 0; w < RVE_SCHED_PASSES; ++w) h->var[w] = variants[w];
+  h->tuned = 0;
   return RVE_OK;
 }
 
@@ -1891,6 +1926,7 @@ int rve_set_operator_form(rve_t h, int form) {
   if (form != RVE_FORM_STRESS && (h->deriv != D_FE || h->finite)) return RVE_ERR_ARG;
   if (int jr = join_user(h)) return jr;
   CK(cudaStreamSynchronize(h->stream));
+  if (form != h->op_form) retune(h);
   h->op_form = form;
   return RVE_OK;
 }
@@ -1906,6 +1942,7 @@ int rve_set_derivative(rve_t h, int derivative) {
   static_assert((int)RVE_DERIV_FE == (int)D_FE && (int)RVE_DERIV_FOURIER2 == (int)D_FOURIER2, "derivative codes");
   const int nq = (derivative == RVE_DERIV_FE) ? (h->dim == 2 ? 2 : 6) : (derivative == RVE_DERIV_FOURIER2 ? 2 : 1);
   if (derivative != h->deriv) {
+    retune(h);
     // the field layout depends on n_q: drop the per-load-case buffers and any solution
     free_L(h);
     h->solved = false;
