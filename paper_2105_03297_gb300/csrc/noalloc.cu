@@ -135,7 +135,7 @@ extern "C" int rve_apply_operator_2d_static(const int64_t* n, const double* leng
   a.cgphase = 0;
   a.grads = 1;
   a.pdl = 1;
-  a.force = 1;
+  a.force = 4;
   cudaError_t e = launch_force_2d<float>(a, s);
   if (e == cudaSuccess) e = launch_pass_c_2d<float>(a, s);
   if (e == cudaSuccess) e = launch_pass_e_2d<float>(a, s);

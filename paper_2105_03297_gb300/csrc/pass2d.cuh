@@ -365,9 +365,10 @@ __device__ __forceinline__ void publish_rr(const PassArgs<T>& a, CgState* cg, co
 // registers at 512 and 1024 points: six blocks of four warps per SM; at 150
 // registers and three blocks the 1024^2 pass took 65 us, now 48 with the
 // combination of all six components it then still did).
-// W = 4 (P = 1) writes the differences d_a w_j along the element edges,
-// d_a = (exp(i k_a h_a) - 1)/h_a, as components 2 a + j: the last pass then
-// only picks them up at the right nodes.  Differences of w itself, taken there
+// W = 4 (P = 1) reads the edge sums s_aj in components 2 a + j (S_EDGE of
+// pass_force.cuh), t_j = sum_a conj(d_a) s_aj, d_a = (exp(i k_a h_a) - 1)/h_a,
+// and writes the differences d_a w_j along the element edges there: the last
+// pass then only picks them up at the right nodes.  Differences of w itself, taken there
 // in real space, round like eps n_a |w|: up to 8 times the error on a smooth
 // field (measured at 1024^2 in FP32: 1.0e-5 against 1.2e-6 of the 2-norm; on
 // white noise 4.3e-7 against 3.1e-7).  Inside the CG that error is corrected
@@ -377,7 +378,7 @@ __device__ __forceinline__ void publish_rr(const PassArgs<T>& a, CgState* cg, co
 template <typename T, int NY, int P, int NT, int V, int W>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) pass_c_2d_fe(PassArgs<T> a) {
   using C = cplx<T>;
-  constexpr int R = 2 * P;
+  constexpr int R = W * P;
   static_assert(W == 2 || (W == 4 && P == 1), "differences: one column per block");
   constexpr int LD = FftSplit<NY, V>::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
   C* base = a.spec + ((int64_t)l * a.m * KX + kx0) * NY;
   auto st_s = [&](int b, int k, C v) { buf[b * LD + k] = v; };
   auto ld_s = [&](int b, int y) -> C { return buf[b * LD + y]; };
-  if (a.resid) {   // nodal state: keep the residual force R and transform it (as pass_y_3d)
+  if (W == 2 && a.resid) {   // nodal state: keep the residual force R and transform it (as pass_y_3d)
     const bool upd = a.resid == 2;
     const T alpha = upd ? cg_alpha<T>(cg) : (T)1;
     constexpr int TOT = R * NY, U = 4;
@@ -424,7 +425,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
     fft4<T, NY, R, LD, NT, -1, true, true, false, false, V>(buf, a.tw[1], ld_s, st_s);
   } else {
     auto ld_g = [&](int b, int y) -> C {
-      return (kx0 + b / 2 < KX) ? base[(b % 2) * cstride + (int64_t)(b / 2) * NY + y] : mkc<T>(0, 0);
+      return (kx0 + b / W < KX) ? base[(b % W) * cstride + (int64_t)(b / W) * NY + y] : mkc<T>(0, 0);
     };
     fft4<T, NY, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[1], ld_g, st_s);
   }
@@ -433,6 +434,14 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
     const int pc = i / NY, ky = i % NY, kx = kx0 + pc;
     if (kx >= KX) continue;
     C t[2] = {buf[2 * pc * LD + ky], buf[(2 * pc + 1) * LD + ky]};
+    C d0, d1;
+    if constexpr (W == 4) {
+      const C one = mkc<T>(1, 0);
+      d0 = cscale(csub(a.ph[0][kx], one), a.ih[0]);
+      d1 = cscale(csub(a.ph[1][ky], one), a.ih[1]);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) t[j] = cadd(cjmul(d0, t[j]), cjmul(d1, buf[(2 + j) * LD + ky]));
+    }
     const C r0 = t[0], r1 = t[1];
     if (kx == 0 && ky == 0) {
       t[0] = t[1] = mkc<T>(0, 0);   // k = 0: no mean
@@ -449,8 +458,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NY >= 512 ? 6 : 4) : 1) 
       acc.add(kx == 0 || kx == KX - 1 ? d : (T)2 * d);
     }
     if constexpr (W == 4) {
-      const C one = mkc<T>(1, 0);
-      const C d0 = cscale(csub(a.ph[0][kx], one), a.ih[0]), d1 = cscale(csub(a.ph[1][ky], one), a.ih[1]);
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         buf[j * LD + ky] = cmul(d0, t[j]);

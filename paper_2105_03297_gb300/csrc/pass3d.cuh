@@ -141,13 +141,17 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT <= 256 ? 4 : 2) : 1) 
   // TZB contiguous y-pencils (one request); inverse, its NY z-chunks of TZB
   // values
   int zb2, kx2, lc2;
+  // the component that holds the second part of component i's nodal forces
+  // (pair 1) or edge sums (pair 2: of x and y), less i; 0 where there is none
+  auto second = [&](int i) -> int { return a.pair == 1 ? 3 : a.pair == 2 && i < 6 ? 9 : 0; };
   if (a.pf_ahead > 0 && grid_ahead(a, zb2, kx2, lc2) && slot_runs(a, lc2 / Cc)) {
     static_assert((TZB * sizeof(C)) % 16 == 0, "bulk prefetch sizes are multiples of 16 bytes");
     const int64_t cb2 = (((int64_t)(lc2 / Cc) * a.m + lc2 % Cc) * KX + kx2);
     const int z2 = zb2 * TZB;
     if (FWD) {
-      if (threadIdx.x < (a.pair ? 2 : 1))
-        prefetch_l2_bulk(a.spec + ((cb2 + 3 * (int64_t)threadIdx.x * KX) * nz + z2) * NY, (unsigned)(TZB * NY * sizeof(C)));
+      const int s2 = second(lc2 % Cc);
+      if (threadIdx.x < (s2 ? 2 : 1))
+        prefetch_l2_bulk(a.spec + ((cb2 + s2 * (int64_t)threadIdx.x * KX) * nz + z2) * NY, (unsigned)(TZB * NY * sizeof(C)));
     } else {
       for (int k = threadIdx.x; k < NY; k += blockDim.x)
         prefetch_l2_bulk(a.spec2 + cb2 * NY * nz + z2 + (int64_t)k * nz, (unsigned)(TZB * sizeof(C)));
@@ -190,8 +194,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (NT <= 256 ? 4 : 2) : 1) 
       __syncthreads();
       auto ld = [&](int zz, int y) -> C { return buf[zz * LD + y]; };
       fft4<T, NY, TZB, LD, NT, -1, true, false, false, true, V>(buf, a.tw[1], ld, st);
-    } else if (a.pair) {   // the two parts of the nodal forces (force_3d)
-      const C* other = pencils + 3 * (int64_t)KX * nz * NY;
+    } else if (const int s2 = second(c)) {   // the two parts of the sums over elements (force_3d)
+      const C* other = pencils + s2 * (int64_t)KX * nz * NY;
       auto ld = [&](int zz, int y) -> C {
         return cadd(pencils[(int64_t)zz * NY + y], other[(int64_t)zz * NY + y]);
       };
@@ -366,12 +370,13 @@ __device__ __forceinline__ void solve_3d(cplx<T>* col, const cplx<T>* e, const T
 // Pass C of the finite elements: forward FFT along z, w^ = (B^H B)^-1 t^,
 // inverse FFT, on the three nodal components; P pencils (k_x, k_y0 + i), i <
 // P, per block.  Row b of the buffer is component b % 3 of pencil b / 3.  W =
-// 9 (P = 1) writes the differences d_a w_j along the element edges as
-// components 3 a + j (see pass_c_2d_fe).  grid (n_x/2+1, n_y/P, L).
+// 9 (P = 1) reads the edge sums s_aj and writes the differences d_a w_j along
+// the element edges as components 3 a + j (see pass_c_2d_fe).
+// grid (n_x/2+1, n_y/P, L).
 template <typename T, int NZ, int P, int NT, int V, int W>
 __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 384 ? 2 : 1) pass_c_3d_nodal(PassArgs<T> a) {
   using C = cplx<T>;
-  constexpr int R = 3 * P;
+  constexpr int R = W * P;
   static_assert(W == 3 || (W == 9 && P == 1), "differences: one pencil per block");
   constexpr int LD = FftSplit<NZ, V>::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -387,7 +392,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 38
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t stride_c = (int64_t)KX * ny * NZ;
   C* base = a.spec2 + (int64_t)l * a.m * stride_c + ((int64_t)kx * ny + ky0) * NZ;
-  auto ld_g = [&](int b, int z) -> C { return base[(b % 3) * stride_c + (b / 3) * NZ + z]; };
+  auto ld_g = [&](int b, int z) -> C { return base[(b % W) * stride_c + (b / W) * NZ + z]; };
   auto st_s = [&](int b, int k, C v) { buf[b * LD + k] = v; };
   fft4<T, NZ, R, LD, NT, -1, false, true, false, false, V>(buf, a.tw[2], ld_g, st_s);
   Acc<T> acc;
@@ -399,6 +404,16 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 1 : W == 9 ? 8 : NT <= 38
       for (int j = 0; j < W; ++j) col[j * LD] = mkc<T>(0, 0);
     } else {
       const C e[3] = {a.ph[0][kx], a.ph[1][ky0 + pc], a.ph[2][kz]};
+      if constexpr (W == 9) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          C t = mkc<T>(0, 0);
+#pragma unroll
+          for (int ax = 0; ax < 3; ++ax)
+            t = cadd(t, cjmul(cscale(csub(e[ax], mkc<T>(1, 0)), a.ih[ax]), col[(3 * ax + j) * LD]));
+          col[j * LD] = t;
+        }
+      }
       const C t[3] = {col[0], col[LD], col[2 * LD]};
       solve_3d<T, LD>(col, e, a.ih, a.inv_n);
       if (a.dot) {
@@ -835,7 +850,7 @@ cudaError_t launch_y_3d_v(const PassArgs<T>& a, cudaStream_t s) {
     set_smem_attrs(k, sm);
     if (dev >= 0 && dev < kMaxDevices) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[dev], k, NT, sm);
   });
-  const int Cc = !fe_path(a) ? a.m : (!FWD && a.grads) ? 9 : 3;   // finite elements: w or its edge differences
+  const int Cc = !fe_path(a) ? a.m : a.grads ? 9 : 3;   // finite elements: edge sums and differences, or t and w
   dim3 grid(a.n[2] / TZB, a.kx, a.L * Cc);
   if (sizeof(T) == 4) {
     PassArgs<T> b = a;

@@ -20,9 +20,9 @@
 //
 // Source of the corner forces (SRC):
 //   S_STRAIN  CG on strain fields: x += alpha_prev p_old, p = r + beta p_old,
-//             sigma = C p, <p, sigma> -> alpha (A_CG); or sigma = C in
-//             (A_FIELD), sigma = in (A_BARE).  p_old and p_new are different
-//             arrays: the row below the tile is read by two blocks.
+//             sigma = C p, <p, sigma> -> alpha (A_CG); or sigma = in (A_BARE).
+//             p_old and p_new are different arrays: the row below the tile is
+//             read by two blocks.
 //             Bound by the 5 m N values per iteration (256 x 256 x 64 in FP32:
 //             622 us, 4.9 TB/s of r, p_old, x in and p, x out; a probe that
 //             marches the same rows without the arithmetic reaches 5.6: each
@@ -30,6 +30,24 @@
 //   S_NODAL   CG on nodal fields: pi = rho + beta pi_old, xi += alpha_prev
 //             pi_old, sigma = C B pi, <B pi, sigma> -> alpha.  Bound by issue:
 //             about 300 arithmetic instructions per voxel.
+//   S_EDGE    rve_apply_operator and its 2D entry point without a handle, whose
+//             result leaves the library as it is: sigma = C in (A_FIELD), sigma =
+//             in (A_BARE).  The factors of B^H are taken apart, f_j = sum_a
+//             d_a^H s_aj, with s_aj the sum of the stresses of the elements at
+//             the edge of axis a that starts at the node; the D^2 sums s_aj are
+//             transformed, and pass C applies conj(d_a) per wavevector.  In f
+//             itself the differences along the short side of a voxel, 1/h_a
+//             times larger, leave their rounding error to the wavevectors of
+//             the long side (FP32, white noise on the unit cell, 2-norm of the
+//             error with f and with s: 1024 x 16 1.1e-6, 2.5e-7; 256 x 16
+//             5.3e-7, 2.1e-7; 64 x 64 2.6e-7, 2.1e-7; 16 x 16 x 256 5.2e-7,
+//             2.3e-7).  It costs the transforms and the traffic of 9 components
+//             instead of 3 (2D: 4 instead of 2): us with f and with s, FP32,
+//             256 x 256 x 64: this pass 188, 267, pass B 54, 78, C 97, 108, the
+//             call 748, 871; 128^3 486, 551; 1024^2 88, 90.
+//             3D: s_x and s_y again in two parts (planes z and z + 1), s_z in
+//             one: 15 real rows, 8 complex transforms, components 3 a + j and
+//             (second parts) 9 + 3 a + j.
 //   S_GRAD    finite strain (2D): the divergence of the stress field in, 4
 //             components P_ia per triangle.
 #pragma once
@@ -37,7 +55,7 @@
 
 namespace rve {
 
-enum { S_STRAIN = 0, S_NODAL = 1, S_GRAD = 2 };
+enum { S_STRAIN = 0, S_NODAL = 1, S_GRAD = 2, S_EDGE = 3 };
 
 // Value of the previous (next) column of the same row; at the row's start (end)
 // inside a warp the row wraps, at a warp's first (last) lane of a longer row
@@ -67,6 +85,22 @@ __device__ __forceinline__ void tet_forces(int t, const T S[3][3], const T* ih, 
   }
 }
 
+// Edges of a voxel: the k-th one of axis a starts at the k-th corner without
+// bit a (corner dx + 2 dy + 4 dz).
+__host__ __device__ constexpr int edge_of(int a, int c) { return a == 0 ? c >> 1 : a == 1 ? (c & 1) + 2 * (c >> 2) : c & 3; }
+
+// Stresses of tetrahedron t, added to the sums g[axis][edge][j] of its three edges.
+template <typename T> __device__ __forceinline__ void tet_edges(int t, const T S[3][3], T g[3][4][3]) {
+  int at = 0;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int a = kuhn_perm(t, i);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) g[a][edge_of(a, at)][j] += S[a][j];
+    at |= 1 << a;
+  }
+}
+
 // Corner forces of the six tetrahedra of a voxel from its corner displacements
 // and the voxel's share of <B u, C B u>.  Tetrahedra that share an edge share
 // its difference (12 edges instead of 18) and its force is summed over them
@@ -75,7 +109,6 @@ template <typename T>
 __device__ __forceinline__ T voxel_forces_3d(const T uc[8][3], T e, T lam, T mu2, const T* ih, T f[8][3]) {
   T d[3][4][3];   // d[a][k][j]: difference of u_j along the edge of axis a at the k-th corner without bit a
   auto corner = [](int a, int k) { return a == 0 ? 2 * k : a == 1 ? (k & 1) + 4 * (k >> 1) : k; };
-  auto edge = [](int a, int c) { return a == 0 ? c >> 1 : a == 1 ? (c & 1) + 2 * (c >> 2) : c & 3; };
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -97,7 +130,7 @@ __device__ __forceinline__ T voxel_forces_3d(const T uc[8][3], T e, T lam, T mu2
     int ke[3];   // edge index of the tetrahedron's edge along each axis
     int at = 0;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) { ke[ax[i]] = edge(ax[i], at); at |= 1 << ax[i]; }
+    for (int i = 0; i < 3; ++i) { ke[ax[i]] = edge_of(ax[i], at); at |= 1 << ax[i]; }
     const T exx = d[0][ke[0]][0], eyy = d[1][ke[1]][1], ezz = d[2][ke[2]][2];
     const T yz = d[1][ke[1]][2] + d[2][ke[2]][1], xz = d[0][ke[0]][2] + d[2][ke[2]][0];
     const T xy = d[0][ke[0]][1] + d[1][ke[1]][0];
@@ -114,11 +147,11 @@ __device__ __forceinline__ T voxel_forces_3d(const T uc[8][3], T e, T lam, T mu2
   for (int c = 0; c < 8; ++c)
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      T v = ih[0] * S[0][edge(0, c & ~1)][j];
+      T v = ih[0] * S[0][edge_of(0, c & ~1)][j];
       if (!(c & 1)) v = -v;
 #pragma unroll
       for (int a = 1; a < 3; ++a) {
-        const T p = S[a][edge(a, c & ~(1 << a))][j];
+        const T p = S[a][edge_of(a, c & ~(1 << a))][j];
         v = (c >> a) & 1 ? v + ih[a] * p : v - ih[a] * p;
       }
       f[c][j] = v;
@@ -133,11 +166,13 @@ template <typename T, int NX, int TY> __host__ __device__ constexpr int force_ld
   constexpr int M = sizeof(T) == 4 ? 16 : 8, want = TY >= M ? 1 : M / TY;
   return FftSplit<NX>::LD + (want - FftSplit<NX>::LD % M + M) % M;
 }
-// Stages of the strain source's ring (18 values a thread each).
+// Stages of the ring of the strain and edge sources, and their values a thread each.
 template <typename T> __host__ __device__ constexpr int force_stages() { return sizeof(T) == 4 ? 3 : 2; }
+template <int SRC> __host__ __device__ constexpr int force_slots() { return SRC == S_STRAIN ? 18 : SRC == S_EDGE ? 6 : 0; }
+template <int SRC> __host__ __device__ constexpr int force_rows() { return SRC == S_EDGE ? 8 : 3; }   // complex rows per y
 template <typename T, int NX, int TY, int NT, int VL, int SRC> constexpr size_t force_3d_smem() {
-  return (SRC == S_STRAIN ? sizeof(T) * force_stages<T>() * 18 * NT * VL : 0) +
-         sizeof(cplx<T>) * 3 * TY * force_ld<T, NX, TY>() +
+  return sizeof(T) * force_stages<T>() * force_slots<SRC>() * NT * VL +
+         sizeof(cplx<T>) * force_rows<SRC>() * TY * force_ld<T, NX, TY>() +
          sizeof(T) * 12 * (NX / VL > 32 ? (TY + NT * VL / NX) * (NX / VL / 32) : 0);
 }
 
@@ -153,9 +188,11 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
   constexpr int NW = TPR > 32 ? TPR / 32 : 1;    // warps per row
   static_assert(NT % TPR == 0 && TY % LN == 0, "threads cover whole rows");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);                        // [3][TY][LD]
-  T* edge = reinterpret_cast<T*>(buf + 3 * TY * LD);              // [LN][TYL + 1][NW][12], TPR > 32
-  T* ring = edge + (TPR > 32 ? 12 * (TY + LN) * NW : 0);          // strain source: [stages][18][NT] x VL
+  constexpr bool EDGES = SRC == S_EDGE;
+  constexpr int CR = force_rows<SRC>(), SL = force_slots<SRC>();
+  C* buf = reinterpret_cast<C*>(smem_raw);                        // [CR][TY][LD]
+  T* edge = reinterpret_cast<T*>(buf + CR * TY * LD);             // [LN][TYL + 1][NW][12], TPR > 32
+  T* ring = edge + (TPR > 32 ? 12 * (TY + LN) * NW : 0);          // [stages][SL][NT] x VL
   __shared__ double red[NT / 32];
   __shared__ T cols[NT];
   __shared__ int flag;
@@ -168,29 +205,36 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
   const int64_t N = a.N;
   const int tx = threadIdx.x % TPR, ln = threadIdx.x / TPR, x = tx * VL;
   const int lane = threadIdx.x & 31;
-  const bool cgm = a.amode == A_CG;
+  const bool cgm = !EDGES && a.amode == A_CG;
   const bool use_old = cgm && cg->it > 0;
   const T beta = use_old ? cg_beta<T>(cg) : (T)0, alpha_prev = use_old ? cg_alpha<T>(cg) : (T)0;
   const T ih[3] = {a.ih[0], a.ih[1], a.ih[2]};
   const T* Ep = a.E + (int64_t)(l / a.lcs) * N + (int64_t)z * ny * NX + x;
   const int first = ln * TYL - 1, end = (ln + 1) * TYL;
   Acc<T> acc;
-  T carry[VL][2][3];   // [column][dz][j]: dy = 1 corners of the row below
+  // dy = 1 corners of the row below: [column][dz][j]; edge sums: s_x [dz][j], s_z [2][j]
+  constexpr int CY = EDGES ? 3 : 2;
+  T carry[VL][CY][3];
 #pragma unroll
   for (int k = 0; k < VL; ++k)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) carry[k][0][j] = carry[k][1][j] = 0;
+    for (int j = 0; j < 3 * CY; ++j) carry[k][j / 3][j % 3] = 0;
   auto load_e = [&](int yy, T* e) { vloadn<T, VL>(e, Ep + (int64_t)((y0 + yy) & (ny - 1)) * NX); };
 
-  // corners with dx = 1 of the last column (f) -> first column of the next thread
-  auto pass_on = [&](int yy, const T f[8][3], T pv[2][2][3]) {
+  // corners with dx = 1 of the last column (f: [8][3] corner forces; edge sums
+  // [3][4][3]: s_y of dz = 0 and 1, s_z of dy = 0 and 1) -> first column of the
+  // next thread
+  auto right_of = [&](const T* f, int i, int k, int j) -> T {
+    return EDGES ? f[(i + 1) * 12 + (1 + 2 * k) * 3 + j] : f[(1 + 2 * i + 4 * k) * 3 + j];
+  };
+  auto pass_on = [&](int yy, const T* f, T pv[2][2][3]) {
 #pragma unroll
     for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
       for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          const T u = f[1 + 2 * dy + 4 * dz][j];
+          const T u = right_of(f, dy, dz, j);
           T q = from_prev<TPR>(u);
           if constexpr (TPR > 32) {
             if (lane == 31) edge[((ln * (TYL + 1) + yy - first) * NW + tx / 32) * 12 + dy * 6 + dz * 3 + j] = u;
@@ -203,32 +247,55 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
         }
   };
   // column k of row yy: corners dx = 0 of its voxel (f) and dx = 1 of the voxel before (pv)
-  auto put_column = [&](int yy, int k, const T f[8][3], const T pv[2][2][3]) {
+  auto put_column = [&](int yy, int k, const T* f, const T pv[2][2][3]) {
     const bool own = yy > first;
-    T v[2][3];
-#pragma unroll
-    for (int dz = 0; dz < 2; ++dz)
+    if constexpr (EDGES) {
+      auto g = [&](int ax, int e, int j) -> T { return f[ax * 12 + e * 3 + j]; };
+      T sz[3];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        v[dz][j] = f[4 * dz][j] + pv[0][dz][j] + carry[k][dz][j];
-        carry[k][dz][j] = f[2 + 4 * dz][j] + pv[1][dz][j];
+        const C sx = mkc<T>(g(0, 0, j) + carry[k][0][j], g(0, 2, j) + carry[k][1][j]);   // x edges dy + 2 dz
+        const C sy = mkc<T>(g(1, 0, j) + pv[0][0][j], g(1, 2, j) + pv[0][1][j]);         // y edges dx + 2 dz
+        sz[j] = g(2, 0, j) + pv[1][0][j] + carry[k][2][j];                               // z edges dx + 2 dy
+        carry[k][0][j] = g(0, 1, j);
+        carry[k][1][j] = g(0, 3, j);
+        carry[k][2][j] = g(2, 2, j) + pv[1][1][j];
+        if (own) {
+          buf[(j * TY + yy) * LD + x + k] = sx;
+          buf[((3 + j) * TY + yy) * LD + x + k] = sy;
+        }
       }
-    if (own) {
+      if (own) {
+        buf[(6 * TY + yy) * LD + x + k] = mkc<T>(sz[0], sz[1]);
+        buf[(7 * TY + yy) * LD + x + k] = mkc<T>(sz[2], (T)0);
+      }
+    } else {
+      T v[2][3];
 #pragma unroll
-      for (int j = 0; j < 3; ++j) buf[(j * TY + yy) * LD + x + k] = mkc<T>(v[0][j], v[1][j]);
+      for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          v[dz][j] = f[12 * dz + j] + pv[0][dz][j] + carry[k][dz][j];
+          carry[k][dz][j] = f[6 + 12 * dz + j] + pv[1][dz][j];
+        }
+      if (own) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) buf[(j * TY + yy) * LD + x + k] = mkc<T>(v[0][j], v[1][j]);
+      }
     }
   };
-  auto right = [&](const T f[8][3], T pv[2][2][3]) {   // within the thread
+  auto right = [&](const T* f, T pv[2][2][3]) {   // within the thread
 #pragma unroll
     for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
       for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) pv[dy][dz][j] = f[1 + 2 * dy + 4 * dz][j];
+        for (int j = 0; j < 3; ++j) pv[dy][dz][j] = right_of(f, dy, dz, j);
   };
 
-  if constexpr (SRC == S_STRAIN) {
-    // A step is one tetrahedron of one row: 6 values each of r, p_old and x.
+  if constexpr (SRC == S_STRAIN || SRC == S_EDGE) {
+    // A step is one tetrahedron of one row: 6 values each of r, p_old and x
+    // (edge source: of the field in).
     // Every thread copies its own values of the next ST - 1 steps into its own
     // slots of the ring (cp.async: no registers are held, and since no thread
     // reads another's slot there is no barrier).
@@ -240,14 +307,14 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
     T* xp = a.x + base;
     const bool mat = a.amode != A_BARE;
     auto off = [&](int yy) -> unsigned { return (unsigned)(((y0 + yy) & (ny - 1)) * NX + x); };
-    auto slot = [&](int t, int s) -> T* { return ring + (((t % ST) * 18 + s) * NT + threadIdx.x) * VL; };
+    auto slot = [&](int t, int s) -> T* { return ring + (((t % ST) * SL + s) * NT + threadIdx.x) * VL; };
     auto issue = [&](int yy, int t) {   // step (yy, t) into slot t % ST
       if (yy < end) {
         const unsigned o = off(yy);
         constexpr int B = VL * (int)sizeof(T);
 #pragma unroll
         for (int s = 0; s < 6; ++s) copy_async<B>(slot(t, s), rp + (6 * t + s) * N + o);
-        if (use_old) {
+        if (!EDGES && use_old) {
 #pragma unroll
           for (int s = 0; s < 6; ++s) copy_async<B>(slot(t, 6 + s), po + (6 * t + s) * N + o);
           if (yy > first) {
@@ -269,11 +336,12 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
       const bool own = yy > first;
       const unsigned o = off(yy);
       if (mat && yy + 1 < end) load_e(yy + 1, en);
-      T f[VL][8][3];
+      constexpr int NF = EDGES ? 36 : 24;   // edge sums [3][4][3] or corner forces [8][3]
+      T f[VL][NF];
 #pragma unroll
       for (int k = 0; k < VL; ++k)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) f[k][c][0] = f[k][c][1] = f[k][c][2] = 0;
+        for (int c = 0; c < NF; ++c) f[k][c] = 0;
       T pq = 0;
 #pragma unroll
       for (int t = 0; t < 6; ++t) {
@@ -282,7 +350,7 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
         T p[6][VL];
 #pragma unroll
         for (int s = 0; s < 6; ++s) vloadn<T, VL>(p[s], slot(t, s));
-        if (use_old) {
+        if (!EDGES && use_old) {
 #pragma unroll
           for (int s = 0; s < 6; ++s) {
             T v[VL];
@@ -310,7 +378,7 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
 #pragma unroll
             for (int s = 0; s < 6; ++s) sg[s] = s < 3 ? tr + me * p[s][k] : me * p[s][k];
 #pragma unroll
-            for (int s = 0; s < 6; ++s) pq += p[s][k] * sg[s];
+            for (int s = 0; s < 6; ++s) pq += EDGES ? (T)0 : p[s][k] * sg[s];
           } else {
 #pragma unroll
             for (int s = 0; s < 6; ++s) sg[s] = p[s][k];
@@ -318,10 +386,11 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
           T S[3][3];
           S[0][0] = sg[0]; S[1][1] = sg[1]; S[2][2] = sg[2];
           S[1][2] = S[2][1] = r2 * sg[3]; S[0][2] = S[2][0] = r2 * sg[4]; S[0][1] = S[1][0] = r2 * sg[5];
-          tet_forces<T>(t, S, ih, f[k]);
+          if constexpr (EDGES) tet_edges<T>(t, S, reinterpret_cast<T(*)[4][3]>(f[k]));
+          else tet_forces<T>(t, S, ih, reinterpret_cast<T(*)[3]>(f[k]));
         }
       }
-      if (own) acc.add(pq);
+      if (!EDGES && own) acc.add(pq);
       T pv[2][2][3];
       pass_on(yy, f[VL - 1], pv);
 #pragma unroll
@@ -434,17 +503,17 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
 #pragma unroll
           for (int j = 0; j < 3; ++j) uc[c][j] = ((c >> 1) & 1 ? hi : lo)[c >> 2][k + (c & 1)][j];
         pq += voxel_forces_3d<T>(uc, e[k], a.lam, a.mu2, ih, f);
-        if (k == VL - 1) pass_on(yy, f, pv1);
+        if (k == VL - 1) pass_on(yy, f[0], pv1);
         if (k < VL - 1) {   // finish column k + 1
           T g[8][3], pr[2][2][3];
-          right(f, pr);
+          right(f[0], pr);
 #pragma unroll
           for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
             for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
               for (int j = 0; j < 3; ++j) g[2 * dy + 4 * dz][j] = keep[dy][dz][j];
-          put_column(yy, k + 1, g, pr);
+          put_column(yy, k + 1, g[0], pr);
         }
 #pragma unroll
         for (int dy = 0; dy < 2; ++dy)
@@ -453,7 +522,7 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
 #pragma unroll
             for (int j = 0; j < 3; ++j) keep[dy][dz][j] = f[2 * dy + 4 * dz][j];
       }
-      put_column(yy, 0, f, pv1);
+      put_column(yy, 0, f[0], pv1);
       if (own) acc.add(pq);
 #pragma unroll
       for (int k = 0; k < VL; ++k) e[k] = en[k];
@@ -468,19 +537,41 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
 
   __syncthreads();
   if constexpr (TPR > 32) {
-    for (int i = threadIdx.x; i < 3 * TY * NW; i += NT) {
+    for (int i = threadIdx.x; i < (EDGES ? 5 : 3) * TY * NW; i += NT) {
       const int w = i % NW, yy = (i / NW) % TY, j = i / (NW * TY);
       const int q = yy / TYL, lr = yy % TYL + 1;   // the lane's rows: 0 is the row below its first
       const int wp = (w + NW - 1) % NW;
-      const T* r0 = edge + ((q * (TYL + 1) + lr) * NW + wp) * 12 + j;        // dy = 0 of row yy
-      const T* r1 = edge + ((q * (TYL + 1) + lr - 1) * NW + wp) * 12 + 6 + j;   // dy = 1 of row yy - 1
-      C* p = buf + (j * TY + yy) * LD + 32 * VL * w;
-      *p = mkc<T>(p->x + r0[0] + r1[0], p->y + r0[3] + r1[3]);
+      const T* r0 = edge + ((q * (TYL + 1) + lr) * NW + wp) * 12;        // dy = 0 of row yy
+      const T* r1 = edge + ((q * (TYL + 1) + lr - 1) * NW + wp) * 12;    // dy = 1 of row yy - 1
+      if constexpr (EDGES) {   // j < 3: s_y; 3, 4: the two rows of s_z
+        C* p = buf + ((3 + j) * TY + yy) * LD + 32 * VL * w;
+        if (j < 3) *p = mkc<T>(p->x + r0[j], p->y + r0[3 + j]);
+        else if (j == 3) *p = mkc<T>(p->x + r0[6] + r1[9], p->y + r0[7] + r1[10]);
+        else p->x += r0[8] + r1[11];
+      } else {
+        C* p = buf + (j * TY + yy) * LD + 32 * VL * w;
+        *p = mkc<T>(p->x + r0[j] + r1[6 + j], p->y + r0[3 + j] + r1[9 + j]);
+      }
     }
     __syncthreads();
   }
-  smem_fft<T, NX, 3 * TY, LD, NT, -1>(buf, a.tw[0]);
-  {
+  smem_fft<T, NX, CR * TY, LD, NT, -1>(buf, a.tw[0]);
+  if constexpr (EDGES) {
+    const int64_t cs = (int64_t)KX * nz * ny;
+    C* p0 = a.spec + (int64_t)l * a.m * cs + (int64_t)z * ny + y0;
+    C* p1 = a.spec + (int64_t)l * a.m * cs + (int64_t)((z + 1) & (nz - 1)) * ny + y0;
+    for (int i = threadIdx.x; i < 8 * KX * TY; i += NT) {
+      const int yy = i % TY, k = (i / TY) % KX, j = i / (TY * KX);
+      const C* row = buf + (j * TY + yy) * LD;
+      const C A = row[k], B = cconj(row[(NX - k) & (NX - 1)]);
+      const C d = csub(A, B);
+      const int64_t o = (int64_t)k * nz * ny + yy;
+      p0[(j == 7 ? 8 : j) * cs + o] = cscale(cadd(A, B), (T)0.5);
+      const C im = mkc<T>((T)0.5 * d.y, (T)-0.5 * d.x);
+      if (j < 6) p1[(9 + j) * cs + o] = im;
+      else if (j == 6) p0[7 * cs + o] = im;
+    }
+  } else {
     C* s0 = a.spec + ((int64_t)l * a.m * KX * nz + z) * ny + y0;
     C* s1 = a.spec + ((((int64_t)l * a.m + 3) * KX) * nz + ((z + 1) & (nz - 1))) * ny + y0;
     for (int i = threadIdx.x; i < 3 * KX * TY; i += NT) {
@@ -521,8 +612,26 @@ __device__ __forceinline__ void pixel_forces(const T S[2][3], T ihx, T ihy, T f[
   f[3][1] = ihx * S[1][2] + ihy * S[1][1];
 }
 
-template <typename T, int NX, int TY, int LN> constexpr size_t force_2d_smem() {
-  return sizeof(cplx<T>) * TY * force_ld<T, NX, TY>() + sizeof(T) * 4 * (NX > 32 ? (TY + LN) * (NX / 32) : 0);
+// The same pixel's stresses at the edges they act on, f[c][2 a + j] = s_aj of
+// corner c: element 0 has its x and y edges at the pixel's own node, element 1
+// the x edge at corner dy = 1 and the y edge at corner dx = 1.  S[q][a][j].
+template <typename T> __device__ __forceinline__ void pixel_edges(const T S[2][2][2], T f[4][4]) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    f[0][j] = S[0][0][j];
+    f[0][2 + j] = S[0][1][j];
+    f[1][j] = 0;
+    f[1][2 + j] = S[1][1][j];
+    f[2][j] = S[1][0][j];
+    f[2][2 + j] = f[3][j] = f[3][2 + j] = 0;
+  }
+}
+
+// Real rows of a node row: the forces f_j or the edge sums s_aj.
+template <int SRC> __host__ __device__ constexpr int force_comps2() { return SRC == S_EDGE ? 4 : 2; }
+template <typename T, int NX, int TY, int LN, int NC> constexpr size_t force_2d_smem() {
+  return sizeof(cplx<T>) * (NC / 2) * TY * force_ld<T, NX, TY>() +
+         sizeof(T) * 2 * NC * (NX > 32 ? (TY + LN) * (NX / 32) : 0);
 }
 
 // The same for a field of first Piola-Kirchhoff stresses P[q][i][a] (finite
@@ -551,8 +660,10 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
   constexpr int NW = NX > 32 ? NX / 32 : 1;
   static_assert((NT % NX == 0 || NX % NT == 0) && TY % LN == 0, "threads cover whole rows");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);             // [TY][LD]: f_0 + i f_1
-  T* edge = reinterpret_cast<T*>(buf + TY * LD);       // [LN][TYL + 1][NW][4], NX > 32
+  constexpr int NC = force_comps2<SRC>();
+  constexpr bool EDGES = NC == 4;
+  C* buf = reinterpret_cast<C*>(smem_raw);             // [NC / 2][TY][LD]: f_0 + i f_1, or s_a0 + i s_a1
+  T* edge = reinterpret_cast<T*>(buf + NC / 2 * TY * LD);   // [LN][TYL + 1][NW][2 NC], NX > 32
   __shared__ double red[NT / 32];
   __shared__ T cols[NT];
   __shared__ int flag;
@@ -564,7 +675,7 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
   if (a.cgphase && cg->status != ST_RUN) return;
   const int64_t N = a.N;
   const int ln = LN > 1 ? threadIdx.x / NX : 0, lane = threadIdx.x & 31;
-  const bool cgm = a.amode == A_CG;
+  const bool cgm = !EDGES && a.amode == A_CG;
   const bool use_old = cgm && cg->it > 0;
   const T beta = cgm ? cg_beta<T>(cg) : (T)0, alpha_prev = cgm ? cg_alpha<T>(cg) : (T)0;
   const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
@@ -574,17 +685,23 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
   for (int cx = 0; cx < CPT; ++cx) {
     const int x = LN > 1 ? threadIdx.x % NX : cx * NT + threadIdx.x;
     const T* Ep = a.E + (int64_t)(l / a.lcs) * N + x;
-    T carry[2] = {0, 0};
-    auto node_row = [&](int yy, const T f[4][2], bool own) {
-      T s[2][2];   // [dy][j]
+    T carry[NC];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) carry[j] = 0;
+    auto node_row = [&](int yy, const T f[4][NC], bool own) {
+      T s[2][NC];   // [dy][j]
 #pragma unroll
       for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
+        for (int j = 0; j < NC; ++j) {
+          if (EDGES && (dy == 1 || j < 2)) {   // nothing at dx = 1 (see pixel_edges)
+            s[dy][j] = f[2 * dy][j];
+            continue;
+          }
           const T u = f[1 + 2 * dy][j];
           T p = from_prev<NX>(u);
           if constexpr (NX > 32) {
-            if (lane == 31) edge[((ln * (TYL + 1) + yy + 1 - ln * TYL) * NW + x / 32) * 4 + dy * 2 + j] = u;
+            if (lane == 31) edge[((ln * (TYL + 1) + yy + 1 - ln * TYL) * NW + x / 32) * 2 * NC + dy * NC + j] = u;
             if (lane == 0) p = 0;
           } else if constexpr (NX == 32) {
             const T w = __shfl_sync(0xffffffffu, u, 31);
@@ -592,9 +709,13 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
           }
           s[dy][j] = f[2 * dy][j] + p;
         }
-      if (own) buf[yy * LD + x] = mkc<T>(s[0][0] + carry[0], s[0][1] + carry[1]);
-      carry[0] = s[1][0];
-      carry[1] = s[1][1];
+      if (own) {
+#pragma unroll
+        for (int c = 0; c < NC / 2; ++c)
+          buf[(c * TY + yy) * LD + x] = mkc<T>(s[0][2 * c] + carry[2 * c], s[0][2 * c + 1] + carry[2 * c + 1]);
+      }
+#pragma unroll
+      for (int j = 0; j < NC; ++j) carry[j] = s[1][j];
     };
     if constexpr (SRC == S_GRAD) {
       const T* __restrict__ in = a.in + (int64_t)l * a.m * N + x;
@@ -606,7 +727,7 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
         pixel_divergence<T>(P, ihx, ihy, f);
         node_row(yy, f, yy >= ln * TYL);
       }
-    } else if constexpr (SRC == S_STRAIN) {
+    } else if constexpr (SRC == S_STRAIN || SRC == S_EDGE) {
       const int64_t base = (int64_t)l * a.m * N + x;
       const T* __restrict__ rp = (cgm ? a.r : a.in) + base;
       const T* __restrict__ po = a.pold + base;
@@ -648,7 +769,7 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
             for (int s = 0; s < 6; ++s) xp[o + s * N] = xs[s];
           }
         }
-        T S[2][3], f[4][2], pq = 0;
+        T S[2][3], f[4][NC], pq = 0;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           if (mat) {
@@ -662,8 +783,13 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
             S[q][0] = p[3 * q]; S[q][1] = p[3 * q + 1]; S[q][2] = r2 * p[3 * q + 2];
           }
         }
-        pixel_forces<T>(S, ihx, ihy, f);
-        if (own) acc.add(pq);
+        if constexpr (EDGES) {
+          const T G[2][2][2] = {{{S[0][0], S[0][2]}, {S[0][2], S[0][1]}}, {{S[1][0], S[1][2]}, {S[1][2], S[1][1]}}};
+          pixel_edges<T>(G, f);
+        } else {
+          pixel_forces<T>(S, ihx, ihy, f);
+          if (own) acc.add(pq);
+        }
         node_row(yy, f, own);
       }
     } else {
@@ -756,27 +882,28 @@ __global__ void __launch_bounds__(NT, MB) force_2d(PassArgs<T> a) {
   if constexpr (NX > 32) {
     for (int i = threadIdx.x; i < TY * NW; i += NT) {
       const int w = i % NW, yy = i / NW, q = yy / TYL, lr = yy % TYL + 1, wp = (w + NW - 1) % NW;
-      const T* r0 = edge + ((q * (TYL + 1) + lr) * NW + wp) * 4;
-      const T* r1 = edge + ((q * (TYL + 1) + lr - 1) * NW + wp) * 4 + 2;
-      C* p = buf + yy * LD + 32 * w;
-      *p = mkc<T>(p->x + r0[0] + r1[0], p->y + r0[1] + r1[1]);
+      const T* r0 = edge + ((q * (TYL + 1) + lr) * NW + wp) * 2 * NC;            // dy = 0 of row yy
+      const T* r1 = edge + ((q * (TYL + 1) + lr - 1) * NW + wp) * 2 * NC + NC;   // dy = 1 of row yy - 1
+      C* p = buf + ((EDGES ? TY : 0) + yy) * LD + 32 * w;                        // edge sums: s_y only
+      if constexpr (EDGES) *p = mkc<T>(p->x + r0[2], p->y + r0[3]);
+      else *p = mkc<T>(p->x + r0[0] + r1[0], p->y + r0[1] + r1[1]);
     }
     __syncthreads();
   }
-  if constexpr (sizeof(T) == 4 && (NX == 512 || NX == 1024) && NT == 2 * FftSplit<NX>::N1 * TY)
+  if constexpr (!EDGES && sizeof(T) == 4 && (NX == 512 || NX == 1024) && NT == 2 * FftSplit<NX>::N1 * TY)
     smem_fft_pair<T, NX, TY, LD, NT, -1>(buf, a.tw[0]);
   else
-    smem_fft<T, NX, TY, LD, NT, -1>(buf, a.tw[0]);
+    smem_fft<T, NX, NC / 2 * TY, LD, NT, -1>(buf, a.tw[0]);
   {
     C* s0 = a.spec + (int64_t)l * a.m * KX * ny + y0;
-    C* s1 = s0 + (int64_t)KX * ny;
-    for (int i = threadIdx.x; i < KX * TY; i += NT) {
-      const int yy = i % TY, k = i / TY;
-      const C* row = buf + yy * LD;
+    for (int i = threadIdx.x; i < NC / 2 * KX * TY; i += NT) {
+      const int yy = i % TY, k = (i / TY) % KX, c = i / (TY * KX);
+      const C* row = buf + (c * TY + yy) * LD;
       const C A = row[k], B = cconj(row[(NX - k) & (NX - 1)]);
       const C d = csub(A, B);
-      s0[(int64_t)k * ny + yy] = cscale(cadd(A, B), (T)0.5);
-      s1[(int64_t)k * ny + yy] = mkc<T>((T)0.5 * d.y, (T)-0.5 * d.x);
+      C* o = s0 + ((int64_t)2 * c * KX + k) * ny + yy;
+      o[0] = cscale(cadd(A, B), (T)0.5);
+      o[(int64_t)KX * ny] = mkc<T>((T)0.5 * d.y, (T)-0.5 * d.x);
     }
   }
   if (cgm) {
@@ -823,6 +950,9 @@ cudaError_t launch_force_3d_n(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int VS = force_cols3<T, NX>();
   constexpr int NT = force_threads3<NX, VS>();
   if (a.force == 2) return launch_force_3d_t<T, NX, TY, NT, VS, S_NODAL>(a, s);
+  // edge sums: 8 complex rows per row of the tile, so fewer rows (256 x 256 x 64,
+  // FP32: 4 rows 267 us, 8 rows 378; two columns per thread 289)
+  if (a.force == 4) return launch_force_3d_t<T, NX, NX >= 128 ? 4 : 8, force_threads3<NX, 1>(), 1, S_EDGE>(a, s);
   if constexpr (NX >= 64) {
     if (a.var_a == 1) return launch_force_3d_t<T, NX, TY / 2, NT, VS, S_STRAIN>(a, s);
     if constexpr (NX >= 128 && sizeof(T) == 4) {
@@ -842,7 +972,8 @@ template <typename T> cudaError_t launch_force_3d(const PassArgs<T>& a, cudaStre
 template <typename T, int NX, int TY, int NT, int SRC>
 cudaError_t launch_force_2d_t(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int MB = sizeof(T) == 8 ? 1 : NT <= 64 ? 8 : NT <= 128 ? 4 : NT <= 512 ? 2 : 1;
-  constexpr size_t sm = force_2d_smem<T, NX, TY, (NT > NX ? NT / NX : 1)>();
+  constexpr size_t sm = force_2d_smem<T, NX, TY, (NT > NX ? NT / NX : 1), force_comps2<SRC>()>();
+  static_assert(sm <= 222 * 1024, "shared memory of the tile");
   auto k = force_2d<T, NX, TY, NT, MB, SRC>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
@@ -859,11 +990,14 @@ template <typename T, int NX, int TY, int SRC> cudaError_t launch_force_2d_r(con
 // Default rows: 8 (FP64: 4) where that gives every SM a block, else half, else
 // a quarter.  A tile computes one row more than it owns, so fewer rows mean
 // more work, but on small grids an idle SM costs more (FP64, 512 x 256, one
-// load case: 64 blocks of 4 rows against 128 of 2).
+// load case: 64 blocks of 4 rows against 128 of 2).  The edge sources have two
+// complex rows per node row: at most half the rows.
 template <typename T, int NX, int SRC> cudaError_t launch_force_2d_auto(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int TY = sizeof(T) == 4 ? 8 : 4;
   const int64_t sms = device_sm_count(), rows = (int64_t)a.n[1] * a.L;
-  if (rows / TY >= sms) return launch_force_2d_r<T, NX, TY, SRC>(a, s);
+  if constexpr (force_comps2<SRC>() == 2) {
+    if (rows / TY >= sms) return launch_force_2d_r<T, NX, TY, SRC>(a, s);
+  }
   if (TY == 4 || rows / (TY / 2) < sms) return launch_force_2d_r<T, NX, 2, SRC>(a, s);
   return launch_force_2d_r<T, NX, TY / 2, SRC>(a, s);
 }
@@ -874,6 +1008,7 @@ template <typename T, int NX>
 cudaError_t launch_force_2d_n(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int TY = sizeof(T) == 4 ? 8 : 4;
   if (a.force == 2) return launch_force_2d_auto<T, NX, S_NODAL>(a, s);
+  if (a.force == 4) return launch_force_2d_auto<T, NX, S_EDGE>(a, s);
   if constexpr (sizeof(T) == 8) {
     if (a.force == 3) return launch_force_2d_auto<T, NX, S_GRAD>(a, s);
   }

@@ -328,6 +328,14 @@ template <typename T> void set_force(const rve_s* h, PassArgs<T>& a, int q) {
   a.pnew = P[q];
 }
 
+// The pass arguments of a single operator application: edge sums in, edge
+// differences out.
+template <typename T> void set_edges(const rve_s* h, PassArgs<T>& a) {
+  a.force = 4;
+  a.pair = h->dim == 3 ? 2 : 0;
+  a.grads = 1;
+}
+
 template <typename T> PassArgs<T> pass_args(const rve_s* h, int L, double* u, const double* emac) {
   PassArgs<T> a;
   std::memset(&a, 0, sizeof(a));
@@ -1881,16 +1889,16 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
   if (!din) CK(cudaMemcpyAsync(h->fbuf, p, bytes, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
   if (h->tsize == 4) {
     PassArgs<float> a = pass_args<float>(h, 1, h->u, h->emac_d);
-    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = P_G; a.emode = E_OUT; a.grads = 1;
-    set_force(h, a, 0);
+    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = P_G; a.emode = E_OUT;
+    set_edges(h, a);
     a.cg = h->cg_op;
     a.pdl = !h->timing;
     a.in = (const float*)in; a.out = (float*)out;
     CK(apply_passes<float>(h, a));
   } else {
     PassArgs<double> a = pass_args<double>(h, 1, h->u, h->emac_d);
-    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = h->finite ? P_FINITE : P_G; a.emode = E_OUT; a.grads = 1;
-    if (force_pass(h, 0)) set_force(h, a, 0);
+    a.amode = apply_material ? A_FIELD : A_BARE; a.pmode = h->finite ? P_FINITE : P_G; a.emode = E_OUT;
+    if (force_pass(h, 0)) set_edges(h, a);
     a.cg = h->cg_op;
     a.in = (const double*)in; a.out = (double*)out;
     CK(apply_passes<double>(h, a));

@@ -72,17 +72,18 @@ template <typename T> struct PassArgs {
                      // TMA unit to prefetch into L2, 0 = none
   int deriv;         // Deriv
   int force;         // first pass of the finite elements: 1 strain fields, 2 nodal fields, 3 stress
-                     // field of finite strain (2D) (pass_force.cuh)
+                     // field of finite strain (2D), 4 edge sums of a strain field (pass_force.cuh)
   const T* pold;     // previous and new search direction of the force pass (different arrays)
   T* pnew;
   const T* rho;      // nodal state: residual and iterate of the force pass
   T* xi;
-  int pair;          // 3D: the spectrum holds F0 and F1 (components j and 3 + j), pass B adds them
+  int pair;          // 3D: the spectrum holds the sums over elements in two parts, pass B adds them: 1 nodal
+                     // forces (components j and 3 + j), 2 edge sums of x and y (i and 9 + i, i < 6)
   int pdl;           // launch with the programmatic-serialization attribute (see pdl_begin)
   int resid;         // nodal state: the pass that loads the x spectra keeps the residual force R(k_x, ..) there
                      // (components 2 D .. 3 D - 1 in 3D, D .. 2 D - 1 in 2D): 1 R = -f, 2 R -= alpha f
   int dot;           // nodal state: pass C sums <rho, R> = |B rho|^2 -> beta (2: start of an inner solve)
-  int grads;         // finite elements: passes C, D and E carry the D^2 edge differences of w instead of its D
+  int grads;         // finite elements: the passes carry D^2 edge sums and edge differences of w instead of D
                      // components (see pass_c_2d_fe), for results that leave the library as they are
 };
 
