@@ -575,13 +575,21 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pas
 }
 
 // Last pass of the finite elements: from w(k_x, z, y) of the three nodal
-// components (pass D) the inverse x FFT of TY + 1 rows of planes z and z + 1
-// (the two planes share one complex transform), then in real space the strains
-// q = B w of the six tetrahedra of every voxel of the TY rows and the update of
-// all 36 components.  Transforming w needs 3 (TY + 1) transforms where the
-// components need 18 TY, and reads 1/12 of the spectrum; what is left is the r
-// traffic (read and written once), which bounds it.  W = 9: the spectrum holds
-// the edge differences of w instead (see pass_c_2d_fe).
+// components (pass D) the inverse x FFT of TY + 1 rows of planes z and z + 1,
+// then in real space the strains q = B w of the six tetrahedra of every voxel of
+// the TY rows and the update of all 36 components.  Transforming w needs 3 TY + 4
+// transforms where the components need 18 TY, and reads 1/12 of the spectrum;
+// what is left is the r traffic (read and written once), which bounds it.
+// Two real rows share a complex transform: w_0 and w_1 of a row, and w_2 of rows
+// 2 i and 2 i + 1.  Every node's values then come from the same transforms in
+// all blocks that use them (a tile's last row is the next one's first, plane z +
+// 1 is the next block's plane z), and q is the strain of one nodal field.
+// Pairing planes z and z + 1 (3 TY + 3 transforms) rounds a node's values
+// differently in the two blocks: the differences of that are no strain field, CG
+// cannot remove them from r, and on flat voxels (1 : 1000, FP32) it did not
+// converge.
+// W = 9: the spectrum holds the edge differences of w instead (see
+// pass_c_2d_fe); plane z in the real, plane z + 1 in the imaginary part.
 // grid (n_y/TY, n_z, L).
 // In FP32 the r loads of the update go through a ring of the thread's own
 // shared-memory slots (cp.async, six tetrahedra deep): issued before the
@@ -592,6 +600,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pas
 template <typename T, int NT, int W> __host__ __device__ constexpr bool e_fe_ring() {
   return sizeof(T) == 4 && W == 3 && NT <= 256;   // else it does not fit beside the rows
 }
+template <int W, int TY> __host__ __device__ constexpr int e_fe_rows() { return W == 3 ? 3 * TY + 4 : W * (TY + 1); }
 template <int NX> __host__ __device__ constexpr int e_fe_ld() {
   // 9 (mod 16): the TY + 1 rows that consecutive lanes unpack at one column
   // fall on different banks
@@ -602,10 +611,12 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   using C = cplx<T>;
   constexpr int KX = NX / 2 + 1;
   constexpr int NR = TY + 1;
-  constexpr int R = W * NR;
+  constexpr int NP = TY / 2 + 1;   // row pairs of w_2
+  constexpr int R = e_fe_rows<W, TY>();
+  static_assert(W == 9 || R == 2 * (NR + NP), "rows of the two planes");
   constexpr int LD = e_fe_ld<NX>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NR][LD]
+  C* buf = reinterpret_cast<C*>(smem_raw);  // W = 3: [2][NR] rows (w_0, w_1), [2][NP] pairs of w_2; 9: [W][NR]
   __shared__ double red[NT / 32];
   __shared__ T cols[NT];
   __shared__ int flag;
@@ -640,29 +651,47 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   {
     const C* pa = a.spec + ((int64_t)l * a.m * KX * nz + z) * ny;
     const C* pb = a.spec + ((int64_t)l * a.m * KX * nz + ((z + 1) & (nz - 1))) * ny;
-    constexpr int TOT = W * KX * NR, UB = 4;
-    for (int i0 = threadIdx.x; i0 < TOT; i0 += UB * NT) {
-      C xa[UB], xb[UB];
+    const int64_t cs = (int64_t)KX * nz * ny;
+    auto pack = [&](C* row, int k, C va, C vb) {
+      if (k == 0 || k == NX / 2) { va.y = 0; vb.y = 0; }  // C2R ignores these imaginary parts
+      row[k] = mkc<T>(va.x - vb.y, va.y + vb.x);                                  // X_a + i X_b
+      if (k > 0 && k < NX / 2) row[NX - k] = mkc<T>(va.x + vb.y, vb.x - va.y);    // conj(X_a) + i conj(X_b)
+    };
+    // items i -> (row b of NB rows a plane or component, k_x, plane or component p),
+    // loaded UB at a time
+    constexpr int UB = 4;
+    auto unpack = [&](auto nb, int np, C* dst, auto&& load) {
+      constexpr int NB = decltype(nb)::value;
+      const int tot = np * KX * NB;
+      for (int i0 = threadIdx.x; i0 < tot; i0 += UB * NT) {
+        C v[UB][2];
 #pragma unroll
-      for (int u = 0; u < UB; ++u) {
-        const int i = i0 + u * NT;
-        if (i < TOT) {
-          const int64_t o = (int64_t)(i / NR) * nz * ny + ((y0 + i % NR) & (ny - 1));   // i / NR = j KX + k_x
-          xa[u] = pa[o]; xb[u] = pb[o];
+        for (int u = 0; u < UB; ++u) {
+          const int i = i0 + u * NT;
+          if (i < tot) load(v[u], i % NB, (i / NB) % KX, i / (NB * KX));
+        }
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+          const int i = i0 + u * NT;
+          if (i < tot) pack(dst + ((i / (NB * KX)) * NB + i % NB) * LD, (i / NB) % KX, v[u][0], v[u][1]);
         }
       }
-#pragma unroll
-      for (int u = 0; u < UB; ++u) {
-        const int i = i0 + u * NT;
-        if (i < TOT) {
-          const int k = (i / NR) % KX, j = i / (NR * KX);
-          C va = xa[u], vb = xb[u];
-          if (k == 0 || k == NX / 2) { va.y = 0; vb.y = 0; }  // C2R ignores these imaginary parts
-          C* row = buf + (j * NR + i % NR) * LD;
-          row[k] = mkc<T>(va.x - vb.y, va.y + vb.x);                                  // X_a + i X_b
-          if (k > 0 && k < NX / 2) row[NX - k] = mkc<T>(va.x + vb.y, vb.x - va.y);    // conj(X_a) + i conj(X_b)
-        }
-      }
+    };
+    if constexpr (W == 3) {
+      unpack(std::integral_constant<int, NR>{}, 2, buf, [&](C* v, int y, int k, int p) {
+        const C* s = (p ? pb : pa) + (int64_t)k * nz * ny + ((y0 + y) & (ny - 1));
+        v[0] = s[0];
+        v[1] = s[cs];
+      });
+      unpack(std::integral_constant<int, NP>{}, 2, buf + 2 * NR * LD, [&](C* v, int pr, int k, int p) {
+        cload2<T>(v, (p ? pb : pa) + 2 * cs + (int64_t)k * nz * ny + ((y0 + 2 * pr) & (ny - 1)));
+      });
+    } else {
+      unpack(std::integral_constant<int, NR>{}, W, buf, [&](C* v, int y, int k, int j) {
+        const int64_t o = j * cs + (int64_t)k * nz * ny + ((y0 + y) & (ny - 1));
+        v[0] = pa[o];
+        v[1] = pb[o];
+      });
     }
   }
   __syncthreads();
@@ -674,17 +703,27 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   for (int i = threadIdx.x; i < UNITS; i += NT) {
     const int yy = i / (NX / VL), x = (i % (NX / VL)) * VL;
     const int64_t v0 = vox0 + (int64_t)yy * NX + x;
-    // node values at (x + q, y + dy): planes z (.x) and z + 1 (.y)
-    C n[W][2][VL + 1];
+    // node values at (x + q, y + dy), planes z and z + 1
+    constexpr int NV = W == 3 ? 2 : W;
+    C n[NV][2][VL + 1];         // W = 3: [dz] (w_0, w_1); 9: [component] (z, z + 1)
+    T n2[2][2][VL + 1];         // W = 3: w_2, [dz]
 #pragma unroll
-    for (int j = 0; j < W; ++j)
+    for (int j = 0; j < NV; ++j)
 #pragma unroll
       for (int dy = 0; dy < 2; ++dy)
 #pragma unroll
-        for (int q = 0; q <= VL; ++q) n[j][dy][q] = buf[(j * NR + yy + dy) * LD + ((x + q) & (NX - 1))];
+        for (int q = 0; q <= VL; ++q) {
+          const int xq = (x + q) & (NX - 1);
+          n[j][dy][q] = buf[(j * NR + yy + dy) * LD + xq];
+          if constexpr (W == 3) {
+            const C* w = buf + (2 * NR + j * NP + (yy + dy) / 2) * LD + xq;
+            n2[j][dy][q] = ((yy + dy) & 1) ? w->y : w->x;
+          }
+        }
     auto corner = [&](int c, int j, int q) -> T {   // corner c = dx + 2 dy + 4 dz of voxel x + q
-      const C v = n[j][(c >> 1) & 1][q + (c & 1)];
-      return (c & 4) ? v.y : v.x;
+      const int dx = c & 1, dy = (c >> 1) & 1, dz = (c >> 2) & 1;
+      if constexpr (W == 3) return j == 0 ? n[dz][dy][q + dx].x : j == 1 ? n[dz][dy][q + dx].y : n2[dz][dy][q + dx];
+      else return dz ? n[j][dy][q + dx].y : n[j][dy][q + dx].x;
     };
     T vs = 0;
 #pragma unroll
@@ -782,7 +821,7 @@ cudaError_t launch_e_3d_t(const PassArgs<T>& a, cudaStream_t s) {
 }
 template <typename T, int NX, int TY, int W = 3>
 cudaError_t launch_e_3d_fe_t(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int R = W * (TY + 1);
+  constexpr int R = e_fe_rows<W, TY>();
   constexpr int NT = fft_threads<NX, R>();
   constexpr size_t sm = sizeof(cplx<T>) * R * e_fe_ld<NX>() + (e_fe_ring<T, NT, W>() ? sizeof(T) * 36 * (NX >= 256 ? 2 : 1) * NT : 0);
     constexpr int MB = sizeof(T) == 8 ? 1 : W == 9 ? (NT <= 448 ? 2 : 1) : NT <= 256 ? (NX >= 256 ? 2 : 4) : NT <= 448 ? 2 : 1;
