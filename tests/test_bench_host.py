@@ -126,3 +126,24 @@ def test_iteration_bytes_per_form():
     mb = bench.model_bytes(3, n, 4, 1, "nodal")
     b2, note2 = bench.iteration_bytes(3, n, 4, "nodal", mb)
     assert b2 == sum(mb.values()) and "nodal" in note2 and b2 < 0.2 * b
+
+
+def test_pass_bytes():
+    """Counted by hand: real streams of N values, spectra of (n_x/2 + 1) n_y n_z
+    complex ones.  The first pass reads r, p_old, x (nodal: rho, pi_old, xi) and
+    E, writes p and x (pi, xi) and the force spectra."""
+    n, s = (64, 32, 16), 4
+    N, spec = 32768, 33 * 512 * 2 * s
+    assert bench.pass_bytes(3, n, s) == {
+        "pass_a": 181 * N * s + 6 * spec, "pass_b": 9 * spec, "pass_c": 6 * spec, "pass_d": 6 * spec,
+        "pass_e": 72 * N * s + 3 * spec}
+    assert bench.pass_bytes(3, n, s, "nodal") == {
+        "force_stencil": 16 * N * s + 6 * spec, "pass_b": 15 * spec, "pass_c": 6 * spec, "pass_d": 6 * spec,
+        "pass_e": 3 * N * s + 3 * spec}
+    pipe = bench.pass_bytes(3, n, s, pipelined=True)
+    assert pipe["pass_a"] == 181 * N * s + 36 * spec and pipe["pass_b"] == 39 * spec
+    N, spec = 2048, 33 * 32 * 2 * s
+    assert bench.pass_bytes(2, n[:2], s, "factored") == {
+        "force_stencil": 31 * N * s + 2 * spec, "pass_c": 4 * spec, "pass_e": 12 * N * s + 2 * spec}
+    assert bench.pass_bytes(2, n[:2], s, "nodal") == {
+        "force_stencil": 11 * N * s + 2 * spec, "pass_c": 8 * spec, "pass_e": 2 * N * s + 2 * spec}
