@@ -643,8 +643,10 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
 
 // Update of VL consecutive values of one strain component by q (modes of the
 // last pass): CG r -= alpha q, INIT r = -q and x = 0, OUT out = q.  rv holds r
-// in CG mode.  Returns the share of <r, r>.
-template <typename T, int VL>
+// in CG mode.  ANY: out may have any element alignment (a separate instance: the
+// branch in that of the CG iterations cost 3 us of 52 at 1024^2).  Returns the
+// share of <r, r>.
+template <typename T, int VL, bool ANY = false>
 __device__ __forceinline__ T strain_update(const PassArgs<T>& a, int64_t idx, T* rv, const T* q, T alpha) {
   T s = 0;
   if (a.emode == E_CG) {
@@ -657,7 +659,7 @@ __device__ __forceinline__ T strain_update(const PassArgs<T>& a, int64_t idx, T*
     for (int i = 0; i < VL; ++i) { n[i] = -q[i]; z[i] = 0; s += q[i] * q[i]; }
     vstoren<T, VL>(a.r + idx, n);
     vstoren<T, VL>(a.x + idx, z);
-  } else if (VL > 1 && (reinterpret_cast<uintptr_t>(a.out) & 15)) {
+  } else if (ANY && VL > 1 && (reinterpret_cast<uintptr_t>(a.out) & 15)) {
     // a caller's own field (the entry point without a handle) of any element
     // alignment; the handle's and the other fields are 16-byte aligned
 #pragma unroll
@@ -754,7 +756,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
     }
     T s = 0;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) s += strain_update<T, VL>(a, v0 + c * a.N, rv[c], q[c], alpha);
+    for (int c = 0; c < NC; ++c) s += strain_update<T, VL, W == 4>(a, v0 + c * a.N, rv[c], q[c], alpha);
     if (GRAD && a.emode == E_INIT) {   // the padding component
       T z[VL];
 #pragma unroll
