@@ -678,16 +678,20 @@ __device__ __forceinline__ T strain_update(const PassArgs<T>& a, int64_t idx, T*
 // the strains needs TY + 2 row pairs where the components need 3 TY, and reads
 // a third of the spectrum.  Bound by the r traffic (read and write, 16-byte
 // accesses).  W = 4: the spectrum holds the edge differences of w instead (see
-// pass_c_2d_fe).  grid (n_y/TY, L).
+// pass_c_2d_fe).  TY = 1 (few rows): w_0 and w_1 of a row share a transform, two
+// rows, where a pair of rows beside the tile's would be half unused.
+// grid (n_y/TY, L).
 template <typename T, int NX, int TY, int NT, int W, bool GRAD = false>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pass_e_2d_fe(PassArgs<T> a) {
   using C = cplx<T>;
+  constexpr bool ROWS = TY == 1;
+  static_assert(!ROWS || W == 2, "single rows: the two components of w");
   constexpr int NPR = TY / 2 + 1;
   constexpr int KX = NX / 2 + 1;
   constexpr int LD = ae_ld<NX>();
   constexpr int VL = sizeof(T) == 4 ? 4 : 1;   // FP64: more, shorter work items
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NPR][LD]
+  C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NPR][LD]; ROWS: [2 rows][LD]
   __shared__ double red[NT / 32];
   __shared__ T cols[NT];
   __shared__ int flag;
@@ -697,9 +701,22 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   pdl_begin();
   if (!cg->active) return;
   if (a.cgphase && cg->status != ST_RUN) return;
-  pass_e_unpack<T, NX, 2 * NPR, NT, LD>(buf, a.spec + (int64_t)l * a.m * KX * ny, W, (int64_t)KX * ny, ny, y0, ny - 1);
+  const C* spec = a.spec + (int64_t)l * a.m * KX * ny;
+  if constexpr (ROWS) {
+    for (int i = threadIdx.x; i < 2 * KX; i += NT) {
+      const int y = i & 1, k = i >> 1;
+      const C* s = spec + (int64_t)k * ny + ((y0 + y) & (ny - 1));
+      C xa = s[0], xb = s[(int64_t)KX * ny];
+      if (k == 0 || k == NX / 2) { xa.y = 0; xb.y = 0; }  // C2R ignores these imaginary parts
+      C* row = buf + y * LD;
+      row[k] = mkc<T>(xa.x - xb.y, xa.y + xb.x);
+      if (k > 0 && k < NX / 2) row[NX - k] = mkc<T>(xa.x + xb.y, xb.x - xa.y);
+    }
+  } else {
+    pass_e_unpack<T, NX, 2 * NPR, NT, LD>(buf, spec, W, (int64_t)KX * ny, ny, y0, ny - 1);
+  }
   __syncthreads();
-  smem_fft<T, NX, W * NPR, LD, NT, +1>(buf, a.tw[0]);
+  smem_fft<T, NX, ROWS ? 2 : W * NPR, LD, NT, +1>(buf, a.tw[0]);
   const bool cgm = a.emode == E_CG;
   const T alpha = cgm ? cg_alpha<T>(cg) : (T)0;
   const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
@@ -720,9 +737,15 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
     for (int j = 0; j < W; ++j)
 #pragma unroll
       for (int k = 0; k <= VL; ++k) {
-        const C* w = buf + (j * NPR + pr) * LD + ((x0 + k) & (NX - 1));
-        lo[j][k] = (yy & 1) ? w->y : w->x;
-        hi[j][k] = (yy & 1) ? w[LD].x : w->y;
+        if constexpr (ROWS) {
+          const C* w = buf + ((x0 + k) & (NX - 1));
+          lo[j][k] = j ? w->y : w->x;
+          hi[j][k] = j ? w[LD].y : w[LD].x;
+        } else {
+          const C* w = buf + (j * NPR + pr) * LD + ((x0 + k) & (NX - 1));
+          lo[j][k] = (yy & 1) ? w->y : w->x;
+          hi[j][k] = (yy & 1) ? w[LD].x : w->y;
+        }
       }
 #pragma unroll
     for (int k = 0; k < VL; ++k) {
@@ -857,7 +880,7 @@ cudaError_t launch_a_2d_n(const PassArgs<T>& a, cudaStream_t s) {
 }
 template <typename T, int NX, int TY, int W, bool GRAD = false>
 cudaError_t launch_e_2d_fe_w(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int R = W * (TY / 2 + 1);
+  constexpr int R = TY == 1 ? 2 : W * (TY / 2 + 1);
   constexpr int NT = fft_threads<NX, R>();
   const size_t sm = sizeof(cplx<T>) * R * ae_ld<NX>();
   auto k = pass_e_2d_fe<T, NX, TY, NT, W, GRAD>;
@@ -885,9 +908,17 @@ cudaError_t launch_e_2d_n(const PassArgs<T>& a, cudaStream_t s) {
       if (a.var_e == 1) return launch_e_2d_fe_t<T, NX, tile_rows<T>(1)>(a, s);
       if (a.var_e == 2 && a.n[1] >= tile_rows<T>(2)) return launch_e_2d_fe_t<T, NX, tile_rows<T>(2)>(a, s);
     }
-    // variant 0: half the rows where the default ones leave SMs without a block
-    if ((int64_t)a.n[1] * a.L / tile_rows<T>(0) < device_sm_count()) return launch_e_2d_fe_t<T, NX, tile_rows<T>(1)>(a, s);
-    return launch_e_2d_fe_t<T, NX, tile_rows<T>(0)>(a, s);
+    // variant 0: half the rows where the default ones leave SMs without a block;
+    // one row, on long rows, where every row gets an SM of its own (FP32, bound by
+    // latency: two rows share one; us, FP64 and FP32: 1024 x 16 half the rows
+    // 63.9, 17.2, one row 48.9, 13.6; 512 x 64 44.9, 14.8 and 36.4, 11.8, FP32 with
+    // three load cases 15.1, 13.2)
+    const int64_t rows = (int64_t)a.n[1] * a.L, sms = device_sm_count();
+    if (rows / tile_rows<T>(0) >= sms) return launch_e_2d_fe_t<T, NX, tile_rows<T>(0)>(a, s);
+    if constexpr (NX >= 64) {
+      if (rows <= (sizeof(T) == 4 ? 2 : 1) * sms) return launch_e_2d_fe_t<T, NX, 1>(a, s);
+    }
+    return launch_e_2d_fe_t<T, NX, tile_rows<T>(1)>(a, s);
   }
   if constexpr (NX >= 64) {
     if (a.var_e == 1) return launch_e_2d_t<T, NX, tile_rows<T>(1)>(a, s);

@@ -167,11 +167,13 @@ template <typename T, int NX, int TY> __host__ __device__ constexpr int force_ld
   return FftSplit<NX>::LD + (want - FftSplit<NX>::LD % M + M) % M;
 }
 // Stages of the ring of the strain and edge sources, and their values a thread each.
-template <typename T> __host__ __device__ constexpr int force_stages() { return sizeof(T) == 4 ? 3 : 2; }
+template <typename T, int NX, int TY> __host__ __device__ constexpr int force_stages() {
+  return NX < 64 && TY == 4 ? 6 : sizeof(T) == 4 ? 3 : 2;
+}
 template <int SRC> __host__ __device__ constexpr int force_slots() { return SRC == S_STRAIN ? 18 : SRC == S_EDGE ? 6 : 0; }
 template <int SRC> __host__ __device__ constexpr int force_rows() { return SRC == S_EDGE ? 8 : 3; }   // complex rows per y
 template <typename T, int NX, int TY, int NT, int VL, int SRC> constexpr size_t force_3d_smem() {
-  return sizeof(T) * force_stages<T>() * force_slots<SRC>() * NT * VL +
+  return sizeof(T) * force_stages<T, NX, TY>() * force_slots<SRC>() * NT * VL +
          sizeof(cplx<T>) * force_rows<SRC>() * TY * force_ld<T, NX, TY>() +
          sizeof(T) * 12 * (NX / VL > 32 ? (TY + NT * VL / NX) * (NX / VL / 32) : 0);
 }
@@ -299,7 +301,8 @@ __global__ void __launch_bounds__(NT, MB) force_3d(PassArgs<T> a) {
     // Every thread copies its own values of the next ST - 1 steps into its own
     // slots of the ring (cp.async: no registers are held, and since no thread
     // reads another's slot there is no barrier).
-    constexpr int ST = force_stages<T>();
+    constexpr int ST = force_stages<T, NX, TY>();
+    static_assert(6 % ST == 0, "step t of every row uses slot t % ST");
     const int64_t base = (int64_t)l * a.m * N + (int64_t)z * ny * NX;
     const T* rp = (cgm ? a.r : a.in) + base;
     const T* po = a.pold + base;
@@ -963,6 +966,17 @@ cudaError_t launch_force_3d_n(const PassArgs<T>& a, cudaStream_t s) {
       if (a.var_a == 4) return launch_force_3d_t<T, NX, TY / 2, 2 * NT, VS, S_STRAIN>(a, s);
     }
   }
+  // Short rows: 16 of them are marched as 4 (n_x = 16) or 8 steps one after the
+  // other, so few blocks leave most SMs idle: 8 rows, or 4 in single steps, all
+  // of whose loads are in flight at once (us, 16 rows and 4: 16^3 FP64 68, 32,
+  // FP32 16.6, 11.5; 32 x 16 x 16 FP64 127, 35; 32^3 FP64 127, 63)
+  if constexpr (NX < 64) {
+    const int64_t rows = (int64_t)a.n[1] * a.n[2] * a.L, sms = device_sm_count();
+    if (rows / TY < sms) {
+      if (rows / 8 >= sms) return launch_force_3d_t<T, NX, 8, NT, VS, S_STRAIN>(a, s);
+      return launch_force_3d_t<T, NX, 4, 4 * NX, VS, S_STRAIN>(a, s);
+    }
+  }
   return launch_force_3d_t<T, NX, TY, NT, VS, S_STRAIN>(a, s);
 }
 template <typename T> cudaError_t launch_force_3d(const PassArgs<T>& a, cudaStream_t s) {
@@ -979,24 +993,33 @@ cudaError_t launch_force_2d_t(const PassArgs<T>& a, cudaStream_t s) {
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
   return launch_pass(a.pdl, k, dim3(a.n[1] / TY, a.L), NT, sm, s, a);
 }
-// Threads: at most two rows in a row of steps (TY = 2: one lane per row).
+// Threads: at most two rows in a row of steps (TY <= 2: one lane per row).
 template <int NX, int TY> constexpr int force_threads2() {
-  return NX >= 256 ? 256 : NX >= 128 ? (TY > 2 ? 128 : 256) : NX * (TY > 2 ? (NX == 64 ? 2 : 4) : 2) < 64 ? 64 : NX * (TY > 2 ? (NX == 64 ? 2 : 4) : 2);
+  if (NX >= 256) return 256;
+  if (NX >= 128) return TY > 2 ? 128 : 256;
+  const int t = NX * (TY > 2 ? (NX == 64 ? 2 : 4) : 2);
+  return t < 64 ? 64 : t;
 }
 template <typename T, int NX, int TY, int SRC> cudaError_t launch_force_2d_r(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int NT0 = force_threads2<NX, TY>(), NT = NT0 > NX * TY ? NX * TY : NT0;
   return launch_force_2d_t<T, NX, TY, NT, SRC>(a, s);
 }
 // Default rows: 8 (FP64: 4) where that gives every SM a block, else half, else
-// a quarter.  A tile computes one row more than it owns, so fewer rows mean
-// more work, but on small grids an idle SM costs more (FP64, 512 x 256, one
-// load case: 64 blocks of 4 rows against 128 of 2).  The edge sources have two
-// complex rows per node row: at most half the rows.
+// a quarter; one, on long rows, where every row gets an SM of its own.  A tile
+// computes one row more than it owns, so fewer rows mean more work, but on small
+// grids an idle SM costs more (FP64, 512 x 256, one load case: 64 blocks of 4
+// rows against 128 of 2; with one row, 256 blocks, 193 us a call against 171.
+// FP64, us, two rows and one: 1024 x 16 82, 61, 512 x 64 54, 44, 256 x 64 32,
+// 26).  The edge sources have two complex rows per node row: at most half the
+// rows.
 template <typename T, int NX, int SRC> cudaError_t launch_force_2d_auto(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int TY = sizeof(T) == 4 ? 8 : 4;
   const int64_t sms = device_sm_count(), rows = (int64_t)a.n[1] * a.L;
   if constexpr (force_comps2<SRC>() == 2) {
     if (rows / TY >= sms) return launch_force_2d_r<T, NX, TY, SRC>(a, s);
+  }
+  if constexpr (NX >= 64) {   // (at least two warps a row)
+    if (rows <= sms) return launch_force_2d_r<T, NX, 1, SRC>(a, s);
   }
   if (TY == 4 || rows / (TY / 2) < sms) return launch_force_2d_r<T, NX, 2, SRC>(a, s);
   return launch_force_2d_r<T, NX, TY / 2, SRC>(a, s);
