@@ -175,7 +175,7 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
 /* Schedule of the FFT passes: tile shapes, threads and radix schedules.
  * variants[RVE_SCHED_PASSES] holds
  *  [0] the first pass (material, nodal forces, x FFT): 0 default rows per
- *      block, 1 half, 2 double; with n_x >= 64 also 3 and 4, the same tiles
+ *      block (fewer where they leave SMs idle), 1 half, 2 double; with n_x >= 64 also 3 and 4, the same tiles
  *      with other threads per block; in 3D with RVE_MIXED and n_x >= 128 also 5, a
  *      persistent pipelined pass that transforms every stress component and
  *      whose next tile's rows arrive by bulk copies while the current tile is
@@ -191,6 +191,8 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
  *      split, 1 half N1 and twice N2 (16 = 2 x 8, 32 = 2 x 16, 64 = 4 x 16,
  *      128 = 4 x 32, 256 = 8 x 32; lengths 512 and 1024 have only split 0);
  *  [3] in 3D the same choice for the y transforms (0 or 1); 0 in 2D.
+ * A single operator application has first and last passes of its own, which
+ * [0] and [1] do not change.
  * -1 = choose by timing the candidates on the handle's buffers at the next
  * solve, with that solve's load cases (at most 8) (the default; the choice is
  * cached per grid, precision, number of load cases timed, operator form and
@@ -368,9 +370,10 @@ int rve_batch_effective_tangent(rve_batch_t b, int index, double* C);
  * state record with a small kernel; make that first call before any stream
  * capture.  Later calls copy nothing from the host and are three launches.  All
  * calls share the array and it keeps the contents of the last call (each call
- * rewrites the spectrum it reads), so calls that overlap on the GPU -- on different streams, or from
- * different host threads -- race; serialise them.  Not usable after
- * cudaDeviceReset on that device.  Returns without waiting for the GPU. */
+ * rewrites the spectrum it reads), so calls that overlap on the GPU -- on
+ * different streams, or from different host threads -- race; serialise them.
+ * Not usable after cudaDeviceReset on that device.  Returns without waiting for
+ * the GPU. */
 int rve_apply_operator_2d_static(const int64_t* n, const double* length, const float* E, double nu,
                                  const float* p, float* q, int apply_material, void* cuda_stream);
 

@@ -326,7 +326,7 @@ class RVE:
         return out
 
     # kind 7: the first pass (with its x transform) of the factored and nodal forms,
-    # and the material kernel of finite strain; kind 8 is not used any more
+    # and the material kernel of finite strain; kind 8 is never recorded
     KINDS = ("pass_a", "pass_b", "pass_c", "pass_d", "pass_e", "residual", "other", "force_stencil",
              "strain_update")
 

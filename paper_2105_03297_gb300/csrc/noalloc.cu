@@ -49,8 +49,8 @@ std::atomic<bool> g_tables_written[kMaxDevices];
 // every length, and the CG-state record (active, everything else zero; no mode
 // of this entry point changes it), written on the device at set-up.  sincospi
 // is CUDA's own FP64 function; its results are rounded to FP32 like the host
-// tables of the handle path.  They used to be rewritten by every call: without
-// that launch a 64 x 64 call is three launches instead of four.
+// tables of the handle path.  Written by every call they would be a fourth
+// launch beside the three of a 64 x 64 call.
 __global__ void fill_static_tables(float2* tables, CgState* cg) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kTableLen; i += gridDim.x * blockDim.x) {
     int n = 16;

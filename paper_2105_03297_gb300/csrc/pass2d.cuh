@@ -11,9 +11,11 @@
 //      and <r, r> (q never touches memory).  x += alpha p of iteration k is
 //      deferred to pass A of iteration k+1, which reads p anyway (one vector
 //      stream less per iteration); cg_finish_x applies the last one.
-// The other derivatives and finite strain carry all their components through C
-// (with the projection) and E.  Measured at 1024^2, three load cases, FP32, us
-// per iteration: all six components through A 113, C 80 and E 85, now A 108, C 35 and E 61.
+// The other derivatives, and the operator on finite-strain fields, carry all
+// their components through C (with the projection) and E; the Newton steps of
+// finite strain take the D nodal ones.  Measured at 1024^2, three load cases,
+// FP32, us per iteration: all six components through A 113, C 80 and E 85, the
+// nodal ones A 108, C 35 and E 61.
 // DFT convention of Appendix A; the 1/N of the inverse is applied in pass C.
 // Two real rows (y, y+1) share one complex FFT (X_y + i X_{y+1}).
 #pragma once
@@ -362,9 +364,9 @@ __device__ __forceinline__ void publish_rr(const PassArgs<T>& a, CgState* cg, co
 // Pass C of the finite elements: w^ = (B^H B)^-1 t^ for P k_x columns per
 // block, from t(k_x, y) in components 0 and 1 of the spectrum (pass A or the
 // force pass) to w(k_x, y) in place.  Bound by the FFT arithmetic (80
-// registers at 512 and 1024 points: six blocks of four warps per SM; at 150
-// registers and three blocks the 1024^2 pass took 65 us, now 48 with the
-// combination of all six components it then still did).
+// registers at 512 and 1024 points: six blocks of four warps per SM; with the
+// six stress components still read and combined here, 1024^2 took 65 us at 150
+// registers and three blocks, 48 at 80 and six).
 // W = 4 (P = 1) reads the edge sums s_aj in components 2 a + j (S_EDGE of
 // pass_force.cuh), t_j = sum_a conj(d_a) s_aj, d_a = (exp(i k_a h_a) - 1)/h_a,
 // and writes the differences d_a w_j along the element edges there: the last

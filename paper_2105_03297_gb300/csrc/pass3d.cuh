@@ -17,8 +17,8 @@
 // The other derivatives (one evaluation point) and finite strain carry all
 // their components through B, C (with the projection), D and E.
 // Measured at 256 x 256 x 64, one load case, FP32, us per iteration: all 36
-// components through every pass A 656, B 168, C 371, D 184, E 388; now A 622,
-// B 38, C 50, D 28, E 289.
+// components through every pass A 656, B 168, C 371, D 184, E 388; the nodal
+// ones A 622, B 38, C 50, D 28, E 289.
 #pragma once
 #include "pass2d.cuh"
 #include "pass3d_pipe.cuh"
@@ -594,8 +594,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pas
 // In FP32 the r loads of the update go through a ring of the thread's own
 // shared-memory slots (cp.async, six tetrahedra deep): issued before the
 // spectrum is unpacked, they keep DRAM busy during the transforms, and in the
-// update every store no longer waits for the loads behind it (us per iteration,
-// without and with: 256 x 256 x 64 309, 289; 128^3 156, 149; 64^3, six load
+// update no store waits for the loads behind it (us per iteration, without and
+// with: 256 x 256 x 64 309, 289; 128^3 156, 149; 64^3, six load
 // cases 147, 114).
 template <typename T, int NT, int W> __host__ __device__ constexpr bool e_fe_ring() {
   return sizeof(T) == 4 && W == 3 && NT <= 256;   // else it does not fit beside the rows
@@ -824,7 +824,7 @@ cudaError_t launch_e_3d_fe_t(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int R = e_fe_rows<W, TY>();
   constexpr int NT = fft_threads<NX, R>();
   constexpr size_t sm = sizeof(cplx<T>) * R * e_fe_ld<NX>() + (e_fe_ring<T, NT, W>() ? sizeof(T) * 36 * (NX >= 256 ? 2 : 1) * NT : 0);
-    constexpr int MB = sizeof(T) == 8 ? 1 : W == 9 ? (NT <= 448 ? 2 : 1) : NT <= 256 ? (NX >= 256 ? 2 : 4) : NT <= 448 ? 2 : 1;
+  constexpr int MB = sizeof(T) == 8 ? 1 : W == 9 ? (NT <= 448 ? 2 : 1) : NT <= 256 ? (NX >= 256 ? 2 : 4) : NT <= 448 ? 2 : 1;
   auto k = pass_e_3d_fe<T, NX, TY, NT, MB, W>;
   static DeviceOnce attr;
   attr.run(current_device(), [&] { set_smem_attrs(k, sm); });
@@ -898,13 +898,12 @@ cudaError_t launch_y_3d_v(const PassArgs<T>& a, cudaStream_t s) {
   } else {
     return launch_pass(a.pdl, k, grid, NT, sm, s, a, Cc);
   }
-  return cudaGetLastError();
 }
 // Pass B of the finite elements from all components (forward).
 template <typename T, int NY, int V>
 cudaError_t launch_b_3d_fe(const PassArgs<T>& a, cudaStream_t s) {
   constexpr int TZB = Tile3D<T>::TZB;
-    constexpr int NT = NY >= 128 ? NY : 128;
+  constexpr int NT = NY >= 128 ? NY : 128;
   constexpr size_t sm = sizeof(cplx<T>) * (3 * TZB * FftSplit<NY, V>::LDO + 3 * TZB * (NY > 32 ? NY / 32 : 1));
   auto k = pass_b_3d_fe<T, NY, TZB, NT, V>;
   static DeviceOnce attr;
