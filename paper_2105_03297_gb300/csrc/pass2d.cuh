@@ -673,27 +673,27 @@ __device__ __forceinline__ T strain_update(const PassArgs<T>& a, int64_t idx, T*
 }
 
 // Last pass of the finite elements: from w(k_x, y) of the two nodal components
-// (pass C) the inverse x FFT of rows y0 .. y0 + TY + 1 (two rows per complex
-// transform; the row past the tile and its partner complete the last pair),
-// then in real space the strains q = B w of both triangles of every pixel of
-// the TY rows and the update of all six components.  Transforming w instead of
-// the strains needs TY + 2 row pairs where the components need 3 TY, and reads
-// a third of the spectrum.  Bound by the r traffic (read and write, 16-byte
-// accesses).  W = 4: the spectrum holds the edge differences of w instead (see
-// pass_c_2d_fe).  TY = 1 (few rows): w_0 and w_1 of a row share a transform, two
-// rows, where a pair of rows beside the tile's would be half unused.
-// grid (n_y/TY, L).
+// (pass C) the inverse x FFT of rows y0 .. y0 + TY, then in real space the
+// strains q = B w of both triangles of every pixel of the TY rows and the update
+// of all six components.  Transforming w instead of the strains needs TY + 1
+// complex transforms where the components need 3 TY, and reads a third of the
+// spectrum.  Bound by the r traffic (read and write, 16-byte accesses).  w_0 and
+// w_1 of a row share a transform, so that a node's values are rounded alike in
+// every tile that uses them, whatever its height.
+// W = 4: the spectrum holds the edge differences of w instead (see
+// pass_c_2d_fe); two rows of a component share a transform (the row past the
+// tile and its partner complete the last pair).  grid (n_y/TY, L).
 template <typename T, int NX, int TY, int NT, int W, bool GRAD = false>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pass_e_2d_fe(PassArgs<T> a) {
   using C = cplx<T>;
-  constexpr bool ROWS = TY == 1;
-  static_assert(!ROWS || W == 2, "single rows: the two components of w");
-  constexpr int NPR = TY / 2 + 1;
+  constexpr bool ROWS = W == 2;
+  static_assert(ROWS || TY > 1, "pairs of rows");
+  constexpr int NPR = TY / 2 + 1, NR = TY + 1;
   constexpr int KX = NX / 2 + 1;
   constexpr int LD = ae_ld<NX>();
   constexpr int VL = sizeof(T) == 4 ? 4 : 1;   // FP64: more, shorter work items
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);  // [W][NPR][LD]; ROWS: [2 rows][LD]
+  C* buf = reinterpret_cast<C*>(smem_raw);  // W = 2: [NR][LD]; W = 4: [W][NPR][LD]
   __shared__ double red[NT / 32];
   __shared__ T cols[NT];
   __shared__ int flag;
@@ -705,20 +705,45 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
   if (a.cgphase && cg->status != ST_RUN) return;
   const C* spec = a.spec + (int64_t)l * a.m * KX * ny;
   if constexpr (ROWS) {
-    for (int i = threadIdx.x; i < 2 * KX; i += NT) {
-      const int y = i & 1, k = i >> 1;
-      const C* s = spec + (int64_t)k * ny + ((y0 + y) & (ny - 1));
-      C xa = s[0], xb = s[(int64_t)KX * ny];
-      if (k == 0 || k == NX / 2) { xa.y = 0; xb.y = 0; }  // C2R ignores these imaginary parts
-      C* row = buf + y * LD;
-      row[k] = mkc<T>(xa.x - xb.y, xa.y + xb.x);
-      if (k > 0 && k < NX / 2) row[NX - k] = mkc<T>(xa.x + xb.y, xb.x - xa.y);
+    // items of YL rows of both components at one k_x (TY > 1: 16-byte loads; the
+    // last one's second row is not needed), UB items in flight
+    constexpr int YL = TY > 1 ? 2 : 1, NI = TY / YL + 1, TOT = KX * NI, UB = 8 / YL;
+    for (int i0 = threadIdx.x; i0 < TOT; i0 += UB * NT) {
+      C va[UB][YL], vb[UB][YL];
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int i = i0 + u * NT;
+        if (i < TOT) {
+          const C* s = spec + (int64_t)(i / NI) * ny + ((y0 + YL * (i % NI)) & (ny - 1));
+          if constexpr (YL == 2) {
+            cload2<T>(va[u], s);
+            cload2<T>(vb[u], s + (int64_t)KX * ny);
+          } else {
+            va[u][0] = s[0];
+            vb[u][0] = s[(int64_t)KX * ny];
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UB; ++u) {
+        const int i = i0 + u * NT, k = i / NI;
+#pragma unroll
+        for (int h = 0; h < YL; ++h) {
+          const int y = YL * (i % NI) + h;
+          if (i >= TOT || y >= NR) continue;
+          C xa = va[u][h], xb = vb[u][h];
+          if (k == 0 || k == NX / 2) { xa.y = 0; xb.y = 0; }  // C2R ignores these imaginary parts
+          C* row = buf + y * LD;
+          row[k] = mkc<T>(xa.x - xb.y, xa.y + xb.x);                                  // X_0 + i X_1
+          if (k > 0 && k < NX / 2) row[NX - k] = mkc<T>(xa.x + xb.y, xb.x - xa.y);    // conj(X_0) + i conj(X_1)
+        }
+      }
     }
   } else {
     pass_e_unpack<T, NX, 2 * NPR, NT, LD>(buf, spec, W, (int64_t)KX * ny, ny, y0, ny - 1);
   }
   __syncthreads();
-  smem_fft<T, NX, ROWS ? 2 : W * NPR, LD, NT, +1>(buf, a.tw[0]);
+  smem_fft<T, NX, ROWS ? NR : W * NPR, LD, NT, +1>(buf, a.tw[0]);
   const bool cgm = a.emode == E_CG;
   const T alpha = cgm ? cg_alpha<T>(cg) : (T)0;
   const T ihx = a.ih[0], ihy = a.ih[1], r2 = (T)kInvSqrt2;
@@ -732,15 +757,15 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 2 : 1) pas
 #pragma unroll
       for (int c = 0; c < NC; ++c) vloadn<T, VL>(rv[c], a.r + v0 + c * a.N);
     }
-    // node rows yy and yy + 1 at columns x0 .. x0 + VL: rows 2 pr and 2 pr + 1
-    // are the two parts of pair pr
+    // node rows yy and yy + 1 at columns x0 .. x0 + VL (W = 4: rows 2 pr and
+    // 2 pr + 1 are the two parts of pair pr)
     T lo[W][VL + 1], hi[W][VL + 1];
 #pragma unroll
     for (int j = 0; j < W; ++j)
 #pragma unroll
       for (int k = 0; k <= VL; ++k) {
         if constexpr (ROWS) {
-          const C* w = buf + ((x0 + k) & (NX - 1));
+          const C* w = buf + yy * LD + ((x0 + k) & (NX - 1));
           lo[j][k] = j ? w->y : w->x;
           hi[j][k] = j ? w[LD].y : w[LD].x;
         } else {
@@ -882,7 +907,7 @@ cudaError_t launch_a_2d_n(const PassArgs<T>& a, cudaStream_t s) {
 }
 template <typename T, int NX, int TY, int W, bool GRAD = false>
 cudaError_t launch_e_2d_fe_w(const PassArgs<T>& a, cudaStream_t s) {
-  constexpr int R = TY == 1 ? 2 : W * (TY / 2 + 1);
+  constexpr int R = W == 2 ? TY + 1 : W * (TY / 2 + 1);
   constexpr int NT = fft_threads<NX, R>();
   const size_t sm = sizeof(cplx<T>) * R * ae_ld<NX>();
   auto k = pass_e_2d_fe<T, NX, TY, NT, W, GRAD>;
