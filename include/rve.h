@@ -195,9 +195,9 @@ int rve_apply_operator(rve_t h, const void* p, void* q, int apply_material, int 
  * [0] and [1] do not change.
  * -1 = choose by timing the candidates on the handle's buffers at the next
  * solve, with that solve's load cases (at most 8) (the default; the choice is
- * cached per grid, precision, number of load cases timed, operator form and
- * derivative for the process, and made again after a change of form or
- * derivative).  rve_set_schedule rejects a variant the grid does not have.
+ * cached per grid, precision, number of load cases timed, kernels of the
+ * operator form and derivative for the process, and looked up or made again
+ * after a change of form or derivative).  rve_set_schedule rejects a variant the grid does not have.
  * rve_schedule also returns the measured candidate times
  * candidate_ms[RVE_SCHED_PASSES][RVE_SCHED_VARIANTS] (0 where a candidate does
  * not exist, runs as another one or was not timed; where variant 5 of the first

@@ -498,13 +498,13 @@ int write_state(rve_s* h, int L) {
 // the first pass is timed together with pass B, which then has 36 components to
 // read instead of two force spectra (256 x 256 x 64: 168 against 38 us).
 // Choices are cached for the process per grid, precision, load cases timed,
-// operator form and derivative: the variants of the form's or derivative's own
-// kernels are not those of another.
+// kernels of the operator form (the strain forms share them, but for A 5) and
+// derivative: the variants of one's kernels are not those of another.
 struct TuneKey {
-  int dim, n0, n1, n2, tsize, nl, form, deriv;
+  int dim, n0, n1, n2, tsize, nl, route, deriv;
   bool operator<(const TuneKey& o) const {
-    return std::tie(dim, n0, n1, n2, tsize, nl, form, deriv) <
-           std::tie(o.dim, o.n0, o.n1, o.n2, o.tsize, o.nl, o.form, o.deriv);
+    return std::tie(dim, n0, n1, n2, tsize, nl, route, deriv) <
+           std::tie(o.dim, o.n0, o.n1, o.n2, o.tsize, o.nl, o.route, o.deriv);
   }
 };
 std::map<TuneKey, std::array<int, RVE_SCHED_PASSES>> g_tuned;
@@ -548,7 +548,9 @@ constexpr int kTuneMaxL = 8;
 
 template <typename T> int autotune(rve_s* h, int L) {
   const int Lt = L < 1 ? 1 : (L > kTuneMaxL ? kTuneMaxL : L);
-  const TuneKey key{h->dim, h->n[0], h->n[1], h->n[2], (int)h->tsize, Lt, h->op_form, h->deriv};
+  // nodal state; strain forms; those with candidate A 5, and the other derivatives
+  const int route = h->op_form == RVE_FORM_NODAL ? 2 : force_pass(h, 5) ? 1 : 0;
+  const TuneKey key{h->dim, h->n[0], h->n[1], h->n[2], (int)h->tsize, Lt, route, h->deriv};
   auto choose = [&](const std::array<int, RVE_SCHED_PASSES>& c) {
     for (int w = 0; w < RVE_SCHED_PASSES; ++w)
       if (h->var[w] < 0) { h->var[w] = c[w]; h->tuned |= 1u << w; }
