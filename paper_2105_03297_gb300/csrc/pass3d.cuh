@@ -18,7 +18,7 @@
 // their components through B, C (with the projection), D and E.
 // Measured at 256 x 256 x 64, one load case, FP32, us per iteration: all 36
 // components through every pass A 656, B 168, C 371, D 184, E 388; the nodal
-// ones A 622, B 38, C 50, D 28, E 289.
+// ones A 622, B 38, C 50, D 28, E 297.
 #pragma once
 #include "pass2d.cuh"
 #include "pass3d_pipe.cuh"
@@ -595,8 +595,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 && NT <= 384) ? 3 : 1) pas
 // shared-memory slots (cp.async, six tetrahedra deep): issued before the
 // spectrum is unpacked, they keep DRAM busy during the transforms, and in the
 // update no store waits for the loads behind it (us per iteration, without and
-// with: 256 x 256 x 64 309, 289; 128^3 156, 149; 64^3, six load
-// cases 147, 114).
+// with, taken with the planes paired: 256 x 256 x 64 309, 289; 128^3 156, 149;
+// 64^3, six load cases 147, 114.  Paired within a plane: 297, 154, 115).
 template <typename T, int NT, int W> __host__ __device__ constexpr bool e_fe_ring() {
   return sizeof(T) == 4 && W == 3 && NT <= 256;   // else it does not fit beside the rows
 }
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(NT, MB) pass_e_3d_fe(PassArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);  // W = 3: [2][NR] rows (w_0, w_1), [2][NP] pairs of w_2; 9: [W][NR]
   __shared__ double red[NT / 32];
-  __shared__ T cols[NT];
+  __shared__ T cols[sizeof(T) == 4 ? NT / 16 : NT];   // (1 KB less holds a fourth block at n_x = 128)
   __shared__ int flag;
   const int l = blockIdx.z, z = blockIdx.y, y0 = blockIdx.x * TY;
   const int ny = a.n[1], nz = a.n[2];

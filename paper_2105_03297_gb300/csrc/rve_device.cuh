@@ -746,7 +746,8 @@ template <typename T> struct Acc {
 // Block sum of such pairs (valid in thread 0).  FP32: every warp adds its lanes
 // as two-sum pairs, so the FP64 pipe (16 cycles per warp instruction) sees only
 // one pair per warp; FP64: block_sum_cols.
-template <int NT, typename T> __device__ __forceinline__ double block_sum_acc(const Acc<T>& v, T* cols /*[NT]*/) {
+template <int NT, typename T>
+__device__ __forceinline__ double block_sum_acc(const Acc<T>& v, T* cols /*[FP32: NT / 16, FP64: NT]*/) {
   if constexpr (sizeof(T) == 4) {
     T hi = v.hi, lo = v.lo;
 #pragma unroll
